@@ -143,7 +143,8 @@ def hbm_peak():
 # the sources that define the planned-plan kernels' device code (and the
 # launch shapes chosen for them); host-only files do not change the counters
 KERNEL_SOURCES = ("common.cuh", "fft.cuh", "fft_fixed.cuh", "search_common.cuh",
-                  "search_fixed.cu", "search_fixed.h", "tma.cuh")
+                  "search_fixed.cu", "search_fixed.cuh", "search_fixed.h", "search_fixed_256.cu",
+                  "search_fixed_720.cu", "search_fixed_1080.cu", "search_fixed_2160.cu", "tma.cuh")
 
 
 def csrc_digest():

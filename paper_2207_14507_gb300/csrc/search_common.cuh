@@ -1,5 +1,5 @@
 // search_common.cuh -- device helpers shared by the wave kernels (search.cu),
-// the compile-time-planned kernels and the persistent kernel (search_fixed.cu).
+// the compile-time-planned kernels and the persistent kernel (search_fixed.cuh).
 #pragma once
 #include <float.h>
 #include <limits.h>

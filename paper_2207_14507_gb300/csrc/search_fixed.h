@@ -1,10 +1,19 @@
-// search_fixed.h -- registry of the compile-time-planned kernels (search_fixed.cu).
+// search_fixed.h -- registry of the compile-time-planned kernels (search_fixed.cuh).
 #pragma once
 #include <vector>
 
 #include "internal.h"
 
 namespace prnu {
+
+// Rows per TMA box of an H-row strip of NC columns (float2): a divisor of H of
+// at most 256 rows whose box size is a multiple of 128 bytes, so that every
+// box lands 128-byte aligned in shared memory.
+__host__ __device__ constexpr int tma_box_rows(int H, int NC, int esize = 8) {
+  for (int br = 256; br >= 1; --br)
+    if (H % br == 0 && (br * NC * esize) % 128 == 0) return br;
+  return 0;
+}
 
 // one instantiated column-pass variant: columns per block, threads, shared
 // memory; with tma the kernel moves its strip by TMA tile copies of br rows
@@ -73,6 +82,12 @@ struct FixedShape {
     return rows.front();
   }
 };
+
+// one frame size's instantiated kernels each
+FixedShape fixed_shape_256();
+FixedShape fixed_shape_720();
+FixedShape fixed_shape_1080();
+FixedShape fixed_shape_2160();
 
 // The instantiated kernels for frames of H x W, or nullptr.
 const FixedShape* find_fixed(int H, int W);
