@@ -168,10 +168,11 @@ Tuning tuning_for(prnu_ctx* c, int H, int W) {
   // the planned kernels run one row pair per block best; waves of up to 1024
   // candidates (up to 16 GB of spectra) amortise the per-wave finalisation and
   // tail: 1024 against 512 gains 0.7% at 1080p, 512 against 129 1% at 4K
-  t.ppb = find_fixed(H, W) ? 1 : 2;
+  const FixedShape* fs = find_fixed(H, W);
+  t.ppb = fs ? 1 : 2;
   // sizes without compile-time-planned kernels run the generic ones (-1), so
   // that what prnu_get_tuning reports is accepted by prnu_set_tuning
-  t.variant = find_fixed(H, W) ? 0 : -1;
+  t.variant = fs ? fs->default_col : -1;
   // within a quarter of the context's HBM budget (spectra and row statistics)
   const size_t per_item = (size_t)H * (W / 2) * sizeof(float2) + (size_t)H * sizeof(RowStat);
   t.wave = (int)std::max<size_t>(1, std::min<size_t>((size_t)default_wave(H, W), c->budget / 4 / per_item));

@@ -1,0 +1,318 @@
+// col_pass.cuh -- the column pass of the compile-time-planned kernels: forward
+// column FFT, product with the fingerprint's spectrum, inverse column FFT of a
+// strip of NC columns of one candidate's packed half spectrum.
+//
+// The transform of H = RA * RB points takes two stages each way, one thread
+// per column and butterfly, a whole radix-RA or radix-RB butterfly in its
+// registers (30 to 48 points): the strip crosses shared memory 6 times (plus
+// the fingerprint's once) where three stages with two columns per thread
+// crossed it 10 times.  Those were bound by the L1 data pipe
+// (67% of its peak, a quarter of it bank conflicts and spilled registers) and
+// by the barriers between its stages.  At 1080p FP32 (ncu, 64 candidates):
+// 3.5 M -> 2.3 M warp instructions a candidate, L1 data pipe 67% -> 49%, L1 hit
+// rate of the twiddles 49% -> 99%, 5.38 -> 4.25 us a candidate.  What bounds it
+// now is latency: 13.5 warps per SM (registers and the strips' shared memory),
+// no unit above 50%.  Each size's variants and their times stand at its
+// registry entry (search_fixed_<rows>.cu).
+//
+//   stage A : butterfly j < RB reads x[j + r RB], r < RA; writes j RA + r
+//   stage B : butterfly j < RA reads x[j + r RA], r < RB, twiddle w_H^(rj);
+//             leaves bins j + r RA in its registers
+//   product : with the fingerprint's bins j + r RA
+//   inverse stage B: the same thread's bins; writes j RB + r
+//   inverse stage A: butterfly j < RB reads x[j + r RB], twiddle w_H^(-rj);
+//             leaves rows j + r RB
+//
+// Between two stages the strip lies in rows of NC elements in groups of RA
+// (RB) rows at an odd pitch LA (LB), so that the threads of a warp, which hold
+// consecutive j and columns, store to distinct banks; TMA's side of the strip
+// is dense.  Every shared address is a per-thread base plus a constant.
+#pragma once
+#include "common.cuh"
+#include "fft_fixed.cuh"
+#include "fft_packed.cuh"
+#include "search_common.cuh"
+#include "search_fixed.h"
+#include "tma.cuh"
+
+namespace prnu {
+
+namespace {
+
+template <int H_, int RA_, int RB_>
+struct ColPlan {
+  static constexpr int H = H_, RA = RA_, RB = RB_;
+  static constexpr int LA = RA | 1, LB = RB | 1;
+  static constexpr int rows = RB * LA > RA * LB ? RB * LA : RA * LB;   // of the strip buffer
+  static constexpr int lanes = RA > RB ? RA : RB;                      // threads per column
+  static_assert(RA * RB == H, "two radices");
+};
+
+// The product for the packed column 0 (DC + i*Nyquist columns of two real
+// spectra in one complex column): F, Fm the frame bins i and H - i, S, Sm the
+// fingerprint bins; unpack both, conj-multiply each real column's spectrum,
+// repack.
+__device__ __forceinline__ float2 packed_col0_product(float2 F, float2 Fm, float2 S, float2 Sm) {
+  const float2 Aa = make_float2(0.5f * (F.x + Fm.x), 0.5f * (F.y - Fm.y));
+  const float2 Bb = make_float2(0.5f * (F.y + Fm.y), 0.5f * (Fm.x - F.x));
+  const float2 Ka = make_float2(0.5f * (S.x + Sm.x), 0.5f * (S.y - Sm.y));
+  const float2 Kb = make_float2(0.5f * (S.y + Sm.y), 0.5f * (Sm.x - S.x));
+  const float2 p1 = c_conj_mul(Aa, Ka), p2 = c_conj_mul(Bb, Kb);
+  return make_float2(p1.x - p2.y, p1.y + p2.x);
+}
+
+// bytes per fingerprint bin of the separate fingerprint region (MODE 3: FP32
+// or FP16 bins; MODE 4: FP16 bins only)
+__host__ __device__ constexpr int fp_region_bin(int mode) { return mode == 3 ? 8 : mode == 4 ? 4 : 0; }
+// the strip buffer, 128-byte aligned; then MODE 2: the two packed column-0
+// scratch columns, MODE 3 and 4: the fingerprint strip
+template <class CP>
+__host__ __device__ constexpr size_t col_buf_bytes(int nc) {
+  return ((size_t)CP::rows * nc * sizeof(float2) + 127) / 128 * 128;
+}
+template <class CP>
+__host__ __device__ constexpr size_t col_pass_smem(int nc, int mode) {
+  return col_buf_bytes<CP>(nc) + (mode == 2 ? 2 * (size_t)CP::H * sizeof(float2) : (size_t)CP::H * nc * fp_region_bin(mode));
+}
+constexpr long long kTmaWaitPolls = 1ll << 20;   // polls of mbarrier.try_wait before giving up
+
+// Every thread of the block: wait for phase `ph` of `bar`; on a wait that
+// runs out anywhere the error flag goes up, the copies get one more bounded
+// wait to land (and those of bar2), and false comes back to all.  Holds a
+// barrier.
+__device__ __forceinline__ bool block_wait(uint64_t* bar, uint32_t ph, int* err, uint64_t* bar2 = nullptr) {
+  const bool ok = mbar_wait_bounded(bar, ph, kTmaWaitPolls);
+  if (__syncthreads_or(!ok)) {
+    if (threadIdx.x == 0) {
+      if (err) atomicExch(err, 1);
+      mbar_wait_bounded(bar, ph, kTmaWaitPolls);
+      if (bar2) mbar_wait_bounded(bar2, 0, kTmaWaitPolls);
+    }
+    __syncthreads();
+    return false;
+  }
+  return true;
+}
+
+// the fingerprint's strip by TMA to shared memory at dst, completing on bar
+template <int H, int NC>
+__device__ __forceinline__ void load_fp_strip(const FpDesc& fp, int c0, char* dst, uint64_t* bar) {
+  const CUtensorMap* fm = reinterpret_cast<const CUtensorMap*>(fp.tmaps) + fp_tmap_index(NC);
+  const int es = fp.dtype == kF32 ? 8 : 4, br = tma_box_rows(H, NC, es);
+  asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"(reinterpret_cast<uint64_t>(fm))
+               : "memory");
+  mbar_expect_tx(bar, H * NC * es);
+#pragma unroll 1
+  for (int b = 0; b < H / br; ++b) tma_load_2d(dst + (size_t)b * br * NC * es, fm, 2 * c0, b * br, bar);
+}
+
+// Columns bx*NC .. bx*NC+NC-1 of candidate `is` in workspace slot `ws`, by
+// T >= NC * CP::lanes threads.
+// MODE 0: every thread loads and stores its own elements.  MODE >= 1: the
+// strip comes into shared memory by TMA tile copies through `map` (the
+// workspace spectra as a [slots*H][W] float tensor) and leaves the same way.
+// MODE 2: the fingerprint strip too comes by TMA, into the strip buffer once
+// stage B has taken its inputs (the packed column-0 scratch then sits after
+// the buffer).  MODE 3 and 4: the fingerprint strip comes by TMA into its own
+// region after the strip buffer, copied from the start together with the
+// strip (MODE 4 sizes the region for FP16 bins: FP32 fingerprints are then
+// loaded per thread).  A TMA wait that runs out raises a.err and abandons the
+// candidate.
+// PART splits the pass for forward units (candidates that share a frame and
+// a grid node): PART 1 runs the forward column FFT only and stores its
+// output, in natural order, back to slot ws; PART 2 loads that output from
+// slot src_ws and runs the product and the inverse FFT into slot ws.  PART 1
+// then PART 2 compute bit for bit what PART 0 (the whole pass) computes.
+// PART 1 and 2 need TMA (MODE >= 1); PART 2 takes MODE >= 2.
+// PFD > 0: each block also asks for the strip PFD strips on (of the wave's
+// slots) to be brought into L2; PART 0 only.
+template <class CP, int W, int NC, int MODE = 0, int PART = 0, int PFD = 0>
+__device__ __forceinline__ void col_body(const PassArgs& a, int is, int ws, int bx, float2* sm,
+                                         const CUtensorMap* map = nullptr, int src_ws = -1) {
+  constexpr bool TMA = MODE >= 1, FPT = MODE >= 2 && PART != 1, FPSEP = MODE >= 3 && PART != 1;
+  static_assert(PFD == 0 || (TMA && PART == 0), "prefetches go with the whole pass by TMA");
+  static_assert(PART == 0 || TMA, "the split column pass moves its strips by TMA");
+  constexpr int H = CP::H, Wh = W / 2, RA = CP::RA, RB = CP::RB, LA = CP::LA, LB = CP::LB;
+  static_assert(Wh % NC == 0, "strips tile the half spectrum");
+  if (src_ws < 0) src_ws = ws;
+  const int t = threadIdx.x, c = t % NC, j = t / NC;
+  const bool act_a = j < RB, act_b = j < RA;
+  const int c0 = bx * NC, col = c0 + c;
+  const WorkItem wi = item_of(a, is);
+  const FpDesc fp = a.fps[wi.fp];
+  char* const fpsm = reinterpret_cast<char*>(sm) + (FPSEP ? col_buf_bytes<CP>(NC) : 0);
+
+  constexpr int BR = tma_box_rows(H, NC);
+  __shared__ uint64_t s_bar, s_fbar;
+  const int fes = fp.dtype == kF32 ? 8 : 4;
+  // the fingerprint strip comes by TMA (boxes of at least 16 bytes; MODE 3/4:
+  // a region sized for its bins), else by per-thread loads
+  const bool fp_tma = FPT && fp.tmaps != nullptr && NC * fes >= 16 && (!FPSEP || fes <= fp_region_bin(MODE));
+  if constexpr (TMA) {
+    static_assert(BR > 0, "no TMA box for this strip");
+    if (t == 0) {
+      mbar_init(&s_bar, 1);
+      if (FPT) mbar_init(&s_fbar, 1);
+      fence_mbar_init();
+    }
+    __syncthreads();
+    if (t == 0) {
+      mbar_expect_tx(&s_bar, H * NC * 8 + (a.stall ? 16 : 0));   // the test hook waits for bytes that never come
+#pragma unroll 1
+      for (int b = 0; b < H / BR; ++b) tma_load_2d(sm + b * BR * NC, map, 2 * c0, src_ws * H + b * BR, &s_bar);
+      if (FPSEP && fp_tma) load_fp_strip<H, NC>(fp, c0, fpsm, &s_fbar);
+      if constexpr (PFD > 0) {   // the strip PFD strips on, into L2
+        const int n = is * (Wh / NC) + bx + PFD, s2 = n / (Wh / NC), b2 = n - s2 * (Wh / NC);
+        if (s2 < a.nitems) {
+#pragma unroll 1
+          for (int b = 0; b < H / BR; ++b) tma_prefetch_2d(map, 2 * b2 * NC, s2 * H + b * BR);
+        }
+      }
+    }
+    if (!block_wait(&s_bar, 0, a.err, FPSEP && fp_tma ? &s_fbar : nullptr)) return;
+  }
+
+  float2* Z = a.spec + (size_t)ws * H * Wh;
+  float2 v[1][RB];   // bins j + r RA
+  if constexpr (PART != 2) {
+    {
+      float2 u[RA];
+      if (act_a) {
+        if constexpr (TMA) {
+          const float2* src = sm + j * NC + c;
+#pragma unroll
+          for (int r = 0; r < RA; ++r) u[r] = src[r * RB * NC];
+        } else {
+          const float2* src = Z + (size_t)j * Wh + col;
+#pragma unroll
+          for (int r = 0; r < RA; ++r) u[r] = __ldg(src + (size_t)r * RB * Wh);
+        }
+      }
+      if constexpr (TMA) __syncthreads();
+      if (act_a) {
+        DftP<RA, false>::run(u);
+        float2* dst = sm + j * LA * NC + c;
+#pragma unroll
+        for (int r = 0; r < RA; ++r) dst[r * NC] = u[r];
+      }
+    }
+    __syncthreads();
+    if (act_b) {
+      const float2* src = sm + j * NC + c;
+#pragma unroll
+      for (int r = 0; r < RB; ++r) v[0][r] = src[r * LA * NC];
+    }
+  } else if (act_b) {
+    const float2* src = sm + j * NC + c;
+#pragma unroll
+    for (int r = 0; r < RB; ++r) v[0][r] = src[r * RA * NC];
+  }
+  if constexpr (FPT && !FPSEP) {   // the strip buffer is free: the fingerprint's strip goes there
+    if (fp_tma) {
+      fence_proxy_async_smem();
+      __syncthreads();
+      if (t == 0) load_fp_strip<H, NC>(fp, c0, fpsm, &s_fbar);
+    }
+  }
+  if constexpr (PART != 2) {
+    if (act_b) {
+      twiddle_tab<RB, RA, false, 1>(v, j);
+      DftP<RB, false>::run(v[0]);
+    }
+  }
+
+  if constexpr (PART == 1) {
+    __syncthreads();
+    if (act_b) {
+      float2* dst = sm + j * NC + c;
+#pragma unroll
+      for (int r = 0; r < RB; ++r) dst[r * RA * NC] = v[0][r];
+    }
+  } else {
+    // fingerprint bin i of column cc of the strip
+    auto fp_bin = [&](int i, int cc) -> float2 {
+      if (fp_tma) {
+        if (fp.dtype == kF32) return reinterpret_cast<const float2*>(fpsm)[i * NC + cc];
+        return __half22float2(reinterpret_cast<const __half2*>(fpsm)[i * NC + cc]);
+      }
+      return load_spec(fp.spec, fp.dtype, (size_t)i * Wh + c0 + cc);
+    };
+    if (FPT && fp_tma) {
+      if (!block_wait(&s_fbar, 0, a.err)) return;
+    } else {
+      __syncthreads();   // every strip value read
+    }
+    if (c0 == 0) {
+      // packed column 0 (DC + i*Nyquist): the product needs bin H - i as
+      // well, through two scratch columns (in the strip buffer where it is
+      // free): the bins, and each thread's products
+      float2* X0 = FPT && !FPSEP ? reinterpret_cast<float2*>(reinterpret_cast<char*>(sm) + col_buf_bytes<CP>(NC)) : sm;
+      if (c == 0 && act_b) {
+#pragma unroll
+        for (int r = 0; r < RB; ++r) X0[j + r * RA] = v[0][r];
+      }
+      __syncthreads();
+      if (c == 0 && act_b) {
+#pragma unroll 1
+        for (int i = j; i < H; i += RA) {
+          const int im = i == 0 ? 0 : H - i;
+          X0[H + i] = packed_col0_product(X0[i], X0[im], fp_bin(i, 0), fp_bin(im, 0));
+        }
+#pragma unroll
+        for (int r = 0; r < RB; ++r) v[0][r] = X0[H + j + r * RA];
+      }
+      __syncthreads();
+    }
+    if (act_b && col != 0) {
+      if (fp_tma && fp.dtype == kF32) {
+        const float2* f = reinterpret_cast<const float2*>(fpsm) + j * NC + c;
+#pragma unroll
+        for (int r = 0; r < RB; ++r) v[0][r] = c_conj_mul(v[0][r], f[r * RA * NC]);
+      } else if (fp_tma) {
+        const __half2* f = reinterpret_cast<const __half2*>(fpsm) + j * NC + c;
+#pragma unroll
+        for (int r = 0; r < RB; ++r) v[0][r] = c_conj_mul(v[0][r], __half22float2(f[r * RA * NC]));
+      } else {
+#pragma unroll
+        for (int r = 0; r < RB; ++r)
+          v[0][r] = c_conj_mul(v[0][r], load_spec(fp.spec, fp.dtype, (size_t)(j + r * RA) * Wh + col));
+      }
+    }
+    if (FPT && !FPSEP && fp_tma) __syncthreads();   // every fingerprint bin read before the buffer is rewritten
+    if (act_b) {
+      DftP<RB, true>::run(v[0]);
+      float2* dst = sm + j * LB * NC + c;
+#pragma unroll
+      for (int r = 0; r < RB; ++r) dst[r * NC] = v[0][r];
+    }
+    __syncthreads();
+    float2 u[1][RA];
+    if (act_a) {
+      const float2* src = sm + j * NC + c;
+#pragma unroll
+      for (int r = 0; r < RA; ++r) u[0][r] = src[r * LB * NC];
+    }
+    if constexpr (TMA) __syncthreads();
+    if (act_a) {
+      twiddle_tab<RA, RB, true, 1>(u, j);
+      DftP<RA, true>::run(u[0]);
+      float2* dst = TMA ? sm + j * NC + c : Z + (size_t)j * Wh + col;
+#pragma unroll
+      for (int r = 0; r < RA; ++r) dst[(size_t)r * RB * (TMA ? NC : Wh)] = u[0][r];
+    }
+  }
+  if constexpr (TMA) {
+    fence_proxy_async_smem();
+    __syncthreads();
+    if (t == 0) {
+#pragma unroll 1
+      for (int b = 0; b < H / BR; ++b) tma_store_2d(map, 2 * c0, ws * H + b * BR, sm + b * BR * NC);
+      bulk_commit();
+      bulk_wait_read();
+    }
+  }
+}
+
+}  // namespace
+
+}  // namespace prnu

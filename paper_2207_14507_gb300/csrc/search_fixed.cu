@@ -106,12 +106,15 @@ void launch_fixed_wave(const PassArgs& a, const FixedShape& fs, int col_variant,
   int v = std::max(0, std::min(col_variant, (int)fs.cols.size() - 1));
   // a variant whose fingerprint region holds FP16 bins only (mode 4) steps
   // aside for FP32 fingerprints: the first variant that copies FP32 bins by TMA
-  if (fs.cols[v].mode == 4 && a.fp_f32)
-    for (int k = 0; k < (int)fs.cols.size(); ++k)
-      if (fs.cols[k].mode == 2 || fs.cols[k].mode == 3) {
-        v = k;
-        break;
-      }
+  // into a region of their own, else into the strip buffer
+  if (fs.cols[v].mode == 4 && a.fp_f32) {
+    auto first = [&](int mode) {
+      for (int k = 0; k < (int)fs.cols.size(); ++k)
+        if (fs.cols[k].mode == mode) return k;
+      return -1;
+    };
+    v = first(3) >= 0 ? first(3) : first(2) >= 0 ? first(2) : v;
+  }
   const FixedCol& fv = fs.cols[v];
   // forward units take the split pass (its inverse half in the variant's fingerprint mode)
   const bool sep = fv.mode >= 3 && fs.col_inv_sep.fn && (fs.col_inv_sep.mode == 3 || !a.fp_f32);

@@ -8,13 +8,7 @@
 // fewer shared-memory passes:
 //   row_forward_body : stage 0 of the row FFT takes its inputs straight from
 //                      the bilinear warp (no shared-memory fill);
-//   col_body         : stage 0 loads the strip from global memory; the last
-//                      forward stage, the spectrum product and the first
-//                      inverse stage stay in registers (the inverse plan is
-//                      the forward plan reversed, so every thread already
-//                      holds its inputs); the last inverse stage stores to
-//                      global memory; stages in between run in place; each
-//                      thread works on a pair of adjacent columns;
+//   col_body         : (col_pass.cuh) two long stages each way in registers;
 //   row_inverse_body : stage 0 rebuilds the two rows' full spectrum straight
 //                      from global memory; the last stage's outputs are
 //                      reduced to the row statistics from registers.
@@ -27,6 +21,7 @@
 #include <algorithm>
 #include <vector>
 
+#include "col_pass.cuh"
 #include "fft_fixed.cuh"
 #include "internal.h"
 #include "search_common.cuh"
@@ -43,11 +38,6 @@ namespace {
 // earlier launch.
 template <bool CG>
 __device__ __forceinline__ float2 ld_spec(const float2* p) {
-  if constexpr (CG) return __ldcg(p);
-  else return __ldg(p);
-}
-template <bool CG>
-__device__ __forceinline__ float4 ld_spec4(const float4* p) {
   if constexpr (CG) return __ldcg(p);
   else return __ldg(p);
 }
@@ -194,428 +184,6 @@ __device__ __forceinline__ void row_forward_body(const PassArgs& a, int is, int 
   }
 }
 
-// ---------------------------------------------------------------- column pass
-
-// The fingerprint bins (i, col0) and (i, col0 + 1) for i = j + r*NS.
-template <int R, int NS, int Wh>
-__device__ __forceinline__ void load_fp_pair(const FpDesc& fp, int j, int col0, float2 (&s)[2][R]) {
-  const size_t b = ((size_t)j * Wh + col0) / 2;
-  if (fp.dtype == kF32) {
-    const float4* p = reinterpret_cast<const float4*>(fp.spec) + b;
-#pragma unroll
-    for (int r = 0; r < R; ++r) split2(__ldg(p + (size_t)r * NS * (Wh / 2)), s[0][r], s[1][r]);
-  } else {
-    const float2* p = reinterpret_cast<const float2*>(fp.spec) + b;   // two __half2
-#pragma unroll
-    for (int r = 0; r < R; ++r) {
-      const float2 u = __ldg(p + (size_t)r * NS * (Wh / 2));
-      s[0][r] = __half22float2(*reinterpret_cast<const __half2*>(&u.x));
-      s[1][r] = __half22float2(*reinterpret_cast<const __half2*>(&u.y));
-    }
-  }
-}
-
-// The product for the packed column 0 (DC + i*Nyquist columns of two real
-// spectra in one complex column): F, Fm the frame bins i and H - i, S, Sm the
-// fingerprint bins; unpack both, conj-multiply each real column's spectrum,
-// repack.
-__device__ __forceinline__ float2 packed_col0_product(float2 F, float2 Fm, float2 S, float2 Sm) {
-  const float2 Aa = make_float2(0.5f * (F.x + Fm.x), 0.5f * (F.y - Fm.y));
-  const float2 Bb = make_float2(0.5f * (F.y + Fm.y), 0.5f * (Fm.x - F.x));
-  const float2 Ka = make_float2(0.5f * (S.x + Sm.x), 0.5f * (S.y - Sm.y));
-  const float2 Kb = make_float2(0.5f * (S.y + Sm.y), 0.5f * (Sm.x - S.x));
-  const float2 p1 = c_conj_mul(Aa, Ka), p2 = c_conj_mul(Bb, Kb);
-  return make_float2(p1.x - p2.y, p1.y + p2.x);
-}
-
-__host__ __device__ constexpr int fp_tmap_index(int NC) { return NC == 2 ? 0 : NC == 4 ? 1 : NC == 8 ? 2 : 3; }
-__host__ __device__ constexpr size_t col_fx_smem_fpt(int H, int nc) { return (size_t)H * (nc + 1) * sizeof(float2); }
-// bytes per fingerprint bin of the separate fingerprint region (MODE 3: FP32
-// or FP16 bins; MODE 4: FP16 bins only)
-__host__ __device__ constexpr int fp_region_bin(int mode) { return mode == 3 ? 8 : mode == 4 ? 4 : 0; }
-__host__ __device__ constexpr size_t col_fx_smem_sep(int H, int nc, int mode) {
-  return (size_t)H * nc * (sizeof(float2) + fp_region_bin(mode));
-}
-constexpr long long kTmaWaitPolls = 1ll << 20;   // polls of mbarrier.try_wait before giving up
-
-// The column pass from the last forward stage on, for the strip of NC
-// columns from c0 whose forward stages have run in the strip buffer sm (PART
-// 2: which holds the last forward stage's outputs): the last forward stage,
-// the product with the fingerprint fp, the inverse stages; the last inverse
-// stage leaves the strip in sm (MODE >= 1) or in Z (MODE 0).  PART 1 stops
-// after the last forward stage and leaves its outputs in sm, in natural
-// order.  With MODE 2 the fingerprint strip comes by TMA into sm once every
-// thread holds its inputs (fp_tma_ok: the caller allows it), completing the
-// mbarrier bar (its completions so far: bar_uses, advanced here when the copy
-// is made, the same on every thread); X0 is the packed column-0 scratch (H
-// float2 that the fingerprint strip does not cover).  With MODE 3 and 4 the
-// caller has already issued the fingerprint strip's copy into its own region
-// after the strip (fp_tma_ok: it did), completing fbar once; X0 is then the
-// strip buffer itself, free once every thread holds its inputs (PART 2 needs
-// no X0: it multiplies as it loads).  hook() runs on every thread right after
-// the barrier that follows the loads of the last forward stage (the strip
-// buffer's old contents are then no longer needed).
-// t = threadIdx.x.  Returns false if the fingerprint copy did not land in
-// time (a.err raised).
-template <class SP, int W, int NC, int T, int MODE, int PART, class Hook>
-__device__ __forceinline__ bool col_tail(const PassArgs& a, const FpDesc& fp, int c0, float2* sm, float2* Z,
-                                         uint64_t* bar, int& bar_uses, bool fp_tma_ok, float2* X0, Hook&& hook,
-                                         int t, uint64_t* fbar = nullptr) {
-  constexpr bool TMA = MODE >= 1, FPT = MODE >= 2 && PART != 1, FPSEP = MODE >= 3;
-  constexpr int H = SP::N, Wh = W / 2;
-  using IS = typename SP::Rev;
-  using M = ColMap<NC, T>;
-  constexpr int NP = M::NP, TJ = M::TJ;
-  const int cp = t % NP, j0 = t / NP;
-  const int col0 = c0 + 2 * cp;
-  float4* sm4 = reinterpret_cast<float4*>(sm);
-  // last forward stage -> spectrum product -> first inverse stage, in registers
-  using FL = Stg<SP, SP::S - 1>;
-  using I0 = Stg<IS, 0>;
-  static_assert(I0::R == FL::R && I0::NB == FL::NB && FL::NB == FL::NS, "register hand-off needs the reversed plan");
-  constexpr int IT = (FL::NB + TJ - 1) / TJ;
-  float2 v[IT][2][FL::R];
-  // The fingerprint strip comes by TMA (into the strip buffer with MODE 2,
-  // into its own region with MODE 3/4), else by per-thread loads.
-  const bool fp_tma = FPT && fp_tma_ok && fp.tmaps != nullptr && NC * (fp.dtype == kF32 ? 8 : 4) >= 16;
-  char* const fpsm = reinterpret_cast<char*>(sm) + (FPSEP ? (size_t)H * NC * sizeof(float2) : 0);
-  // fingerprint bin (i, col) of this strip
-  auto fp_bin = [&](int i, int col) -> float2 {
-    if (fp_tma) {
-      if (fp.dtype == kF32) return reinterpret_cast<const float2*>(fpsm)[i * NC + (col - c0)];
-      return __half22float2(reinterpret_cast<const __half2*>(fpsm)[i * NC + (col - c0)]);
-    }
-    return load_spec(fp.spec, fp.dtype, (size_t)i * Wh + col);
-  };
-  // the fingerprint bins (j + r*NS, col0) and (j + r*NS, col0 + 1) from the TMA'd strip
-  auto fp_pair = [&](int j, int r, float2& s0, float2& s1) {
-    if (fp.dtype == kF32) {
-      split2(reinterpret_cast<const float4*>(fpsm)[(j + r * FL::NS) * NP + cp], s0, s1);
-    } else {
-      const float2 u = reinterpret_cast<const float2*>(fpsm)[(j + r * FL::NS) * NP + cp];   // two __half2
-      s0 = __half22float2(*reinterpret_cast<const __half2*>(&u.x));
-      s1 = __half22float2(*reinterpret_cast<const __half2*>(&u.y));
-    }
-  };
-  if constexpr (PART == 2 && FPSEP) {
-    // The strip holds the last forward stage's outputs in natural order and
-    // the fingerprint strip has its own region: each bin is multiplied as it
-    // is loaded, and column 0's mirror bins H - i are read from the strip.
-    if (fp_tma) {
-      const bool ok = mbar_wait_bounded(fbar, 0, kTmaWaitPolls);
-      if (__syncthreads_or(!ok)) {
-        if (t == 0) {
-          if (a.err) atomicExch(a.err, 1);
-          mbar_wait_bounded(fbar, 0, kTmaWaitPolls);
-        }
-        __syncthreads();
-        return false;
-      }
-    }
-#pragma unroll
-    for (int it = 0; it < IT; ++it) {
-      const int j = j0 + it * TJ;
-      if (FL::NB % TJ != 0 && j >= FL::NB) continue;
-      const float4* src = sm4 + j * NP + cp;
-      float2 sf[2][FL::R];
-      if (!fp_tma) load_fp_pair<FL::R, FL::NS, Wh>(fp, j, col0, sf);
-#pragma unroll
-      for (int r = 0; r < FL::R; ++r) {
-        float2 F0, F1, s0, s1;
-        split2(src[r * FL::NB * NP], F0, F1);
-        if (fp_tma) fp_pair(j, r, s0, s1);
-        else {
-          s0 = sf[0][r];
-          s1 = sf[1][r];
-        }
-        if (col0 == 0) {
-          const int i = j + r * FL::NS, im = i == 0 ? 0 : H - i;
-          v[it][0][r] = packed_col0_product(F0, sm[im * NC], fp_bin(i, 0), fp_bin(im, 0));
-        } else {
-          v[it][0][r] = c_conj_mul(F0, s0);
-        }
-        v[it][1][r] = c_conj_mul(F1, s1);
-      }
-    }
-    __syncthreads();   // every strip value read before the first inverse stage rewrites the strip
-    hook();
-  } else {
-#pragma unroll
-  for (int it = 0; it < IT; ++it) {
-    const int j = j0 + it * TJ;
-    if (FL::NB % TJ != 0 && j >= FL::NB) continue;
-    const float4* src = sm4 + j * NP + cp;
-#pragma unroll
-    for (int r = 0; r < FL::R; ++r) split2(src[r * FL::NB * NP], v[it][0][r], v[it][1][r]);
-  }
-  __syncthreads();
-  hook();
-  if constexpr (FPT && !FPSEP) {
-    if (fp_tma && t == 0) {
-      const CUtensorMap* fm = reinterpret_cast<const CUtensorMap*>(fp.tmaps) + fp_tmap_index(NC);
-      const int es = fp.dtype == kF32 ? 8 : 4, fbr = tma_box_rows(H, NC, es);
-      asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"(reinterpret_cast<uint64_t>(fm))
-                   : "memory");
-      mbar_expect_tx(bar, H * NC * es);
-#pragma unroll 1
-      for (int b = 0; b < H / fbr; ++b)
-        tma_load_2d(reinterpret_cast<char*>(sm) + (size_t)b * fbr * NC * es, fm, 2 * c0, b * fbr, bar);
-    }
-  }
-  if constexpr (PART != 2) {   // PART 2: the strip held the outputs of this stage
-#pragma unroll
-    for (int it = 0; it < IT; ++it) {
-      const int j = j0 + it * TJ;
-      if (FL::NB % TJ != 0 && j >= FL::NB) continue;
-      twiddle_tab<FL::R, FL::NS, false, 2>(v[it], j);
-      Dft<FL::R, false>::run(v[it][0]);
-      Dft<FL::R, false>::run(v[it][1]);
-    }
-  }
-  if constexpr (PART == 1) {
-    // outputs i = j + r*NS go back where the stage took its inputs (NB == NS)
-#pragma unroll
-    for (int it = 0; it < IT; ++it) {
-      const int j = j0 + it * TJ;
-      if (FL::NB % TJ != 0 && j >= FL::NB) continue;
-      float4* dst = sm4 + j * NP + cp;
-#pragma unroll
-      for (int r = 0; r < FL::R; ++r) dst[r * FL::NS * NP] = join2(v[it][0][r], v[it][1][r]);
-    }
-    return true;
-  }
-  if constexpr (FPT) {
-    if (fp_tma) {
-      uint64_t* const wb = FPSEP ? fbar : bar;
-      const int ph = FPSEP ? 0 : bar_uses & 1;
-      if (!FPSEP) ++bar_uses;
-      const bool ok = mbar_wait_bounded(wb, ph, kTmaWaitPolls);
-      if (__syncthreads_or(!ok)) {
-        if (t == 0) {
-          if (a.err) atomicExch(a.err, 1);
-          mbar_wait_bounded(wb, ph, kTmaWaitPolls);
-        }
-        __syncthreads();
-        return false;
-      }
-    }
-  }
-  // thread holds bins i = j + r*NS of columns col0 and col0 + 1
-  if (c0 == 0) {
-    // packed column 0 (DC + i*Nyquist): the product needs bin H - i as well
-    if (cp == 0) {
-#pragma unroll
-      for (int it = 0; it < IT; ++it) {
-        const int j = j0 + it * TJ;
-        if (FL::NB % TJ != 0 && j >= FL::NB) continue;
-#pragma unroll
-        for (int r = 0; r < FL::R; ++r) X0[j + r * FL::NS] = v[it][0][r];
-      }
-    }
-    __syncthreads();
-    if (cp == 0) {
-#pragma unroll
-      for (int it = 0; it < IT; ++it) {
-        const int j = j0 + it * TJ;
-        if (FL::NB % TJ != 0 && j >= FL::NB) continue;
-#pragma unroll
-        for (int r = 0; r < FL::R; ++r) {
-          const int i = j + r * FL::NS;
-          const int im = i == 0 ? 0 : H - i;
-          v[it][0][r] = packed_col0_product(v[it][0][r], X0[im], fp_bin(i, 0), fp_bin(im, 0));
-        }
-      }
-    }
-    __syncthreads();
-  }
-  const bool col0_done = col0 == 0;
-#pragma unroll
-  for (int it = 0; it < IT; ++it) {
-    const int j = j0 + it * TJ;
-    if (FL::NB % TJ != 0 && j >= FL::NB) continue;
-    if (fp_tma) {
-#pragma unroll
-      for (int r = 0; r < FL::R; ++r) {
-        float2 s0, s1;
-        fp_pair(j, r, s0, s1);
-        if (!col0_done) v[it][0][r] = c_conj_mul(v[it][0][r], s0);
-        v[it][1][r] = c_conj_mul(v[it][1][r], s1);
-      }
-    } else {
-      float2 sf[2][FL::R];
-      load_fp_pair<FL::R, FL::NS, Wh>(fp, j, col0, sf);
-#pragma unroll
-      for (int r = 0; r < FL::R; ++r) {
-        if (!col0_done) v[it][0][r] = c_conj_mul(v[it][0][r], sf[0][r]);
-        v[it][1][r] = c_conj_mul(v[it][1][r], sf[1][r]);
-      }
-    }
-  }
-  if (!FPSEP && fp_tma) __syncthreads();   // every fingerprint bin read before the strip buffer is rewritten
-  }
-#pragma unroll
-  for (int it = 0; it < IT; ++it) {
-    const int j = j0 + it * TJ;
-    if (FL::NB % TJ != 0 && j >= FL::NB) continue;
-    Dft<FL::R, true>::run(v[it][0]);
-    Dft<FL::R, true>::run(v[it][1]);
-    float4* dst = sm4 + j * FL::R * NP + cp;
-#pragma unroll
-    for (int r = 0; r < FL::R; ++r) dst[r * NP] = join2(v[it][0][r], v[it][1][r]);
-  }
-  __syncthreads();
-  ColStages<IS, 1, IS::S - 1, T, NC, true>::run(sm4, t);
-
-  {  // last inverse stage: shared memory -> global memory
-    using G = Stg<IS, IS::S - 1>;
-    static_assert(G::NB == G::NS, "last stage");
-    constexpr int ITL = (G::NB + TJ - 1) / TJ;
-#pragma unroll
-    for (int it = 0; it < ITL; ++it) {
-      const int j = j0 + it * TJ;
-      if (G::NB % TJ != 0 && j >= G::NB) continue;
-      float2 w[2][G::R];
-      const float4* src = sm4 + j * NP + cp;
-#pragma unroll
-      for (int r = 0; r < G::R; ++r) split2(src[r * G::NB * NP], w[0][r], w[1][r]);
-      twiddle_tab<G::R, G::NS, true, 2>(w, j);
-      Dft<G::R, true>::run(w[0]);
-      Dft<G::R, true>::run(w[1]);
-      if constexpr (TMA) {
-        // outputs j + r*Ns sit where this thread's inputs were: no barrier needed
-        float4* dst = sm4 + j * NP + cp;
-#pragma unroll
-        for (int r = 0; r < G::R; ++r) dst[r * G::NS * NP] = join2(w[0][r], w[1][r]);
-      } else {
-        float4* dst = reinterpret_cast<float4*>(Z + (size_t)j * Wh + col0);
-#pragma unroll
-        for (int r = 0; r < G::R; ++r) dst[(size_t)r * G::NS * (Wh / 2)] = join2(w[0][r], w[1][r]);
-      }
-    }
-  }
-  return true;
-}
-
-
-// Columns bx*NC .. bx*NC+NC-1 of candidate `is` in workspace slot `ws`.
-// MODE 0: every thread loads and stores its own elements.  MODE >= 1: the
-// strip comes into shared memory by TMA tile copies through `map` (the
-// workspace spectra as a [slots*H][W] float tensor) and leaves the same way.
-// MODE 2: the fingerprint strip too comes by TMA, into the strip buffer once
-// the last forward stage has taken its inputs (the packed column-0 scratch then
-// sits after the strip).  MODE 3 and 4: the fingerprint strip comes by TMA
-// into its own region after the strip buffer, copied from the start together
-// with the strip (MODE 4 sizes the region for FP16 bins: FP32 fingerprints
-// are then loaded per thread).  A TMA wait that runs out raises a.err and
-// abandons the candidate.
-// PART splits the pass for forward units (candidates that share a frame and
-// a grid node): PART 1 runs the forward column FFT only and stores its
-// output, in natural order, back to slot ws; PART 2 loads that output from
-// slot src_ws, where each thread finds the values the last forward stage
-// leaves in its registers, and runs the product and the inverse FFT into slot
-// ws.  PART 1 then PART 2 compute bit for bit what PART 0 (the whole pass)
-// computes.  PART 1 and 2 need TMA (MODE >= 1); PART 2 takes MODE 2.
-template <class SP, int W, int NC, int T, bool CG = false, int MODE = 0, int PART = 0>
-__device__ __forceinline__ void col_body(const PassArgs& a, int is, int ws, int bx, float2* sm,
-                                         const CUtensorMap* map = nullptr, int src_ws = -1) {
-  constexpr bool TMA = MODE >= 1, FPT = MODE >= 2 && PART != 1, FPSEP = MODE >= 3 && PART != 1;
-  static_assert(PART == 0 || TMA, "the split column pass moves its strips by TMA");
-  if (src_ws < 0) src_ws = ws;
-  constexpr int H = SP::N, Wh = W / 2;
-  using IS = typename SP::Rev;
-  using M = ColMap<NC, T>;
-  constexpr int NP = M::NP, TJ = M::TJ;
-  static_assert(Wh % NC == 0, "strips tile the half spectrum");
-  const int t = threadIdx.x;
-  const int c0 = bx * NC;
-  const int cp = t % NP, j0 = t / NP;
-  const int col0 = c0 + 2 * cp;
-  float2* Z = a.spec + (size_t)ws * H * Wh;
-  float4* sm4 = reinterpret_cast<float4*>(sm);
-  const WorkItem wi = item_of(a, is);
-  const FpDesc fp = a.fps[wi.fp];
-
-  constexpr int BR = tma_box_rows(H, NC);
-  __shared__ uint64_t s_bar, s_fbar;
-  // MODE 3/4: the fingerprint strip's copy goes out with the strip's (a
-  // region sized for its bins, boxes of at least 16 bytes)
-  const int fes = fp.dtype == kF32 ? 8 : 4;
-  const bool fp_sep = FPSEP && fp.tmaps != nullptr && fes <= fp_region_bin(MODE) && NC * fes >= 16;
-  if constexpr (TMA) {
-    static_assert(BR > 0, "no TMA box for this strip");
-    static_assert(!FPSEP || (H * NC * sizeof(float2)) % 128 == 0, "the fingerprint region starts 128-byte aligned");
-    if (t == 0) {
-      mbar_init(&s_bar, 1);
-      if (FPSEP) mbar_init(&s_fbar, 1);
-      fence_mbar_init();
-    }
-    __syncthreads();
-    if (t == 0) {
-      mbar_expect_tx(&s_bar, H * NC * 8 + (a.stall ? 16 : 0));   // the test hook waits for bytes that never come
-#pragma unroll 1
-      for (int b = 0; b < H / BR; ++b) tma_load_2d(sm + b * BR * NC, map, 2 * c0, src_ws * H + b * BR, &s_bar);
-      if (fp_sep) {
-        const CUtensorMap* fm = reinterpret_cast<const CUtensorMap*>(fp.tmaps) + fp_tmap_index(NC);
-        const int fbr = tma_box_rows(H, NC, fes);
-        char* dst = reinterpret_cast<char*>(sm) + (size_t)H * NC * sizeof(float2);
-        asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"(reinterpret_cast<uint64_t>(fm))
-                     : "memory");
-        mbar_expect_tx(&s_fbar, H * NC * fes);
-#pragma unroll 1
-        for (int b = 0; b < H / fbr; ++b) tma_load_2d(dst + (size_t)b * fbr * NC * fes, fm, 2 * c0, b * fbr, &s_fbar);
-      }
-    }
-    const bool ok = mbar_wait_bounded(&s_bar, 0, kTmaWaitPolls);
-    if (__syncthreads_or(!ok)) {
-      if (t == 0) {
-        if (a.err) atomicExch(a.err, 1);
-        mbar_wait_bounded(&s_bar, 0, kTmaWaitPolls);   // let the copies land before the block leaves
-        if (fp_sep) mbar_wait_bounded(&s_fbar, 0, kTmaWaitPolls);
-      }
-      __syncthreads();
-      return;
-    }
-    if constexpr (PART != 2) ColStages<SP, 0, SP::S - 1, T, NC, false>::run(sm4, t);
-  } else {  // forward stage 0 from global memory
-    using G = Stg<SP, 0>;
-    constexpr int IT = (G::NB + TJ - 1) / TJ;
-#pragma unroll
-    for (int it = 0; it < IT; ++it) {
-      const int j = j0 + it * TJ;
-      if (G::NB % TJ != 0 && j >= G::NB) continue;
-      float2 v[2][G::R];
-      const float4* src = reinterpret_cast<const float4*>(Z + (size_t)j * Wh + col0);
-#pragma unroll
-      for (int r = 0; r < G::R; ++r) split2(ld_spec4<CG>(src + (size_t)r * G::NB * (Wh / 2)), v[0][r], v[1][r]);
-      Dft<G::R, false>::run(v[0]);
-      Dft<G::R, false>::run(v[1]);
-      float4* dst = sm4 + j * G::R * NP + cp;
-#pragma unroll
-      for (int r = 0; r < G::R; ++r) dst[r * NP] = join2(v[0][r], v[1][r]);
-    }
-    __syncthreads();
-    ColStages<SP, 1, SP::S - 1, T, NC, false>::run(sm4, t);
-  }
-
-  // the rest of the pass (PART 1 leaves its outputs in the strip buffer)
-  float2* X0 = FPT && !FPSEP ? sm + H * NC : sm;   // with MODE 2 the strip buffer holds the fingerprint
-  int bar_uses = 1;                                  // s_bar completed once (the strip)
-  if (!col_tail<SP, W, NC, T, MODE, PART>(a, fp, c0, sm, Z, &s_bar, bar_uses, FPSEP ? fp_sep : true, X0, [] {}, t,
-                                          &s_fbar))
-    return;
-  if constexpr (TMA) {
-    fence_proxy_async_smem();
-    __syncthreads();
-    if (t == 0) {
-#pragma unroll 1
-      for (int b = 0; b < H / BR; ++b) tma_store_2d(map, 2 * c0, ws * H + b * BR, sm + b * BR * NC);
-      bulk_commit();
-      if constexpr (CG) bulk_wait_all();
-      else bulk_wait_read();
-    }
-  }
-}
-
 // ---------------------------------------------------------------- row inverse + statistics
 
 // Inverse row FFT of z = G_a + i G_b, the full spectrum of the packed rows
@@ -742,40 +310,38 @@ __global__ void __launch_bounds__(T * PPB) k_row_forward_fx(PassArgs a) {
                                    reinterpret_cast<float2*>(smem4), threadIdx.x);
 }
 
-template <class SP, int W, int NC, int T, int MINB>
-__global__ void __launch_bounds__(T, MINB) k_col_fx(PassArgs a) {
+template <class CP, int W, int NC, int MINB>
+__global__ void __launch_bounds__(NC* CP::lanes, MINB) k_col_fx(PassArgs a) {
   extern __shared__ float4 smem4[];
   if (past_count(a, blockIdx.y, 0)) return;
-  col_body<SP, W, NC, T>(a, blockIdx.y, blockIdx.y, blockIdx.x, reinterpret_cast<float2*>(smem4));
+  col_body<CP, W, NC>(a, blockIdx.y, blockIdx.y, blockIdx.x, reinterpret_cast<float2*>(smem4));
 }
 
-template <class SP, int W, int NC, int T, int MINB, int MODE>
-__global__ void __launch_bounds__(T, MINB) k_col_tma_fx(PassArgs a, const __grid_constant__ CUtensorMap map) {
+template <class CP, int W, int NC, int MINB, int MODE, int PFD>
+__global__ void __launch_bounds__(NC* CP::lanes, MINB) k_col_tma_fx(PassArgs a, const __grid_constant__ CUtensorMap map) {
   extern __shared__ __align__(1024) float4 smem4t[];
   if (past_count(a, blockIdx.y, 0)) return;
-  col_body<SP, W, NC, T, false, MODE>(a, blockIdx.y, blockIdx.y, blockIdx.x, reinterpret_cast<float2*>(smem4t),
-                                      &map);
+  col_body<CP, W, NC, MODE, 0, PFD>(a, blockIdx.y, blockIdx.y, blockIdx.x, reinterpret_cast<float2*>(smem4t), &map);
 }
 
 // Forward units (see col_body PART): the forward column FFT of unit
 // blockIdx.y, in place in its slot a.nitems + u; then, per candidate slot
 // blockIdx.y, the product with its fingerprint and the inverse FFT from its
 // unit's slot into its own.
-template <class SP, int W, int NC, int T, int MINB>
-__global__ void __launch_bounds__(T, MINB) k_col_fwd_fx(PassArgs a, const __grid_constant__ CUtensorMap map) {
+template <class CP, int W, int NC, int MINB>
+__global__ void __launch_bounds__(NC* CP::lanes, MINB) k_col_fwd_fx(PassArgs a, const __grid_constant__ CUtensorMap map) {
   extern __shared__ __align__(1024) float4 smem4f[];
   const int u = blockIdx.y;
   if (past_count(a, u, 1)) return;
-  col_body<SP, W, NC, T, false, 1, 1>(a, unit_first(a, u), a.nitems + u, blockIdx.x,
-                                      reinterpret_cast<float2*>(smem4f), &map);
+  col_body<CP, W, NC, 1, 1>(a, unit_first(a, u), a.nitems + u, blockIdx.x, reinterpret_cast<float2*>(smem4f), &map);
 }
-template <class SP, int W, int NC, int T, int MINB, int MODE>
-__global__ void __launch_bounds__(T, MINB) k_col_inv_fx(PassArgs a, const __grid_constant__ CUtensorMap map) {
+template <class CP, int W, int NC, int MINB, int MODE>
+__global__ void __launch_bounds__(NC* CP::lanes, MINB) k_col_inv_fx(PassArgs a, const __grid_constant__ CUtensorMap map) {
   extern __shared__ __align__(1024) float4 smem4i[];
   const int s = blockIdx.y;
   if (past_count(a, s, 0)) return;
-  col_body<SP, W, NC, T, false, MODE, 2>(a, s, s, blockIdx.x, reinterpret_cast<float2*>(smem4i), &map,
-                                         a.nitems + unit_of_slot(a, s));
+  col_body<CP, W, NC, MODE, 2>(a, s, s, blockIdx.x, reinterpret_cast<float2*>(smem4i), &map,
+                               a.nitems + unit_of_slot(a, s));
 }
 
 template <class SP, int T, int PPB>
@@ -805,9 +371,156 @@ template <int DT, class SP, int T, int PPB>
 __device__ __forceinline__ void row_forward_task(const PassArgs& a, int is, int ws, int bx, float2* smem, int tx) {
   row_forward_body<DT, SP, T, PPB>(a, is, ws, bx, smem, tx);
 }
+// The column pass as a task of the persistent kernel, whose register bound
+// (80 at 1080p) holds no 30-point butterfly: three radix stages, a pair of
+// adjacent columns per thread, loads and stores by every thread itself, L2
+// only.  The same steps as col_body (col_pass.cuh).
+
+// The fingerprint bins (i, col0) and (i, col0 + 1) for i = j + r*NS.
+template <int R, int NS, int Wh>
+__device__ __forceinline__ void load_fp_pair(const FpDesc& fp, int j, int col0, float2 (&s)[2][R]) {
+  const size_t b = ((size_t)j * Wh + col0) / 2;
+  if (fp.dtype == kF32) {
+    const float4* p = reinterpret_cast<const float4*>(fp.spec) + b;
+#pragma unroll
+    for (int r = 0; r < R; ++r) split2(__ldg(p + (size_t)r * NS * (Wh / 2)), s[0][r], s[1][r]);
+  } else {
+    const float2* p = reinterpret_cast<const float2*>(fp.spec) + b;   // two __half2
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      const float2 u = __ldg(p + (size_t)r * NS * (Wh / 2));
+      s[0][r] = __half22float2(*reinterpret_cast<const __half2*>(&u.x));
+      s[1][r] = __half22float2(*reinterpret_cast<const __half2*>(&u.y));
+    }
+  }
+}
+
 template <class SP, int W, int NC, int T>
-__device__ __forceinline__ void col_task(const PassArgs& a, int is, int ws, int bx, float2* smem) {
-  col_body<SP, W, NC, T, true>(a, is, ws, bx, smem);
+__device__ __forceinline__ void col_task(const PassArgs& a, int is, int ws, int bx, float2* sm) {
+  constexpr int H = SP::N, Wh = W / 2;
+  using IS = typename SP::Rev;
+  using M = ColMap<NC, T>;
+  constexpr int NP = M::NP, TJ = M::TJ;
+  static_assert(Wh % NC == 0, "strips tile the half spectrum");
+  const int t = threadIdx.x;
+  const int c0 = bx * NC;
+  const int cp = t % NP, j0 = t / NP;
+  const int col0 = c0 + 2 * cp;
+  float2* Z = a.spec + (size_t)ws * H * Wh;
+  float4* sm4 = reinterpret_cast<float4*>(sm);
+  const WorkItem wi = item_of(a, is);
+  const FpDesc fp = a.fps[wi.fp];
+  {  // forward stage 0 from global memory
+    using G = Stg<SP, 0>;
+    constexpr int IT = (G::NB + TJ - 1) / TJ;
+#pragma unroll
+    for (int it = 0; it < IT; ++it) {
+      const int j = j0 + it * TJ;
+      if (G::NB % TJ != 0 && j >= G::NB) continue;
+      float2 v[2][G::R];
+      const float4* src = reinterpret_cast<const float4*>(Z + (size_t)j * Wh + col0);
+#pragma unroll
+      for (int r = 0; r < G::R; ++r) split2(__ldcg(src + (size_t)r * G::NB * (Wh / 2)), v[0][r], v[1][r]);
+      Dft<G::R, false>::run(v[0]);
+      Dft<G::R, false>::run(v[1]);
+      float4* dst = sm4 + j * G::R * NP + cp;
+#pragma unroll
+      for (int r = 0; r < G::R; ++r) dst[r * NP] = join2(v[0][r], v[1][r]);
+    }
+  }
+  __syncthreads();
+  ColStages<SP, 1, SP::S - 1, T, NC, false>::run(sm4, t);
+  // last forward stage -> spectrum product -> first inverse stage, in registers
+  using FL = Stg<SP, SP::S - 1>;
+  using I0 = Stg<IS, 0>;
+  static_assert(I0::R == FL::R && I0::NB == FL::NB && FL::NB == FL::NS, "register hand-off needs the reversed plan");
+  constexpr int IT = (FL::NB + TJ - 1) / TJ;
+  float2 v[IT][2][FL::R];
+#pragma unroll
+  for (int it = 0; it < IT; ++it) {
+    const int j = j0 + it * TJ;
+    if (FL::NB % TJ != 0 && j >= FL::NB) continue;
+    const float4* src = sm4 + j * NP + cp;
+#pragma unroll
+    for (int r = 0; r < FL::R; ++r) split2(src[r * FL::NB * NP], v[it][0][r], v[it][1][r]);
+  }
+  __syncthreads();
+#pragma unroll
+  for (int it = 0; it < IT; ++it) {
+    const int j = j0 + it * TJ;
+    if (FL::NB % TJ != 0 && j >= FL::NB) continue;
+    twiddle_tab<FL::R, FL::NS, false, 2>(v[it], j);
+    Dft<FL::R, false>::run(v[it][0]);
+    Dft<FL::R, false>::run(v[it][1]);
+  }
+  // thread holds bins i = j + r*NS of columns col0 and col0 + 1
+  if (c0 == 0) {
+    // packed column 0 (DC + i*Nyquist): the product needs bin H - i as well
+    if (cp == 0) {
+#pragma unroll
+      for (int it = 0; it < IT; ++it) {
+        const int j = j0 + it * TJ;
+        if (FL::NB % TJ != 0 && j >= FL::NB) continue;
+#pragma unroll
+        for (int r = 0; r < FL::R; ++r) sm[j + r * FL::NS] = v[it][0][r];
+      }
+    }
+    __syncthreads();
+    if (cp == 0) {
+#pragma unroll
+      for (int it = 0; it < IT; ++it) {
+        const int j = j0 + it * TJ;
+        if (FL::NB % TJ != 0 && j >= FL::NB) continue;
+#pragma unroll
+        for (int r = 0; r < FL::R; ++r) {
+          const int i = j + r * FL::NS;
+          const int im = i == 0 ? 0 : H - i;
+          v[it][0][r] = packed_col0_product(v[it][0][r], sm[im], load_spec(fp.spec, fp.dtype, (size_t)i * Wh),
+                                            load_spec(fp.spec, fp.dtype, (size_t)im * Wh));
+        }
+      }
+    }
+    __syncthreads();
+  }
+#pragma unroll
+  for (int it = 0; it < IT; ++it) {
+    const int j = j0 + it * TJ;
+    if (FL::NB % TJ != 0 && j >= FL::NB) continue;
+    float2 sf[2][FL::R];
+    load_fp_pair<FL::R, FL::NS, Wh>(fp, j, col0, sf);
+#pragma unroll
+    for (int r = 0; r < FL::R; ++r) {
+      if (col0 != 0) v[it][0][r] = c_conj_mul(v[it][0][r], sf[0][r]);
+      v[it][1][r] = c_conj_mul(v[it][1][r], sf[1][r]);
+    }
+    Dft<FL::R, true>::run(v[it][0]);
+    Dft<FL::R, true>::run(v[it][1]);
+    float4* dst = sm4 + j * FL::R * NP + cp;
+#pragma unroll
+    for (int r = 0; r < FL::R; ++r) dst[r * NP] = join2(v[it][0][r], v[it][1][r]);
+  }
+  __syncthreads();
+  ColStages<IS, 1, IS::S - 1, T, NC, true>::run(sm4, t);
+  {  // last inverse stage: shared memory -> global memory
+    using G = Stg<IS, IS::S - 1>;
+    static_assert(G::NB == G::NS, "last stage");
+    constexpr int ITL = (G::NB + TJ - 1) / TJ;
+#pragma unroll
+    for (int it = 0; it < ITL; ++it) {
+      const int j = j0 + it * TJ;
+      if (G::NB % TJ != 0 && j >= G::NB) continue;
+      float2 w[2][G::R];
+      const float4* src = sm4 + j * NP + cp;
+#pragma unroll
+      for (int r = 0; r < G::R; ++r) split2(src[r * G::NB * NP], w[0][r], w[1][r]);
+      twiddle_tab<G::R, G::NS, true, 2>(w, j);
+      Dft<G::R, true>::run(w[0]);
+      Dft<G::R, true>::run(w[1]);
+      float4* dst = reinterpret_cast<float4*>(Z + (size_t)j * Wh + col0);
+#pragma unroll
+      for (int r = 0; r < G::R; ++r) dst[(size_t)r * G::NS * (Wh / 2)] = join2(w[0][r], w[1][r]);
+    }
+  }
 }
 template <class SP, int T, int PPB>
 __device__ __forceinline__ void row_inverse_task(const PassArgs& a, int ws, int bx, float2* smem, int tx) {
@@ -1038,33 +751,31 @@ void allow(K k) {
 constexpr int kFinPairs = 3;
 
 // RT threads per row pair in the row forward kernel, RTI in the row inverse
-// (and in the finalisation)
-template <class RS, int RT, class CS, int RTI = RT>
+// (and in the finalisation); CP the column pass's plan, CS the three-stage
+// plan of the persistent kernel's column task
+template <class RS, int RT, class CP, class CS, int RTI = RT>
 struct ShapeDef {
-  static constexpr int W = RS::N, H = CS::N;
-  // NC columns per block, CT threads, at least MINB resident blocks per SM
+  static constexpr int W = RS::N, H = CP::H;
+  static_assert(CS::N == H, "column plans of one length");
+  // NC columns per block, at least MINB resident blocks per SM
   // MODE: 0 plain loads and stores, 1 strip by TMA, 2 strip and fingerprint by TMA
-  static FixedCol col_entry(void* fn, int nc, int ct, size_t smem, int mode) {
+  static FixedCol col_entry(void* fn, int nc, int mode) {
     allow_max_dynamic_smem(fn);
-    FixedCol c{nc, ct, smem, fn, mode != 0, tma_box_rows(H, nc), mode};
-    return c;
+    return FixedCol{nc, nc * CP::lanes, col_pass_smem<CP>(nc, mode), fn, mode != 0, tma_box_rows(H, nc), mode};
   }
-  static constexpr size_t col_smem(int nc, int mode) {
-    return mode >= 3 ? col_fx_smem_sep(H, nc, mode) : mode == 2 ? col_fx_smem_fpt(H, nc) : col_fx_smem(H, nc);
-  }
-  template <int NC, int CT, int MINB, int MODE>
+  template <int NC, int MINB, int MODE, int PFD = 0>
   static FixedCol col() {
-    void* fn = MODE ? (void*)k_col_tma_fx<CS, W, NC, CT, MINB, MODE> : (void*)k_col_fx<CS, W, NC, CT, MINB>;
-    return col_entry(fn, NC, CT, col_smem(NC, MODE), MODE);
+    if constexpr (MODE > 0) return col_entry((void*)k_col_tma_fx<CP, W, NC, MINB, MODE, PFD>, NC, MODE);
+    else return col_entry((void*)k_col_fx<CP, W, NC, MINB>, NC, MODE);
   }
-  // the split column pass of forward units (NC columns, CT threads, MINB blocks)
-  template <int NC, int CT, int MINB>
+  // the split column pass of forward units (NC columns, MINB blocks)
+  template <int NC, int MINB>
   static FixedCol col_fwd() {
-    return col_entry((void*)k_col_fwd_fx<CS, W, NC, CT, MINB>, NC, CT, col_fx_smem(H, NC), 1);
+    return col_entry((void*)k_col_fwd_fx<CP, W, NC, MINB>, NC, 1);
   }
-  template <int NC, int CT, int MINB, int MODE = 2>
+  template <int NC, int MINB, int MODE = 2>
   static FixedCol col_inv() {
-    return col_entry((void*)k_col_inv_fx<CS, W, NC, CT, MINB, MODE>, NC, CT, col_smem(NC, MODE), MODE);
+    return col_entry((void*)k_col_inv_fx<CP, W, NC, MINB, MODE>, NC, MODE);
   }
   // RIMB: resident row-inverse blocks per SM to allocate registers for (0: no bound)
   template <int PPB, int RIMB = 0>

@@ -15,6 +15,9 @@ __host__ __device__ constexpr int tma_box_rows(int H, int NC, int esize = 8) {
   return 0;
 }
 
+// the descriptor of strips of NC columns among a fingerprint's four
+__host__ __device__ constexpr int fp_tmap_index(int NC) { return NC == 2 ? 0 : NC == 4 ? 1 : NC == 8 ? 2 : 3; }
+
 // one instantiated column-pass variant: columns per block, threads, shared
 // memory; with tma the kernel moves its strip by TMA tile copies of br rows
 // and takes a CUtensorMap of the workspace spectra as a second argument,
@@ -69,6 +72,7 @@ struct FixedShape {
   int W, H;
   std::vector<FixedRow> rows;
   std::vector<FixedCol> cols;
+  int default_col;           // the column variant of the default tuning
   FixedCol col_fwd, col_inv; // the column pass split for forward units (k_col_fwd_fx, k_col_inv_fx)
   FixedCol col_inv_sep;      // k_col_inv_fx with the fingerprint strip in its own region (mode 3/4), taken
                              // with a column variant of that mode; fn null where none is instantiated

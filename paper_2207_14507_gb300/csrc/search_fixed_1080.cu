@@ -4,12 +4,16 @@
 namespace prnu {
 
 FixedShape fixed_shape_1080() {
-  using D = ShapeDef<Spec<1920, 16, 12, 10>, 192, Spec<1080, 9, 12, 10>, 160>;
+  using D = ShapeDef<Spec<1920, 16, 12, 10>, 192, ColPlan<1080, 36, 30>, Spec<1080, 9, 12, 10>, 160>;
+  // us per candidate of the column variants (FP32 / FP16 fingerprints, waves of
+  // 512): 4-column strips, mode 4 with 4 blocks per SM - / 3.83, mode 3 with 3
+  // blocks 4.25 / 4.33, mode 2 4.70 / 4.83, mode 1 4.61 / 4.73, mode 0 5.50,
+  // 8-column strips 7.40 (mode 1), 6.7 (mode 3), 4.04 (mode 4, 2 blocks).  The
+  // three-stage plan: 5.38 / 5.30.
   return D::make({D::row<2>(), D::row<1, 8>()},
-                 {D::col<4, 240, 3, 3>(), D::col<4, 240, 3, 2>(), D::col<4, 240, 3, 1>(),
-                  D::col<4, 240, 3, 0>(), D::col<8, 480, 1, 1>()},
-                 {D::col_fwd<4, 240, 3>(), D::col_inv<4, 240, 3>(), D::col_inv<4, 240, 3, 3>(),
-                  D::col_inv<4, 240, 4, 4>()},
+                 {D::col<4, 4, 4>(), D::col<4, 3, 2>(), D::col<4, 3, 1>(), D::col<4, 3, 0>(), D::col<8, 1, 1>(),
+                  D::col<4, 3, 3>()},
+                 {D::col_fwd<4, 4>(), D::col_inv<4, 3>(), D::col_inv<4, 3, 3>(), D::col_inv<4, 4, 4>()},
                  D::persist<192, 2, 4>());
 }
 

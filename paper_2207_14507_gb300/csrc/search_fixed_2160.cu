@@ -4,12 +4,13 @@
 namespace prnu {
 
 FixedShape fixed_shape_2160() {
-  using D = ShapeDef<Spec<3840, 16, 16, 15>, 256, Spec<2160, 15, 12, 12>>;
+  using D = ShapeDef<Spec<3840, 16, 16, 15>, 256, ColPlan<2160, 48, 45>, Spec<2160, 15, 12, 12>>;
+  // us per candidate (FP32 / FP16 fingerprints), 2 blocks per SM: mode 4 - / 18.8,
+  // with the L2 prefetch 18.0; mode 2 20.7 / 20.5; mode 1 25.2 / 25.0; mode 0 26
+  // (8-column strips, 1 block: 24 to 28).  The three-stage plan: 21.9 (FP16).
   return D::make({D::row<2>(), D::row<1, 5>()},
-                 {D::col<4, 360, 2, 4>(), D::col<4, 360, 2, 2>(), D::col<4, 360, 2, 1>(),
-                  D::col<4, 360, 2, 0>()},
-                 {D::col_fwd<4, 360, 2>(), D::col_inv<4, 360, 2>(), D::col_inv<4, 360, 2, 4>()},
-                 D::persist<256, 2, 4>());
+                 {D::col<4, 2, 4, 152>(), D::col<4, 2, 2, 152>(), D::col<4, 2, 1>(), D::col<4, 2, 0>()},
+                 {D::col_fwd<4, 2>(), D::col_inv<4, 2>(), D::col_inv<4, 2, 4>()}, D::persist<256, 2, 4>());
 }
 
 }  // namespace prnu

@@ -4,12 +4,14 @@
 namespace prnu {
 
 FixedShape fixed_shape_720() {
-  using D = ShapeDef<Spec<1280, 16, 10, 8>, 160, Spec<720, 9, 10, 8>>;
+  using D = ShapeDef<Spec<1280, 16, 10, 8>, 160, ColPlan<720, 30, 24>, Spec<720, 9, 10, 8>>;
+  // us per candidate (FP32 / FP16 fingerprints): 8-column strips, mode 4 with 3
+  // blocks per SM - / 1.56, mode 3 with 2 blocks 1.79 / 1.80, mode 2 2.27, mode 1
+  // 2.12 / 1.99; 4-column strips, mode 3 1.77 / 1.82, mode 4 1.66 to 1.69, mode 2 2.18.
   return D::make({D::row<2>(), D::row<1>()},
-                 {D::col<8, 360, 2, 3>(), D::col<8, 360, 2, 1>(), D::col<8, 360, 2, 2>(),
-                  D::col<8, 360, 2, 0>(), D::col<4, 180, 4, 2>(), D::col<8, 360, 3, 4>()},
-                 {D::col_fwd<4, 180, 4>(), D::col_inv<4, 180, 4>(), D::col_inv<4, 180, 4, 3>(),
-                  D::col_inv<4, 180, 5, 4>()},
+                 {D::col<8, 3, 4>(), D::col<8, 2, 1>(), D::col<8, 2, 2>(), D::col<8, 2, 0>(), D::col<4, 4, 2>(),
+                  D::col<4, 4, 3>()},
+                 {D::col_fwd<8, 3>(), D::col_inv<8, 2>(), D::col_inv<8, 2, 3>(), D::col_inv<8, 3, 4>()},
                  D::persist<160, 2, 4>());
 }
 
