@@ -28,6 +28,7 @@
 #include <type_traits>
 
 #include "fft.cuh"
+#include "fft_packed.cuh"
 
 namespace prnu {
 
@@ -175,70 +176,53 @@ __device__ __forceinline__ void row_store16(float2* out, int j, const float2 (&v
   for (int m = 0; m < 8; ++m) d[m] = make_float4(v[2 * m].x, v[2 * m].y, v[2 * m + 1].x, v[2 * m + 1].y);
 }
 
-// Stage I (>= 1) of row plan SP on one transform, T threads (thread t),
-// in -> out, both in the row layout.
-template <class SP, int I, int T, bool INV>
-__device__ __forceinline__ void row_stage(const float2* __restrict__ in, float2* __restrict__ out, int t) {
-  using G = Stg<SP, I>;
-  static_assert(G::NB % 16 == 0 && G::NS % 16 == 0 && T % 16 == 0, "row stages need 16-element blocks");
-  constexpr int IT = (G::NB + T - 1) / T;
-  constexpr int LB = G::NB / 16 * 18, LS = G::NS / 16 * 18;
-#pragma unroll
-  for (int it = 0; it < IT; ++it) {
-    const int j = t + it * T;
-    if (G::NB % T != 0 && j >= G::NB) break;
-    float2 v[1][G::R];
-    const float2* src = in + rp2(j);
-#pragma unroll
-    for (int r = 0; r < G::R; ++r) v[0][r] = src[r * LB];
-    const int k = (G::NB == G::NS) ? j : j % G::NS;
-    twiddle_tab<G::R, G::NS, INV, 1>(v, k);
-    Dft<G::R, INV>::run(v[0]);
-    float2* dst = out + rp2((j - k) * G::R + k);
-#pragma unroll
-    for (int r = 0; r < G::R; ++r) dst[r * LS] = v[0][r];
-  }
-}
-
-// Stage I (>= 1) of row plan SP in place on `buf`, one butterfly per thread
-// (NB <= T): every thread loads its inputs, the block synchronises, then every
-// thread stores its outputs.  One row buffer instead of two, for one more
-// barrier.  Called by every thread of the block.
+// Stage I (>= 1) of row plan SP in place on `buf`, butterflies j = t + it*T:
+// every thread loads its inputs, the block synchronises, then every thread
+// stores its outputs.  One row buffer instead of two, for one more barrier.
+// Called by every thread of the block.
 template <class SP, int I, int T, bool INV>
 __device__ __forceinline__ void row_stage_ip(float2* buf, int t) {
   using G = Stg<SP, I>;
   static_assert(G::NB % 16 == 0 && G::NS % 16 == 0 && T % 16 == 0, "row stages need 16-element blocks");
-  static_assert(G::NB <= T, "in-place row stages hold one butterfly per thread");
+  constexpr int IT = (G::NB + T - 1) / T;
+  static_assert(IT <= 2, "an in-place row stage holds two butterflies per thread at most");
   constexpr int LB = G::NB / 16 * 18, LS = G::NS / 16 * 18;
-  const bool act = G::NB == T || t < G::NB;
-  const int j = t;
-  const int k = (G::NB == G::NS) ? j : j % G::NS;
-  float2 v[1][G::R];
-  if (act) {
+  float2 v[IT][1][G::R];
+#pragma unroll
+  for (int it = 0; it < IT; ++it) {
+    const int j = t + it * T;
+    if ((it + 1) * T > G::NB && j >= G::NB) continue;
     const float2* src = buf + rp2(j);
 #pragma unroll
-    for (int r = 0; r < G::R; ++r) v[0][r] = src[r * LB];
+    for (int r = 0; r < G::R; ++r) v[it][0][r] = src[r * LB];
   }
   __syncthreads();
-  if (act) {
-    twiddle_tab<G::R, G::NS, INV, 1>(v, k);
-    Dft<G::R, INV>::run(v[0]);
+#pragma unroll
+  for (int it = 0; it < IT; ++it) {
+    const int j = t + it * T;
+    if ((it + 1) * T > G::NB && j >= G::NB) continue;
+    const int k = (G::NB == G::NS) ? j : j % G::NS;
+    twiddle_tab<G::R, G::NS, INV, 1>(v[it], k);
+    DftP<G::R, INV>::run(v[it][0]);
     float2* dst = buf + rp2((j - k) * G::R + k);
 #pragma unroll
-    for (int r = 0; r < G::R; ++r) dst[r * LS] = v[0][r];
+    for (int r = 0; r < G::R; ++r) dst[r * LS] = v[it][0][r];
   }
 }
 
-// Last stage of row plan SP (Ns = n/R): butterflies j = t + it*T, outputs
-// x = j + r*Ns stay in registers, v[it]; `last_valid` tells which are real.
+// Last stage of row plan SP (Ns = n/R): butterflies j = t + it*STEP, outputs
+// x = j + r*Ns stay in registers, v[it]; `valid` tells which are real.  Where
+// two butterflies per thread cover the stage, half of them is the step (even
+// loads); else T.
 template <class SP, int T>
 struct RowLast {
   using G = Stg<SP, SP::S - 1>;
   static constexpr int R = G::R;
   static constexpr int NS = G::NS;
-  static constexpr int IT = (G::NB + T - 1) / T;
+  static constexpr int STEP = (G::NB > T && G::NB % 2 == 0 && G::NB / 2 <= T) ? G::NB / 2 : T;
+  static constexpr int IT = (G::NB + STEP - 1) / STEP;
   static_assert(G::NB == G::NS && G::NB % 16 == 0, "last stage: k = j");
-  __device__ __forceinline__ static bool valid(int t, int it) { return G::NB % T == 0 || t + it * T < G::NB; }
+  __device__ __forceinline__ static bool valid(int t, int it) { return t < STEP && t + it * STEP < G::NB; }
 };
 
 template <class SP, int T, bool INV>
@@ -249,13 +233,13 @@ __device__ __forceinline__ void row_stage_last(const float2* __restrict__ in, in
 #pragma unroll
   for (int it = 0; it < L::IT; ++it) {
     if (!L::valid(t, it)) break;
-    const int j = t + it * T;
+    const int j = t + it * L::STEP;
     const float2* src = in + rp2(j);
     float2 u[1][L::R];
 #pragma unroll
     for (int r = 0; r < L::R; ++r) u[0][r] = src[r * LB];
     twiddle_tab<L::R, L::NS, INV, 1>(u, j);
-    Dft<L::R, INV>::run(u[0]);
+    DftP<L::R, INV>::run(u[0]);
 #pragma unroll
     for (int r = 0; r < L::R; ++r) v[it][r] = u[0][r];
   }

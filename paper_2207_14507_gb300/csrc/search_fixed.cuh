@@ -109,78 +109,109 @@ __device__ __forceinline__ void row_forward_body(const PassArgs& a, int is, int 
   float2* o0 = a.spec + ((size_t)ws * H + y0) * Wh;
   float2* o1 = o0 + Wh;
   using LS = Stg<SP, SP::S - 1>;
-  constexpr bool kShflSplit = SP::S == 3 && LS::NB == T && T % 32 == 0 && LS::R % 2 == 0;
-  if constexpr (kShflSplit) {
-    // The last stage with butterflies j and Ns - j on partner lanes l and
-    // l ^ 16 of one warp (j = 0 and Ns/2, their own mirrors, share lane pair
-    // 0): output x = j + r*Ns has its mirror W - x at r' = R-1-r of butterfly
-    // Ns - j, so the split of z = G_a + i G_b takes the mirror bins by shuffle
-    // instead of a shared-memory round trip.
+  constexpr int R = LS::R, NS = LS::NS, LB = NS / 16 * 18;
+  // Split z = G_a + i G_b into the two rows' half spectra (packed: bin 0 holds
+  // (DC, Nyquist)): bin x < W/2 from z(x) and z(W - x).
+  auto put = [&](int x, float2 zk, float2 zm) {
+    o0[x] = make_float2(0.5f * (zk.x + zm.x), 0.5f * (zk.y - zm.y));
+    o1[x] = make_float2(0.5f * (zk.y + zm.y), 0.5f * (zm.x - zk.x));
+  };
+  auto put0 = [&](float2 z0, float2 zn) {
+    o0[0] = make_float2(z0.x, zn.x);
+    o1[0] = make_float2(z0.y, zn.y);
+  };
+  if constexpr (SP::S == 3) {
     row_stage_ip<SP, 1, T, false>(A, t);
     __syncthreads();
-    constexpr int R = LS::R, NS = LS::NS, LB = NS / 16 * 18;
+  }
+  // Output x = j + r*Ns of the last stage has its mirror W - x at r' = R-1-r of
+  // butterfly Ns - j; j = 0 and Ns/2 are their own mirrors.
+  if constexpr (R % 2 == 0 && NS % 2 == 0 && NS / 2 <= T && NS > T) {
+    // a thread holds both butterflies of a mirror pair: no exchange
+    if (t < NS / 2) {
+      const int ja = t, jb = t == 0 ? NS / 2 : NS - t;
+      float2 va[1][R], vb[1][R];
+      const float2 *sa = A + rp2(ja), *sb = A + rp2(jb);
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        va[0][r] = sa[r * LB];
+        vb[0][r] = sb[r * LB];
+      }
+      twiddle_tab<R, NS, false, 1>(va, ja);
+      DftP<R, false>::run(va[0]);
+      twiddle_tab<R, NS, false, 1>(vb, jb);
+      DftP<R, false>::run(vb[0]);
+      if (t == 0) {
+        put0(va[0][0], va[0][R / 2]);
+#pragma unroll
+        for (int r = 1; r < R / 2; ++r) put(r * NS, va[0][r], va[0][R - r]);
+#pragma unroll
+        for (int r = 0; r < R / 2; ++r) put(NS / 2 + r * NS, vb[0][r], vb[0][R - 1 - r]);
+      } else {
+#pragma unroll
+        for (int r = 0; r < R / 2; ++r) {
+          put(ja + r * NS, va[0][r], vb[0][R - 1 - r]);
+          put(jb + r * NS, vb[0][r], va[0][R - 1 - r]);
+        }
+      }
+    }
+  } else if constexpr (R % 2 == 0 && NS % 2 == 0 && T % 32 == 0 && (NS / 2 + 15) / 16 * 32 <= T) {
+    // one butterfly per thread, those of a mirror pair on lanes l and l ^ 16 of
+    // one warp (j = 0 and Ns/2 share lane pair 0): mirror bins by shuffle
     const int p = (t >> 5) * 16 + (t & 15), h = (t >> 4) & 1;
     const int j = p == 0 ? (h ? NS / 2 : 0) : (h ? NS - p : p);
     float2 v[1][R];
-    const float2* src = A + rp2(j);
+    if (p < NS / 2) {
+      const float2* src = A + rp2(j);
 #pragma unroll
-    for (int r = 0; r < R; ++r) v[0][r] = src[r * LB];
-    twiddle_tab<R, NS, false, 1>(v, j);
-    Dft<R, false>::run(v[0]);
+      for (int r = 0; r < R; ++r) v[0][r] = src[r * LB];
+      twiddle_tab<R, NS, false, 1>(v, j);
+      DftP<R, false>::run(v[0]);
+    }
     float2 m[R / 2];
 #pragma unroll
     for (int r = 0; r < R / 2; ++r) {
       m[r].x = __shfl_xor_sync(0xffffffffu, v[0][R - 1 - r].x, 16);
       m[r].y = __shfl_xor_sync(0xffffffffu, v[0][R - 1 - r].y, 16);
     }
+    if (p < NS / 2) {
+#pragma unroll
+      for (int r = 0; r < R / 2; ++r) {
+        if (j == 0 && r == 0) put0(v[0][0], v[0][R / 2]);
+        else put(j + r * NS, v[0][r], j == 0 ? v[0][R - r] : j == NS / 2 ? v[0][R - 1 - r] : m[r]);
+      }
+    }
+  } else if constexpr (R % 2 == 0 && NS == 16 && T == 16) {
+    // one butterfly per thread of a half warp: the mirror's lane is 16 - t
+    float2 v[1][R];
+    const float2* src = A + rp2(t);
+#pragma unroll
+    for (int r = 0; r < R; ++r) v[0][r] = src[r * LB];
+    twiddle_tab<R, NS, false, 1>(v, t);
+    DftP<R, false>::run(v[0]);
 #pragma unroll
     for (int r = 0; r < R / 2; ++r) {
-      const int x = j + r * NS;   // < W/2
-      const float2 zk = v[0][r];
-      float2 P, Q;
-      if (j == 0 && r == 0) {     // bin 0 packs (DC, Nyquist); the Nyquist bin W/2 is r = R/2 here
-        const float2 zn = v[0][R / 2];
-        P = make_float2(zk.x, zn.x);
-        Q = make_float2(zk.y, zn.y);
-      } else {
-        const float2 zm = j == 0 ? v[0][R - r] : j == NS / 2 ? v[0][R - 1 - r] : m[r];
-        P = make_float2(0.5f * (zk.x + zm.x), 0.5f * (zk.y - zm.y));
-        Q = make_float2(0.5f * (zk.y + zm.y), 0.5f * (zm.x - zk.x));
-      }
-      o0[x] = P;
-      o1[x] = Q;
+      float2 m;
+      m.x = __shfl_sync(0xffffffffu, v[0][R - 1 - r].x, (16 - t) & 15, 16);
+      m.y = __shfl_sync(0xffffffffu, v[0][R - 1 - r].y, (16 - t) & 15, 16);
+      if (t == 0 && r == 0) put0(v[0][0], v[0][R / 2]);
+      else put(t + r * NS, v[0][r], t == 0 ? v[0][(R - r) % R] : m);
     }
-    return;
-  }
-  const float2* res = A;
-  row_stage_ip<SP, 1, T, false>(A, t);
-  __syncthreads();
-  if constexpr (SP::S == 3) {
-    row_stage_ip<SP, 2, T, false>(A, t);
+  } else {
+    // the last stage through shared memory
+    row_stage_ip<SP, SP::S - 1, T, false>(A, t);
     __syncthreads();
-  }
-  // split z = G_a + i G_b into the two rows' half spectra (packed: bin 0
-  // holds (DC, Nyquist))
-  constexpr int MI = (Wh + T - 1) / T;
-  const float2* rk = res + rp2(t);
-  const float2* rm = res - t + 2 * ((-t) >> 4);   // + rp2(X) gives rp2(X - t) for X = 0 mod 16
+    constexpr int MI = (Wh + T - 1) / T;
+    const float2* rk = A + rp2(t);
+    const float2* rm = A - t + 2 * ((-t) >> 4);   // + rp2(X) gives rp2(X - t) for X = 0 mod 16
 #pragma unroll
-  for (int m = 0; m < MI; ++m) {
-    const int k = t + m * T;
-    if (Wh % T != 0 && k >= Wh) break;
-    const float2 zk = rk[m * (T / 16 * 18)];
-    float2 P, Q;
-    if (m == 0 && t == 0) {
-      const float2 zn = res[rp2(Wh)];
-      P = make_float2(zk.x, zn.x);
-      Q = make_float2(zk.y, zn.y);
-    } else {
-      const float2 zm = rm[rp2(W - m * T)];
-      P = make_float2(0.5f * (zk.x + zm.x), 0.5f * (zk.y - zm.y));
-      Q = make_float2(0.5f * (zk.y + zm.y), 0.5f * (zm.x - zk.x));
+    for (int m = 0; m < MI; ++m) {
+      const int k = t + m * T;
+      if (Wh % T != 0 && k >= Wh) break;
+      const float2 zk = rk[m * (T / 16 * 18)];
+      if (m == 0 && t == 0) put0(zk, A[rp2(Wh)]);
+      else put(k, zk, rm[rp2(W - m * T)]);
     }
-    o0[k] = P;
-    o1[k] = Q;
   }
 }
 
@@ -229,7 +260,7 @@ __device__ __forceinline__ void row_inverse_fft(const float2* pa, const float2* 
       u[0] = make_float2(a0.x, b0.x);
       u[8] = make_float2(a0.y, b0.y);
     }
-    Dft<16, true>::run(u);
+    DftP<16, true>::run(u);
     row_store16(A, t, u);
   }
   __syncthreads();
@@ -244,7 +275,7 @@ template <class SP, int T, int PPB, bool CG = false>
 __device__ __forceinline__ void row_inverse_body(const PassArgs& a, int ws, int bx, float2* smem, int tx) {
   constexpr int W = SP::N, Wh = W / 2, L = row_len2(W);
   using GL = RowLast<SP, T>;
-  static_assert(PPB == 1 || T % 32 == 0, "row-pair groups must not share a warp (warp-level reductions)");
+  static_assert(T % 16 == 0 && T * PPB % 32 == 0, "row-pair groups in half warps, whole warps in all");
   const int grp = tx / T, t = tx - grp * T;
   const int H = a.H;
   const int pair = bx * PPB + grp;
@@ -254,18 +285,18 @@ __device__ __forceinline__ void row_inverse_body(const PassArgs& a, int ws, int 
   float2 v[GL::IT][GL::R];
   row_inverse_fft<SP, T, CG>(pa, pa + Wh, A, t, v);
   // per thread: max, first arg-max and energy of each row over its outputs,
-  // visited in increasing x (x = t + it*T + r*NS with t + it*T < NS), so a
+  // visited in increasing x (x = t + it*STEP + r*NS with t + it*STEP < NS), so a
   // strictly larger value is the only one that moves the arg-max: the first
   // maximum is kept without comparing indices
   float ma = -INFINITY, mb = -INFINITY;
   int ia = INT_MAX, ib = INT_MAX;
-  float sa = 0.f, sb = 0.f;
+  float2 sq = make_float2(0.f, 0.f);
 #pragma unroll
   for (int r = 0; r < GL::R; ++r) {
 #pragma unroll
     for (int it = 0; it < GL::IT; ++it) {
       if (!GL::valid(t, it)) continue;
-      const int x = t + it * T + r * GL::NS;
+      const int x = t + it * GL::STEP + r * GL::NS;
       const float2 u = v[it][r];
       if (u.x > ma) {
         ma = u.x;
@@ -275,25 +306,36 @@ __device__ __forceinline__ void row_inverse_body(const PassArgs& a, int ws, int 
         mb = u.y;
         ib = x;
       }
-      sa = fmaf(u.x, u.x, sa);
-      sb = fmaf(u.y, u.y, sb);
+      sq = __ffma2_rn(u, u, sq);
     }
   }
   // across the warp: the max by an integer reduction of the order-preserving
-  // key, then the least index among the lanes that hold it; energies by an
-  // FP32 butterfly (warps are combined in double by row_stats_final)
-  const int ka = __reduce_max_sync(0xffffffffu, float_key(ma));
-  const int kb = __reduce_max_sync(0xffffffffu, float_key(mb));
-  ia = __reduce_min_sync(0xffffffffu, float_key(ma) == ka ? ia : INT_MAX);
-  ib = __reduce_min_sync(0xffffffffu, float_key(mb) == kb ? ib : INT_MAX);
+  // key, then the least index among the lanes that hold it (across the half
+  // warp by shuffles where groups share warps); energies by an FP32 butterfly (warps are combined
+  // in double by row_stats_final)
+  constexpr int SEG = T % 32 == 0 ? 32 : 16;
+  if constexpr (SEG == 32) {
+    const int ka = __reduce_max_sync(0xffffffffu, float_key(ma));
+    const int kb = __reduce_max_sync(0xffffffffu, float_key(mb));
+    ia = __reduce_min_sync(0xffffffffu, float_key(ma) == ka ? ia : INT_MAX);
+    ib = __reduce_min_sync(0xffffffffu, float_key(mb) == kb ? ib : INT_MAX);
+    ma = key_float(ka);
+    mb = key_float(kb);
+  } else {
 #pragma unroll
-  for (int o = 16; o; o >>= 1) {
-    sa += __shfl_xor_sync(0xffffffffu, sa, o);
-    sb += __shfl_xor_sync(0xffffffffu, sb, o);
+    for (int o = SEG / 2; o; o >>= 1) {
+      better_f(ma, ia, __shfl_xor_sync(0xffffffffu, ma, o), __shfl_xor_sync(0xffffffffu, ia, o));
+      better_f(mb, ib, __shfl_xor_sync(0xffffffffu, mb, o), __shfl_xor_sync(0xffffffffu, ib, o));
+    }
   }
-  if ((t & 31) == 0) red[t >> 5] = RowRed{key_float(ka), ia, key_float(kb), ib, sa, 0.f, sb, 0.f};
+#pragma unroll
+  for (int o = SEG / 2; o; o >>= 1) {
+    sq.x += __shfl_xor_sync(0xffffffffu, sq.x, o);
+    sq.y += __shfl_xor_sync(0xffffffffu, sq.y, o);
+  }
+  if (t % SEG == 0) red[t / SEG] = RowRed{ma, ia, mb, ib, sq.x, 0.f, sq.y, 0.f};
   __syncthreads();
-  if (t == 0) row_stats_final(red, (T + 31) / 32, a.stats + (size_t)ws * H + 2 * pair);
+  if (t == 0) row_stats_final(red, (T + SEG - 1) / SEG, a.stats + (size_t)ws * H + 2 * pair);
 }
 
 // ---------------------------------------------------------------- wave kernels
@@ -301,13 +343,25 @@ __device__ __forceinline__ void row_inverse_body(const PassArgs& a, int ws, int 
 // blockIdx.y = candidate slot, or with forward units the unit u, whose row
 // spectrum goes to slot a.nitems + u
 template <int DT, class SP, int T, int PPB>
-__global__ void __launch_bounds__(T * PPB) k_row_forward_fx(PassArgs a) {
-  extern __shared__ float4 smem4[];
+__device__ __forceinline__ void row_forward_block(const PassArgs& a, float2* smem) {
   const bool units = a.units || a.share > 1;
   const int u = blockIdx.y;
   if (past_count(a, u, units ? 1 : 0)) return;
-  row_forward_body<DT, SP, T, PPB>(a, units ? unit_first(a, u) : u, units ? a.nitems + u : u, blockIdx.x,
-                                   reinterpret_cast<float2*>(smem4), threadIdx.x);
+  row_forward_body<DT, SP, T, PPB>(a, units ? unit_first(a, u) : u, units ? a.nitems + u : u, blockIdx.x, smem,
+                                   threadIdx.x);
+}
+template <int DT, class SP, int T, int PPB>
+__global__ void __launch_bounds__(T * PPB) k_row_forward_fx(PassArgs a) {
+  extern __shared__ float4 smem4[];
+  row_forward_block<DT, SP, T, PPB>(a, reinterpret_cast<float2*>(smem4));
+}
+// the same with registers allocated for MINB resident blocks per SM (a
+// separate kernel: an explicit bound of 1 changes the allocation of the
+// unbounded one)
+template <int DT, class SP, int T, int PPB, int MINB>
+__global__ void __launch_bounds__(T * PPB, MINB) k_row_forward_mb(PassArgs a) {
+  extern __shared__ float4 smem4[];
+  row_forward_block<DT, SP, T, PPB>(a, reinterpret_cast<float2*>(smem4));
 }
 
 template <class CP, int W, int NC, int MINB>
@@ -350,9 +404,6 @@ __global__ void __launch_bounds__(T * PPB) k_row_inverse_fx(PassArgs a) {
   if (past_count(a, blockIdx.y, 0)) return;
   row_inverse_body<SP, T, PPB>(a, blockIdx.y, blockIdx.x, reinterpret_cast<float2*>(smem4), threadIdx.x);
 }
-// the same with registers allocated for MINB resident blocks per SM (a
-// separate kernel: an explicit bound of 1 changes the allocation of the
-// unbounded one)
 template <class SP, int T, int PPB, int MINB>
 __global__ void __launch_bounds__(T * PPB, MINB) k_row_inverse_mb(PassArgs a) {
   extern __shared__ float4 smem4[];
@@ -590,7 +641,7 @@ __device__ __forceinline__ void finalize_task(const PassArgs& a, int is, int ws,
         if (!SL::valid(tg, it)) break;
 #pragma unroll
         for (int r = 0; r < SL::R; ++r) {
-          const int x = tg + it * T + r * SL::NS;
+          const int x = tg + it * SL::STEP + r * SL::NS;
           if (cdist(x, px, W) <= kHalfWindow) continue;
           if (cdist(2 * p, py, H) <= kHalfWindow) e += (double)V[it][r].x * V[it][r].x;
           if (cdist(2 * p + 1, py, H) <= kHalfWindow) e += (double)V[it][r].y * V[it][r].y;
@@ -756,6 +807,7 @@ constexpr int kFinPairs = 3;
 template <class RS, int RT, class CP, class CS, int RTI = RT>
 struct ShapeDef {
   static constexpr int W = RS::N, H = CP::H;
+  static constexpr int FT = (RTI + 31) / 32 * 32;   // of a row pair in the finalisation: whole warps
   static_assert(CS::N == H, "column plans of one length");
   // NC columns per block, at least MINB resident blocks per SM
   // MODE: 0 plain loads and stores, 1 strip by TMA, 2 strip and fingerprint by TMA
@@ -777,36 +829,40 @@ struct ShapeDef {
   static FixedCol col_inv() {
     return col_entry((void*)k_col_inv_fx<CP, W, NC, MINB, MODE>, NC, MODE);
   }
-  // RIMB: resident row-inverse blocks per SM to allocate registers for (0: no bound)
-  template <int PPB, int RIMB = 0>
+  // RIMB, RFMB: resident row-inverse and row-forward blocks per SM to allocate
+  // registers for (0: no bound)
+  template <int DT, int PPB, int RFMB>
+  static void* row_fwd() {
+    void* f;
+    if constexpr (RFMB > 0) f = (void*)k_row_forward_mb<DT, RS, RT, PPB, RFMB>;
+    else f = (void*)k_row_forward_fx<DT, RS, RT, PPB>;
+    allow_max_dynamic_smem(f);
+    return f;
+  }
+  template <int PPB, int RIMB = 0, int RFMB = 0>
   static FixedRow row() {
     FixedRow r{};
     r.ppb = PPB;
     r.threads = RT;
     r.threads_inv = RTI;
     r.smem = row_fx_smem<W>(PPB);
-    r.fwd[kF32] = (void*)k_row_forward_fx<kF32, RS, RT, PPB>;
-    r.fwd[kF16] = (void*)k_row_forward_fx<kF16, RS, RT, PPB>;
-    r.fwd[kBF16] = (void*)k_row_forward_fx<kBF16, RS, RT, PPB>;
-    r.fwd[kF16P] = (void*)k_row_forward_fx<kF16P, RS, RT, PPB>;
-    r.fwd[kBF16P] = (void*)k_row_forward_fx<kBF16P, RS, RT, PPB>;
+    r.fwd[kF32] = row_fwd<kF32, PPB, RFMB>();
+    r.fwd[kF16] = row_fwd<kF16, PPB, RFMB>();
+    r.fwd[kBF16] = row_fwd<kBF16, PPB, RFMB>();
+    r.fwd[kF16P] = row_fwd<kF16P, PPB, RFMB>();
+    r.fwd[kBF16P] = row_fwd<kBF16P, PPB, RFMB>();
     if constexpr (RIMB > 0) r.inv = (void*)k_row_inverse_mb<RS, RTI, PPB, RIMB>;
     else r.inv = (void*)k_row_inverse_fx<RS, RTI, PPB>;
-    r.fin = (void*)k_finalize_fx<RS, RTI, kFinPairs>;
-    r.fin_threads = RTI * kFinPairs;
+    r.fin = (void*)k_finalize_fx<RS, FT, kFinPairs>;
+    r.fin_threads = FT * kFinPairs;
     r.fin_smem = row_fx_smem<W>(kFinPairs);
-    allow(k_finalize_fx<RS, RTI, kFinPairs>);
-    allow(k_row_forward_fx<kF32, RS, RT, PPB>);
-    allow(k_row_forward_fx<kF16, RS, RT, PPB>);
-    allow(k_row_forward_fx<kBF16, RS, RT, PPB>);
-    allow(k_row_forward_fx<kF16P, RS, RT, PPB>);
-    allow(k_row_forward_fx<kBF16P, RS, RT, PPB>);
+    allow(k_finalize_fx<RS, FT, kFinPairs>);
     allow_max_dynamic_smem(r.inv);
     return r;
   }
   // PRT threads per row pair (PRT * PPB per block, also the column task's
   // threads): chosen so that every stage holds one butterfly per thread
-  template <int PRT, int PPB, int NC>
+  template <int PRT, int PPB, int NC, class PRS = RS>
   static FixedPersist persist() {
     FixedPersist f{};
     f.ppb = PPB;
@@ -816,9 +872,9 @@ struct ShapeDef {
     const size_t cs = col_fx_smem(H, NC);
     const size_t fs = row_fx_smem<W>(PPB);
     f.smem = std::max(rs, std::max(cs, fs));
-    f.fn[kF32] = (void*)k_persist<kF32, RS, PRT, PPB, CS, NC>;
-    f.fn[kF16] = (void*)k_persist<kF16, RS, PRT, PPB, CS, NC>;
-    f.fn[kBF16] = (void*)k_persist<kBF16, RS, PRT, PPB, CS, NC>;
+    f.fn[kF32] = (void*)k_persist<kF32, PRS, PRT, PPB, CS, NC>;
+    f.fn[kF16] = (void*)k_persist<kF16, PRS, PRT, PPB, CS, NC>;
+    f.fn[kBF16] = (void*)k_persist<kBF16, PRS, PRT, PPB, CS, NC>;
     for (int d = 0; d < 3; ++d) {
       allow_max_dynamic_smem(f.fn[d]);
       int nb = 0;

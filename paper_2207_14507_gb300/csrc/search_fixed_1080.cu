@@ -4,17 +4,23 @@
 namespace prnu {
 
 FixedShape fixed_shape_1080() {
-  using D = ShapeDef<Spec<1920, 16, 12, 10>, 192, ColPlan<1080, 36, 30>, Spec<1080, 9, 12, 10>, 160>;
+  // Rows of 1920 = 16 x 15 x 8 points by 128 threads a row pair: 120, 128 and
+  // 2 x 120 butterflies, where 16 x 12 x 10 by 192 threads left 72 of them idle
+  // in the warp's gathers.  Row forward 4.71 -> 4.18 us a candidate (FP32; FP16
+  // 4.30 -> 3.68), row inverse 2.50 -> 2.30.  Registers for 8 blocks per SM each:
+  // the row inverse takes 2.46 unbounded (50 registers, 10 blocks), 2.33 for 7,
+  // the row forward 4.43 unbounded, 4.17 for 7, 4.30 for 9.
+  using D = ShapeDef<Spec<1920, 16, 15, 8>, 128, ColPlan<1080, 36, 30>, Spec<1080, 9, 12, 10>>;
   // us per candidate of the column variants (FP32 / FP16 fingerprints, waves of
   // 512): 4-column strips, mode 4 with 4 blocks per SM - / 3.83, mode 3 with 3
   // blocks 4.25 / 4.33, mode 2 4.70 / 4.83, mode 1 4.61 / 4.73, mode 0 5.50,
   // 8-column strips 7.40 (mode 1), 6.7 (mode 3), 4.04 (mode 4, 2 blocks).  The
   // three-stage plan: 5.38 / 5.30.
-  return D::make({D::row<2>(), D::row<1, 8>()},
+  return D::make({D::row<2>(), D::row<1, 8, 8>()},
                  {D::col<4, 4, 4>(), D::col<4, 3, 2>(), D::col<4, 3, 1>(), D::col<4, 3, 0>(), D::col<8, 1, 1>(),
                   D::col<4, 3, 3>()},
                  {D::col_fwd<4, 4>(), D::col_inv<4, 3>(), D::col_inv<4, 3, 3>(), D::col_inv<4, 4, 4>()},
-                 D::persist<192, 2, 4>());
+                 D::persist<192, 2, 4, Spec<1920, 16, 12, 10>>());
 }
 
 }  // namespace prnu
