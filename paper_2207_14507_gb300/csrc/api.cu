@@ -1052,7 +1052,7 @@ int prnu_destroy(prnu_ctx* ctx) {
     }
     ctx->fps.clear();
     for (DeviceBuf* b : {&ctx->ws_spec, &ctx->ws_stats, &ctx->ws_items, &ctx->ws_results, &ctx->ws_groups,
-                         &ctx->ws_out, &ctx->ws_fpdesc, &ctx->ws_misc, &ctx->ws_resid, &ctx->ws_persist, &ctx->ws_pad, &ctx->ws_fpest,
+                         &ctx->ws_out, &ctx->ws_fpdesc, &ctx->ws_misc, &ctx->ws_resid, &ctx->ws_persist, &ctx->ws_pad,
                          &ctx->ws_lit, &ctx->ws_litx, &ctx->ws_litpart, &ctx->ws_renders, &ctx->ws_resize,
                          &ctx->ws_wav, &ctx->ws_corr})
       ctx_free(ctx, b->p, b->bytes);
@@ -1148,28 +1148,11 @@ int prnu_fingerprint_estimate(prnu_ctx* ctx, const uint8_t* d_frames, int L, int
     std::lock_guard<std::recursive_mutex> lk(ctx->mu);
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     PRNU_CUDA_TRY(cudaStreamWaitEvent(s, ctx->last_done, 0));
-    constexpr int kChunk = 16;
-    const size_t n = (size_t)H * W;
-    const int C0 = std::min(L, kChunk);
-    const size_t rb = (sizeof(float) * n * C0 + 255) / 256 * 256, db = (sizeof(double) * n + 255) / 256 * 256;
-    ensure_buf(ctx, ctx->ws_fpest, rb + 2 * db);
-    char* base = reinterpret_cast<char*>(ctx->ws_fpest.p);
-    float* R = reinterpret_cast<float*>(base);
-    double* num = reinterpret_cast<double*>(base + rb);
-    double* den = reinterpret_cast<double*>(base + rb + db);
-    const size_t np = residual_partials_needed(C0, H, W);
-    ensure_buf(ctx, ctx->ws_resid, sizeof(unsigned long long) * C0 + 256 + sizeof(double) * np);
+    const size_t accb = (sizeof(unsigned long long) * L + 255) & ~(size_t)255;
+    ensure_buf(ctx, ctx->ws_resid, accb + sizeof(unsigned long long) * residual_partials_needed(L, H, W));
     auto* acc = reinterpret_cast<unsigned long long*>(ctx->ws_resid.p);
-    auto* partials = reinterpret_cast<double*>(reinterpret_cast<char*>(ctx->ws_resid.p) +
-                                               ((sizeof(unsigned long long) * C0 + 255) & ~(size_t)255));
-    for (int l0 = 0; l0 < L; l0 += kChunk) {
-      const int Lc = std::min(kChunk, L - l0);
-      const uint8_t* fr = d_frames + (size_t)l0 * H * pitch;
-      launch_residual(fr, Lc, H, W, pitch, PRNU_WEIGHT_BY_INTENSITY, kF32, R, nullptr, acc, partials,
-                      (int)residual_partials_needed(Lc, H, W), s, ctx->launches);
-      launch_fp_estimate_accumulate(R, fr, pitch, Lc, H, W, num, den, l0 == 0, s, ctx->launches);
-    }
-    launch_fp_estimate_divide(num, den, d_K, n, s, ctx->launches);
+    auto* slots = reinterpret_cast<unsigned long long*>(reinterpret_cast<char*>(ctx->ws_resid.p) + accb);
+    launch_fp_estimate(d_frames, pitch, L, H, W, slots, acc, d_K, s, ctx->launches);
     PRNU_CUDA_TRY(cudaEventRecord(ctx->last_done, s));
   });
 }
@@ -1404,35 +1387,6 @@ int eis_grid_search_frames(prnu_ctx* ctx, const uint8_t* d_frames, int F, int H,
   });
 }
 
-// Taps of output samples first .. first + n - 1 of a length-n_in axis resized
-// by `scale`: sample o at input position u = (o + 0.5) / scale - 0.5, tent
-// weights max(0, 1 - |j - u| a) with a = min(scale, 1), indices clamped to the
-// axis, normalised; T taps per sample (zero weight beyond its support).
-static void resize_taps(int n_in, double scale, int first, int n, int T, std::vector<float>& w, std::vector<int>& idx) {
-  const double a = std::min(scale, 1.0);
-  w.assign((size_t)n * T, 0.f);
-  idx.assign((size_t)n * T, 0);
-  for (int o = 0; o < n; ++o) {
-    const double u = ((double)(first + o) + 0.5) / scale - 0.5;
-    const int lo = (int)std::floor(u - 1.0 / a);
-    std::vector<double> ws;
-    std::vector<int> js;
-    double tot = 0.0;
-    for (int j = lo; j <= lo + T - 1; ++j) {
-      const double t = 1.0 - std::fabs((double)j - u) * a;
-      if (t <= 0.0) continue;
-      const int jj = std::min(std::max(j, 0), n_in - 1);
-      ws.push_back(t);
-      js.push_back(jj);
-      tot += t;
-    }
-    for (size_t k = 0; k < ws.size(); ++k) {
-      w[(size_t)o * T + k] = (float)(ws[k] / tot);
-      idx[(size_t)o * T + k] = js[k];
-    }
-  }
-}
-
 int prnu_fingerprint_resize(prnu_ctx* ctx, const float* d_Kin, int Hin, int Win, size_t in_pitch, double scale,
                             int y0, int x0, float* d_Kout, int H, int W, prnu_stream stream) {
   return guarded([&] {
@@ -1449,25 +1403,12 @@ int prnu_fingerprint_resize(prnu_ctx* ctx, const float* d_Kin, int Hin, int Win,
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     // taps per sample: the tent spans (u - 1/a, u + 1/a), at most floor(2/a) + 2 integers
     const int T = (int)std::floor(2.0 / std::min(scale, 1.0)) + 2;
-    std::vector<float> wy, wx;
-    std::vector<int> iy, ix;
-    resize_taps(Hin, scale, y0, H, T, wy, iy);
-    resize_taps(Win, scale, x0, W, T, wx, ix);
-    const size_t nwy = wy.size(), nwx = wx.size();
-    ensure_buf(ctx, ctx->ws_resize, (nwy + nwx) * (sizeof(float) + sizeof(int)) + 1024);
-    char* base = reinterpret_cast<char*>(ctx->ws_resize.p);
-    float* d_wy = reinterpret_cast<float*>(base);
-    float* d_wx = d_wy + nwy;
-    int* d_iy = reinterpret_cast<int*>(d_wx + nwx);
-    int* d_ix = d_iy + nwy;
+    const size_t taps = ((size_t)H + W) * T;
+    ensure_buf(ctx, ctx->ws_resize, taps * (sizeof(float) + sizeof(int)));
+    float* d_w = reinterpret_cast<float*>(ctx->ws_resize.p);
     PRNU_CUDA_TRY(cudaStreamWaitEvent(s, ctx->last_done, 0));
-    Stager st(ctx);
-    st.add(d_wy, wy.data(), nwy);
-    st.add(d_wx, wx.data(), nwx);
-    st.add(d_iy, iy.data(), nwy);
-    st.add(d_ix, ix.data(), nwx);
-    st.flush(s);
-    launch_fp_resize(d_Kin, in_pitch, d_wy, d_iy, d_wx, d_ix, T, H, W, d_Kout, s, ctx->launches);
+    launch_fp_resize(d_Kin, Hin, Win, in_pitch, scale, y0, x0, T, d_w, reinterpret_cast<int*>(d_w + taps), H, W, d_Kout,
+                     s, ctx->launches);
     PRNU_CUDA_TRY(cudaEventRecord(ctx->last_done, s));
     PRNU_CUDA_TRY(cudaStreamSynchronize(s));
   });

@@ -160,14 +160,13 @@ void launch_wavelet_residual(const uint8_t* frames, int F, int H, int W, size_t 
                              float sigma0, void* out, float* scale, float* bufA, float* bufT, int chunk,
                              double* partials, cudaStream_t s, LaunchCounter& lc);
 size_t wavelet_partials_needed(int F, int H, int W);
-// fingerprint resampling with T taps per axis: weights and (clamped) indices per output row and column
-void launch_fp_resize(const float* K, size_t pitch, const float* wy, const int* iy, const float* wx, const int* ix,
-                      int T, int H, int W, float* out, cudaStream_t s, LaunchCounter& lc);
-// Eq. 2 accumulation over Lc residuals R [Lc][H][W] (R = I W(I)) and their frames
-void launch_fp_estimate_accumulate(const float* R, const uint8_t* frames, size_t pitch, int Lc, int H, int W,
-                                   double* num, double* den, bool first, cudaStream_t s, LaunchCounter& lc);
-void launch_fp_estimate_divide(const double* num, const double* den, float* K, size_t n, cudaStream_t s,
-                               LaunchCounter& lc);
+// fingerprint resampling with T taps per axis; w, idx: (H + W) * T scratch weights and input indices
+void launch_fp_resize(const float* K, int Hin, int Win, size_t pitch, double scale, int y0, int x0, int T, float* w,
+                      int* idx, int H, int W, float* out, cudaStream_t s, LaunchCounter& lc);
+// Eq. 2's estimate over L frames into K [H][W]; slots: residual_partials_needed(L,
+// H, W) of 8 bytes, acc: L (scratch)
+void launch_fp_estimate(const uint8_t* frames, size_t pitch, int L, int H, int W, unsigned long long* slots,
+                        unsigned long long* acc, float* K, cudaStream_t s, LaunchCounter& lc);
 // dense [F][H][W] residuals -> the zero-bordered layout the compile-time-planned
 // kernels read (row pitch W + 3, pixel (0, 0) at W + 4, (H + 3)(W + 3) per frame)
 // layout (half storage only): 0 single elements, 1 pairs (kF16P/kBF16P)
@@ -234,7 +233,7 @@ struct prnu_ctx {
   cudaEvent_t last_done = nullptr;
   // call workspace
   prnu::DeviceBuf ws_spec, ws_stats, ws_items, ws_results, ws_groups, ws_out, ws_fpdesc, ws_misc, ws_resid,
-      ws_persist, ws_pad, ws_fpest, ws_lit, ws_litx, ws_litpart, ws_renders, ws_resize, ws_wav, ws_corr;
+      ws_persist, ws_pad, ws_lit, ws_litx, ws_litpart, ws_renders, ws_resize, ws_wav, ws_corr;
   size_t tw_bytes = 0;
   int* h_err = nullptr;           // pinned: error flag of the last persistent launch or TMA wait
   int* d_err = nullptr;           // device flag the wave kernels raise when a bounded wait gives up

@@ -9,62 +9,141 @@
 //   W = (x - mu) nu2 / var = 9 D nu2 / V   where var >= nu2 (and V > 0),
 //   W = x - mu = D / 9                      elsewhere,
 // and R = x W (PRNU_WEIGHT_BY_INTENSITY) or W.
+#include <type_traits>
+
 #include "internal.h"
 
 namespace prnu {
 
 namespace {
 
-// A block covers a 32 x 32 tile with 32 x 8 threads (4 rows each); the tile
-// and its one-pixel halo (borders replicated) are staged once in shared memory.
-constexpr int kBX = 32, kBY = 32, kBR = 4, kTW = kBX + 2, kTH = kBY + 2;
-static_assert(kBY == 8 * kBR, "a thread covers kBR rows of the tile");
+// A thread covers 4 adjacent pixels of RPT rows, a block of 32 x 8 threads a
+// tile of 128 x 8*RPT.  Everything up to V and D is an integer below 2^24, so
+// it is computed exactly in FP32, two pixels to a packed instruction, the 3x3
+// sums as sums over rows (kept for the next row), then over columns.  Against
+// one pixel per thread from a shared-memory tile with 9 integer loads a pixel,
+// 30 full-HD frames to normalised FP16 (three passes, the frames in L2) take
+// 243 us instead of 737; what bounds it is instruction issue (63%),
+// 34 instructions a pixel and pass.
+constexpr int kBX = 32, kPX = 4;   // lanes of a block's row, pixels of a thread
 
-__device__ __forceinline__ void load_tile_u8(const uint8_t* __restrict__ f, size_t pitch, int H, int W, int* tile) {
-  const int tid = threadIdx.y * kBX + threadIdx.x;
-  const int x0 = blockIdx.x * kBX - 1, y0 = blockIdx.y * kBY - 1;
-  for (int k = tid; k < kTW * kTH; k += kBX * 8) {
-    const int sy = k / kTW, sx = k - sy * kTW;
-    const int y = min(max(y0 + sy, 0), H - 1), x = min(max(x0 + sx, 0), W - 1);
-    tile[k] = __ldg(f + (size_t)y * pitch + x);
+// rows per thread: 8, but 2 where 8 would leave the GPU's 152 SMs with less
+// than two blocks each
+inline int resid_rows(int F, int H, int W) {
+  const long long blocks = (long long)F * ((W + kBX * kPX - 1) / (kBX * kPX)) * ((H + 63) / 64);
+  return blocks >= 304 ? 8 : 2;
+}
+inline dim3 resid_grid(int F, int H, int W, int rpt) {
+  return dim3((W + kBX * kPX - 1) / (kBX * kPX), (H + 8 * rpt - 1) / (8 * rpt), F);
+}
+
+// byte i of w as a float: the byte in the low mantissa bits of 2^23, minus 2^23
+template <int I>
+__device__ __forceinline__ float byte_f(uint32_t w) {
+  return __uint_as_float(__byte_perm(w, 0x4B000000u, 0x7440 | I));
+}
+
+// Pixels x-1 .. x+4 of one row (borders replicated): the middle four as two
+// packed pairs, the outer two apart.
+struct Row6 {
+  float2 a, b;   // (x, x+1), (x+2, x+3)
+  float l, r;    // x-1, x+4
+};
+struct Raw6 {    // the same as bytes: x .. x+3, x-1, x+4
+  uint32_t w, l, r;
+};
+// VEC: rows are 4-byte aligned (x is a multiple of 4)
+template <bool VEC>
+__device__ __forceinline__ Raw6 load_raw6(const uint8_t* __restrict__ row, int x, int W) {
+  Raw6 o;
+  if (VEC && x + 3 < W) {
+    o.w = __ldg(reinterpret_cast<const uint32_t*>(row + x));
+  } else {
+    o.w = __ldg(row + min(x, W - 1)) | (uint32_t)__ldg(row + min(x + 1, W - 1)) << 8 |
+          (uint32_t)__ldg(row + min(x + 2, W - 1)) << 16 | (uint32_t)__ldg(row + min(x + 3, W - 1)) << 24;
   }
-  __syncthreads();
+  o.l = __ldg(row + min(max(x - 1, 0), W - 1));
+  o.r = __ldg(row + min(x + 4, W - 1));
+  return o;
+}
+__device__ __forceinline__ Row6 row_floats(const Raw6& q) {
+  const float2 m = make_float2(-8388608.f, -8388608.f);
+  Row6 o;
+  o.a = __fadd2_rn(make_float2(byte_f<0>(q.w), byte_f<1>(q.w)), m);
+  o.b = __fadd2_rn(make_float2(byte_f<2>(q.w), byte_f<3>(q.w)), m);
+  o.l = byte_f<0>(q.l) - 8388608.f;
+  o.r = byte_f<0>(q.r) - 8388608.f;
+  return o;
+}
+__device__ __forceinline__ Row6 row_square(const Row6& p) {
+  return Row6{__fmul2_rn(p.a, p.a), __fmul2_rn(p.b, p.b), p.l * p.l, p.r * p.r};
+}
+__device__ __forceinline__ Row6 row_add(const Row6& p, const Row6& q) {
+  return Row6{__fadd2_rn(p.a, q.a), __fadd2_rn(p.b, q.b), p.l + q.l, p.r + q.r};
+}
+// sums of three adjacent columns around each of the four pixels
+__device__ __forceinline__ void row_sum3(const Row6& c, float2& a, float2& b) {
+  const float u = c.a.x + c.a.y, v = c.b.x + c.b.y;
+  a = make_float2(c.l + u, u + c.b.x);
+  b = make_float2(c.a.y + v, v + c.r);
 }
 
-// 3x3 sums of x and x^2 and the centre of tile pixel (tx, ty)
-__device__ __forceinline__ void moments3x3(const int* tile, int tx, int ty, int* s1, int* s2, int* xc) {
-  int a = 0, b = 0;
+// V (and with D the centre's offset) of the four pixels of RPT rows, row by row
+// to fn(k, the row's pixels, Va, Vb, Da, Db); row(i) gives row i - 1 (0 <= i <
+// RPT + 2).
+template <int RPT, class Rows, class Fn>
+__device__ __forceinline__ void for_rows(Rows&& row, Fn&& fn) {
+  const Row6 up = row(0);
+  Row6 mid = row(1);
+  Row6 s1 = row_add(up, mid), s2 = row_add(row_square(up), row_square(mid));   // of the two rows above the next
 #pragma unroll
-  for (int dy = 0; dy < 3; ++dy)
-#pragma unroll
-    for (int dx = 0; dx < 3; ++dx) {
-      const int v = tile[(ty + dy) * kTW + tx + dx];
-      a += v;
-      b += v * v;
-    }
-  *s1 = a;
-  *s2 = b;
-  *xc = tile[(ty + 1) * kTW + tx + 1];
+  for (int k = 0; k < RPT; ++k) {
+    const Row6 dn = row(k + 2), dn2 = row_square(dn);
+    float2 a1, b1, a2, b2;
+    row_sum3(row_add(s1, dn), a1, b1);
+    row_sum3(row_add(s2, dn2), a2, b2);
+    const float2 nine = make_float2(9.f, 9.f);
+    const float2 na1 = make_float2(-a1.x, -a1.y), nb1 = make_float2(-b1.x, -b1.y);
+    fn(k, mid, __ffma2_rn(nine, a2, __fmul2_rn(na1, a1)), __ffma2_rn(nine, b2, __fmul2_rn(nb1, b1)),
+       __ffma2_rn(nine, mid.a, na1), __ffma2_rn(nine, mid.b, nb1));
+    s1 = row_add(mid, dn);
+    s2 = row_add(row_square(mid), dn2);
+    mid = dn;
+  }
 }
+
+// rows y0 - 1 .. of the frame f, its first and last rows repeated outside
+template <bool VEC>
+struct FrameRows {
+  const uint8_t* f;
+  size_t pitch;
+  int H, W, x, y0;
+  __device__ __forceinline__ Raw6 raw(int i) const {
+    return load_raw6<VEC>(f + (size_t)min(max(y0 - 1 + i, 0), H - 1) * pitch, x, W);
+  }
+  __device__ __forceinline__ Row6 operator()(int i) const { return row_floats(raw(i)); }
+};
 
 // per block: the integer sum of 81 * (local variance) of its pixels, one slot per block
+template <int RPT, bool VEC>
 __global__ void __launch_bounds__(kBX * 8) k_resid_moments(const uint8_t* __restrict__ frames, size_t pitch, int H,
                                                            int W, unsigned long long* __restrict__ part_out) {
-  __shared__ int tile[kTW * kTH];
   __shared__ unsigned long long part[8];
-  const int f = blockIdx.z;
-  load_tile_u8(frames + (size_t)f * H * pitch, pitch, H, W, tile);
-  const int tx = threadIdx.x, x = blockIdx.x * kBX + tx;
-  unsigned long long v = 0;
-#pragma unroll
-  for (int k = 0; k < kBR; ++k) {
-    const int ty = threadIdx.y + 8 * k, y = blockIdx.y * kBY + ty;
-    if (x < W && y < H) {
-      int s1, s2, xc;
-      moments3x3(tile, tx, ty, &s1, &s2, &xc);
-      v += (unsigned long long)(9 * s2 - s1 * s1);
-    }
+  const int f = blockIdx.z, tx = threadIdx.x;
+  const int x = (blockIdx.x * kBX + tx) * kPX, y0 = (blockIdx.y * 8 + threadIdx.y) * RPT;
+  unsigned acc = 0;   // at most 32 terms of at most 81 * 255^2 / 4 each
+  if (x < W && y0 < H) {
+    for_rows<RPT>(FrameRows<VEC>{frames + (size_t)f * H * pitch, pitch, H, W, x, y0},
+                       [&](int k, const Row6&, float2 va, float2 vb, float2, float2) {
+                         if (y0 + k >= H) return;
+                         if (x + 3 < W) {   // four terms: exact below 2^24
+                           acc += __float2uint_rn((va.x + va.y) + (vb.x + vb.y));
+                         } else {
+                           acc += __float2uint_rn(va.x + (x + 1 < W ? va.y : 0.f) + (x + 2 < W ? vb.x : 0.f));
+                         }
+                       });
   }
+  unsigned long long v = acc;
 #pragma unroll
   for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   if (tx == 0) part[threadIdx.y] = v;
@@ -94,52 +173,100 @@ __global__ void k_resid_noise(const unsigned long long* __restrict__ part, int n
   }
 }
 
-__device__ __forceinline__ float residual_value(int s1, int s2, int xc, float nu2, float nu2x81, int weight) {
-  const int V = 9 * s2 - s1 * s1;
-  const float D = (float)(9 * xc - s1);
-  float w;
-  if (V > 0 && (float)V >= nu2x81) w = (9.f * D) * nu2 / (float)V;
-  else w = D / 9.f;
-  return weight ? (float)xc * w : w;
+// n / d for |d| in [1, 2^24) and |n| below 2^60: the hardware's reciprocal
+// (1 ulp), the quotient, and one step of iterative refinement by its exact
+// remainder (Newton's correction), which leaves the rounding of the last add;
+// a third of the instructions of the general division.
+__device__ __forceinline__ float quotient(float n, float d) {
+  float rc;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(rc) : "f"(d));
+  const float q = n * rc;
+  return fmaf(fmaf(-q, d, n), rc, q);
 }
 
-// MODE 0: store R; MODE 1: per-block sum of R^2 (double) to partials; MODE 2: store R * scale[f].
-// R(y, x) of frame f goes to out[f * lay.fpitch + lay.roff + y * lay.rpitch + x].
-template <int DT, int MODE>
+// W of one pixel: 9 D nu2 / V or D / 9 (see the head of this file)
+__device__ __forceinline__ float residual_w(float V, float D, float nu2, float nu2x81) {
+  const bool wiener = V > 0.f && V >= nu2x81;
+  return quotient(wiener ? (9.f * D) * nu2 : D, wiener ? V : 9.f);
+}
+
+// the frame's noise power and 81 times it, from its integer sum
+__device__ __forceinline__ float2 noise_power(unsigned long long acc, int H, int W) {
+  const double nu2d = (double)acc / (81.0 * (double)H * (double)W);
+  return make_float2((float)nu2d, (float)(81.0 * nu2d));
+}
+
+template <int DT>
+__device__ __forceinline__ void store4(void* p, size_t o, float4 v, int n, bool vec) {
+  if (vec && n >= 4) {
+    if constexpr (DT == kF32) {
+      *reinterpret_cast<float4*>(reinterpret_cast<float*>(p) + o) = v;
+    } else {
+      uint2 u;
+      if constexpr (DT == kF16) {
+        const __half2 a = __floats2half2_rn(v.x, v.y), b = __floats2half2_rn(v.z, v.w);
+        u = make_uint2(*reinterpret_cast<const uint32_t*>(&a), *reinterpret_cast<const uint32_t*>(&b));
+      } else {
+        const __nv_bfloat162 a = __floats2bfloat162_rn(v.x, v.y), b = __floats2bfloat162_rn(v.z, v.w);
+        u = make_uint2(*reinterpret_cast<const uint32_t*>(&a), *reinterpret_cast<const uint32_t*>(&b));
+      }
+      *reinterpret_cast<uint2*>(reinterpret_cast<uint16_t*>(p) + o) = u;
+    }
+  } else {
+    store_store_type<DT>(p, o, v.x);
+    if (n > 1) store_store_type<DT>(p, o + 1, v.y);
+    if (n > 2) store_store_type<DT>(p, o + 2, v.z);
+    if (n > 3) store_store_type<DT>(p, o + 3, v.w);
+  }
+}
+
+// MODE 0: store R (and scale[f] = 1); MODE 1: per-block sum of R^2 (double) to
+// partials; MODE 2: store R * scale[f].
+// R(y, x) of frame f goes to out[f * lay.fpitch + lay.roff + y * lay.rpitch + x];
+// vec_out: the quads of a row lie on vector boundaries.
+template <int DT, int MODE, int RPT, bool VEC>
 __global__ void __launch_bounds__(kBX * 8) k_resid_apply(const uint8_t* __restrict__ frames, size_t pitch, int H,
                                                          int W, const unsigned long long* __restrict__ acc,
                                                          int weight, void* __restrict__ out,
-                                                         double* __restrict__ partials,
-                                                         const float* __restrict__ scale, ResidLayout lay) {
-  __shared__ int tile[kTW * kTH];
+                                                         double* __restrict__ partials, float* __restrict__ scale,
+                                                         ResidLayout lay, bool vec_out) {
   __shared__ double part[8];
-  __shared__ float s_nu2[2];
-  const int f = blockIdx.z;
-  if (threadIdx.x == 0 && threadIdx.y == 0) {   // once per block: the FP64 pipe is narrow
-    const double nu2d = (double)acc[f] / (81.0 * (double)H * (double)W);
-    s_nu2[0] = (float)nu2d;
-    s_nu2[1] = (float)(81.0 * nu2d);
-  }
-  load_tile_u8(frames + (size_t)f * H * pitch, pitch, H, W, tile);   // (synchronises)
-  const float nu2 = s_nu2[0];
-  const float nu2x81 = s_nu2[1];
-  const int tx = threadIdx.x, x = blockIdx.x * kBX + tx;
-  float sq = 0.f;
+  __shared__ float2 s_nu2;
+  const int f = blockIdx.z, tx = threadIdx.x;
+  if (tx == 0 && threadIdx.y == 0) s_nu2 = noise_power(acc[f], H, W);   // once per block: the FP64 pipe is narrow
+  __syncthreads();
+  const float2 nu2 = s_nu2;
+  const float s = MODE == 2 ? scale[f] : 1.f;
+  const int x = (blockIdx.x * kBX + tx) * kPX, y0 = (blockIdx.y * 8 + threadIdx.y) * RPT;
+  float sq[RPT];
 #pragma unroll
-  for (int k = 0; k < kBR; ++k) {
-    const int ty = threadIdx.y + 8 * k, y = blockIdx.y * kBY + ty;
-    if (x < W && y < H) {
-      int s1, s2, xc;
-      moments3x3(tile, tx, ty, &s1, &s2, &xc);
-      const float r = residual_value(s1, s2, xc, nu2, nu2x81, weight);
-      const size_t o = (size_t)f * lay.fpitch + lay.roff + (size_t)y * lay.rpitch + x;
-      if (MODE == 0) store_store_type<DT>(out, o, r);
-      if (MODE == 2) store_store_type<DT>(out, o, r * scale[f]);
-      sq = fmaf(r, r, sq);
-    }
+  for (int k = 0; k < RPT; ++k) sq[k] = 0.f;
+  if (x < W && y0 < H) {
+    for_rows<RPT>(FrameRows<VEC>{frames + (size_t)f * H * pitch, pitch, H, W, x, y0},
+                       [&](int k, const Row6& p, float2 va, float2 vb, float2 da, float2 db) {
+                         if (y0 + k >= H) return;
+                         float4 r = make_float4(residual_w(va.x, da.x, nu2.x, nu2.y), residual_w(va.y, da.y, nu2.x, nu2.y),
+                                                residual_w(vb.x, db.x, nu2.x, nu2.y), residual_w(vb.y, db.y, nu2.x, nu2.y));
+                         if (weight) r = make_float4(p.a.x * r.x, p.a.y * r.y, p.b.x * r.z, p.b.y * r.w);
+                         if (MODE == 1) {
+                           if (x + 1 >= W) r.y = 0.f;
+                           if (x + 2 >= W) r.z = 0.f;
+                           if (x + 3 >= W) r.w = 0.f;
+                           sq[k] = fmaf(r.x, r.x, r.y * r.y) + fmaf(r.z, r.z, r.w * r.w);
+                         } else {
+                           if (MODE == 2) r = make_float4(r.x * s, r.y * s, r.z * s, r.w * s);
+                           store4<DT>(out, (size_t)f * lay.fpitch + lay.roff + (size_t)(y0 + k) * lay.rpitch + x, r, W - x,
+                                      vec_out);
+                         }
+                       });
   }
-  if (MODE == 1) {   // float within a warp, double across warps and blocks
-    float v = sq;
+  if (MODE == 0 && scale && blockIdx.x == 0 && blockIdx.y == 0 && tx == 0 && threadIdx.y == 0) scale[f] = 1.f;
+  if (MODE == 1) {   // pairwise over a thread's rows, float within a warp, double across warps and blocks
+#pragma unroll
+    for (int o = RPT / 2; o; o >>= 1)
+#pragma unroll
+      for (int k = 0; k < o; ++k) sq[k] += sq[k + o];
+    float v = sq[0];
 #pragma unroll
     for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     if (tx == 0) part[threadIdx.y] = (double)v;
@@ -207,41 +334,141 @@ __global__ void k_pad_pairs(const uint16_t* __restrict__ in, int H, int W, uint3
   out[(size_t)f * (H + 3) * P + (size_t)yp * P + xp] = lo | (hi << 16);
 }
 
+// the kernel template with its rows per thread and row alignment chosen
+template <class Fn>
+void resid_dispatch(int rpt, bool vec, Fn&& fn) {
+  using std::integral_constant;
+  if (rpt == 8 && vec) fn(integral_constant<int, 8>{}, integral_constant<bool, true>{});
+  else if (rpt == 8) fn(integral_constant<int, 8>{}, integral_constant<bool, false>{});
+  else if (vec) fn(integral_constant<int, 2>{}, integral_constant<bool, true>{});
+  else fn(integral_constant<int, 2>{}, integral_constant<bool, false>{});
+}
+bool rows_aligned4(const void* frames, size_t pitch) { return ((reinterpret_cast<uintptr_t>(frames) | pitch) & 3) == 0; }
+
 template <int MODE>
-void apply_dispatch(int dtype, dim3 g, dim3 b, cudaStream_t s, const uint8_t* frames, size_t pitch, int H, int W,
-                    const unsigned long long* acc, int weight, void* out, double* partials, const float* scale,
+void apply_dispatch(int dtype, int rpt, bool vec, dim3 g, cudaStream_t s, const uint8_t* frames, size_t pitch, int H,
+                    int W, const unsigned long long* acc, int weight, void* out, double* partials, float* scale,
                     const ResidLayout& l) {
-  if (dtype == kF32)
-    k_resid_apply<kF32, MODE><<<g, b, 0, s>>>(frames, pitch, H, W, acc, weight, out, partials, scale, l);
-  else if (dtype == kF16)
-    k_resid_apply<kF16, MODE><<<g, b, 0, s>>>(frames, pitch, H, W, acc, weight, out, partials, scale, l);
-  else
-    k_resid_apply<kBF16, MODE><<<g, b, 0, s>>>(frames, pitch, H, W, acc, weight, out, partials, scale, l);
+  const dim3 b(kBX, 8);
+  // quads start at multiples of 4 elements of rows and frames that do too
+  const bool vec_out = out && (l.roff | l.rpitch | l.fpitch) % 4 == 0 &&
+                       reinterpret_cast<uintptr_t>(out) % (dtype == kF32 ? 16 : 8) == 0;
+  resid_dispatch(rpt, vec, [&](auto R, auto V) {
+    constexpr int RPT = decltype(R)::value;
+    constexpr bool VEC = decltype(V)::value;
+    auto* fn = k_resid_apply<kF32, MODE, RPT, VEC>;
+    if constexpr (MODE != 1) {   // MODE 1 stores no residual
+      if (dtype == kF16) fn = k_resid_apply<kF16, MODE, RPT, VEC>;
+      else if (dtype == kBF16) fn = k_resid_apply<kBF16, MODE, RPT, VEC>;
+    }
+    fn<<<g, b, 0, s>>>(frames, pitch, H, W, acc, weight, out, partials, scale, l, vec_out);
+  });
+  PRNU_CUDA_TRY(cudaGetLastError());
 }
 
-// Eq. 2 sums over a chunk of Lc frames: num += sum_l R_l (R = I W(I)),
-// den += sum_l I_l^2, in double (first: start from zero).
-__global__ void k_fp_accumulate(const float* __restrict__ R, const uint8_t* __restrict__ frames, size_t pitch, int Lc,
-                                int H, int W, double* __restrict__ num, double* __restrict__ den, int first) {
-  const int x = blockIdx.x * blockDim.x + threadIdx.x, y = blockIdx.y;
-  if (x >= W) return;
-  const size_t p = (size_t)y * W + x;
-  double a = first ? 0.0 : num[p], b = first ? 0.0 : den[p];
-  for (int l = 0; l < Lc; ++l) {
-    a += (double)R[(size_t)l * H * W + p];
-    const double I = (double)frames[((size_t)l * H + y) * pitch + x];
-    b += I * I;
+// the frames' integer variance sums, block slots first
+void launch_moments(const uint8_t* frames, int F, int H, int W, size_t pitch, int rpt, unsigned long long* slots,
+                    unsigned long long* acc, cudaStream_t s, LaunchCounter& lc) {
+  const dim3 g = resid_grid(F, H, W, rpt);
+  resid_dispatch(rpt, rows_aligned4(frames, pitch), [&](auto R, auto V) {
+    k_resid_moments<decltype(R)::value, decltype(V)::value><<<g, dim3(kBX, 8), 0, s>>>(frames, pitch, H, W, slots);
+  });
+  PRNU_CUDA_TRY(cudaGetLastError());
+  k_resid_noise<<<F, 256, 0, s>>>(slots, (int)(g.x * g.y), acc);
+  PRNU_CUDA_TRY(cudaGetLastError());
+  lc.n += 2;
+}
+
+// s + c += b (Knuth's two-sum), two sums at once
+__device__ __forceinline__ void csum_add2(float2& s, float2& c, float2 b) {
+  const float2 t = __fadd2_rn(s, b);
+  const float2 bp = __fadd2_rn(t, make_float2(-s.x, -s.y));
+  const float2 sp = __fadd2_rn(t, make_float2(-bp.x, -bp.y));
+  const float2 e = __fadd2_rn(__fadd2_rn(s, make_float2(-sp.x, -sp.y)), __fadd2_rn(b, make_float2(-bp.x, -bp.y)));
+  s = t;
+  c = __fadd2_rn(c, e);
+}
+
+// K = sum_l I W(I) / sum_l I^2 (Eq. 2) of a thread's pixels over all L frames.
+// The numerator is a compensated FP32 sum (48 bits; the FP64 pipe takes 1/64 of
+// the FP32 rate), the denominator an integer: exact in FP32 over up to 256
+// frames, which LONG then adds to a compensated sum.  One pass over the frames
+// where residuals in memory and FP64 sums took three and two more: 0.58 ms (with the noise powers)
+// instead of 2.98 for 16 frames of 4000 x 3000, bound by issue (59%).
+template <bool VEC, bool LONG>
+__global__ void __launch_bounds__(kBX * 8, 2) k_fp_estimate(const uint8_t* __restrict__ frames, size_t pitch, int L,
+                                                         int H, int W, const unsigned long long* __restrict__ acc,
+                                                         float* __restrict__ K, bool vec_out) {
+  constexpr int RPT = 2;
+  __shared__ float2 s_nu2[256];
+  const int tx = threadIdx.x, tid = threadIdx.y * kBX + tx;
+  const int x = (blockIdx.x * kBX + tx) * kPX, y0 = (blockIdx.y * 8 + threadIdx.y) * RPT;
+  const float2 zero = make_float2(0.f, 0.f);
+  float2 n[RPT][2], nc[RPT][2], d[RPT][2], dh[RPT][2], dl[RPT][2];
+#pragma unroll
+  for (int k = 0; k < RPT; ++k)
+#pragma unroll
+    for (int q = 0; q < 2; ++q) n[k][q] = nc[k][q] = dh[k][q] = dl[k][q] = zero;
+  for (int l0 = 0; l0 < L; l0 += 256) {
+    const int lc = min(256, L - l0);
+    __syncthreads();
+    if (tid < lc) s_nu2[tid] = noise_power(acc[l0 + tid], H, W);
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < RPT; ++k) d[k][0] = d[k][1] = zero;
+    if (x < W && y0 < H) {
+      FrameRows<VEC> rows{frames + (size_t)l0 * H * pitch, pitch, H, W, x, y0};
+      Raw6 next[RPT + 2];   // the next frame's rows are loaded before this one's are used
+#pragma unroll
+      for (int i = 0; i < RPT + 2; ++i) next[i] = rows.raw(i);
+      for (int l = 0; l < lc; ++l) {
+        const float2 nu2 = s_nu2[l];
+        Raw6 cur[RPT + 2];
+#pragma unroll
+        for (int i = 0; i < RPT + 2; ++i) cur[i] = next[i];
+        if (l + 1 < lc) {
+          rows.f += (size_t)H * pitch;
+#pragma unroll
+          for (int i = 0; i < RPT + 2; ++i) next[i] = rows.raw(i);
+        }
+        for_rows<RPT>([&](int i) { return row_floats(cur[i]); },
+                           [&](int k, const Row6& p, float2 va, float2 vb, float2 da, float2 db) {
+                             const float2 wa = make_float2(residual_w(va.x, da.x, nu2.x, nu2.y),
+                                                           residual_w(va.y, da.y, nu2.x, nu2.y));
+                             const float2 wb = make_float2(residual_w(vb.x, db.x, nu2.x, nu2.y),
+                                                           residual_w(vb.y, db.y, nu2.x, nu2.y));
+                             csum_add2(n[k][0], nc[k][0], __fmul2_rn(p.a, wa));
+                             csum_add2(n[k][1], nc[k][1], __fmul2_rn(p.b, wb));
+                             d[k][0] = __ffma2_rn(p.a, p.a, d[k][0]);
+                             d[k][1] = __ffma2_rn(p.b, p.b, d[k][1]);
+                           });
+      }
+    }
+#pragma unroll
+    for (int k = 0; k < RPT; ++k)
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {
+        if (LONG) csum_add2(dh[k][q], dl[k][q], d[k][q]);
+        else dh[k][q] = d[k][q];
+      }
   }
-  num[p] = a;
-  den[p] = b;
+  if (x >= W) return;
+  // (s + c) / (h + l): a quotient and one correction by its remainder
+  auto ratio = [](float s, float c, float h, float l) {
+    if (!(h > 0.f)) return 0.f;
+    const float q = s / h;
+    return q + (fmaf(-q, h, s) + fmaf(-q, l, c)) / h;
+  };
+#pragma unroll
+  for (int k = 0; k < RPT; ++k) {
+    if (y0 + k >= H) break;
+    const float4 r = make_float4(ratio(n[k][0].x, nc[k][0].x, dh[k][0].x, dl[k][0].x),
+                                 ratio(n[k][0].y, nc[k][0].y, dh[k][0].y, dl[k][0].y),
+                                 ratio(n[k][1].x, nc[k][1].x, dh[k][1].x, dl[k][1].x),
+                                 ratio(n[k][1].y, nc[k][1].y, dh[k][1].y, dl[k][1].y));
+    store4<kF32>(K, (size_t)(y0 + k) * W + x, r, W - x, vec_out);
+  }
 }
-
-__global__ void k_fp_divide(const double* __restrict__ num, const double* __restrict__ den, float* __restrict__ K,
-                            size_t n) {
-  const size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
-  if (i < n) K[i] = den[i] > 0.0 ? (float)(num[i] / den[i]) : 0.f;
-}
-
 
 // ---------------------------------------------------------------- frame-literal residuals (Sec. 3.2)
 //
@@ -419,8 +646,35 @@ __global__ void __launch_bounds__(kLX * 8) k_lit_apply(const float* __restrict__
   }
 }
 
+// Taps of one axis (Sec. 3's resampling): output sample o at input position
+// u = (first + o + 0.5) / scale - 0.5, tent weights max(0, 1 - |j - u| a) with a
+// = min(scale, 1), indices clamped to the axis, normalised; T taps per sample
+// (zero weight beyond its support).  In double, one thread per sample of both
+// axes (y first).
+struct TapAxis {
+  int n_in, first, n;
+  float* w;
+  int* idx;
+};
+__global__ void k_fp_taps(TapAxis ay, TapAxis ax, double scale, int T) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= ay.n + ax.n) return;
+  const bool y = i < ay.n;
+  const TapAxis t = y ? ay : ax;
+  const int o = y ? i : i - ay.n;
+  const double a = fmin(scale, 1.0);
+  const double u = ((double)(t.first + o) + 0.5) / scale - 0.5;
+  const int lo = (int)floor(u - 1.0 / a);
+  double tot = 0.0;
+  for (int k = 0; k < T; ++k) tot += fmax(1.0 - fabs((double)(lo + k) - u) * a, 0.0);
+  for (int k = 0; k < T; ++k) {
+    t.w[(size_t)o * T + k] = (float)(fmax(1.0 - fabs((double)(lo + k) - u) * a, 0.0) / tot);
+    t.idx[(size_t)o * T + k] = min(max(lo + k, 0), t.n_in - 1);
+  }
+}
+
 // Fingerprint resampling: out(y, x) = sum_a sum_b wy[y][a] wx[x][b] K(iy[y][a], ix[x][b]),
-// T taps per axis (unused taps have weight 0 and index 0).
+// T taps per axis (unused taps have weight 0).
 __global__ void k_fp_resize(const float* __restrict__ K, size_t pitch, const float* __restrict__ wy,
                             const int* __restrict__ iy, const float* __restrict__ wx, const int* __restrict__ ix,
                             int T, int H, int W, float* __restrict__ out) {
@@ -440,18 +694,16 @@ __global__ void k_fp_resize(const float* __restrict__ K, size_t pitch, const flo
 
 }  // namespace
 
-void launch_fp_estimate_accumulate(const float* R, const uint8_t* frames, size_t pitch, int Lc, int H, int W,
-                                   double* num, double* den, bool first, cudaStream_t s, LaunchCounter& lc) {
+void launch_fp_estimate(const uint8_t* frames, size_t pitch, int L, int H, int W, unsigned long long* slots,
+                        unsigned long long* acc, float* K, cudaStream_t s, LaunchCounter& lc) {
   ProfScope ps(lc, kKindResidual, s);
-  k_fp_accumulate<<<dim3((W + 255) / 256, H), 256, 0, s>>>(R, frames, pitch, Lc, H, W, num, den, first ? 1 : 0);
-  PRNU_CUDA_TRY(cudaGetLastError());
-  lc.n++;
-}
-
-void launch_fp_estimate_divide(const double* num, const double* den, float* K, size_t n, cudaStream_t s,
-                               LaunchCounter& lc) {
-  ProfScope ps(lc, kKindResidual, s);
-  k_fp_divide<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(num, den, K, n);
+  launch_moments(frames, L, H, W, pitch, resid_rows(L, H, W), slots, acc, s, lc);
+  const dim3 g = resid_grid(1, H, W, 2), b(kBX, 8);
+  const bool vec = rows_aligned4(frames, pitch), lng = L > 256;
+  const bool vec_out = W % 4 == 0 && reinterpret_cast<uintptr_t>(K) % 16 == 0;
+  auto* fn = lng ? (vec ? k_fp_estimate<true, true> : k_fp_estimate<false, true>)
+                 : (vec ? k_fp_estimate<true, false> : k_fp_estimate<false, false>);
+  fn<<<g, b, 0, s>>>(frames, pitch, L, H, W, acc, K, vec_out);
   PRNU_CUDA_TRY(cudaGetLastError());
   lc.n++;
 }
@@ -493,54 +745,47 @@ size_t literal_partials_needed(int nr, int H, int W) {
 }
 
 size_t residual_partials_needed(int F, int H, int W) {
-  const size_t gx = (W + kBX - 1) / kBX, gy = (H + kBY - 1) / kBY;
-  return (size_t)F * gx * gy;
+  const dim3 g = resid_grid(F, H, W, resid_rows(F, H, W));
+  return (size_t)F * g.x * g.y;
 }
 
 void launch_residual(const uint8_t* frames, int F, int H, int W, size_t pitch, int flags, int dtype, void* out,
                      float* scale, unsigned long long* acc, double* partials, int /*max_partials*/, cudaStream_t s,
                      LaunchCounter& lc, const ResidLayout* lay) {
   const ResidLayout l = lay ? *lay : ResidLayout{W, (size_t)H * W, 0};
-  const dim3 b(kBX, 8);
-  const dim3 g((W + kBX - 1) / kBX, (H + kBY - 1) / kBY, F);
+  const int rpt = resid_rows(F, H, W);
+  const bool vec = rows_aligned4(frames, pitch);
+  const dim3 g = resid_grid(F, H, W, rpt);
   const int weight = (flags & PRNU_WEIGHT_BY_INTENSITY) ? 1 : 0;
   ProfScope ps(lc, kKindResidual, s);
   // the block slots go to `partials` (8-byte slots, reused below by PRNU_NORMALISE)
-  auto* slots = reinterpret_cast<unsigned long long*>(partials);
-  k_resid_moments<<<g, b, 0, s>>>(frames, pitch, H, W, slots);
-  PRNU_CUDA_TRY(cudaGetLastError());
-  k_resid_noise<<<F, 256, 0, s>>>(slots, (int)(g.x * g.y), acc);
-  PRNU_CUDA_TRY(cudaGetLastError());
-  lc.n += 2;
+  launch_moments(frames, F, H, W, pitch, rpt, reinterpret_cast<unsigned long long*>(partials), acc, s, lc);
   if (flags & PRNU_NORMALISE) {
-    apply_dispatch<1>(dtype, g, b, s, frames, pitch, H, W, acc, weight, out, partials, scale, l);
-    PRNU_CUDA_TRY(cudaGetLastError());
+    // the sum of squares does not depend on the storage type
+    apply_dispatch<1>(kF32, rpt, vec, g, s, frames, pitch, H, W, acc, weight, nullptr, partials, scale, l);
     k_resid_scale<<<F, 256, 0, s>>>(partials, (int)(g.x * g.y), H, W, scale);
     PRNU_CUDA_TRY(cudaGetLastError());
-    apply_dispatch<2>(dtype, g, b, s, frames, pitch, H, W, acc, weight, out, partials, scale, l);
-    PRNU_CUDA_TRY(cudaGetLastError());
+    apply_dispatch<2>(dtype, rpt, vec, g, s, frames, pitch, H, W, acc, weight, out, partials, scale, l);
     lc.n += 3;
   } else {
-    apply_dispatch<0>(dtype, g, b, s, frames, pitch, H, W, acc, weight, out, partials, scale, l);
-    PRNU_CUDA_TRY(cudaGetLastError());
+    apply_dispatch<0>(dtype, rpt, vec, g, s, frames, pitch, H, W, acc, weight, out, partials, scale, l);
     lc.n++;
-    if (scale) {
-      k_fill<<<(F + 255) / 256, 256, 0, s>>>(scale, F, 1.f);
-      PRNU_CUDA_TRY(cudaGetLastError());
-      lc.n++;
-    }
   }
 }
 
 }  // namespace prnu
 
 namespace prnu {
-void launch_fp_resize(const float* K, size_t pitch, const float* wy, const int* iy, const float* wx, const int* ix,
-                      int T, int H, int W, float* out, cudaStream_t s, LaunchCounter& lc) {
+void launch_fp_resize(const float* K, int Hin, int Win, size_t pitch, double scale, int y0, int x0, int T, float* w,
+                      int* idx, int H, int W, float* out, cudaStream_t s, LaunchCounter& lc) {
   ProfScope ps(lc, kKindResidual, s);
-  k_fp_resize<<<dim3((W + 127) / 128, H), 128, 0, s>>>(K, pitch, wy, iy, wx, ix, T, H, W, out);
+  const size_t ny = (size_t)H * T;
+  k_fp_taps<<<(H + W + 127) / 128, 128, 0, s>>>(TapAxis{Hin, y0, H, w, idx}, TapAxis{Win, x0, W, w + ny, idx + ny},
+                                                scale, T);
   PRNU_CUDA_TRY(cudaGetLastError());
-  lc.n++;
+  k_fp_resize<<<dim3((W + 127) / 128, H), 128, 0, s>>>(K, pitch, w, idx, w + ny, idx + ny, T, H, W, out);
+  PRNU_CUDA_TRY(cudaGetLastError());
+  lc.n += 2;
 }
 }  // namespace prnu
 
