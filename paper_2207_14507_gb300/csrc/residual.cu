@@ -173,21 +173,10 @@ __global__ void k_resid_noise(const unsigned long long* __restrict__ part, int n
   }
 }
 
-// n / d for |d| in [1, 2^24) and |n| below 2^60: the hardware's reciprocal
-// (1 ulp), the quotient, and one step of iterative refinement by its exact
-// remainder (Newton's correction), which leaves the rounding of the last add;
-// a third of the instructions of the general division.
-__device__ __forceinline__ float quotient(float n, float d) {
-  float rc;
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(rc) : "f"(d));
-  const float q = n * rc;
-  return fmaf(fmaf(-q, d, n), rc, q);
-}
-
 // W of one pixel: 9 D nu2 / V or D / 9 (see the head of this file)
 __device__ __forceinline__ float residual_w(float V, float D, float nu2, float nu2x81) {
   const bool wiener = V > 0.f && V >= nu2x81;
-  return quotient(wiener ? (9.f * D) * nu2 : D, wiener ? V : 9.f);
+  return refined_quotient(wiener ? (9.f * D) * nu2 : D, wiener ? V : 9.f);
 }
 
 // the frame's noise power and 81 times it, from its integer sum

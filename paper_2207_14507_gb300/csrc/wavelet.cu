@@ -14,8 +14,13 @@
 //      outside the band; the last low-low band replaced by 0;
 //   4. the inverse transform of those noise parts: W(I) = I - F(I) (the
 //      transform is linear), cropped to H x W; R = I W(I) or W(I).
-// Two Hp x Wp buffers per frame: the coefficients (A) and a scratch (T); the
-// noise parts and the inverse run in T and A alternately.
+// Two Hp x Wp buffers per frame.  Forward: the detail bands of every level in
+// the quadrant layout (pitch Wp) in A, each level's low-low band, the next
+// level's input, in T.  Then the noise parts in the quadrant layout in T, and
+// the inverse's intermediate images in A; its last level goes straight to the
+// residual.  Each level is one kernel each way: a block filters a tile along
+// rows and columns through shared memory, two elements to a packed FP32
+// instruction.
 #include <algorithm>
 
 #include "internal.h"
@@ -26,253 +31,367 @@ namespace {
 
 // Daubechies' scaling filter with 4 vanishing moments, sum sqrt(2); wavelet
 // filter g[k] = (-1)^k h[7 - k]
-__constant__ float c_h[8] = {0.2303778133088964f,  0.7148465705529154f,  0.6308807679298587f,
-                             -0.0279837694168599f, -0.1870348117190931f, 0.0308413818355607f,
-                             0.0328830116668852f,  -0.0105974017850690f};
-__device__ __forceinline__ float wav_g(int k) { return (k & 1) ? -c_h[7 - k] : c_h[7 - k]; }
-
-constexpr int kWB = 128;
-
-__global__ void k_wav_pad(const uint8_t* __restrict__ frames, size_t pitch, int H, int W, int Hp, int Wp,
-                          float* __restrict__ A) {
-  const int x = blockIdx.x * kWB + threadIdx.x, y = blockIdx.y, f = blockIdx.z;
-  if (x >= Wp) return;
-  const int ys = y < H ? y : 2 * H - 1 - y, xs = x < W ? x : 2 * W - 1 - x;   // half-sample mirror
-  A[((size_t)f * Hp + y) * Wp + x] = (float)frames[((size_t)f * H + ys) * pitch + xs];
+__host__ __device__ constexpr float wav_h(int k) {
+  constexpr float h[8] = {0.2303778133088964f,  0.7148465705529154f,  0.6308807679298587f,
+                          -0.0279837694168599f, -0.1870348117190931f, 0.0308413818355607f,
+                          0.0328830116668852f,  -0.0105974017850690f};
+  return h[k];
 }
+__host__ __device__ constexpr float wav_g(int k) { return (k & 1) ? -wav_h(7 - k) : wav_h(7 - k); }
+// (value, value) or (a pair of coefficients) for the packed instructions
+__device__ __forceinline__ float2 dup(float v) { return make_float2(v, v); }
 
-// rows of the h x w top-left region of X (pitch Wp) -> T: [low w/2 | high w/2]
-__global__ void k_wav_rows(const float* __restrict__ X, int w, int Hp, int Wp, float* __restrict__ T) {
-  const int n = blockIdx.x * kWB + threadIdx.x, y = blockIdx.y, f = blockIdx.z;
-  const int w2 = w / 2;
-  if (n >= w2) return;
-  const float* row = X + ((size_t)f * Hp + y) * Wp;
-  float a = 0.f, d = 0.f;
+constexpr int kTS = 32;              // coefficients of a band per block and axis: 64 x 64 pixels
+constexpr int kIn = 2 * kTS + 6;     // input samples of the analysis
+constexpr int kPairs = kIn / 2;
+constexpr int kBand = kTS + 3;       // coefficients of the synthesis
+constexpr int kLevels = 4;
+
+// index i >= 0 of an axis of n samples, periodic
+__device__ __forceinline__ int wrap_up(int i, int n) { return i < n ? i : i % n; }
+// index i >= -3, periodic
+__device__ __forceinline__ int wrap_both(int i, int n) { return i >= 0 ? wrap_up(i, n) : ((i % n) + n) % n; }
+// sample i < 2 n of an axis of n samples, mirrored at its end (half-sample)
+__device__ __forceinline__ int mirror(int i, int n) { return i < n ? i : 2 * n - 1 - i; }
+
+// One level of the analysis: the h x w image (LEVEL0: the uint8 frame, mirrored
+// to that size; else X, dense, of frame stride fstride) to its three detail
+// bands in A (quadrant layout, pitch Wp) and, unless LL is null, its low-low
+// band (dense h/2 x w/2).  8 full-HD frames, all levels: 84 us, where a
+// kernel per axis with 8 global loads an output took 255.
+template <bool LEVEL0>
+__global__ void __launch_bounds__(256) k_wav_analyse(const uint8_t* __restrict__ frames, size_t pitch, int H, int W,
+                                                     const float* __restrict__ X, size_t fstride, int h, int w, int Wp,
+                                                     float* __restrict__ A, float* __restrict__ LL) {
+  __shared__ __align__(16) float2 in[kPairs * (kIn + 2)];   // (row 2p, row 2p + 1) at column x
+  __shared__ float2 T[2][kPairs][kTS];                      // the same after the row filters, low and high
+  const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
+  const int n0 = blockIdx.x * kTS, m0 = blockIdx.y * kTS, f = blockIdx.z;
+  const int w2 = w / 2, h2 = h / 2;
+  auto sample = [&](int y, int x) -> float {
+    if (LEVEL0) return (float)__ldg(frames + ((size_t)f * H + mirror(y, H)) * pitch + mirror(x, W));
+    return __ldg(X + (size_t)f * fstride + (size_t)y * w + x);
+  };
+  for (int p = wp; p < kPairs; p += 8) {
+    const int ya = wrap_up(2 * (m0 + p), h), yb = wrap_up(2 * (m0 + p) + 1, h);
 #pragma unroll
-  for (int k = 0; k < 8; ++k) {
-    const float v = row[(2 * n + k) % w];
-    a = fmaf(c_h[k], v, a);
-    d = fmaf(wav_g(k), v, d);
-  }
-  float* o = T + ((size_t)f * Hp + y) * Wp;
-  o[n] = a;
-  o[w2 + n] = d;
-}
-
-// columns of the h x w top-left region of T -> X: low h/2 rows over high h/2 rows
-__global__ void k_wav_cols(const float* __restrict__ T, int h, int w, int Hp, int Wp, float* __restrict__ X) {
-  const int x = blockIdx.x * kWB + threadIdx.x, n = blockIdx.y, f = blockIdx.z;
-  if (x >= w) return;
-  const float* base = T + (size_t)f * Hp * Wp + x;
-  float a = 0.f, d = 0.f;
-#pragma unroll
-  for (int k = 0; k < 8; ++k) {
-    const float v = base[(size_t)((2 * n + k) % h) * Wp];
-    a = fmaf(c_h[k], v, a);
-    d = fmaf(wav_g(k), v, d);
-  }
-  float* o = X + (size_t)f * Hp * Wp + x;
-  o[(size_t)n * Wp] = a;
-  o[(size_t)(h / 2 + n) * Wp] = d;
-}
-
-// inverse of k_wav_cols: X (h x w region, low over high) -> T
-__global__ void k_wav_icols(const float* __restrict__ X, int h, int w, int Hp, int Wp, float* __restrict__ T) {
-  const int x = blockIdx.x * kWB + threadIdx.x, m = blockIdx.y, f = blockIdx.z;
-  if (x >= w) return;
-  const int h2 = h / 2;
-  const float* base = X + (size_t)f * Hp * Wp + x;
-  float v = 0.f;
-#pragma unroll
-  for (int k = (m & 1); k < 8; k += 2) {   // output m takes input 2n + k = m (mod h)
-    const int n = (((m - k) / 2) % h2 + h2) % h2;
-    v = fmaf(c_h[k], base[(size_t)n * Wp], v);
-    v = fmaf(wav_g(k), base[(size_t)(h2 + n) * Wp], v);
-  }
-  T[((size_t)f * Hp + m) * Wp + x] = v;
-}
-
-// inverse of k_wav_rows: T (h x w region, [low | high]) -> X
-__global__ void k_wav_irows(const float* __restrict__ T, int w, int Hp, int Wp, float* __restrict__ X) {
-  const int m = blockIdx.x * kWB + threadIdx.x, y = blockIdx.y, f = blockIdx.z;
-  if (m >= w) return;
-  const int w2 = w / 2;
-  const float* row = T + ((size_t)f * Hp + y) * Wp;
-  float v = 0.f;
-#pragma unroll
-  for (int k = (m & 1); k < 8; k += 2) {
-    const int n = (((m - k) / 2) % w2 + w2) % w2;
-    v = fmaf(c_h[k], row[n], v);
-    v = fmaf(wav_g(k), row[w2 + n], v);
-  }
-  X[((size_t)f * Hp + y) * Wp + m] = v;
-}
-
-// noise parts of the three detail bands (h2 x w2 each) of one level: band b of
-// frame f = blockIdx.z: 0 (rows high, columns low) at (0, w2), 1 at (h2, 0),
-// 2 at (h2, w2); reads A, writes T
-constexpr int kSX = 32, kSY = 8, kSR = 4;
-__global__ void __launch_bounds__(kSX * kSY) k_wav_shrink(const float* __restrict__ A, int h2, int w2, int Hp, int Wp,
-                                                        float s0sq, float* __restrict__ T) {
-  __shared__ float sq[(kSY + 2 * kSR) * (kSX + 2 * kSR)];
-  const int f = blockIdx.z / 3, b = blockIdx.z - 3 * f;
-  const int oy = b == 0 ? 0 : h2, ox = b == 1 ? 0 : w2;
-  const float* band = A + ((size_t)f * Hp + oy) * Wp + ox;
-  const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * kSX + tx;
-  const int bx0 = blockIdx.x * kSX - kSR, by0 = blockIdx.y * kSY - kSR;
-  constexpr int SW = kSX + 2 * kSR, SN = (kSY + 2 * kSR) * SW;
-  for (int k = tid; k < SN; k += kSX * kSY) {
-    const int sy = k / SW, sx = k - sy * SW;
-    const int y = by0 + sy, x = bx0 + sx;
-    float v = 0.f;
-    if (y >= 0 && y < h2 && x >= 0 && x < w2) {
-      const float c = band[(size_t)y * Wp + x];
-      v = c * c;
+    for (int q = 0; q < 3; ++q) {
+      const int i = lane + 32 * q;
+      if (i >= kIn) break;
+      const int x = wrap_up(2 * n0 + i, w);
+      in[p * (kIn + 2) + i] = make_float2(sample(ya, x), sample(yb, x));
     }
-    sq[k] = v;
   }
   __syncthreads();
-  const int x = blockIdx.x * kSX + tx, y = blockIdx.y * kSY + ty;
-  if (x >= w2 || y >= h2) return;
-  // window sums of radius 1..4 around (ty, tx) + kSR, ring by ring
-  float sum = 0.f, s2 = INFINITY;
-  const float* cen = sq + (ty + kSR) * SW + tx + kSR;
-  sum = cen[0];
+  for (int p = wp; p < kPairs; p += 8) {
+    const float4* src = reinterpret_cast<const float4*>(in + p * (kIn + 2)) + lane;
+    float2 lo = dup(0.f), hi = dup(0.f);
 #pragma unroll
-  for (int r = 1; r <= kSR; ++r) {
-#pragma unroll
-    for (int d = -r; d <= r; ++d) {
-      sum += cen[-r * SW + d] + cen[r * SW + d];
-      if (d > -r && d < r) sum += cen[d * SW - r] + cen[d * SW + r];
+    for (int j = 0; j < 4; ++j) {
+      const float4 v = src[j];
+      const float2 a = make_float2(v.x, v.y), b = make_float2(v.z, v.w);
+      lo = __ffma2_rn(a, dup(wav_h(2 * j)), lo);
+      lo = __ffma2_rn(b, dup(wav_h(2 * j + 1)), lo);
+      hi = __ffma2_rn(a, dup(wav_g(2 * j)), hi);
+      hi = __ffma2_rn(b, dup(wav_g(2 * j + 1)), hi);
     }
-    const float nw = (float)((2 * r + 1) * (2 * r + 1));
-    s2 = fminf(s2, fmaxf(sum / nw - s0sq, 0.f));
+    T[0][p][lane] = lo;
+    T[1][p][lane] = hi;
   }
-  const float c = band[(size_t)y * Wp + x];
-  const float den = s2 + s0sq;
-  T[((size_t)f * Hp + oy + y) * Wp + ox + x] = den > 0.f ? c * s0sq / den : 0.f;
+  __syncthreads();
+  // columns: a warp takes the low or the high half, 8 output rows of each kind
+  const int half = wp & 1, g = (wp >> 1) * 8, n = n0 + lane;
+  if (n >= w2) return;
+  float2 t[11];
+#pragma unroll
+  for (int i = 0; i < 11; ++i) t[i] = T[half][g + i][lane];
+  const size_t fo = (size_t)f * fstride;
+#pragma unroll
+  for (int k = 0; k < 8; ++k) {
+    const int m = m0 + g + k;
+    if (m >= h2) break;
+    float2 lo = dup(0.f), hi = dup(0.f);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      lo = __ffma2_rn(t[k + j], make_float2(wav_h(2 * j), wav_h(2 * j + 1)), lo);
+      hi = __ffma2_rn(t[k + j], make_float2(wav_g(2 * j), wav_g(2 * j + 1)), hi);
+    }
+    const float l = lo.x + lo.y, d = hi.x + hi.y;
+    if (half) A[fo + (size_t)m * Wp + w2 + n] = l;
+    else if (LL) LL[fo + (size_t)m * w2 + n] = l;
+    A[fo + (size_t)(h2 + m) * Wp + (half ? w2 : 0) + n] = d;
+  }
 }
 
-__global__ void k_wav_zero(int h, int w, int Hp, int Wp, float* __restrict__ T) {
-  const int x = blockIdx.x * kWB + threadIdx.x, y = blockIdx.y, f = blockIdx.z;
-  if (x < w) T[((size_t)f * Hp + y) * Wp + x] = 0.f;
+// Noise parts of the three detail bands of every level: band b of frame f,
+// blockIdx.z = 3 f + b: 0 (rows high, columns low) at (0, w2), 1 at (h2, 0), 2 at
+// (h2, w2) of a level of h2 x w2 coefficients a band; blockIdx.x counts the
+// levels' tiles, finest level first.  Reads A, writes T.  The sums of c^2 over
+// the 3, 5, 7 and 9 wide windows go along rows first (four sums a pixel, each a
+// pair more than the last), then along columns.  The smallest of max(0, mean -
+// s0) is max(0, smallest mean - s0): subtraction and max are monotone in
+// floating point too.  8 full-HD frames: 121 us; 80 shared loads a
+// coefficient in a kernel per level took 211.
+constexpr int kSX = 32, kSY = 32, kSR = 4;
+// FAST: the quotients c s0 / den have no subnormal or overflowing part
+template <bool FAST>
+__global__ void __launch_bounds__(256) k_wav_shrink(const float* __restrict__ A, int Hp, int Wp, size_t fstride, float s0sq,
+                                                    float* __restrict__ T) {
+  // row pitches that put 8 lanes of consecutive rows in distinct 16-byte banks
+  constexpr int SW = kSX + 2 * kSR + 4, SH = kSY + 2 * kSR, HW = kSX + 1;
+  __shared__ __align__(16) float sq[SH * SW];
+  __shared__ __align__(16) float4 hs[SH * HW];
+  const int f = blockIdx.z / 3, b = blockIdx.z - 3 * f;
+  int h2 = Hp / 2, w2 = Wp / 2, tile = blockIdx.x, tx = (w2 + kSX - 1) / kSX, n = tx * ((h2 + kSY - 1) / kSY);
+  while (tile >= n) {   // the level of this tile
+    tile -= n;
+    h2 /= 2;
+    w2 /= 2;
+    tx = (w2 + kSX - 1) / kSX;
+    n = tx * ((h2 + kSY - 1) / kSY);
+  }
+  const int by0 = tile / tx * kSY, bx0 = (tile - tile / tx * tx) * kSX;
+  const int oy = b == 0 ? 0 : h2, ox = b == 1 ? 0 : w2;
+  const float* band = A + (size_t)f * fstride + (size_t)oy * Wp + ox;
+  const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
+  for (int sy = wp; sy < SH; sy += 8) {
+    const int y = by0 + sy - kSR;
+    const float* row = band + (size_t)y * Wp;
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      const int sx = lane + 32 * q, x = bx0 + sx - kSR;
+      if (sx >= kSX + 2 * kSR) break;
+      float c = 0.f;
+      if ((unsigned)y < (unsigned)h2 && (unsigned)x < (unsigned)w2) c = __ldg(row + x);
+      sq[sy * SW + sx] = c * c;
+    }
+  }
+  __syncthreads();
+  for (int sy = lane; sy < SH; sy += 32) {   // four adjacent pixels of a row, a lane per row
+    const int x4 = wp * 4;
+    const float4* p = reinterpret_cast<const float4*>(sq + sy * SW + x4);
+    const float4 q0 = p[0], q1 = p[1], q2 = p[2];
+    const float v[12] = {q0.x, q0.y, q0.z, q0.w, q1.x, q1.y, q1.z, q1.w, q2.x, q2.y, q2.z, q2.w};
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const float s1 = v[i + 3] + v[i + 4] + v[i + 5], s2 = s1 + (v[i + 2] + v[i + 6]);
+      const float s3 = s2 + (v[i + 1] + v[i + 7]);
+      hs[sy * HW + x4 + i] = make_float4(s1, s2, s3, s3 + (v[i] + v[i + 8]));
+    }
+  }
+  __syncthreads();
+  const int x = bx0 + lane;
+  if (x >= w2) return;
+  // four adjacent rows of a column
+  const int y0 = wp * 4;
+  float2 ra[12], rb[12];   // (3, 5) and (7, 9) wide sums
+#pragma unroll
+  for (int i = 0; i < 12; ++i) {
+    const float4 q = hs[(y0 + i) * HW + lane];
+    ra[i] = make_float2(q.x, q.y);
+    rb[i] = make_float2(q.z, q.w);
+  }
+  float* const To = T + (size_t)f * fstride + (size_t)oy * Wp + ox;
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const int y = by0 + y0 + k, i = k + 4;
+    if (y >= h2) break;
+    const float c = __ldg(band + (size_t)y * Wp + x);
+    float2 ma = __fadd2_rn(ra[i], __fadd2_rn(ra[i - 1], ra[i + 1]));
+    float2 mb = __fadd2_rn(rb[i], __fadd2_rn(rb[i - 1], rb[i + 1]));
+    ma.y += ra[i - 2].y + ra[i + 2].y;
+    mb = __fadd2_rn(mb, __fadd2_rn(rb[i - 2], rb[i + 2]));
+    mb = __fadd2_rn(mb, __fadd2_rn(rb[i - 3], rb[i + 3]));
+    mb.y += rb[i - 4].y + rb[i + 4].y;
+    const float m = fminf(fminf(ma.x * (1.f / 9.f), ma.y * (1.f / 25.f)), fminf(mb.x * (1.f / 49.f), mb.y * (1.f / 81.f)));
+    const float den = fmaxf(m - s0sq, 0.f) + s0sq, num = c * s0sq;
+    float r;
+    if (FAST) r = refined_quotient(num, den);
+    else r = den > 0.f ? num / den : 0.f;
+    To[(size_t)y * Wp + x] = r;
+  }
 }
 
-// R = I W (or W) of frame f0 + blockIdx.z into out (dense [F][H][W] of type DT).
-// MODE 0: store R; MODE 1: per-block sum of R^2 to partials; MODE 2: store R * scale[f].
-template <int DT, int MODE>
-__global__ void k_wav_out(const float* __restrict__ Wr, const uint8_t* __restrict__ frames, size_t pitch, int H, int W,
-                          int Hp, int Wp, int f0, int weight, void* __restrict__ out, double* __restrict__ partials,
-                          const float* __restrict__ scale) {
-  __shared__ double part[kWB / 32];
-  const int x = blockIdx.x * kWB + threadIdx.x, y = blockIdx.y, fl = blockIdx.z, f = f0 + fl;
-  float r = 0.f;
-  if (x < W) {
-    const float w = Wr[((size_t)fl * Hp + y) * Wp + x];
-    r = weight ? (float)frames[((size_t)f * H + y) * pitch + x] * w : w;
-    const size_t o = ((size_t)f * H + y) * W + x;
-    if (MODE == 0) store_store_type<DT>(out, o, r);
-    if (MODE == 2) store_store_type<DT>(out, o, r * scale[f]);
+// One level of the synthesis: the noise parts in D (quadrant layout, pitch Wp)
+// and the low-low image LL (dense h/2 x w/2; null: zero) to the h x w image.
+// OUT 0: dense into Y.  The last level: OUT 1 stores R = I W (or W) in `out`
+// (dense [F][H][W]), OUT 2 the per-block sum of R^2 in partials, OUT 3
+// R * scale[f].  8 full-HD frames, all levels: 104 us, where a kernel per
+// axis and one for the residual took 400.
+template <int DT, int OUT>
+__global__ void __launch_bounds__(256) k_wav_synth(const float* __restrict__ D, const float* __restrict__ LL, size_t fstride,
+                                                   int h, int w, int Wp, float* __restrict__ Y,
+                                                   const uint8_t* __restrict__ frames, size_t pitch, int H, int W, int f0,
+                                                   int weight, void* __restrict__ out, double* __restrict__ partials,
+                                                   const float* __restrict__ scale) {
+  __shared__ __align__(16) float B[4][kBand][kTS + 4];         // the four bands, coefficient n at n - n0 + 3
+  __shared__ __align__(16) float2 T[kTS][2][kTS + 4];          // (row 2i, row 2i + 1) after the column filters
+  __shared__ double part[8];
+  const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
+  const int n0 = blockIdx.x * kTS, m0 = blockIdx.y * kTS, fl = blockIdx.z, f = f0 + fl;
+  const int w2 = w / 2, h2 = h / 2;
+  const size_t fo = (size_t)fl * fstride;
+  for (int r = wp; r < kBand; r += 8) {
+    const int m = wrap_both(m0 + r - 3, h2);
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      const int c = lane + 32 * q;
+      if (c >= kTS + 4) break;
+      const int n = wrap_both(n0 + c - 3, w2);
+      B[0][r][c] = LL ? __ldg(LL + fo + (size_t)m * w2 + n) : 0.f;
+      B[1][r][c] = __ldg(D + fo + (size_t)(h2 + m) * Wp + n);
+      B[2][r][c] = __ldg(D + fo + (size_t)m * Wp + w2 + n);
+      B[3][r][c] = __ldg(D + fo + (size_t)(h2 + m) * Wp + w2 + n);
+    }
   }
-  if (MODE == 1) {   // float within a warp, double across warps and blocks
-    float v = r * r;
+  __syncthreads();
+  // columns: outputs 2i and 2i + 1 take coefficients i - 3 .. i; a thread takes
+  // two adjacent columns of the low or the high half, 5 values of i
+  constexpr int kCP = (kTS + 4) / 2, kG = 5;
+  if (threadIdx.x < 2 * kCP * 7) {
+    const int q = threadIdx.x % (2 * kCP), g = threadIdx.x / (2 * kCP) * kG;
+    const int half = q / kCP, c = (q - half * kCP) * 2;
+    float2 lo[kG + 3], hi[kG + 3];
+#pragma unroll
+    for (int i = 0; i < kG + 3; ++i) {
+      const int r = min(g + i, kBand - 1);
+      lo[i] = *reinterpret_cast<const float2*>(&B[2 * half][r][c]);
+      hi[i] = *reinterpret_cast<const float2*>(&B[2 * half + 1][r][c]);
+    }
+#pragma unroll
+    for (int i = 0; i < kG; ++i) {
+      if (g + i >= kTS) break;
+      float2 a = dup(0.f), b = dup(0.f);
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        a = __ffma2_rn(lo[i + 3 - j], dup(wav_h(2 * j)), a);
+        a = __ffma2_rn(hi[i + 3 - j], dup(wav_g(2 * j)), a);
+        b = __ffma2_rn(lo[i + 3 - j], dup(wav_h(2 * j + 1)), b);
+        b = __ffma2_rn(hi[i + 3 - j], dup(wav_g(2 * j + 1)), b);
+      }
+      *reinterpret_cast<float4*>(&T[g + i][half][c]) = make_float4(a.x, b.x, a.y, b.y);
+    }
+  }
+  __syncthreads();
+  // rows: a warp takes a pair of rows, a lane outputs 2n and 2n + 1 of both
+  const int x = 2 * (n0 + lane);
+  const float s = OUT == 3 ? scale[f] : 1.f;
+  float sq[kTS / 8];
+#pragma unroll
+  for (int k = 0; k < kTS / 8; ++k) {
+    const int i = wp + 8 * k, y = 2 * (m0 + i);
+    sq[k] = 0.f;
+    if (OUT == 0 ? (y >= h || x >= w) : (y >= H || x >= W)) continue;
+    float2 a = dup(0.f), b = dup(0.f);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const float2 l = T[i][0][lane + 3 - j], d = T[i][1][lane + 3 - j];
+      a = __ffma2_rn(l, dup(wav_h(2 * j)), a);
+      a = __ffma2_rn(d, dup(wav_g(2 * j)), a);
+      b = __ffma2_rn(l, dup(wav_h(2 * j + 1)), b);
+      b = __ffma2_rn(d, dup(wav_g(2 * j + 1)), b);
+    }
+    if (OUT == 0) {
+      *reinterpret_cast<float2*>(Y + fo + (size_t)y * w + x) = make_float2(a.x, b.x);
+      *reinterpret_cast<float2*>(Y + fo + (size_t)(y + 1) * w + x) = make_float2(a.y, b.y);
+    } else {
+#pragma unroll
+      for (int e = 0; e < 2; ++e) {
+        if (y + e >= H) break;
+        float2 r = e ? make_float2(a.y, b.y) : make_float2(a.x, b.x);
+        const bool two = x + 1 < W;
+        if (weight) {
+          const uint8_t* I = frames + ((size_t)f * H + y + e) * pitch + x;
+          r.x *= (float)__ldg(I);
+          r.y *= two ? (float)__ldg(I + 1) : 0.f;
+        }
+        if (OUT == 2) {
+          sq[k] += fmaf(r.x, r.x, two ? r.y * r.y : 0.f);
+        } else {
+          const size_t o = ((size_t)f * H + y + e) * W + x;
+          store_store_type<DT>(out, o, r.x * s);
+          if (two) store_store_type<DT>(out, o + 1, r.y * s);
+        }
+      }
+    }
+  }
+  if (OUT == 2) {   // pairwise in a thread, float within a warp, double across warps and blocks
+    float v = (sq[0] + sq[1]) + (sq[2] + sq[3]);
 #pragma unroll
     for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = (double)v;
+    if (lane == 0) part[wp] = (double)v;
     __syncthreads();
     if (threadIdx.x == 0) {
-      double s = 0.0;
-      for (int k = 0; k < kWB / 32; ++k) s += part[k];
-      partials[(size_t)f * gridDim.x * gridDim.y + (size_t)y * gridDim.x + blockIdx.x] = s;
+      double t = 0.0;
+      for (int k = 0; k < 8; ++k) t += part[k];
+      partials[(size_t)f * gridDim.x * gridDim.y + blockIdx.y * gridDim.x + blockIdx.x] = t;
     }
   }
 }
 
-template <int MODE>
-void wav_out(int dtype, dim3 g, cudaStream_t s, const float* Wr, const uint8_t* frames, size_t pitch, int H, int W,
-             int Hp, int Wp, int f0, int weight, void* out, double* partials, const float* scale) {
-  if (dtype == kF32)
-    k_wav_out<kF32, MODE><<<g, kWB, 0, s>>>(Wr, frames, pitch, H, W, Hp, Wp, f0, weight, out, partials, scale);
-  else if (dtype == kF16)
-    k_wav_out<kF16, MODE><<<g, kWB, 0, s>>>(Wr, frames, pitch, H, W, Hp, Wp, f0, weight, out, partials, scale);
-  else
-    k_wav_out<kBF16, MODE><<<g, kWB, 0, s>>>(Wr, frames, pitch, H, W, Hp, Wp, f0, weight, out, partials, scale);
-  PRNU_CUDA_TRY(cudaGetLastError());
-}
+int pad16(int n) { return (n + 15) / 16 * 16; }
+dim3 tiles(int h, int w, int n) { return dim3((w / 2 + kTS - 1) / kTS, (h / 2 + kTS - 1) / kTS, n); }
 
 }  // namespace
 
-size_t wavelet_partials_needed(int F, int H, int W) { return (size_t)F * H * ((W + kWB - 1) / kWB); }
-
-namespace {
-
-// W(I) of nf frames into bufT (pitch Wp, frame stride Hp*Wp); bufA is scratch
-void wavelet_chunk(const uint8_t* fr, int nf, int H, int W, size_t pitch, float s0sq, float* bufA, float* bufT,
-                   cudaStream_t s, LaunchCounter& lc) {
-  constexpr int kLevels = 4;
-  const int Hp = (H + 15) / 16 * 16, Wp = (W + 15) / 16 * 16;
-  k_wav_pad<<<dim3((Wp + kWB - 1) / kWB, Hp, nf), kWB, 0, s>>>(fr, pitch, H, W, Hp, Wp, bufA);
-  PRNU_CUDA_TRY(cudaGetLastError());
-  lc.n++;
-  for (int l = 0; l < kLevels; ++l) {   // forward: A -> T (rows) -> A (columns)
-    const int h = Hp >> l, w = Wp >> l;
-    k_wav_rows<<<dim3((w / 2 + kWB - 1) / kWB, h, nf), kWB, 0, s>>>(bufA, w, Hp, Wp, bufT);
-    k_wav_cols<<<dim3((w + kWB - 1) / kWB, h / 2, nf), kWB, 0, s>>>(bufT, h, w, Hp, Wp, bufA);
-    PRNU_CUDA_TRY(cudaGetLastError());
-    lc.n += 2;
-  }
-  for (int l = 0; l < kLevels; ++l) {   // noise parts of the detail bands: A -> T
-    const int h2 = (Hp >> l) / 2, w2 = (Wp >> l) / 2;
-    k_wav_shrink<<<dim3((w2 + kSX - 1) / kSX, (h2 + kSY - 1) / kSY, 3 * nf), dim3(kSX, kSY), 0, s>>>(
-        bufA, h2, w2, Hp, Wp, s0sq, bufT);
-    PRNU_CUDA_TRY(cudaGetLastError());
-    lc.n++;
-  }
-  {
-    const int h = Hp >> kLevels, w = Wp >> kLevels;
-    k_wav_zero<<<dim3((w + kWB - 1) / kWB, h, nf), kWB, 0, s>>>(h, w, Hp, Wp, bufT);
-    PRNU_CUDA_TRY(cudaGetLastError());
-    lc.n++;
-  }
-  for (int l = kLevels - 1; l >= 0; --l) {   // inverse: T (columns) -> A (rows) -> T
-    const int h = Hp >> l, w = Wp >> l;
-    k_wav_icols<<<dim3((w + kWB - 1) / kWB, h, nf), kWB, 0, s>>>(bufT, h, w, Hp, Wp, bufA);
-    k_wav_irows<<<dim3((w + kWB - 1) / kWB, h, nf), kWB, 0, s>>>(bufA, w, Hp, Wp, bufT);
-    PRNU_CUDA_TRY(cudaGetLastError());
-    lc.n += 2;
-  }
+size_t wavelet_partials_needed(int F, int H, int W) {
+  const dim3 g = tiles(pad16(H), pad16(W), 1);
+  return (size_t)F * g.x * g.y;
 }
-
-}  // namespace
 
 void launch_wavelet_residual(const uint8_t* frames, int F, int H, int W, size_t pitch, int flags, int dtype,
                              float sigma0, void* out, float* scale, float* bufA, float* bufT, int chunk,
                              double* partials, cudaStream_t s, LaunchCounter& lc) {
-  const int Hp = (H + 15) / 16 * 16, Wp = (W + 15) / 16 * 16;
+  const int Hp = pad16(H), Wp = pad16(W);
+  const size_t fs = (size_t)Hp * Wp;
   const int weight = (flags & PRNU_WEIGHT_BY_INTENSITY) ? 1 : 0;
   const bool norm = (flags & PRNU_NORMALISE) != 0;
   const float s0sq = sigma0 * sigma0;
-  const int gx = (W + kWB - 1) / kWB;
+  // offset of level l's dense image (l >= 1) in its buffer
+  auto off = [&](int l) {
+    size_t o = 0;
+    for (int k = 1; k < l; ++k) o += (size_t)(Hp >> k) * (Wp >> k);
+    return o;
+  };
+  const dim3 g0 = tiles(Hp, Wp, 1);
+  const int nblk = (int)(g0.x * g0.y);
   ProfScope ps(lc, kKindResidual, s);
   for (int f0 = 0; f0 < F; f0 += chunk) {
     const int nf = std::min(chunk, F - f0);
-    wavelet_chunk(frames + (size_t)f0 * H * pitch, nf, H, W, pitch, s0sq, bufA, bufT, s, lc);
-    if (norm) wav_out<1>(dtype, dim3(gx, H, nf), s, bufT, frames, pitch, H, W, Hp, Wp, f0, weight, out, partials, scale);
-    else wav_out<0>(dtype, dim3(gx, H, nf), s, bufT, frames, pitch, H, W, Hp, Wp, f0, weight, out, partials, scale);
-    lc.n++;
-  }
-  if (norm) {   // s = 1 / RMS(R) per frame, then the scaled store
-    launch_resid_scale(partials, gx * H, F, H, W, scale, s, lc);
-    for (int f0 = 0; f0 < F; f0 += chunk) {
-      const int nf = std::min(chunk, F - f0);
-      if (F > chunk)   // the buffers hold the last chunk only: recompute
-        wavelet_chunk(frames + (size_t)f0 * H * pitch, nf, H, W, pitch, s0sq, bufA, bufT, s, lc);
-      wav_out<2>(dtype, dim3(gx, H, nf), s, bufT, frames, pitch, H, W, Hp, Wp, f0, weight, out, partials, scale);
-      lc.n++;
+    const uint8_t* fr = frames + (size_t)f0 * H * pitch;
+    for (int l = 0; l < kLevels; ++l) {
+      const int h = Hp >> l, w = Wp >> l;
+      float* ll = l + 1 < kLevels ? bufT + off(l + 1) : nullptr;
+      if (l == 0) k_wav_analyse<true><<<tiles(h, w, nf), 256, 0, s>>>(fr, pitch, H, W, nullptr, fs, h, w, Wp, bufA, ll);
+      else k_wav_analyse<false><<<tiles(h, w, nf), 256, 0, s>>>(fr, pitch, H, W, bufT + off(l), fs, h, w, Wp, bufA, ll);
+      PRNU_CUDA_TRY(cudaGetLastError());
     }
-  } else if (scale) {
-    launch_fill(scale, F, 1.f, s, lc);
+    unsigned ntiles = 0;
+    for (int l = 0; l < kLevels; ++l)
+      ntiles += (((Wp >> (l + 1)) + kSX - 1) / kSX) * (((Hp >> (l + 1)) + kSY - 1) / kSY);
+    // |c| <= 16 * 255 (four levels of gain 2), so den <= 2^25 + s0 and c s0 <= 2^12 s0
+    auto* shrink = s0sq >= 1e-18f && s0sq <= 1e18f ? k_wav_shrink<true> : k_wav_shrink<false>;
+    shrink<<<dim3(ntiles, 1, 3 * nf), 256, 0, s>>>(bufA, Hp, Wp, fs, s0sq, bufT);
+    PRNU_CUDA_TRY(cudaGetLastError());
+    auto synth = [&](auto* fn, int l) {
+      const int h = Hp >> l, w = Wp >> l;
+      fn<<<tiles(h, w, nf), 256, 0, s>>>(bufT, l + 1 < kLevels ? bufA + off(l + 1) : nullptr, fs, h, w, Wp,
+                                         l ? bufA + off(l) : nullptr, frames, pitch, H, W, f0, weight, out, partials, scale);
+      PRNU_CUDA_TRY(cudaGetLastError());
+      lc.n++;
+    };
+    for (int l = kLevels - 1; l >= 1; --l) synth(k_wav_synth<kF32, 0>, l);
+    lc.n += kLevels + 1;
+    if (!norm) {
+      synth(dtype == kF32 ? k_wav_synth<kF32, 1> : dtype == kF16 ? k_wav_synth<kF16, 1> : k_wav_synth<kBF16, 1>, 0);
+      continue;
+    }
+    // s = 1 / RMS(R) per frame, then the last level again with the scaled store
+    synth(k_wav_synth<kF32, 2>, 0);
+    launch_resid_scale(partials + (size_t)f0 * nblk, nblk, nf, H, W, scale + f0, s, lc);
+    synth(dtype == kF32 ? k_wav_synth<kF32, 3> : dtype == kF16 ? k_wav_synth<kF16, 3> : k_wav_synth<kBF16, 3>, 0);
   }
+  if (!norm && scale) launch_fill(scale, F, 1.f, s, lc);
 }
 
 }  // namespace prnu
