@@ -358,7 +358,9 @@ void enqueue_search(prnu_ctx* c, const SearchCall& call, prnu_result* d_out, dou
     launch_pad_frames(call.resid, call.rdtype, call.F, H, W, c->ws_pad.p, s, c->launches, pairs ? 1 : 0);
     a.resid = c->ws_pad.p;
   }
-  a.rdtype = pairs ? (call.rdtype == kF16 ? kF16P : kBF16P) : call.rdtype;
+  a.rdtype = pairs ? (call.rdtype == kF16 ? kF16P : kBF16P)
+             : call.prepadded && fs && !persistent ? (int)kF32I   // renders: identity warps
+                                                   : call.rdtype;
   a.rpitch = lay.rpitch;
   a.fpitch = lay.fpitch;
   a.roff = lay.roff;

@@ -14,7 +14,10 @@ enum StoreType { kF32 = 0, kF16 = 1, kBF16 = 2 };
 // half storage: element x holds the pair (R[x], R[x + 1]) as one 4-byte
 // word, so a bilinear sample takes one aligned load per row.
 enum PairStoreType { kF16P = 3, kBF16P = 4 };
-constexpr int kNumStoreLayouts = 5;
+// FP32 residuals in the zero-bordered layout whose items all warp by the
+// identity: the planned row kernels read each pixel itself.
+enum { kF32I = 5 };
+constexpr int kNumStoreLayouts = 6;
 
 // One candidate of the search: which frame, which fingerprint, which grid
 // node, where its result goes, and the inverse-warp matrix

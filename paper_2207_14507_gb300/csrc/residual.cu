@@ -470,12 +470,16 @@ __global__ void __launch_bounds__(kBX * 8, 2) k_fp_estimate(const uint8_t* __res
 // X is not an integer image, so the moments are taken in float from the
 // differences to the window's centre (d = x_k - x_c: mean m1 = sum d / 9,
 // variance sum d^2 / 9 - m1^2), which keeps the cancellation small.  A block
-// warps its 32x8 tile plus a one-pixel halo into shared memory; halo pixels
+// warps a 64 x 64 tile plus a one-pixel halo into shared memory; halo pixels
 // outside the frame are the warped values at the clamped position (the
-// replicated border).
+// replicated border).  A thread takes two adjacent columns, packed, down 8
+// rows.  At 1080p a render takes 6.3 us of warp and moments and 3.3 us
+// of residual (one pixel a thread from shared memory and general bounds tests
+// everywhere: 11.4 and 7.4), both bound by issue.
 
-constexpr int kLX = 32, kLY = 32, kLR = 4, kLTX = kLX + 2, kLTY = kLY + 2;   // 32 x 8 threads, 4 rows each
-static_assert(kLY == 8 * kLR, "a thread covers kLR rows of the tile");
+constexpr int kLX = 64, kLY = 64, kLR = 8;
+constexpr int kLP = kLX + 4, kLTY = kLY + 2;   // tile pitch and rows: pixel (x, y) of the tile at (x + 2, y + 1)
+static_assert(kLX == 2 * 32 && kLY == 8 * kLR, "a lane takes a column pair, each of 8 warps kLR rows");
 
 // uint8 -> float without a conversion instruction: the byte in the low
 // mantissa bits of 2^23 (exact for every byte value)
@@ -502,78 +506,124 @@ __device__ __forceinline__ float warp_u8(const uint8_t* __restrict__ fr, int pit
   return fmaf(fy, bot, (1.f - fy) * top);
 }
 
-// the warped tile with its halo, tile[(ty + 1) * kLTX + tx + 1] = X(x, y)
-__device__ __forceinline__ void warp_tile(const uint8_t* __restrict__ frames, size_t pitch, int H, int W,
-                                          const WorkItem& it, float* tile) {
-  const uint8_t* fr = frames + (size_t)it.frame * H * pitch;
-  const float cx = 0.5f * (float)(W - 1), cy = 0.5f * (float)(H - 1);
-  const int tid = threadIdx.y * kLX + threadIdx.x;
-  const int x0 = blockIdx.x * kLX - 1, y0 = blockIdx.y * kLY - 1;
-#pragma unroll
-  for (int k0 = 0; k0 < kLTX * kLTY; k0 += kLX * 8) {
-    const int k = k0 + tid;
-    if (k < kLTX * kLTY) {
-      const int sy = k / kLTX, sx = k - sy * kLTX;
-      const int y = min(max(y0 + sy, 0), H - 1), x = min(max(x0 + sx, 0), W - 1);
-      tile[k] = warp_u8(fr, (int)pitch, H, W, it, cx, cy, x, y);
-    }
-  }
-  __syncthreads();
+// warp_u8 where the four taps lie inside the frame: floor(q) by rounding q - 1/2
+// to an integer at 1.5 * 2^23 (an integer q may give q - 1 and weight 1 on its
+// own tap: the same value), whose mantissa holds the tap's index
+__device__ __forceinline__ float warp_u8_inside(const uint8_t* __restrict__ fr, int pitch, float qx, float qy) {
+  constexpr float kRound = 12582912.f;
+  constexpr int kBits = 0x4B400000;
+  const float tx = (qx - 0.5f) + kRound, ty = (qy - 0.5f) + kRound;
+  const float fx = qx - (tx - kRound), fy = qy - (ty - kRound);
+  const uint8_t* p = fr + ((__float_as_int(ty) - kBits) * pitch + (__float_as_int(tx) - kBits));
+  const uint8_t* r = p + pitch;
+  const float v00 = u8f(__ldg(p)), v01 = u8f(__ldg(p + 1)), v10 = u8f(__ldg(r)), v11 = u8f(__ldg(r + 1));
+  const float top = fmaf(fx, v01 - v00, v00), bot = fmaf(fx, v11 - v10, v10);
+  return fmaf(fy, bot - top, top);
 }
 
-// centre value, window mean offset m1 and population variance of tile pixel (tx, ty)
-__device__ __forceinline__ void tile_moments(const float* tile, int tx, int ty, float* xc, float* m1, float* var) {
-  const float c = tile[(ty + 1) * kLTX + tx + 1];
-  float s1 = 0.f, s2 = 0.f;
-#pragma unroll
-  for (int dy = 0; dy < 3; ++dy)
-#pragma unroll
-    for (int dx = 0; dx < 3; ++dx) {
-      const float d = tile[(ty + dy) * kLTX + tx + dx] - c;
-      s1 += d;
-      s2 = fmaf(d, d, s2);
-    }
-  const float m = s1 * (1.f / 9.f);
-  *xc = c;
-  *m1 = m;
-  *var = fmaf(-m, m, s2 * (1.f / 9.f));
+// Window mean offset m1 and population variance of a column pair's pixels,
+// from the rows above, at and below: l, c, r the pairs (x-1, x), (x, x+1) and
+// (x+1, x+2).
+struct PairRow {
+  float2 l, c, r;
+};
+__device__ __forceinline__ void pair_moments(const PairRow& up, const PairRow& mid, const PairRow& dn, float2& m1,
+                                             float2& var) {
+  const float2 nc = make_float2(-mid.c.x, -mid.c.y);
+  float2 s1 = make_float2(0.f, 0.f), s2 = s1;
+  auto term = [&](float2 v) {
+    const float2 d = __fadd2_rn(v, nc);
+    s1 = __fadd2_rn(s1, d);
+    s2 = __ffma2_rn(d, d, s2);
+  };
+  term(up.l);
+  term(up.c);
+  term(up.r);
+  term(mid.l);
+  term(mid.r);
+  term(dn.l);
+  term(dn.c);
+  term(dn.r);
+  const float2 ninth = make_float2(1.f / 9.f, 1.f / 9.f);
+  m1 = __fmul2_rn(s1, ninth);
+  var = __ffma2_rn(make_float2(-m1.x, -m1.y), m1, __fmul2_rn(s2, ninth));
 }
 
 // per block: sum of the local variances of its pixels (double), one slot per
 // block; the warped frame itself to X[r][H][W] for the second pass
-__global__ void __launch_bounds__(kLX * 8) k_lit_moments(const uint8_t* __restrict__ frames, size_t pitch, int H,
-                                                         int W, const WorkItem* __restrict__ renders,
-                                                         double* __restrict__ partials, float* __restrict__ X) {
-  __shared__ float tile[kLTX * kLTY];
+__global__ void __launch_bounds__(256) k_lit_moments(const uint8_t* __restrict__ frames, size_t pitch, int H, int W,
+                                                     const WorkItem* __restrict__ renders,
+                                                     double* __restrict__ partials, float* __restrict__ X) {
+  __shared__ __align__(16) float tile[kLTY * kLP];
   __shared__ double part[8];
   const WorkItem it = renders[blockIdx.z];
-  warp_tile(frames, pitch, H, W, it, tile);
-  const int tx = threadIdx.x, x = blockIdx.x * kLX + tx;
-  if (x < W) {
-    float* xo = X + (size_t)blockIdx.z * H * W + x;
+  const uint8_t* fr = frames + (size_t)it.frame * H * pitch;
+  const float cx = 0.5f * (float)(W - 1), cy = 0.5f * (float)(H - 1);
+  const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
+  const int x0 = blockIdx.x * kLX, y0 = blockIdx.y * kLY;
+  const int xa = max(x0 - 1, 0), xb = min(x0 + kLX, W - 1), ya = max(y0 - 1, 0), yb = min(y0 + kLY, H - 1);
+  auto map = [&](int x, int y, float& qx, float& qy) {
+    const float dx = (float)x - cx, dy = (float)y - cy;
+    qx = fmaf(it.a11, dx, fmaf(it.a12, dy, cx));
+    qy = fmaf(it.a21, dx, fmaf(it.a22, dy, cy));
+  };
+  // the map is affine: its corners bound the tile
+  bool inside = true;
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    float qx, qy;
+    map(k & 1 ? xb : xa, k & 2 ? yb : ya, qx, qy);
+    inside = inside && qx >= 1.5f && qx <= (float)W - 2.5f && qy >= 1.5f && qy <= (float)H - 2.5f;
+  }
+  auto sample = [&](int sx, int sy) {   // tile pixel (sx - 1, sy - 1)
+    const int x = min(max(x0 + sx - 1, 0), W - 1), y = min(max(y0 + sy - 1, 0), H - 1);
+    float v;
+    if (inside) {
+      float qx, qy;
+      map(x, y, qx, qy);
+      v = warp_u8_inside(fr, (int)pitch, qx, qy);
+    } else {
+      v = warp_u8(fr, (int)pitch, H, W, it, cx, cy, x, y);
+    }
+    tile[sy * kLP + sx + 1] = v;
+  };
+  for (int sy = wp; sy < kLTY; sy += 8) {
+    sample(lane + 1, sy);
+    sample(lane + 33, sy);
+  }
+  if (threadIdx.x < 2 * kLTY) sample(threadIdx.x & 1 ? kLX + 1 : 0, threadIdx.x >> 1);   // the two halo columns
+  __syncthreads();
+  const int x = x0 + 2 * lane, ys = y0 + wp * kLR;
+  float2 acc[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+  if (x < W) {   // W is even: both pixels of the pair
+    auto row = [&](int k) {   // tile row k of this warp's band (0: the row above it)
+      const float2* p = reinterpret_cast<const float2*>(tile + (wp * kLR + k) * kLP) + lane;
+      const float2 a = p[0], c = p[1], b = p[2];
+      return PairRow{make_float2(a.y, c.x), c, make_float2(c.y, b.x)};
+    };
+    PairRow up = row(0), mid = row(1);
+    float* xo = X + ((size_t)blockIdx.z * H + ys) * W + x;
 #pragma unroll
     for (int k = 0; k < kLR; ++k) {
-      const int ty = threadIdx.y + 8 * k, y = blockIdx.y * kLY + ty;
-      if (y < H) xo[(size_t)y * W] = tile[(ty + 1) * kLTX + tx + 1];
+      const PairRow dn = row(k + 2);
+      if (ys + k < H) {
+        *reinterpret_cast<float2*>(xo + (size_t)k * W) = mid.c;
+        float2 m, var;
+        pair_moments(up, mid, dn, m, var);
+        acc[k & 1] = __fadd2_rn(acc[k & 1], var);
+      }
+      up = mid;
+      mid = dn;
     }
   }
-  // float within a warp (128 terms), double across warps and blocks: the FP64
-  // pipe is a small fraction of the FP32 one, so it takes one add per warp
-  float v = 0.f;
-#pragma unroll
-  for (int k = 0; k < kLR; ++k) {
-    const int ty = threadIdx.y + 8 * k, y = blockIdx.y * kLY + ty;
-    if (x < W && y < H) {
-      float c, m, var;
-      tile_moments(tile, tx, ty, &c, &m, &var);
-      v += var;
-    }
-  }
+  // float within a warp, double across warps and blocks: the FP64 pipe is a
+  // small fraction of the FP32 one, so it takes one add per warp
+  float v = (acc[0].x + acc[1].x) + (acc[0].y + acc[1].y);
 #pragma unroll
   for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  if (tx == 0) part[threadIdx.y] = (double)v;
+  if (lane == 0) part[wp] = (double)v;
   __syncthreads();
-  if (threadIdx.y == 0 && tx == 0) {
+  if (threadIdx.x == 0) {
     double s = 0.0;
     for (int k = 0; k < 8; ++k) s += part[k];
     partials[(size_t)blockIdx.z * gridDim.x * gridDim.y + blockIdx.y * gridDim.x + blockIdx.x] = s;
@@ -597,41 +647,42 @@ __global__ void k_lit_noise(const double* __restrict__ partials, int nblk, int H
   }
 }
 
-// R of every pixel into out[r * lay.fpitch + lay.roff + y * lay.rpitch + x] (float)
-// (the tile and its replicated halo read back from X, the first pass's warped frame)
-__global__ void __launch_bounds__(kLX * 8) k_lit_apply(const float* __restrict__ X, int H, int W,
-                                                       const float* __restrict__ nu2, int weight,
-                                                       float* __restrict__ out, ResidLayout lay) {
-  __shared__ float tile[kLTX * kLTY];
-  {
-    const float* xr = X + (size_t)blockIdx.z * H * W;
-    const int tid = threadIdx.y * kLX + threadIdx.x;
-    const int x0 = blockIdx.x * kLX - 1, y0 = blockIdx.y * kLY - 1;
-#pragma unroll
-    for (int k0 = 0; k0 < kLTX * kLTY; k0 += kLX * 8) {
-      const int k = k0 + tid;
-      if (k < kLTX * kLTY) {
-        const int sy = k / kLTX, sx = k - sy * kLTX;
-        const int y = min(max(y0 + sy, 0), H - 1), x = min(max(x0 + sx, 0), W - 1);
-        tile[k] = __ldg(xr + (size_t)y * W + x);
-      }
-    }
-    __syncthreads();
-  }
-  const int tx = threadIdx.x, x = blockIdx.x * kLX + tx;
-  if (x >= W) return;
+// R of every pixel into out[r * lay.fpitch + lay.roff + y * lay.rpitch + x]
+// (float) from X, the first pass's warped frame, a column pair and kLR rows to
+// a thread, straight from global memory
+__global__ void __launch_bounds__(256) k_lit_apply(const float* __restrict__ X, int H, int W,
+                                                   const float* __restrict__ nu2, int weight, float* __restrict__ out,
+                                                   ResidLayout lay) {
+  const int x = blockIdx.x * kLX + 2 * (threadIdx.x & 31), ys = blockIdx.y * kLY + (threadIdx.x >> 5) * kLR;
+  if (x >= W || ys >= H) return;
+  const float* xr = X + (size_t)blockIdx.z * H * W;
+  const int xl = max(x - 1, 0), xh = min(x + 2, W - 1);
+  auto row = [&](int y) {
+    const float* p = xr + (size_t)min(max(y, 0), H - 1) * W;
+    const float2 c = __ldg(reinterpret_cast<const float2*>(p + x));
+    return PairRow{make_float2(__ldg(p + xl), c.x), c, make_float2(c.y, __ldg(p + xh))};
+  };
   const float n2 = nu2[blockIdx.z];
-  float* o = out + (size_t)blockIdx.z * lay.fpitch + lay.roff + x;
-#pragma unroll
-  for (int k = 0; k < kLR; ++k) {
-    const int ty = threadIdx.y + 8 * k, y = blockIdx.y * kLY + ty;
-    if (y >= H) break;
-    float c, m, var;
-    tile_moments(tile, tx, ty, &c, &m, &var);
+  auto wiener = [&](float m, float var) {   // x - (mu + (x - mu) gain), x - mu = -m1
     const float den = fmaxf(var, n2);
     const float gain = den > 0.f ? __fdividef(fmaxf(var - n2, 0.f), den) : 1.f;
-    const float w = -m * (1.f - gain);   // x - (mu + (x - mu) gain), x - mu = -m1
-    o[(size_t)y * lay.rpitch] = weight ? c * w : w;
+    return -m * (1.f - gain);
+  };
+  float* o = out + (size_t)blockIdx.z * lay.fpitch + lay.roff + (size_t)ys * lay.rpitch + x;
+  PairRow up = row(ys - 1), mid = row(ys);
+#pragma unroll
+  for (int k = 0; k < kLR; ++k) {
+    if (ys + k >= H) break;
+    const PairRow dn = row(ys + k + 1);
+    float2 m, var;
+    pair_moments(up, mid, dn, m, var);
+    float2 w = make_float2(wiener(m.x, var.x), wiener(m.y, var.y));
+    if (weight) w = __fmul2_rn(mid.c, w);
+    o[0] = w.x;
+    o[1] = w.y;
+    o += lay.rpitch;
+    up = mid;
+    mid = dn;
   }
 }
 
@@ -719,7 +770,7 @@ void launch_literal_residuals(const uint8_t* frames, size_t pitch, int H, int W,
                               float* nu2, cudaStream_t s, LaunchCounter& lc) {
   if (nr == 0) return;
   ProfScope ps(lc, kKindResidual, s);
-  const dim3 b(kLX, 8), g((W + kLX - 1) / kLX, (H + kLY - 1) / kLY, nr);
+  const dim3 b(256), g((W + kLX - 1) / kLX, (H + kLY - 1) / kLY, nr);
   k_lit_moments<<<g, b, 0, s>>>(frames, pitch, H, W, renders, partials, X);
   PRNU_CUDA_TRY(cudaGetLastError());
   k_lit_noise<<<nr, 256, 0, s>>>(partials, (int)(g.x * g.y), H, W, nu2);

@@ -214,6 +214,8 @@ struct StoreT<kBF16P> {
   using type = __nv_bfloat162;
   __device__ __forceinline__ static float2 ld2(const __nv_bfloat162* p) { return __bfloat1622float2(__ldg(p)); }
 };
+template <>
+struct StoreT<kF32I> : StoreT<kF32> {};
 template <int DT>
 constexpr bool kPairStore = DT == kF16P || DT == kBF16P;
 

@@ -100,7 +100,11 @@ __device__ __forceinline__ void row_forward_body(const PassArgs& a, int is, int 
   if (t < NB0) {
     float2 v[16];
     const float dxj = (float)t - cx;
-    if (inside) warp_row16<DT, W, NB0, false>(fr, H, it, dxj, bx0, by0, bx1, by1, v);
+    if constexpr (DT == kF32I) {
+      const float* p = fr + (size_t)y0 * pad_pitch(W) + t;
+#pragma unroll
+      for (int r = 0; r < 16; ++r) v[r] = make_float2(__ldg(p + r * NB0), __ldg(p + pad_pitch(W) + r * NB0));
+    } else if (inside) warp_row16<DT, W, NB0, false>(fr, H, it, dxj, bx0, by0, bx1, by1, v);
     else warp_row16<DT, W, NB0, true>(fr, H, it, dxj, bx0, by0, bx1, by1, v);
     Dft<16, false>::run(v);
     row_store16(A, t, v);
@@ -851,6 +855,7 @@ struct ShapeDef {
     r.fwd[kBF16] = row_fwd<kBF16, PPB, RFMB>();
     r.fwd[kF16P] = row_fwd<kF16P, PPB, RFMB>();
     r.fwd[kBF16P] = row_fwd<kBF16P, PPB, RFMB>();
+    r.fwd[kF32I] = row_fwd<kF32I, PPB, RFMB>();
     if constexpr (RIMB > 0) r.inv = (void*)k_row_inverse_mb<RS, RTI, PPB, RIMB>;
     else r.inv = (void*)k_row_inverse_fx<RS, RTI, PPB>;
     r.fin = (void*)k_finalize_fx<RS, FT, kFinPairs>;
