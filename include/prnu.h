@@ -417,7 +417,9 @@ int prnu_server_stats_get(prnu_ctx* ctx, prnu_server_stats* out);
 /* ---------------------------------------------------------------- tuning */
 
 /* Launch configuration of the fused path for one frame size: columns per
- * column-pass block and row pairs per row block of the generic kernels, the
+ * column-pass block and row pairs per row block of the generic kernels (sides
+ * that are the product of two radices up to 48 have two-stage passes with
+ * their own blocks and take neither), the
  * candidates per wave (per-candidate spectra kept in the workspace), and which
  * compile-time-planned column kernel to use where the size has them
  * (1920x1080, 1280x720, 3840x2160, 256x256). */

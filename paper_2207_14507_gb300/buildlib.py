@@ -17,8 +17,9 @@ CSRC = os.path.join(HERE, "csrc")
 BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libprnu.so")
 SOURCES = ["search_fixed_2160.cu", "search_fixed_1080.cu", "search_fixed_720.cu", "search_fixed_256.cu",
-           "api.cu", "search.cu", "search_fixed.cu", "residual.cu", "wavelet.cu", "serve.cu", "autotune.cu",
-           "noalloc.cu", "wave_loop.cu"]
+           "api.cu", "search.cu", "col_generic.cu", "row_generic.cu", "row_generic_f32.cu", "row_generic_f16.cu",
+           "row_generic_bf16.cu", "search_fixed.cu", "residual.cu", "wavelet.cu", "serve.cu", "autotune.cu", "noalloc.cu",
+           "wave_loop.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "--expt-relaxed-constexpr",
          "-I" + os.path.join(ROOT, "include")]

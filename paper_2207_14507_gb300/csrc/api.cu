@@ -80,7 +80,7 @@ bool is_5smooth(int n) {
   return n == 1;
 }
 
-FftPlan make_plan(int n, const std::vector<int>& tw_offsets) {
+FftPlan make_plan_at(int n, int tw_base) {
   FftPlan p{};
   PRNU_CHECK_ARG(n >= 2 && n <= kMaxFft && is_5smooth(n), "FFT length must be 5-smooth in [2, 4096]");
   std::vector<int> cur, best;
@@ -88,10 +88,50 @@ FftPlan make_plan(int n, const std::vector<int>& tw_offsets) {
   PRNU_CHECK_ARG(!best.empty() && (int)best.size() <= kMaxStages, "no FFT plan");
   p.n = n;
   p.nstages = (int)best.size();
-  for (int i = 0; i < p.nstages; ++i) p.radix[i] = best[i];
+  int ns = 1, off = tw_base;
+  for (int i = 0; i < p.nstages; ++i) {
+    p.radix[i] = best[i];
+    p.ns[i] = ns;
+    p.inv[i] = ns > 1 ? (unsigned)(((1ull << 32) + ns - 1) / ns) : 0;
+    p.tw[i] = off;
+    off += stage_tw_len(best[i], ns);
+    ns *= best[i];
+  }
   p.min_radix = best.back();
-  p.tw_off = tw_offsets[n];
+  if (col2_radices(n, &p.ra, &p.rb)) {
+    p.tw_fwd = off;
+    p.tw_inv = off + stage_tw_len(p.rb, p.ra);
+  }
   return p;
+}
+
+FftPlan make_plan(int n, const std::vector<int>& tw_offsets) {
+  PRNU_CHECK_ARG(n >= 2 && n <= kMaxFft && tw_offsets[n] >= 0, "no twiddles for this FFT length");
+  return make_plan_at(n, tw_offsets[n]);
+}
+
+// The twiddles of plan p, appended to the table.
+static void append_plan_twiddles(const FftPlan& p, std::vector<float4>& tab) {
+  std::vector<float2> w(p.n);   // exp(-2 pi i k / n)
+  for (int k = 0; k < p.n; ++k) {
+    const double a = 2.0 * 3.14159265358979323846 * (double)k / (double)p.n;
+    w[k] = make_float2((float)cos(a), (float)(-sin(a)));
+  }
+  auto stage = [&](int R, int ns) {
+    const long long unit = p.n / (ns * R);
+    for (int m = 0; m < R / 2; ++m)
+      for (int k = 0; k < ns; ++k) {
+        const float2 u = w[(2 * m + 1) * k * unit % p.n];
+        const float2 v = 2 * m + 2 < R ? w[(2 * m + 2) * k * unit % p.n] : make_float2(0.f, 0.f);
+        tab.push_back(make_float4(u.x, u.y, v.x, v.y));
+      }
+  };
+  for (int i = 0; i < p.nstages; ++i)
+    if (p.ns[i] > 1) stage(p.radix[i], p.ns[i]);
+  if (p.ra) {
+    stage(p.rb, p.ra);
+    stage(p.ra, p.rb);
+  }
 }
 
 void row_launch_shape(const FftPlan& p, int* threads, int* maxb) {
@@ -1009,19 +1049,16 @@ int prnu_create(prnu_ctx** out, int device, size_t hbm_budget_bytes) {
     size_t fr = 0, tot = 0;
     PRNU_CUDA_TRY(cudaMemGetInfo(&fr, &tot));
     c->budget = hbm_budget_bytes ? hbm_budget_bytes : (size_t)(0.9 * (double)fr);
-    // twiddles w_n^k = exp(-2 pi i k / n) for every 5-smooth n <= 4096
+    // stage twiddles of the plans of every length a side can have
     c->tw_off.assign(kMaxFft + 1, -1);
-    std::vector<float2> tw;
-    for (int n = 1; n <= kMaxFft; ++n) {
+    std::vector<float4> tw;
+    for (int n = 16; n <= kMaxFft; n += 2) {
       if (!is_5smooth(n)) continue;
       c->tw_off[n] = (int)tw.size();
-      for (int k = 0; k < n; ++k) {
-        const double a = 2.0 * 3.14159265358979323846 * (double)k / (double)n;
-        tw.push_back(make_float2((float)cos(a), (float)(-sin(a))));
-      }
+      append_plan_twiddles(make_plan(n, c->tw_off), tw);
     }
-    const size_t twb = tw.size() * sizeof(float2);
-    c->d_tw = reinterpret_cast<float2*>(ctx_alloc(c.get(), twb));
+    const size_t twb = tw.size() * sizeof(float4);
+    c->d_tw = reinterpret_cast<float4*>(ctx_alloc(c.get(), twb));
     c->tw_bytes = twb;
     PRNU_CUDA_TRY(cudaMemcpy(c->d_tw, tw.data(), twb, cudaMemcpyHostToDevice));
     PRNU_CUDA_TRY(cudaEventCreateWithFlags(&c->last_done, cudaEventDisableTiming));

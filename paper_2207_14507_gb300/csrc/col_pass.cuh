@@ -28,6 +28,7 @@
 // consecutive j and columns, store to distinct banks; TMA's side of the strip
 // is dense.  Every shared address is a per-thread base plus a constant.
 #pragma once
+#include "col_generic.cuh"
 #include "common.cuh"
 #include "fft_fixed.cuh"
 #include "fft_packed.cuh"
@@ -47,19 +48,6 @@ struct ColPlan {
   static constexpr int lanes = RA > RB ? RA : RB;                      // threads per column
   static_assert(RA * RB == H, "two radices");
 };
-
-// The product for the packed column 0 (DC + i*Nyquist columns of two real
-// spectra in one complex column): F, Fm the frame bins i and H - i, S, Sm the
-// fingerprint bins; unpack both, conj-multiply each real column's spectrum,
-// repack.
-__device__ __forceinline__ float2 packed_col0_product(float2 F, float2 Fm, float2 S, float2 Sm) {
-  const float2 Aa = make_float2(0.5f * (F.x + Fm.x), 0.5f * (F.y - Fm.y));
-  const float2 Bb = make_float2(0.5f * (F.y + Fm.y), 0.5f * (Fm.x - F.x));
-  const float2 Ka = make_float2(0.5f * (S.x + Sm.x), 0.5f * (S.y - Sm.y));
-  const float2 Kb = make_float2(0.5f * (S.y + Sm.y), 0.5f * (Sm.x - S.x));
-  const float2 p1 = c_conj_mul(Aa, Ka), p2 = c_conj_mul(Bb, Kb);
-  return make_float2(p1.x - p2.y, p1.y + p2.x);
-}
 
 // bytes per fingerprint bin of the separate fingerprint region (MODE 3: FP32
 // or FP16 bins; MODE 4: FP16 bins only)

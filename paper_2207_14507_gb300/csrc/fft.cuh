@@ -11,8 +11,8 @@
 // compile time: sizes 2..5 from their closed forms, the others by a two-factor
 // Cooley-Tukey split R = P*Q whose inner twiddles are compile-time constants.
 // Those constants come from a constexpr Taylor series (they are only ever
-// w_R^k for R <= 16); the stage twiddles w_n^k come from a table the host
-// builds in double precision and rounds to float.
+// w_R^k for small R); the stage twiddles come from tables built in double
+// precision and rounded to float.
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -225,142 +225,24 @@ struct Dft {
 constexpr int kMaxStages = 8;
 constexpr int kMaxFft = 4096;
 
-// A length-n plan: radices in execution order and the offset of the w_n^k
-// table (n entries) inside the context's twiddle buffer.
+// A length-n plan: radices in execution order; per stage the product of the
+// earlier radices, ceil(2^32 / ns) (j mod ns by one high multiplication, exact
+// for j < 2^16) and the place of its twiddles in the table (fft_plan.cuh), in
+// float4.  ra, rb: where n is the product of two radices that one thread can
+// hold, the two-stage plan of the column pass (col_generic.cuh), with the
+// twiddles of its second forward and second inverse stage; else 0.
 struct FftPlan {
   int n;
   int nstages;
   int radix[kMaxStages];
-  int tw_off;
+  int ns[kMaxStages];
+  unsigned inv[kMaxStages];
+  int tw[kMaxStages];
   int min_radix;
+  int ra, rb, tw_fwd, tw_inv;
 };
 
-// ---------------------------------------------------------------- stages
-//
-// Stages run out of place between two shared-memory buffers (ping-pong): a
-// thread loads one butterfly's R inputs, transforms them in registers and
-// stores the R outputs before it takes the next butterfly, so no register
-// state crosses a barrier.  Two layouts:
-//  * row layout: one FFT per thread group, element i at i + (i >> 4) (one
-//    float2 of padding every 16 keeps the strided stores off one bank);
-//  * column layout: NC = 1 << lg interleaved FFTs (columns), element i of
-//    column c at i*NC + c; butterflies are spread over all threads of the block.
-
-__device__ __forceinline__ int rpad(int i) { return i + (i >> 4); }
-__host__ __device__ constexpr int row_smem_len(int n) { return n + (n >> 4) + 1; }
-
-template <int R, bool INV>
-__device__ __forceinline__ void twiddle_inputs(float2 (&v)[R], int k, int step_unit,
-                                               const float2* __restrict__ tw) {
-  // v[r] *= w_n^{r * k * step_unit}, step_unit = n / (Ns * R)
-  if (k == 0) return;
-  const int s = k * step_unit;
-#pragma unroll
-  for (int r = 1; r < R; ++r) {
-    float2 w = __ldg(tw + r * s);
-    v[r] = INV ? c_mulc(v[r], w) : c_mul(v[r], w);
-  }
-}
-
-template <int R, bool INV>
-__device__ __forceinline__ void stage_row(const float2* __restrict__ in, float2* __restrict__ out, int n, int ns,
-                                          const float2* __restrict__ tw, int t, int T) {
-  const int nb = n / R;
-  const int unit = n / (ns * R);
-  for (int j = t; j < nb; j += T) {
-    float2 v[R];
-#pragma unroll
-    for (int r = 0; r < R; ++r) v[r] = in[rpad(j + r * nb)];
-    const int k = j % ns;
-    twiddle_inputs<R, INV>(v, k, unit, tw);
-    Dft<R, INV>::run(v);
-    const int base = (j - k) * R + k;
-#pragma unroll
-    for (int r = 0; r < R; ++r) out[rpad(base + r * ns)] = v[r];
-  }
-}
-
-template <int R, bool INV>
-__device__ __forceinline__ void stage_col(const float2* __restrict__ in, float2* __restrict__ out, int n, int ns,
-                                          const float2* __restrict__ tw, int t, int T, int lg) {
-  const int nb = n / R;
-  const int unit = n / (ns * R);
-  const int total = nb << lg;
-  const int cm = (1 << lg) - 1;
-  for (int g = t; g < total; g += T) {
-    const int j = g >> lg, c = g & cm;
-    float2 v[R];
-#pragma unroll
-    for (int r = 0; r < R; ++r) v[r] = in[((j + r * nb) << lg) + c];
-    const int k = j % ns;
-    twiddle_inputs<R, INV>(v, k, unit, tw);
-    Dft<R, INV>::run(v);
-    const int base = (j - k) * R + k;
-#pragma unroll
-    for (int r = 0; r < R; ++r) out[((base + r * ns) << lg) + c] = v[r];
-  }
-}
-
-// Full FFT of the data in `a` (row layout), using `b` as the second buffer.
-// Every thread of the block must call it (it holds barriers); a thread of a
-// group without a row passes t >= n so that it owns no butterfly.  The caller
-// synchronises before the call; the result is in the returned buffer and is
-// visible to the whole block on return.
-template <bool INV>
-__device__ float2* fft_row(float2* a, float2* b, const FftPlan& p, const float2* __restrict__ twtab, int t, int T) {
-  const float2* tw = twtab + p.tw_off;
-  int ns = 1;
-  for (int s = 0; s < p.nstages; ++s) {
-    const int R = p.radix[s];
-    switch (R) {
-      case 2: stage_row<2, INV>(a, b, p.n, ns, tw, t, T); break;
-      case 3: stage_row<3, INV>(a, b, p.n, ns, tw, t, T); break;
-      case 4: stage_row<4, INV>(a, b, p.n, ns, tw, t, T); break;
-      case 5: stage_row<5, INV>(a, b, p.n, ns, tw, t, T); break;
-      case 6: stage_row<6, INV>(a, b, p.n, ns, tw, t, T); break;
-      case 8: stage_row<8, INV>(a, b, p.n, ns, tw, t, T); break;
-      case 9: stage_row<9, INV>(a, b, p.n, ns, tw, t, T); break;
-      case 10: stage_row<10, INV>(a, b, p.n, ns, tw, t, T); break;
-      case 12: stage_row<12, INV>(a, b, p.n, ns, tw, t, T); break;
-      case 15: stage_row<15, INV>(a, b, p.n, ns, tw, t, T); break;
-      default: stage_row<16, INV>(a, b, p.n, ns, tw, t, T); break;
-    }
-    __syncthreads();
-    float2* x = a;
-    a = b;
-    b = x;
-    ns *= R;
-  }
-  return a;
-}
-
-template <bool INV>
-__device__ float2* fft_col(float2* a, float2* b, const FftPlan& p, const float2* __restrict__ twtab, int t, int T,
-                           int lg) {
-  const float2* tw = twtab + p.tw_off;
-  int ns = 1;
-  for (int s = 0; s < p.nstages; ++s) {
-    const int R = p.radix[s];
-    switch (R) {
-      case 2: stage_col<2, INV>(a, b, p.n, ns, tw, t, T, lg); break;
-      case 3: stage_col<3, INV>(a, b, p.n, ns, tw, t, T, lg); break;
-      case 4: stage_col<4, INV>(a, b, p.n, ns, tw, t, T, lg); break;
-      case 5: stage_col<5, INV>(a, b, p.n, ns, tw, t, T, lg); break;
-      case 6: stage_col<6, INV>(a, b, p.n, ns, tw, t, T, lg); break;
-      case 8: stage_col<8, INV>(a, b, p.n, ns, tw, t, T, lg); break;
-      case 9: stage_col<9, INV>(a, b, p.n, ns, tw, t, T, lg); break;
-      case 10: stage_col<10, INV>(a, b, p.n, ns, tw, t, T, lg); break;
-      case 12: stage_col<12, INV>(a, b, p.n, ns, tw, t, T, lg); break;
-      case 15: stage_col<15, INV>(a, b, p.n, ns, tw, t, T, lg); break;
-      default: stage_col<16, INV>(a, b, p.n, ns, tw, t, T, lg); break;
-    }
-    __syncthreads();
-    float2* x = a;
-    a = b;
-    b = x;
-    ns *= R;
-  }
-  return a;
-}
+// float4 entries of a stage's twiddles
+__host__ __device__ constexpr int stage_tw_len(int R, int ns) { return ns > 1 ? (R / 2) * ns : 0; }
 
 }  // namespace prnu

@@ -64,7 +64,7 @@ __host__ __device__ constexpr int prime_power(int r) {
 template <int R, bool INV>
 struct DftP {
   static constexpr int F = prime_power(R);
-  static constexpr int P = F < R ? F : R % 4 == 0 && R > 8 ? 4 : R % 2 == 0 ? 2 : 3;
+  static constexpr int P = F < R ? F : R % 4 == 0 && R > 8 ? 4 : R % 2 == 0 ? 2 : R % 3 == 0 ? 3 : 5;
   static constexpr int Q = R / P;
   static constexpr int UQ = F < R ? Q * ce_inv_mod(Q % P, P) : 1;   // output step of k1 and of k2
   static constexpr int UP = F < R ? P * ce_inv_mod(P % Q, Q) : P;

@@ -37,7 +37,12 @@ void set_error(const std::string& msg);
 
 // ---------------------------------------------------------------- plans
 
+// the plan of length n, its twiddles from entry tw_base (tw_offsets[n]) of the table
+FftPlan make_plan_at(int n, int tw_base);
 FftPlan make_plan(int n, const std::vector<int>& tw_offsets);
+// the two-stage plan of length n (col_generic.cuh, row_generic.cuh), false if it has none
+bool col2_radices(int n, int* ra, int* rb);
+void allow_col2();
 bool is_5smooth(int n);
 // threads per row FFT and registers-per-thread class (1, 2 or 4 butterflies)
 void row_launch_shape(const FftPlan& p, int* threads, int* maxb);
@@ -92,6 +97,13 @@ void launch_row_forward(const PassArgs& a, bool warp, const float* mean_sub, flo
 // mode 4: inverse only, in place (float2)                               [naive path]
 void launch_col(const PassArgs& a, int mode, float2* out_f32, void* out_f16, const float* scale,
                 cudaStream_t s, LaunchCounter& lc);
+// widths with a two-stage plan (a.prow.ra; row_generic.cuh)
+void launch_row_forward2(const PassArgs& a, bool warp, const float* mean_sub, float2* out, cudaStream_t s,
+                         LaunchCounter& lc);
+void launch_row_inverse2(const PassArgs& a, float* c_out, cudaStream_t s, LaunchCounter& lc);
+void allow_row2();
+// mode 0 of a height with a two-stage plan (a.pcol.ra)
+void launch_col2(const PassArgs& a, cudaStream_t s, LaunchCounter& lc);
 void launch_row_inverse(const PassArgs& a, float* c_out, cudaStream_t s, LaunchCounter& lc);
 void launch_finalize(const PassArgs& a, cudaStream_t s, LaunchCounter& lc);
 // groups as SearchCall describes them (share = 1: contiguous)
@@ -227,8 +239,8 @@ struct prnu_ctx {
   std::recursive_mutex mu;
   std::map<uint64_t, std::shared_ptr<prnu::Fingerprint>> fps;
   uint64_t next_handle = 1;
-  float2* d_tw = nullptr;
-  std::vector<int> tw_off;   // offset per length, -1 if not 5-smooth
+  float4* d_tw = nullptr;
+  std::vector<int> tw_off;   // offset per length, -1 where no side has it
   prnu::LaunchCounter launches;
   cudaEvent_t last_done = nullptr;
   // call workspace

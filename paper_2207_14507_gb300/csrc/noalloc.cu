@@ -41,7 +41,7 @@ constexpr size_t kOffSpecX = 0;
 constexpr size_t kOffSpecK = kOffSpecX + kSpecBytes;
 constexpr size_t kOffStats = kOffSpecK + kSpecBytes;
 constexpr size_t kOffTw = kOffStats + (size_t)kMaxSide * sizeof(RowStat);
-constexpr size_t kOffItem = kOffTw + 2 * (size_t)kMaxSide * sizeof(float2);
+constexpr size_t kOffItem = kOffTw + 2 * (size_t)kMaxSide * sizeof(float4);   // a plan takes fewer entries than 4096
 constexpr size_t kOffFp = kOffItem + 256;
 constexpr size_t kOffResult = kOffFp + 256;
 constexpr size_t kOffScal = kOffResult + 256;
@@ -54,12 +54,22 @@ constexpr int kMaxDevices = 64;
 std::mutex g_mu;
 unsigned char* g_addr[kMaxDevices] = {};
 
-// w_n^k = exp(-2 pi i k / n), evaluated in double and rounded to float
-__global__ void k_noalloc_twiddles(float2* __restrict__ tw, int n) {
-  for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
-    double s, c;
-    sincospi(2.0 * (double)k / (double)n, &s, &c);
-    tw[k] = make_float2((float)c, (float)(-s));
+// the stage twiddles of plan p (fft_plan.cuh), evaluated in double and rounded to float
+__global__ void k_noalloc_twiddles(FftPlan p, float4* __restrict__ tw) {
+  const int id = blockIdx.x * blockDim.x + threadIdx.x, T = gridDim.x * blockDim.x;
+  auto stage = [&](int R, int ns, int off) {
+    for (int i = id; i < stage_tw_len(R, ns); i += T) {
+      const int m = i / ns, k = i - m * ns;
+      double s1, c1, s2 = 0.0, c2 = 0.0;
+      sincospi(2.0 * (double)((2 * m + 1) * k) / (double)(ns * R), &s1, &c1);
+      if (2 * m + 2 < R) sincospi(2.0 * (double)((2 * m + 2) * k) / (double)(ns * R), &s2, &c2);
+      tw[off + i] = make_float4((float)c1, (float)(-s1), (float)c2, (float)(-s2));
+    }
+  };
+  for (int s = 0; s < p.nstages; ++s) stage(p.radix[s], p.ns[s], p.tw[s]);
+  if (p.ra) {
+    stage(p.rb, p.ra, p.tw_fwd);
+    stage(p.ra, p.rb, p.tw_inv);
   }
 }
 
@@ -121,7 +131,7 @@ extern "C" int pce_score_noalloc(const float* d_X, const float* d_K, int H, int 
     float2* specX = reinterpret_cast<float2*>(base + kOffSpecX);
     float2* specK = reinterpret_cast<float2*>(base + kOffSpecK);
     RowStat* stats = reinterpret_cast<RowStat*>(base + kOffStats);
-    float2* tw = reinterpret_cast<float2*>(base + kOffTw);
+    float4* tw = reinterpret_cast<float4*>(base + kOffTw);
     WorkItem* ditem = reinterpret_cast<WorkItem*>(base + kOffItem);
     FpDesc* dfp = reinterpret_cast<FpDesc*>(base + kOffFp);
     CandResult* dres = reinterpret_cast<CandResult*>(base + kOffResult);
@@ -130,14 +140,10 @@ extern "C" int pce_score_noalloc(const float* d_X, const float* d_K, int H, int 
 
     // twiddle tables: length W at tw[0], length H at tw[kMaxSide] (the
     // offsets are set here, not looked up, so H == W needs no special case)
-    const std::vector<int> zero_off(kMaxFft + 1, 0);
-    FftPlan prow = make_plan(W, zero_off);
-    FftPlan pcol = make_plan(H, zero_off);
-    prow.tw_off = 0;
-    pcol.tw_off = kMaxSide;
-    k_noalloc_twiddles<<<8, 256, 0, s>>>(tw, W);
+    const FftPlan prow = make_plan_at(W, 0), pcol = make_plan_at(H, kMaxSide);
+    k_noalloc_twiddles<<<8, 256, 0, s>>>(prow, tw);
     PRNU_CUDA_TRY(cudaGetLastError());
-    k_noalloc_twiddles<<<8, 256, 0, s>>>(tw + kMaxSide, H);
+    k_noalloc_twiddles<<<8, 256, 0, s>>>(pcol, tw);
     PRNU_CUDA_TRY(cudaGetLastError());
 
     WorkItem it{};

@@ -30,8 +30,10 @@ namespace prnu {
 // Warp (optional) + row FFT of two rows per thread group; writes the packed
 // half spectrum of both rows.  grid = (ceil((H/2)/ppb), wave), block = ppb*T.
 // Without WARP the input is the single image at a.resid (minus *mean_sub).
+// 64 registers (two blocks of 512): unbounded the kernel takes 68 and loses a
+// third at 1440 x 2560 (21.0 against 14.5 us a candidate)
 template <int DT, bool WARP>
-__global__ void __launch_bounds__(512) k_row_forward(PassArgs a, const float* __restrict__ mean_sub,
+__global__ void __launch_bounds__(512, 2) k_row_forward(PassArgs a, const float* __restrict__ mean_sub,
                                                       float2* __restrict__ out_override) {
   extern __shared__ float2 smem[];
   const int T = a.row_threads;
@@ -93,7 +95,7 @@ __global__ void __launch_bounds__(512) k_row_forward(PassArgs a, const float* __
 // spectrum.  grid = (ceil((W/2) >> lg), wave), block = T.
 // mode 0: fwd FFT, x conj(.) * K0^, inv FFT;  1: fwd FFT to out (fingerprint);
 // 2: product only;  3: fwd FFT only;  4: inv FFT only (modes 2-4 in place).
-__global__ void __launch_bounds__(512) k_col(PassArgs a, int mode, float2* __restrict__ out_f32,
+__global__ void __launch_bounds__(512, 2) k_col(PassArgs a, int mode, float2* __restrict__ out_f32,
                                               __half2* __restrict__ out_f16, const float* __restrict__ out_scale) {
   extern __shared__ float2 smem[];
   const int T = blockDim.x, tid = threadIdx.x;
@@ -163,7 +165,7 @@ __global__ void __launch_bounds__(512) k_col(PassArgs a, int mode, float2* __res
 
 // Inverse row FFT of two rows per group; per-row max / first arg-max / sum of
 // squares into a.stats, or (c_out != nullptr) the rows of C themselves.
-__global__ void __launch_bounds__(512) k_row_inverse(PassArgs a, float* __restrict__ c_out) {
+__global__ void __launch_bounds__(512, 2) k_row_inverse(PassArgs a, float* __restrict__ c_out) {
   extern __shared__ float2 smem[];
   const int T = a.row_threads;
   const int grp = threadIdx.x / T, t = threadIdx.x - grp * T;
@@ -178,8 +180,9 @@ __global__ void __launch_bounds__(512) k_row_inverse(PassArgs a, float* __restri
   const float2* Z = a.spec + (size_t)slot * H * Wh;
   if (active) build_full_row(buf, Z + (size_t)(2 * pair) * Wh, Z + (size_t)(2 * pair + 1) * Wh, W, t, T);
   __syncthreads();
-  buf = fft_row<true>(buf, buf2, a.prow, a.tw, active ? t : (1 << 28), T);
+  const int tl = active ? t : (1 << 28);
   if (c_out) {
+    buf = fft_row<true>(buf, buf2, a.prow, a.tw, tl, T);
     if (active) {
       float* ra = c_out + (size_t)(2 * pair) * W;
       for (int x = t; x < W; x += T) {
@@ -190,18 +193,20 @@ __global__ void __launch_bounds__(512) k_row_inverse(PassArgs a, float* __restri
     }
     return;
   }
+  // the last stage's outputs go to the statistics from registers
   float ma = -INFINITY, mb = -INFINITY;
   int ia = INT_MAX, ib = INT_MAX;
-  float sa = 0.f, sb = 0.f;
-  if (active) {
-    for (int x = t; x < W; x += T) {
-      const float2 v = buf[rpad(x)];
-      if (v.x > ma) { ma = v.x; ia = x; }
-      if (v.y > mb) { mb = v.y; ib = x; }
-      sa = fmaf(v.x, v.x, sa);
-      sb = fmaf(v.y, v.y, sb);
-    }
-  }
+  float2 sq = make_float2(0.f, 0.f);
+  const int last = a.prow.nstages - 1;
+  buf = fft_row<true>(buf, buf2, a.prow, a.tw, tl, T, last);
+  plan_stage_any<true>(
+      a.prow, last, a.tw, tl, T, [=](int i) { return buf[rpad(i)]; },
+      [&](int x, float2 v) {
+        better_f(ma, ia, v.x, x);
+        better_f(mb, ib, v.y, x);
+        sq = __ffma2_rn(v, v, sq);
+      });
+  const float sa = sq.x, sb = sq.y;
   row_stats_warp(ma, ia, mb, ib, sa, sb, t, reinterpret_cast<RowRed*>(red));
   __syncthreads();
   if (active && t == 0) row_stats_final(reinterpret_cast<const RowRed*>(red), T >> 5, a.stats + (size_t)slot * H + 2 * pair);
@@ -359,6 +364,10 @@ __global__ void k_naive_final(const float* __restrict__ C, int H, int W, const W
 
 void launch_row_forward(const PassArgs& a, bool warp, const float* mean_sub, float2* out, cudaStream_t s,
                         LaunchCounter& lc) {
+  if (a.prow.ra) {
+    launch_row_forward2(a, warp, mean_sub, out, s, lc);
+    return;
+  }
   int T, maxb;
   row_launch_shape(a.prow, &T, &maxb);
   PRNU_CHECK_ARG(T == a.row_threads, "row thread count mismatch");
@@ -381,6 +390,10 @@ void launch_row_forward(const PassArgs& a, bool warp, const float* mean_sub, flo
 
 void launch_col(const PassArgs& a, int mode, float2* out_f32, void* out_f16, const float* scale, cudaStream_t s,
                 LaunchCounter& lc) {
+  if (mode == 0 && a.pcol.ra) {
+    launch_col2(a, s, lc);
+    return;
+  }
   int T, maxb;
   col_launch_shape(a.pcol, a.col_log2, &T, &maxb);
   const int Wh = a.W / 2;
@@ -395,6 +408,10 @@ void launch_col(const PassArgs& a, int mode, float2* out_f32, void* out_f16, con
 }
 
 void launch_row_inverse(const PassArgs& a, float* c_out, cudaStream_t s, LaunchCounter& lc) {
+  if (a.prow.ra) {
+    launch_row_inverse2(a, c_out, s, lc);
+    return;
+  }
   int T, maxb;
   row_launch_shape(a.prow, &T, &maxb);
   const int ppb = a.pairs_per_block;
@@ -506,6 +523,8 @@ void set_kernel_attributes() {
   allow_smem(k_col);
   allow_smem(k_row_inverse);
   allow_smem(k_finalize);
+  allow_col2();
+  allow_row2();
   cudaGetLastError();
 }
 

@@ -6,6 +6,7 @@
 #include <math.h>
 
 #include "common.cuh"
+#include "fft_plan.cuh"
 #include "prnu.h"
 
 namespace prnu {
@@ -175,13 +176,21 @@ __device__ __forceinline__ float bilinear(const void* R, size_t base, int H, int
   const float fx0 = floorf(qx), fy0 = floorf(qy);
   const float fx = qx - fx0, fy = qy - fy0;
   const int x0 = (int)fx0, y0 = (int)fy0;
-  const bool xi0 = (unsigned)x0 < (unsigned)W, xi1 = (unsigned)(x0 + 1) < (unsigned)W;
-  const bool yi0 = (unsigned)y0 < (unsigned)H, yi1 = (unsigned)(y0 + 1) < (unsigned)H;
   const size_t r0 = base + (size_t)((long long)y0 * pitch + x0);
-  const float v00 = (yi0 && xi0) ? load_store_type<DT>(R, r0) : 0.f;
-  const float v01 = (yi0 && xi1) ? load_store_type<DT>(R, r0 + 1) : 0.f;
-  const float v10 = (yi1 && xi0) ? load_store_type<DT>(R, r0 + pitch) : 0.f;
-  const float v11 = (yi1 && xi1) ? load_store_type<DT>(R, r0 + pitch + 1) : 0.f;
+  float v00, v01, v10, v11;
+  if ((unsigned)x0 < (unsigned)(W - 1) && (unsigned)y0 < (unsigned)(H - 1)) {   // every tap inside, as for most warps
+    v00 = load_store_type<DT>(R, r0);
+    v01 = load_store_type<DT>(R, r0 + 1);
+    v10 = load_store_type<DT>(R, r0 + pitch);
+    v11 = load_store_type<DT>(R, r0 + pitch + 1);
+  } else {
+    const bool xi0 = (unsigned)x0 < (unsigned)W, xi1 = (unsigned)(x0 + 1) < (unsigned)W;
+    const bool yi0 = (unsigned)y0 < (unsigned)H, yi1 = (unsigned)(y0 + 1) < (unsigned)H;
+    v00 = (yi0 && xi0) ? load_store_type<DT>(R, r0) : 0.f;
+    v01 = (yi0 && xi1) ? load_store_type<DT>(R, r0 + 1) : 0.f;
+    v10 = (yi1 && xi0) ? load_store_type<DT>(R, r0 + pitch) : 0.f;
+    v11 = (yi1 && xi1) ? load_store_type<DT>(R, r0 + pitch + 1) : 0.f;
+  }
   const float gx = 1.f - fx, gy = 1.f - fy;
   return gy * (gx * v00 + fx * v01) + fy * (gx * v10 + fx * v11);
 }
