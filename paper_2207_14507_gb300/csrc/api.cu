@@ -277,7 +277,13 @@ void build_items(const prnu_grid& g, const prnu_window* windows, int F, int P, S
   call.cmax = g.nlam * g.nth;
   std::vector<float> lam(g.nlam), th(g.nth);
   for (int i = 0; i < g.nlam; ++i) lam[i] = (float)((double)g.lam0 + (double)i * (double)g.dlam);
-  for (int j = 0; j < g.nth; ++j) th[j] = (float)((double)g.th0_deg + (double)j * (double)g.dth_deg);
+  std::vector<double> vc(g.nth), vs(g.nth);
+  for (int j = 0; j < g.nth; ++j) {
+    th[j] = (float)((double)g.th0_deg + (double)j * (double)g.dth_deg);
+    const double t = (double)th[j] * 3.14159265358979323846 / 180.0;
+    vc[j] = cos(t);
+    vs[j] = sin(t);
+  }
   for (int f = 0; f < F; ++f) {
     int il = 0, ih = g.nlam - 1, jl = 0, jh = g.nth - 1;
     if (windows) {
@@ -290,8 +296,7 @@ void build_items(const prnu_grid& g, const prnu_window* windows, int F, int P, S
     auto node = [&](int p, int i, int j) {
       const double L = (double)lam[i];
       PRNU_CHECK_ARG(L > 0 && std::isfinite(L), "grid scales must be positive");
-      const double t = (double)th[j] * 3.14159265358979323846 / 180.0;
-      const double cs = cos(t), sn = sin(t);
+      const double cs = vc[j], sn = vs[j];
       WorkItem it;
       it.frame = f;
       it.fp = p;
@@ -623,6 +628,12 @@ static void add_pair_items(SearchCall& call, int f, int p, int group, const std:
 // ---------------------------------------------------------------- the correction as a device-side loop
 
 namespace {
+
+// the work list and fingerprint table of one candidate
+__global__ void k_set_pair(WorkItem it, FpDesc fd, WorkItem* __restrict__ dit, FpDesc* __restrict__ dfd) {
+  *dit = it;
+  *dfd = fd;
+}
 
 constexpr int kCorrHalfLam = 5;   // lambda nodes either side of the estimate (11 in all)
 
@@ -1067,6 +1078,7 @@ int prnu_create(prnu_ctx** out, int device, size_t hbm_budget_bytes) {
     PRNU_CUDA_TRY(cudaEventRecord(c->stage_free, 0));
     PRNU_CUDA_TRY(cudaHostAlloc((void**)&c->h_err, sizeof(int), cudaHostAllocDefault));
     *c->h_err = 0;
+    PRNU_CUDA_TRY(cudaHostAlloc((void**)&c->h_res, sizeof(CandResult), cudaHostAllocDefault));
     c->d_err = reinterpret_cast<int*>(ctx_alloc(c.get(), sizeof(int)));
     PRNU_CUDA_TRY(cudaMemset(c->d_err, 0, sizeof(int)));
     set_kernel_attributes();
@@ -1099,6 +1111,7 @@ int prnu_destroy(prnu_ctx* ctx) {
     ctx_free(ctx, ctx->d_err, sizeof(int));
     if (ctx->h_pinned) cudaFreeHost(ctx->h_pinned);
     if (ctx->h_err) cudaFreeHost(ctx->h_err);
+    if (ctx->h_res) cudaFreeHost(ctx->h_res);
     if (ctx->aux) cudaStreamDestroy(ctx->aux);
     if (ctx->ev_fork) cudaEventDestroy(ctx->ev_fork);
     if (ctx->ev_join) cudaEventDestroy(ctx->ev_join);
@@ -1464,6 +1477,8 @@ int pce_score(prnu_ctx* ctx, const float* d_X, uint64_t fp_handle, int H, int W,
     auto f = find_fp(ctx, fp_handle);
     PRNU_CHECK_ARG(f->H == H && f->W == W, "fingerprint size differs");
     const int Wh = W / 2;
+    if (*ctx->h_err)
+      report_device_abort(ctx, s, "a bounded device-side wait of an earlier call timed out; its results are invalid");
     PRNU_CUDA_TRY(cudaStreamWaitEvent(s, ctx->last_done, 0));
     PRNU_CUDA_TRY(cudaStreamWaitEvent(s, f->ready, 0));
     ensure_buf(ctx, ctx->ws_items, sizeof(WorkItem));
@@ -1474,11 +1489,10 @@ int pce_score(prnu_ctx* ctx, const float* d_X, uint64_t fp_handle, int H, int W,
     WorkItem it{};
     it.a11 = it.a22 = 1.f;
     it.lam = 1.f;
-    FpDesc fd{f->d_spec, f->dtype, f->d_scal + 2};
-    Stager st(ctx);
-    st.add(ctx->ws_items.p, &it, 1);
-    st.add(ctx->ws_fpdesc.p, &fd, 1);
-    st.flush(s);
+    const FpDesc fd = fp_desc(*f);
+    k_set_pair<<<1, 1, 0, s>>>(it, fd, reinterpret_cast<WorkItem*>(ctx->ws_items.p),
+                               reinterpret_cast<FpDesc*>(ctx->ws_fpdesc.p));
+    PRNU_CUDA_TRY(cudaGetLastError());
     const FftPlan prow = make_plan(W, ctx->tw_off), pcol = make_plan(H, ctx->tw_off);
     int rowT, rowMB;
     row_launch_shape(prow, &rowT, &rowMB);
@@ -1486,11 +1500,13 @@ int pce_score(prnu_ctx* ctx, const float* d_X, uint64_t fp_handle, int H, int W,
     PassArgs a{};
     a.resid = d_X;
     a.rdtype = kF32;
+    a.rpitch = W;
+    a.fpitch = (size_t)H * W;
     a.H = H;
     a.W = W;
     a.items = reinterpret_cast<const WorkItem*>(ctx->ws_items.p);
     a.item0 = 0;
-    a.nitems = 1;
+    a.nitems = a.nunits = a.share = 1;
     a.spec = reinterpret_cast<float2*>(ctx->ws_spec.p);
     a.stats = reinterpret_cast<RowStat*>(ctx->ws_stats.p);
     a.results = reinterpret_cast<CandResult*>(ctx->ws_results.p);
@@ -1501,14 +1517,26 @@ int pce_score(prnu_ctx* ctx, const float* d_X, uint64_t fp_handle, int H, int W,
     a.pairs_per_block = tn.ppb;
     a.col_log2 = tn.col_log2;
     a.row_threads = rowT;
-    launch_row_forward(a, false, nullptr, nullptr, s, ctx->launches);
-    launch_col(a, 0, nullptr, nullptr, nullptr, s, ctx->launches);
-    launch_row_inverse(a, nullptr, s, ctx->launches);
-    launch_finalize(a, s, ctx->launches);
-    CandResult r{};
-    PRNU_CUDA_TRY(cudaMemcpyAsync(&r, a.results, sizeof(CandResult), cudaMemcpyDeviceToHost, s));
+    a.err = ctx->d_err;
+    a.stall = ctx->debug_stall;
+    a.fp_f32 = fd.dtype == kF32;
+    const FixedShape* fs = tn.variant >= 0 ? find_fixed(H, W) : nullptr;
+    if (fs && fixed_supports(*fs, H, tn.ppb)) {
+      a.rdtype = kF32I;
+      launch_fixed_wave(a, *fs, tn.variant, s, ctx->launches);
+      PRNU_CUDA_TRY(cudaMemcpyAsync(ctx->h_err, ctx->d_err, sizeof(int), cudaMemcpyDeviceToHost, s));
+    } else {
+      launch_row_forward(a, false, nullptr, nullptr, s, ctx->launches);
+      launch_col(a, 0, nullptr, nullptr, nullptr, s, ctx->launches);
+      launch_row_inverse(a, nullptr, s, ctx->launches);
+      launch_finalize(a, s, ctx->launches);
+    }
+    ctx->launches.n++;
+    PRNU_CUDA_TRY(cudaMemcpyAsync(ctx->h_res, a.results, sizeof(CandResult), cudaMemcpyDeviceToHost, s));
     PRNU_CUDA_TRY(cudaEventRecord(ctx->last_done, s));
     PRNU_CUDA_TRY(cudaStreamSynchronize(s));
+    if (*ctx->h_err) report_device_abort(ctx, s, "a bounded device-side wait timed out; the results are invalid");
+    const CandResult r = *ctx->h_res;
     if (pce) *pce = r.pce;
     if (dy) *dy = r.py < H / 2 ? r.py : r.py - H;
     if (dx) *dx = r.px < W / 2 ? r.px : r.px - W;

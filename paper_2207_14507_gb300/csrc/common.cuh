@@ -14,8 +14,8 @@ enum StoreType { kF32 = 0, kF16 = 1, kBF16 = 2 };
 // half storage: element x holds the pair (R[x], R[x + 1]) as one 4-byte
 // word, so a bilinear sample takes one aligned load per row.
 enum PairStoreType { kF16P = 3, kBF16P = 4 };
-// FP32 residuals in the zero-bordered layout whose items all warp by the
-// identity: the planned row kernels read each pixel itself.
+// FP32 residuals, in any layout, whose items all warp by the identity: the
+// planned row kernels read each pixel itself.
 enum { kF32I = 5 };
 constexpr int kNumStoreLayouts = 6;
 
@@ -142,6 +142,23 @@ __device__ __forceinline__ float refined_quotient(float n, float d) {
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(rc) : "f"(d));
   const float q = n * rc;
   return fmaf(fmaf(-q, d, n), rc, q);
+}
+
+// s + c += b (Knuth's two-sum), two sums at once
+__device__ __forceinline__ void csum_add2(float2& s, float2& c, float2 b) {
+  const float2 t = __fadd2_rn(s, b);
+  const float2 bp = __fadd2_rn(t, make_float2(-s.x, -s.y));
+  const float2 sp = __fadd2_rn(t, make_float2(-bp.x, -bp.y));
+  const float2 e = __fadd2_rn(__fadd2_rn(s, make_float2(-sp.x, -sp.y)), __fadd2_rn(b, make_float2(-bp.x, -bp.y)));
+  s = t;
+  c = __fadd2_rn(c, e);
+}
+
+// s + c += v * v, the square exact (its rounding error goes to c)
+__device__ __forceinline__ void csum_square2(float2& s, float2& c, float2 v) {
+  const float2 p = __fmul2_rn(v, v);
+  c = __fadd2_rn(c, __ffma2_rn(v, v, make_float2(-p.x, -p.y)));
+  csum_add2(s, c, p);
 }
 
 // ---------------------------------------------------------------- storage loads / stores

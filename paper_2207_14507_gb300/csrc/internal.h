@@ -106,6 +106,8 @@ void allow_row2();
 void launch_col2(const PassArgs& a, cudaStream_t s, LaunchCounter& lc);
 void launch_row_inverse(const PassArgs& a, float* c_out, cudaStream_t s, LaunchCounter& lc);
 void launch_finalize(const PassArgs& a, cudaStream_t s, LaunchCounter& lc);
+// the second half of the finalisation of a wave whose candidates' parts several blocks computed
+void launch_finalize_sum(const PassArgs& a, cudaStream_t s, LaunchCounter& lc);
 // groups as SearchCall describes them (share = 1: contiguous)
 void launch_argmax(const CandResult* res, const WorkItem* items, const int* group_start, int ngroups, int share,
                    prnu_result* out, const float* scale, int H, int W, cudaStream_t s, LaunchCounter& lc);
@@ -247,6 +249,7 @@ struct prnu_ctx {
   prnu::DeviceBuf ws_spec, ws_stats, ws_items, ws_results, ws_groups, ws_out, ws_fpdesc, ws_misc, ws_resid,
       ws_persist, ws_pad, ws_lit, ws_litx, ws_litpart, ws_renders, ws_resize, ws_wav, ws_corr;
   size_t tw_bytes = 0;
+  prnu::CandResult* h_res = nullptr;   // pinned: pce_score's result
   int* h_err = nullptr;           // pinned: error flag of the last persistent launch or TMA wait
   int* d_err = nullptr;           // device flag the wave kernels raise when a bounded wait gives up
   int debug_stall = 0;            // prnu_debug_set(PRNU_DEBUG_STALL_DEVICE_WAITS)

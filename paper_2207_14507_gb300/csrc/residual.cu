@@ -368,16 +368,6 @@ void launch_moments(const uint8_t* frames, int F, int H, int W, size_t pitch, in
   lc.n += 2;
 }
 
-// s + c += b (Knuth's two-sum), two sums at once
-__device__ __forceinline__ void csum_add2(float2& s, float2& c, float2 b) {
-  const float2 t = __fadd2_rn(s, b);
-  const float2 bp = __fadd2_rn(t, make_float2(-s.x, -s.y));
-  const float2 sp = __fadd2_rn(t, make_float2(-bp.x, -bp.y));
-  const float2 e = __fadd2_rn(__fadd2_rn(s, make_float2(-sp.x, -sp.y)), __fadd2_rn(b, make_float2(-bp.x, -bp.y)));
-  s = t;
-  c = __fadd2_rn(c, e);
-}
-
 // K = sum_l I W(I) / sum_l I^2 (Eq. 2) of a thread's pixels over all L frames.
 // The numerator is a compensated FP32 sum (48 bits; the FP64 pipe takes 1/64 of
 // the FP32 rate), the denominator an integer: exact in FP32 over up to 256

@@ -212,22 +212,96 @@ __global__ void __launch_bounds__(512, 2) k_row_inverse(PassArgs a, float* __res
   if (active && t == 0) row_stats_final(reinterpret_cast<const RowRed*>(red), T >> 5, a.stats + (size_t)slot * H + 2 * pair);
 }
 
-// One block per candidate of the wave: see finalize_body.
+// Finalisation (search_common.cuh): window pairs b0 .. b1-1 and the row shares of
+// the same numbers of candidate slot `s`, to parts (after the caller's barrier,
+// by thread 0).
+constexpr int kFinMaxWarps = 16;
+__device__ void finalize_parts(const PassArgs& a, int s, const FinPeak& pk, int b0, int b1, float2* smem, double* parts) {
+  __shared__ double red[kFinParts][kFinMaxWarps];
+  const int T = blockDim.x, t = threadIdx.x;
+  const int H = a.H, W = a.W, Wh = W >> 1;
+  const RowStat* st = a.stats + (size_t)s * H;
+  const float2* Z = a.spec + (size_t)s * H * Wh;
+  float2* const bufA = smem;
+  float2* const bufB = smem + row_smem_len(W);
+  for (int b = b0; b < b1; ++b) {
+    if (b < kFinRowParts) part_warp(row_share(st, H, pk.py, b, t, T), t, red[b]);
+    const int p = window_pair(pk.py, b, H);
+    build_full_row(bufA, Z + (size_t)(2 * p) * Wh, Z + (size_t)(2 * p + 1) * Wh, W, t, T);
+    __syncthreads();
+    const float2* buf = fft_row<true>(bufA, bufB, a.prow, a.tw, t, T);
+    PairEnergy e;
+    for (int x = t; x < W; x += T)
+      if (cdist(x, pk.px, W) > kHalfWindow) e.add(buf[rpad(x)]);
+    part_warp(e.total(cdist(2 * p, pk.py, H) <= kHalfWindow, cdist(2 * p + 1, pk.py, H) <= kHalfWindow), t,
+              red[kFinRowParts + b]);
+    __syncthreads();   // the row buffers are free again
+  }
+  if (t == 0)
+    for (int b = b0; b < b1; ++b) {
+      if (b < kFinRowParts) parts[b] = part_total(red[b], T >> 5);
+      parts[kFinRowParts + b] = part_total(red[kFinRowParts + b], T >> 5);
+    }
+}
+
+// One block per candidate of the wave.
 __global__ void __launch_bounds__(512) k_finalize(PassArgs a) {
   extern __shared__ float2 smem[];
-  finalize_body(a, blockIdx.x, blockIdx.x, smem);
+  const FinPeak pk = block_peak(a.stats + (size_t)blockIdx.x * a.H, a.H, a.W, threadIdx.x, blockDim.x,
+                                reinterpret_cast<WarpRed*>(smem + 2 * row_smem_len(a.W)));
+  double parts[kFinParts];
+  finalize_parts(a, blockIdx.x, pk, 0, kFinPairParts, smem, parts);
+  if (threadIdx.x == 0) finish_candidate(a, blockIdx.x, pk, parts);
+}
+
+// One block per window pair (blockIdx.y) of a candidate; k_finalize_sum ends it.
+__global__ void __launch_bounds__(512) k_finalize_part(PassArgs a) {
+  extern __shared__ float2 smem[];
+  const int s = blockIdx.x, b = blockIdx.y;
+  const FinPeak pk = block_peak(a.stats + (size_t)s * a.H, a.H, a.W, threadIdx.x, blockDim.x,
+                                reinterpret_cast<WarpRed*>(smem + 2 * row_smem_len(a.W)));
+  finalize_parts(a, s, pk, b, b + 1, smem, fin_scratch(a, s, pk.py));
+  if (b == 0 && threadIdx.x == 0) park_peak(a, s, pk);
+}
+
+// The results of candidates whose parts several blocks computed, a thread each.
+__global__ void k_finalize_sum(PassArgs a) {
+  const int s = blockIdx.x * blockDim.x + threadIdx.x;
+  if (s >= a.nitems || past_count(a, s, 0)) return;
+  const CandResult* r = result_of(a, s);
+  const FinPeak pk{r->peak, r->py, r->px};
+  double parts[kFinParts];
+  const double* p = fin_scratch(a, s, pk.py);
+#pragma unroll
+  for (int k = 0; k < kFinParts; ++k) parts[k] = p[k];
+  finish_candidate(a, s, pk, parts);
 }
 
 // Best candidate of each (frame, fingerprint) group g: its items are
 // first + k*share (k < count) with first = gstart[g / share] + g % share and
 // count = (gstart[g / share + 1] - gstart[g / share]) / share, in ascending
-// candidate order (share = 1: contiguous groups).  One warp per group.
-__global__ void k_argmax(const CandResult* __restrict__ res, const WorkItem* __restrict__ items,
-                         const int* __restrict__ gstart, int ngroups, int share, prnu_result* __restrict__ out,
-                         int H, int W) {
-  const int g = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  if (g >= ngroups) return;
-  argmax_group(res, items, gstart, share, out, H, W, g, threadIdx.x & 31);
+// candidate order (share = 1: contiguous groups).  One block per group (a warp's
+// chain of loads over 1681 candidates took 24 us).
+__global__ void __launch_bounds__(256) k_argmax(const CandResult* __restrict__ res, const WorkItem* __restrict__ items,
+                                                const int* __restrict__ gstart, int ngroups, int share,
+                                                prnu_result* __restrict__ out, int H, int W) {
+  __shared__ double s_v[8];
+  __shared__ int s_i[8];
+  const int g = blockIdx.x, f = g / share, t = threadIdx.x;
+  const int b = gstart[f] + (g - f * share), n = (gstart[f + 1] - gstart[f]) / share;
+  double bv = -INFINITY;
+  int bi = INT_MAX;
+  for (int k = t; k < n; k += 256) better_d(bv, bi, res[b + k * share].pce, b + k * share);
+  warp_maxarg_d(bv, bi);
+  if ((t & 31) == 0) {
+    s_v[t >> 5] = bv;
+    s_i[t >> 5] = bi;
+  }
+  __syncthreads();
+  if (t == 0) {
+    for (int w = 1; w < 8; ++w) better_d(bv, bi, s_v[w], s_i[w]);
+    out[g] = group_result(res, items, n, bi, H, W);
+  }
 }
 
 __global__ void k_scatter_all(const CandResult* __restrict__ res, int n, int cmax, double* __restrict__ all) {
@@ -423,24 +497,36 @@ void launch_row_inverse(const PassArgs& a, float* c_out, cudaStream_t s, LaunchC
   lc.n++;
 }
 
+void launch_finalize_sum(const PassArgs& a, cudaStream_t s, LaunchCounter& lc) {
+  k_finalize_sum<<<(a.nitems + 63) / 64, 64, 0, s>>>(a);
+  PRNU_LAUNCH_CHECK();
+  lc.n++;
+}
+
 void launch_finalize(const PassArgs& a, cudaStream_t s, LaunchCounter& lc) {
   int T, maxb;
   row_launch_shape(a.prow, &T, &maxb);
-  dim3 g(a.nitems), b(T);
   const size_t sm = row_smem_bytes(a.W, 1);
   ProfScope ps(lc, kKindFinalize, s);
-  k_finalize<<<g, b, sm, s>>>(a);
-  PRNU_LAUNCH_CHECK();
+  // Up to a candidate per SM the block's chain of six row FFTs is the latency: a
+  // block per window pair.  Past that the GPU is full and the peak is searched
+  // once (480 x 640, 1764 candidates: 100 against 132 us).
+  if (a.nitems <= 152) {
+    k_finalize_part<<<dim3(a.nitems, kFinPairParts), T, sm, s>>>(a);
+    PRNU_LAUNCH_CHECK();
+    launch_finalize_sum(a, s, lc);
+  } else {
+    k_finalize<<<a.nitems, T, sm, s>>>(a);
+    PRNU_LAUNCH_CHECK();
+  }
   lc.n++;
 }
 
 void launch_argmax(const CandResult* res, const WorkItem* items, const int* group_start, int ngroups, int share,
                    prnu_result* out, const float* /*scale*/, int H, int W, cudaStream_t s, LaunchCounter& lc) {
   if (ngroups <= 0) return;
-  const int warps = 8;
   ProfScope ps(lc, kKindArgmax, s);
-  k_argmax<<<(ngroups + warps - 1) / warps, warps * 32, 0, s>>>(res, items, group_start, ngroups,
-                                                                std::max(share, 1), out, H, W);
+  k_argmax<<<ngroups, 256, 0, s>>>(res, items, group_start, ngroups, std::max(share, 1), out, H, W);
   PRNU_LAUNCH_CHECK();
   lc.n++;
 }
@@ -523,6 +609,7 @@ void set_kernel_attributes() {
   allow_smem(k_col);
   allow_smem(k_row_inverse);
   allow_smem(k_finalize);
+  allow_smem(k_finalize_part);
   allow_col2();
   allow_row2();
   cudaGetLastError();

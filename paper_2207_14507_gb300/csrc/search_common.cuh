@@ -51,6 +51,28 @@ __device__ __forceinline__ void warp_maxarg_d(double& v, int& i) {
   }
 }
 
+// The result of a group whose best candidate is bi (n candidates in all)
+__device__ __forceinline__ prnu_result group_result(const CandResult* __restrict__ res, const WorkItem* __restrict__ items,
+                                                    int n, int bi, int H, int W) {
+  prnu_result r;
+  if (bi == INT_MAX || n == 0) {
+    r.lam = 0.f; r.th_deg = 0.f; r.dy = 0; r.dx = 0; r.pce = 0.0; r.peak = 0.f; r.cand_idx = -1;
+  } else {
+    const CandResult c = res[bi];
+    const WorkItem it = items[bi];
+    r.lam = it.lam;
+    r.th_deg = it.th_deg;
+    r.dy = c.py < (H + 1) / 2 ? c.py : c.py - H;
+    r.dx = c.px < (W + 1) / 2 ? c.px : c.px - W;
+    if (2 * c.py == H) r.dy = -H / 2;
+    if (2 * c.px == W) r.dx = -W / 2;
+    r.pce = c.pce;
+    r.peak = c.peak;
+    r.cand_idx = c.cand;
+  }
+  return r;
+}
+
 // The best candidate of group g (one frame and fingerprint), by one warp
 // (lane = its lane): the highest PCE, the lowest index among equal ones
 // (candidates gstart[f] + (g - f*share) + k*share of frame f = g / share),
@@ -67,25 +89,7 @@ __device__ __forceinline__ void argmax_group(const CandResult* __restrict__ res,
     better_d(bv, bi, res[i].pce, i);
   }
   warp_maxarg_d(bv, bi);
-  if (lane == 0) {
-    prnu_result r;
-    if (bi == INT_MAX || n == 0) {
-      r.lam = 0.f; r.th_deg = 0.f; r.dy = 0; r.dx = 0; r.pce = 0.0; r.peak = 0.f; r.cand_idx = -1;
-    } else {
-      const CandResult c = res[bi];
-      const WorkItem it = items[bi];
-      r.lam = it.lam;
-      r.th_deg = it.th_deg;
-      r.dy = c.py < (H + 1) / 2 ? c.py : c.py - H;
-      r.dx = c.px < (W + 1) / 2 ? c.px : c.px - W;
-      if (2 * c.py == H) r.dy = -H / 2;
-      if (2 * c.px == W) r.dx = -W / 2;
-      r.pce = c.pce;
-      r.peak = c.peak;
-      r.cand_idx = c.cand;
-    }
-    out[g] = r;
-  }
+  if (lane == 0) out[g] = group_result(res, items, n, bi, H, W);
 }
 __device__ __forceinline__ double warp_sum(double s) {
 #pragma unroll
@@ -307,88 +311,122 @@ __host__ __device__ inline size_t row_smem_bytes(int W, int ppb) {
   return (size_t)ppb * 2 * row_smem_len(W) * sizeof(float2) + (size_t)ppb * 32 * sizeof(WarpRed);
 }
 
-// Peak, energy outside the cyclic 11x11 window and PCE (Eq. 3) of candidate
-// `is` whose row statistics and spectrum sit in workspace slot `ws`; all
-// threads of the block take part (any block size that is a multiple of 32).
-static __device__ __noinline__ void finalize_body(const PassArgs& a, int is, int ws, float2* smem) {
-  __shared__ int s_py, s_px;
-  __shared__ float s_peak;
-  const int T = blockDim.x, t = threadIdx.x;
-  const int H = a.H, W = a.W, Wh = W >> 1;
-  const WorkItem it = item_of(a, is);
-  const RowStat* st = a.stats + (size_t)ws * H;
-  const float2* Z = a.spec + (size_t)ws * H * Wh;
-  float2* const bufA = smem;
-  float2* const bufB = smem + row_smem_len(W);
-  WarpRed* red = reinterpret_cast<WarpRed*>(smem + 2 * row_smem_len(W));
-  const int nw = T >> 5, w = t >> 5;
+// ---------------------------------------------------------------- finalisation
+//
+// Peak, energy outside the cyclic 11x11 window and PCE (Eq. 3) of a candidate
+// whose row statistics and spectrum sit in a workspace slot.  The energy is the
+// sum, in this order, of kFinParts parts: the rows outside the window in three
+// interleaved shares (row y in share (y / T) % 3 for the T threads of a row
+// pair), then the six row pairs that hold the window's rows, recomputed from
+// the spectrum, each without the window's columns.  A part is summed per
+// thread, over its warps and over the T threads the same way wherever it is
+// computed, so one block per candidate and one per window pair, whose parts a
+// second kernel adds up, give the same bits.
 
+constexpr int kFinPairParts = 6, kFinRowParts = 3, kFinParts = kFinRowParts + kFinPairParts;
+
+// the b-th row pair of the window around row py (11 rows cover 6 pairs)
+__device__ __forceinline__ int window_pair(int py, int b, int H) {
+  return (((py - kHalfWindow + H) % H >> 1) + b) % (H >> 1);
+}
+
+struct FinPeak {
+  float peak;
+  int py, px;
+};
+// the first maximum over all rows, by the TB threads of the block; holds barriers
+__device__ __forceinline__ FinPeak block_peak(const RowStat* st, int H, int W, int t, int TB, WarpRed* red) {
+  __shared__ FinPeak s_peak;
   float bv = -INFINITY;
   int bi = INT_MAX;
-  for (int y = t; y < H; y += T) {
-    const RowStat r = st[y];
+  for (int y = t; y < H; y += TB) {
+    const RowStat r = ld_l2(st + y);
     better_f(bv, bi, r.max, y * W + r.arg);
   }
   warp_maxarg(bv, bi);
-  if ((t & 31) == 0) { red[w].ma = bv; red[w].ia = bi; }
+  if ((t & 31) == 0) {
+    red[t >> 5].ma = bv;
+    red[t >> 5].ia = bi;
+  }
   __syncthreads();
   if (t == 0) {
-    for (int k = 1; k < nw; ++k) better_f(bv, bi, red[k].ma, red[k].ia);
+    for (int k = 1; k < TB >> 5; ++k) better_f(bv, bi, red[k].ma, red[k].ia);
     if (bi == INT_MAX) bi = 0;
-    s_peak = bv;
-    s_py = bi / W;
-    s_px = bi - (bi / W) * W;
+    s_peak = FinPeak{bv, bi / W, bi - (bi / W) * W};
   }
   __syncthreads();
-  const int py = s_py, px = s_px;
-  double e = 0.0;
-  for (int y = t; y < H; y += T)
-    if (cdist(y, py, H) > kHalfWindow) e += st[y].sumsq;
-  int prev = -1;
-  for (int d = -kHalfWindow; d <= kHalfWindow; ++d) {
-    const int r = (py + d + H) % H;
-    const int p = r >> 1;
-    if (p == prev) continue;
-    prev = p;
-    build_full_row(bufA, Z + (size_t)(2 * p) * Wh, Z + (size_t)(2 * p + 1) * Wh, W, t, T);
-    __syncthreads();
-    const float2* buf = fft_row<true>(bufA, bufB, a.prow, a.tw, t, T);
-    for (int q = 0; q < 2; ++q) {
-      if (cdist(2 * p + q, py, H) > kHalfWindow) continue;
-      for (int x = t; x < W; x += T) {
-        if (cdist(x, px, W) <= kHalfWindow) continue;
-        const float2 v = buf[rpad(x)];
-        const double c = q ? v.y : v.x;
-        e += c * c;
-      }
-    }
-    __syncthreads();
-  }
-  e = warp_sum(e);
-  if ((t & 31) == 0) red[w].sa = e;
-  __syncthreads();
-  if (t == 0) {
-    double etot = red[0].sa;
-    for (int k = 1; k < nw; ++k) etot += red[k].sa;
-    const double E = etot / ((double)H * (double)W - (double)kWindowCount);
-    const double pk = (double)s_peak;
-    double pce;
-    if (E > 0.0) pce = (pk < 0 ? -1.0 : 1.0) * pk * pk / E;
-    else pce = pk == 0.0 ? 0.0 : (pk < 0 ? -INFINITY : INFINITY);
-    const FpDesc fp = a.fps[it.fp];
-    double pv = pk / ((double)H * (double)W) * (double)(*fp.inv_scale);
-    if (a.scale) pv /= (double)a.scale[it.frame];
-    CandResult r;
-    r.pce = pce;
-    r.peak = (float)pv;
-    r.py = py;
-    r.px = px;
-    r.cand = it.cand;
-    r.group = it.group;
-    r.pad = 0;
-    *result_of(a, is) = r;
-  }
+  return s_peak;
 }
 
+// share q of the energy of the rows outside the window, this thread's part (t < T)
+__device__ __forceinline__ double row_share(const RowStat* st, int H, int py, int q, int t, int T) {
+  double e = 0.0;
+  for (int y = q * T + t; y < H; y += kFinRowParts * T)
+    if (cdist(y, py, H) > kHalfWindow) e += ld_l2(st + y).sumsq;
+  return e;
+}
+
+// Energy of one window pair, this thread's part: squares summed in compensated
+// FP32 (exact products, 48-bit sums; an FP64 add or conversion takes 1/64 of the
+// FP32 rate, which made up a third of the finalisation), rows a and b in the
+// lanes, joined in double.
+struct PairEnergy {
+  float2 s = make_float2(0.f, 0.f), c = make_float2(0.f, 0.f);
+  __device__ __forceinline__ void add(float2 v) { csum_square2(s, c, v); }
+  __device__ __forceinline__ double total(bool row_a, bool row_b) const {
+    return (row_a ? (double)s.x + (double)c.x : 0.0) + (row_b ? (double)s.y + (double)c.y : 0.0);
+  }
+};
+
+// The sums of a group's parts: every warp leaves its own in red[part][warp], and
+// after a barrier one thread adds them up, warps in order.
+__device__ __forceinline__ void part_warp(double e, int t, double* red_part) {
+  e = warp_sum(e);
+  if ((t & 31) == 0) red_part[t >> 5] = e;
+}
+__device__ __forceinline__ double part_total(const double* red_part, int nw) {
+  double e = red_part[0];
+  for (int k = 1; k < nw; ++k) e += red_part[k];
+  return e;
+}
+
+// Where a candidate's parts wait when several blocks compute them: in its own
+// spectrum, dead but for the window's rows, eight rows from the peak.
+__device__ __forceinline__ double* fin_scratch(const PassArgs& a, int ws, int py) {
+  const int H = a.H, row = (py + H / 2) % H & ~1;
+  return reinterpret_cast<double*>(a.spec + ((size_t)ws * H + row) * (a.W >> 1));
+}
+
+// one thread: PCE and result of candidate `is`
+__device__ __forceinline__ void finish_candidate(const PassArgs& a, int is, const FinPeak& p, const double* parts) {
+  double etot = parts[0];
+  for (int k = 1; k < kFinParts; ++k) etot += parts[k];
+  const WorkItem it = item_of(a, is);
+  const int H = a.H, W = a.W;
+  const double E = etot / ((double)H * (double)W - (double)kWindowCount);
+  const double pk = (double)p.peak;
+  double pce;
+  if (E > 0.0) pce = (pk < 0 ? -1.0 : 1.0) * pk * pk / E;
+  else pce = pk == 0.0 ? 0.0 : (pk < 0 ? -INFINITY : INFINITY);
+  const FpDesc fp = a.fps[it.fp];
+  double pv = pk / ((double)H * (double)W) * (double)(*fp.inv_scale);
+  if (a.scale) pv /= (double)a.scale[it.frame];
+  CandResult r;
+  r.pce = pce;
+  r.peak = (float)pv;
+  r.py = p.py;
+  r.px = p.px;
+  r.cand = it.cand;
+  r.group = it.group;
+  r.pad = 0;
+  *result_of(a, is) = r;
+}
+// the peak in the result until k_finalize_sum completes it
+__device__ __forceinline__ void park_peak(const PassArgs& a, int is, const FinPeak& p) {
+  CandResult* r = result_of(a, is);
+  r->peak = p.peak;
+  r->py = p.py;
+  r->px = p.px;
+}
 
 }  // namespace prnu

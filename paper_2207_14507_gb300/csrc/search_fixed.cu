@@ -8,6 +8,7 @@
 #include <mutex>
 
 #include "internal.h"
+#include "search_common.cuh"
 #include "search_fixed.h"
 
 namespace prnu {
@@ -152,7 +153,9 @@ void launch_fixed_wave(const PassArgs& a, const FixedShape& fs, int col_variant,
   }
   {
     ProfScope ps(lc, kKindFinalize, s);
-    PRNU_CUDA_TRY(cudaLaunchKernel(fr.fin, dim3(a.nitems), dim3(fr.fin_threads), args, fr.fin_smem, s));
+    PRNU_CUDA_TRY(cudaLaunchKernel(fr.fin, dim3(a.nitems, fr.fin_split ? kFinPairParts : 1), dim3(fr.fin_threads), args,
+                                   fr.fin_smem, s));
+    if (fr.fin_split) launch_finalize_sum(a, s, lc);
   }
   lc.n += 4;
 }

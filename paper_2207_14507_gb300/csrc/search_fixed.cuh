@@ -101,9 +101,9 @@ __device__ __forceinline__ void row_forward_body(const PassArgs& a, int is, int 
     float2 v[16];
     const float dxj = (float)t - cx;
     if constexpr (DT == kF32I) {
-      const float* p = fr + (size_t)y0 * pad_pitch(W) + t;
+      const float *p = fr + (size_t)y0 * a.rpitch + t, *q = p + a.rpitch;
 #pragma unroll
-      for (int r = 0; r < 16; ++r) v[r] = make_float2(__ldg(p + r * NB0), __ldg(p + pad_pitch(W) + r * NB0));
+      for (int r = 0; r < 16; ++r) v[r] = make_float2(__ldg(p + r * NB0), __ldg(q + r * NB0));
     } else if (inside) warp_row16<DT, W, NB0, false>(fr, H, it, dxj, bx0, by0, bx1, by1, v);
     else warp_row16<DT, W, NB0, true>(fr, H, it, dxj, bx0, by0, bx1, by1, v);
     Dft<16, false>::run(v);
@@ -582,110 +582,84 @@ __device__ __forceinline__ void row_inverse_task(const PassArgs& a, int ws, int 
   row_inverse_body<SP, T, PPB, true>(a, ws, bx, smem, tx);
 }
 
-// finalize_body with the window's rows recomputed by the compile-time-planned
-// inverse row FFT (one row pair per thread group, PPB pairs per round).
+// The energy of window pair `p` outside the window's columns (and of its rows
+// inside the window only), this thread's part; the rows by the planned inverse
+// row FFT of the T threads of a group (thread t) in its buffer A.
+template <class SP, int T>
+__device__ __forceinline__ double window_pair_energy(const PassArgs& a, const float2* Z, const FinPeak& pk, int p, int t,
+                                                     float2* A) {
+  constexpr int W = SP::N, Wh = W / 2;
+  using SL = RowLast<SP, T>;
+  const float2* pa = Z + (size_t)(2 * p) * Wh;
+  float2 V[SL::IT][SL::R];
+  row_inverse_fft<SP, T, true>(pa, pa + Wh, A, t, V);
+  PairEnergy e;
+#pragma unroll
+  for (int it = 0; it < SL::IT; ++it) {
+    if (!SL::valid(t, it)) break;
+#pragma unroll
+    for (int r = 0; r < SL::R; ++r) {
+      const int x = t + it * SL::STEP + r * SL::NS;
+      if (cdist(x, pk.px, W) > kHalfWindow) e.add(V[it][r]);
+    }
+  }
+  return e.total(cdist(2 * p, pk.py, a.H) <= kHalfWindow, cdist(2 * p + 1, pk.py, a.H) <= kHalfWindow);
+}
+
+// One candidate by PPB groups of T threads: group g takes row shares and window
+// pairs g, g + PPB, ..
 template <class SP, int T, int PPB>
 __device__ __forceinline__ void finalize_task(const PassArgs& a, int is, int ws, float2* smem, int tx) {
   constexpr int W = SP::N, Wh = W / 2, L = row_len2(W), TB = T * PPB;
-  using SL = RowLast<SP, T>;
-  __shared__ int s_py, s_px, s_np;
-  __shared__ float s_peak;
-  __shared__ int s_pairs[2 * kHalfWindow + 1];
+  __shared__ double red[kFinParts][T / 32];
   const int t = tx, grp = t / T, tg = t - grp * T;
-  const int H = a.H;
-  const WorkItem it = item_of(a, is);
-  const RowStat* st = a.stats + (size_t)ws * H;
-  const float2* Z = a.spec + (size_t)ws * H * Wh;
-  WarpRed* red = reinterpret_cast<WarpRed*>(smem + (size_t)PPB * L);
-  constexpr int NW = TB / 32;
-  const int w = t >> 5;
-
-  float bv = -INFINITY;
-  int bi = INT_MAX;
-  for (int y = t; y < H; y += TB) {
-    const RowStat r = ld_l2(st + y);
-    better_f(bv, bi, r.max, y * W + r.arg);
+  const RowStat* st = a.stats + (size_t)ws * a.H;
+  const float2* Z = a.spec + (size_t)ws * a.H * Wh;
+  const FinPeak pk = block_peak(st, a.H, W, t, TB, reinterpret_cast<WarpRed*>(smem + (size_t)PPB * L));
+  for (int q = grp; q < kFinRowParts; q += PPB) part_warp(row_share(st, a.H, pk.py, q, tg, T), tg, red[q]);
+#pragma unroll 1
+  for (int b0 = 0; b0 < kFinPairParts; b0 += PPB) {
+    const int b = b0 + grp;
+    const double e = window_pair_energy<SP, T>(a, Z, pk, window_pair(pk.py, b % kFinPairParts, a.H), tg,
+                                               smem + (size_t)grp * L);
+    if (b < kFinPairParts) part_warp(e, tg, red[kFinRowParts + b]);
+    __syncthreads();   // the row buffers are free again
   }
-  warp_maxarg(bv, bi);
-  if ((t & 31) == 0) {
-    red[w].ma = bv;
-    red[w].ia = bi;
-  }
-  __syncthreads();
   if (t == 0) {
-    for (int k = 1; k < NW; ++k) better_f(bv, bi, red[k].ma, red[k].ia);
-    if (bi == INT_MAX) bi = 0;
-    s_peak = bv;
-    s_py = bi / W;
-    s_px = bi - (bi / W) * W;
-    int np = 0, prev = -1;
-    for (int d = -kHalfWindow; d <= kHalfWindow; ++d) {
-      const int p = ((s_py + d + H) % H) >> 1;
-      if (p != prev) s_pairs[np++] = p;
-      prev = p;
-    }
-    s_np = np;
-  }
-  __syncthreads();
-  const int py = s_py, px = s_px, np = s_np;
-  double e = 0.0;
-  for (int y = t; y < H; y += TB)
-    if (cdist(y, py, H) > kHalfWindow) e += ld_l2(st + y).sumsq;
-  for (int r0 = 0; r0 < np; r0 += PPB) {
-    const int k = r0 + grp;
-    const bool act = k < np;
-    const int p = act ? s_pairs[k] : 0;
-    float2* A = smem + (size_t)grp * L;
-    const float2* pa = Z + (size_t)(2 * p) * Wh;
-    float2 V[SL::IT][SL::R];
-    row_inverse_fft<SP, T, true>(pa, pa + Wh, A, tg, V);
-    if (act) {
+    double parts[kFinParts];
 #pragma unroll
-      for (int it = 0; it < SL::IT; ++it) {
-        if (!SL::valid(tg, it)) break;
-#pragma unroll
-        for (int r = 0; r < SL::R; ++r) {
-          const int x = tg + it * SL::STEP + r * SL::NS;
-          if (cdist(x, px, W) <= kHalfWindow) continue;
-          if (cdist(2 * p, py, H) <= kHalfWindow) e += (double)V[it][r].x * V[it][r].x;
-          if (cdist(2 * p + 1, py, H) <= kHalfWindow) e += (double)V[it][r].y * V[it][r].y;
-        }
-      }
-    }
-    __syncthreads();
-  }
-  e = warp_sum(e);
-  if ((t & 31) == 0) red[w].sa = e;
-  __syncthreads();
-  if (t == 0) {
-    double etot = red[0].sa;
-    for (int k = 1; k < NW; ++k) etot += red[k].sa;
-    const double E = etot / ((double)H * (double)W - (double)kWindowCount);
-    const double pk = (double)s_peak;
-    double pce;
-    if (E > 0.0) pce = (pk < 0 ? -1.0 : 1.0) * pk * pk / E;
-    else pce = pk == 0.0 ? 0.0 : (pk < 0 ? -INFINITY : INFINITY);
-    const FpDesc fp = a.fps[it.fp];
-    double pv = pk / ((double)H * (double)W) * (double)(*fp.inv_scale);
-    if (a.scale) pv /= (double)a.scale[it.frame];
-    CandResult res;
-    res.pce = pce;
-    res.peak = (float)pv;
-    res.py = py;
-    res.px = px;
-    res.cand = it.cand;
-    res.group = it.group;
-    res.pad = 0;
-    *result_of(a, is) = res;
+    for (int k = 0; k < kFinParts; ++k) parts[k] = part_total(red[k], T / 32);
+    finish_candidate(a, is, pk, parts);
   }
 }
-// One block per candidate of the wave: finalize_task with PPB row pairs of the
-// window recomputed at a time.
+// One block per candidate of the wave, PPB row pairs of the window at a time.
 template <class SP, int T, int PPB>
 __global__ void __launch_bounds__(T * PPB) k_finalize_fx(PassArgs a) {
   if (past_count(a, blockIdx.x, 0)) return;
   extern __shared__ float4 smem4[];
   finalize_task<SP, T, PPB>(a, blockIdx.x, blockIdx.x, reinterpret_cast<float2*>(smem4), threadIdx.x);
+}
+// One block per window pair (blockIdx.y) of a candidate; k_finalize_sum ends it.
+template <class SP, int T>
+__global__ void __launch_bounds__(T) k_finalize_part_fx(PassArgs a) {
+  if (past_count(a, blockIdx.x, 0)) return;
+  extern __shared__ float4 smem4[];
+  __shared__ double red[2][T / 32];
+  constexpr int W = SP::N, Wh = W / 2, L = row_len2(W);
+  float2* smem = reinterpret_cast<float2*>(smem4);
+  const int s = blockIdx.x, b = blockIdx.y, t = threadIdx.x;
+  const RowStat* st = a.stats + (size_t)s * a.H;
+  const FinPeak pk = block_peak(st, a.H, W, t, T, reinterpret_cast<WarpRed*>(smem + L));
+  if (b < kFinRowParts) part_warp(row_share(st, a.H, pk.py, b, t, T), t, red[0]);
+  part_warp(window_pair_energy<SP, T>(a, a.spec + (size_t)s * a.H * Wh, pk, window_pair(pk.py, b, a.H), t, smem), t,
+            red[1]);
+  __syncthreads();
+  if (t == 0) {
+    double* parts = fin_scratch(a, s, pk.py);
+    if (b < kFinRowParts) parts[b] = part_total(red[0], T / 32);
+    parts[kFinRowParts + b] = part_total(red[1], T / 32);
+  }
+  if (b == 0 && t == 0) park_peak(a, s, pk);
 }
 
 //
@@ -858,10 +832,15 @@ struct ShapeDef {
     r.fwd[kF32I] = row_fwd<kF32I, PPB, RFMB>();
     if constexpr (RIMB > 0) r.inv = (void*)k_row_inverse_mb<RS, RTI, PPB, RIMB>;
     else r.inv = (void*)k_row_inverse_fx<RS, RTI, PPB>;
-    r.fin = (void*)k_finalize_fx<RS, FT, kFinPairs>;
-    r.fin_threads = FT * kFinPairs;
-    r.fin_smem = row_fx_smem<W>(kFinPairs);
-    allow(k_finalize_fx<RS, FT, kFinPairs>);
+    // A block per window pair where a pair's FFT fills one (us per 1000
+    // candidates, one block per candidate first: 1080p 124 -> 69, 4K 258 -> 157,
+    // 720p 112 -> 61; 256, one warp a pair: 35 -> 38)
+    r.fin_split = FT > 32;
+    r.fin_threads = r.fin_split ? FT : FT * kFinPairs;
+    r.fin_smem = row_fx_smem<W>(r.fin_split ? 1 : kFinPairs);
+    if constexpr (FT > 32) r.fin = (void*)k_finalize_part_fx<RS, FT>;
+    else r.fin = (void*)k_finalize_fx<RS, FT, kFinPairs>;
+    allow_max_dynamic_smem(r.fin);
     allow_max_dynamic_smem(r.inv);
     return r;
   }

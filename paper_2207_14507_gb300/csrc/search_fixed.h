@@ -40,7 +40,8 @@ struct FixedRow {
   size_t smem;
   void* fwd[kNumStoreLayouts];   // by residual storage type (kF32, kF16, kBF16, kF16P, kBF16P, kF32I)
   void* inv;
-  void* fin;                 // per-candidate PCE (one block per candidate)
+  void* fin;                 // per-candidate PCE: one block per candidate, or per window pair (fin_split)
+  bool fin_split;
   int fin_threads;
   size_t fin_smem;
 };
