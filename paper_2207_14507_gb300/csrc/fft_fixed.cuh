@@ -210,38 +210,80 @@ __device__ __forceinline__ void row_stage_ip(float2* buf, int t) {
   }
 }
 
-// Last stage of row plan SP (Ns = n/R): butterflies j = t + it*STEP, outputs
-// x = j + r*Ns stay in registers, v[it]; `valid` tells which are real.  Where
-// two butterflies per thread cover the stage, half of them is the step (even
-// loads); else T.
+// The last stage's butterflies ja = t and jb = NS - t (t = 0: 0 and NS/2) from
+// the row layout, their outputs x = j + r*NS in va and vb.  One set of twiddles
+// serves both: with w = exp(-2 pi i / (NS R)), w^(r (NS - k)) = w_R^r conj(w^(rk)), so
+// output q of butterfly NS - k is output q + 1 of the DFT of the inputs times
+// conj(w^(rk)).  (k = NS/2 for t = 0, whose butterfly 0 has no twiddles.)
+template <int R, int NS, bool INV>
+__device__ __forceinline__ void mirror_pair_stage(const float2* __restrict__ in, int t, float2 (&va)[R], float2 (&vb)[R]) {
+  constexpr int LB = NS / 16 * 18, RP = TwTab<R, NS>::RP;
+  const int k = t == 0 ? NS / 2 : t;
+  const float2 *sa = in + rp2(t), *sb = in + rp2(t == 0 ? NS / 2 : NS - t);
+  float2 u[R];
+#pragma unroll
+  for (int r = 0; r < R; ++r) {
+    va[r] = sa[r * LB];
+    u[r] = sb[r * LB];
+  }
+  const float4* p = reinterpret_cast<const float4*>(kStageTw<R, NS>.v) + k;
+#pragma unroll
+  for (int m = 0; m < RP / 2; ++m) {
+    const float4 w = __ldg(p + m * NS);
+    const int r = 2 * m + 1;
+    if (t != 0) va[r] = tw_mul<INV>(va[r], w.x, w.y);
+    u[r] = tw_mul<!INV>(u[r], w.x, w.y);
+    if (r + 1 < R) {
+      if (t != 0) va[r + 1] = tw_mul<INV>(va[r + 1], w.z, w.w);
+      u[r + 1] = tw_mul<!INV>(u[r + 1], w.z, w.w);
+    }
+  }
+  DftP<R, INV>::run(va);
+  DftP<R, INV>::run(u);
+#pragma unroll
+  for (int r = 0; r < R; ++r) vb[r] = u[(r + 1) % R];
+}
+
+// Last stage of row plan SP (Ns = n/R): butterflies of thread t, `it` of them,
+// outputs x(t, it, r), increasing in (r, it), stay in registers, v[it]; `valid`
+// tells which are real.  Where two butterflies per thread cover the stage they
+// are a mirror pair, else j = t + it*T.
 template <class SP, int T>
 struct RowLast {
   using G = Stg<SP, SP::S - 1>;
   static constexpr int R = G::R;
   static constexpr int NS = G::NS;
-  static constexpr int STEP = (G::NB > T && G::NB % 2 == 0 && G::NB / 2 <= T) ? G::NB / 2 : T;
-  static constexpr int IT = (G::NB + STEP - 1) / STEP;
+  static constexpr bool PAIR = G::NB > T && G::NB % 2 == 0 && G::NB / 2 <= T;
+  static constexpr int IT = PAIR ? 2 : (G::NB + T - 1) / T;
   static_assert(G::NB == G::NS && G::NB % 16 == 0, "last stage: k = j");
-  __device__ __forceinline__ static bool valid(int t, int it) { return t < STEP && t + it * STEP < G::NB; }
+  __device__ __forceinline__ static bool valid(int t, int it) { return PAIR ? t < NS / 2 : t + it * T < G::NB; }
+  __device__ __forceinline__ static int x(int t, int it, int r) {
+    if (PAIR) return (it == 0 ? t : t == 0 ? NS / 2 : NS - t) + r * NS;
+    return t + it * T + r * NS;
+  }
 };
 
 template <class SP, int T, bool INV>
 __device__ __forceinline__ void row_stage_last(const float2* __restrict__ in, int t,
                                                float2 (&v)[RowLast<SP, T>::IT][RowLast<SP, T>::R]) {
   using L = RowLast<SP, T>;
-  constexpr int LB = L::NS / 16 * 18;
+  if constexpr (L::PAIR) {
+    if (t < L::NS / 2) mirror_pair_stage<L::R, L::NS, INV>(in, t, v[0], v[1]);
+  } else {
+    constexpr int LB = L::NS / 16 * 18;
 #pragma unroll
-  for (int it = 0; it < L::IT; ++it) {
-    if (!L::valid(t, it)) break;
-    const int j = t + it * L::STEP;
-    const float2* src = in + rp2(j);
-    float2 u[1][L::R];
+    for (int it = 0; it < L::IT; ++it) {
+      if (!L::valid(t, it)) break;
+      const int j = t + it * T;
+      const float2* src = in + rp2(j);
+      float2 u[1][L::R];
 #pragma unroll
-    for (int r = 0; r < L::R; ++r) u[0][r] = src[r * LB];
-    twiddle_tab<L::R, L::NS, INV, 1>(u, j);
-    DftP<L::R, INV>::run(u[0]);
+      for (int r = 0; r < L::R; ++r) u[0][r] = src[r * LB];
+      twiddle_tab<L::R, L::NS, INV, 1>(u, j);
+      DftP<L::R, INV>::run(u[0]);
 #pragma unroll
-    for (int r = 0; r < L::R; ++r) v[it][r] = u[0][r];
+      for (int r = 0; r < L::R; ++r) v[it][r] = u[0][r];
+    }
   }
 }
 

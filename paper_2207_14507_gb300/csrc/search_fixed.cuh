@@ -135,16 +135,7 @@ __device__ __forceinline__ void row_forward_body(const PassArgs& a, int is, int 
     if (t < NS / 2) {
       const int ja = t, jb = t == 0 ? NS / 2 : NS - t;
       float2 va[1][R], vb[1][R];
-      const float2 *sa = A + rp2(ja), *sb = A + rp2(jb);
-#pragma unroll
-      for (int r = 0; r < R; ++r) {
-        va[0][r] = sa[r * LB];
-        vb[0][r] = sb[r * LB];
-      }
-      twiddle_tab<R, NS, false, 1>(va, ja);
-      DftP<R, false>::run(va[0]);
-      twiddle_tab<R, NS, false, 1>(vb, jb);
-      DftP<R, false>::run(vb[0]);
+      mirror_pair_stage<R, NS, false>(A, t, va[0], vb[0]);
       if (t == 0) {
         put0(va[0][0], va[0][R / 2]);
 #pragma unroll
@@ -289,7 +280,7 @@ __device__ __forceinline__ void row_inverse_body(const PassArgs& a, int ws, int 
   float2 v[GL::IT][GL::R];
   row_inverse_fft<SP, T, CG>(pa, pa + Wh, A, t, v);
   // per thread: max, first arg-max and energy of each row over its outputs,
-  // visited in increasing x (x = t + it*STEP + r*NS with t + it*STEP < NS), so a
+  // visited in increasing x (butterfly 0's before butterfly 1's at each r), so a
   // strictly larger value is the only one that moves the arg-max: the first
   // maximum is kept without comparing indices
   float ma = -INFINITY, mb = -INFINITY;
@@ -300,7 +291,7 @@ __device__ __forceinline__ void row_inverse_body(const PassArgs& a, int ws, int 
 #pragma unroll
     for (int it = 0; it < GL::IT; ++it) {
       if (!GL::valid(t, it)) continue;
-      const int x = t + it * GL::STEP + r * GL::NS;
+      const int x = GL::x(t, it, r);
       const float2 u = v[it][r];
       if (u.x > ma) {
         ma = u.x;
@@ -599,7 +590,7 @@ __device__ __forceinline__ double window_pair_energy(const PassArgs& a, const fl
     if (!SL::valid(t, it)) break;
 #pragma unroll
     for (int r = 0; r < SL::R; ++r) {
-      const int x = t + it * SL::STEP + r * SL::NS;
+      const int x = SL::x(t, it, r);
       if (cdist(x, pk.px, W) > kHalfWindow) e.add(V[it][r]);
     }
   }
