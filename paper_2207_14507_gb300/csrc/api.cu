@@ -1225,18 +1225,10 @@ int prnu_fingerprint_term(prnu_ctx* ctx, const float* d_K, int H, int W, int sto
     f->W = W;
     f->dtype = half ? kF16 : kF32;
     f->bytes = (size_t)H * Wh * (half ? sizeof(__half2) : sizeof(float2));
-    // the column pass of the compile-time-planned kernels reads strips of the
-    // spectrum by TMA: its descriptors live right after the spectrum
-    alignas(64) unsigned char tmaps[kFpTmapBytes];
-    const size_t tmap_off = (f->bytes + 127) / 128 * 128;
-    f->bytes = tmap_off + kFpTmapBytes;
+    // the column pass of the compile-time-planned kernels copies whole strips
+    f->strips = find_fixed(H, W) ? 1 : 0;
     f->d_spec = ctx_alloc(ctx, f->bytes);
     try {
-      if (encode_fp_tmaps(f->d_spec, f->dtype, H, W, tmaps)) {
-        PRNU_CUDA_TRY(
-            cudaMemcpy(static_cast<char*>(f->d_spec) + tmap_off, tmaps, kFpTmapBytes, cudaMemcpyHostToDevice));
-        f->tmap_off = tmap_off;
-      }
       f->d_scal = reinterpret_cast<float*>(ctx_alloc(ctx, 3 * sizeof(float)));
     } catch (...) {
       ctx_free(ctx, f->d_spec, f->bytes);
@@ -1269,7 +1261,7 @@ int prnu_fingerprint_term(prnu_ctx* ctx, const float* d_K, int H, int W, int sto
     a.row_threads = rowT;
     launch_row_forward(a, false, f->d_scal, nullptr, s, ctx->launches);
     launch_col(a, 1, half ? nullptr : reinterpret_cast<float2*>(f->d_spec), half ? f->d_spec : nullptr,
-               f->d_scal + 1, s, ctx->launches);
+               f->d_scal + 1, s, ctx->launches, f->strips);
     PRNU_CUDA_TRY(cudaEventRecord(f->ready, s));
     PRNU_CUDA_TRY(cudaEventRecord(ctx->last_done, s));
     f->refs = 1;

@@ -127,8 +127,7 @@ struct Col2 {
 #pragma unroll 1
         for (int i = j; i < H; i += ra) {
           const int im = i == 0 ? 0 : H - i;
-          sm[H + i] = packed_col0_product(sm[i], sm[im], load_spec(fp.spec, fp.dtype, (size_t)i * Wh),
-                                          load_spec(fp.spec, fp.dtype, (size_t)im * Wh));
+          sm[H + i] = packed_col0_product(sm[i], sm[im], load_fp(fp, i, 0, H, Wh), load_fp(fp, im, 0, H, Wh));
         }
 #pragma unroll
         for (int r = 0; r < R; ++r) v[r] = sm[H + j + r * ra];
@@ -137,7 +136,7 @@ struct Col2 {
     }
     if (!act) return;
     if (col != 0 && col < Wh) {
-      const size_t first = (size_t)j * Wh + col, step = (size_t)ra * Wh;
+      const size_t first = fp_index(fp, j, col, H, Wh), step = (size_t)ra * (fp.strips ? 4 : Wh);
       if (fp.dtype == kF32) {
         const float2* s = reinterpret_cast<const float2*>(fp.spec) + first;
 #pragma unroll

@@ -58,9 +58,18 @@ template <class CP>
 __host__ __device__ constexpr size_t col_buf_bytes(int nc) {
   return ((size_t)CP::rows * nc * sizeof(float2) + 127) / 128 * 128;
 }
+// The fingerprint's strips of 4 columns lie one after the other in shared
+// memory, this many bytes apart beyond their own, so that the columns a warp
+// reads together fall in distinct banks.
+__host__ __device__ constexpr int fp_strip_pad(int nc) { return nc > 4 ? 512 / nc : 0; }
+__host__ __device__ constexpr size_t fp_strips_bytes(int H, int nc, int es) {
+  return (size_t)(nc / 4) * ((size_t)H * 4 * es + fp_strip_pad(nc));
+}
 template <class CP>
 __host__ __device__ constexpr size_t col_pass_smem(int nc, int mode) {
-  return col_buf_bytes<CP>(nc) + (mode == 2 ? 2 * (size_t)CP::H * sizeof(float2) : (size_t)CP::H * nc * fp_region_bin(mode));
+  return col_buf_bytes<CP>(nc) + (mode == 2  ? 2 * (size_t)CP::H * sizeof(float2)
+                                  : mode > 2 ? fp_strips_bytes(CP::H, nc, fp_region_bin(mode))
+                                             : 0);
 }
 constexpr long long kTmaWaitPolls = 1ll << 20;   // polls of mbarrier.try_wait before giving up
 
@@ -82,16 +91,17 @@ __device__ __forceinline__ bool block_wait(uint64_t* bar, uint32_t ph, int* err,
   return true;
 }
 
-// the fingerprint's strip by TMA to shared memory at dst, completing on bar
+// the fingerprint's NC columns from c0 to shared memory at dst, completing on
+// bar: a contiguous copy per strip of 4 (the spectrum's own strips come as rows
+// of 32 bytes, of which a TMA unit moves one in about 1.4 cycles: the
+// fingerprint's, copied that way too, took a sixth of the pass)
 template <int H, int NC>
-__device__ __forceinline__ void load_fp_strip(const FpDesc& fp, int c0, char* dst, uint64_t* bar) {
-  const CUtensorMap* fm = reinterpret_cast<const CUtensorMap*>(fp.tmaps) + fp_tmap_index(NC);
-  const int es = fp.dtype == kF32 ? 8 : 4, br = tma_box_rows(H, NC, es);
-  asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"(reinterpret_cast<uint64_t>(fm))
-               : "memory");
-  mbar_expect_tx(bar, H * NC * es);
+__device__ __forceinline__ void load_fp_strips(const FpDesc& fp, int c0, char* dst, uint64_t* bar) {
+  const uint32_t bytes = H * 4 * (fp.dtype == kF32 ? 8 : 4);
+  const char* src = static_cast<const char*>(fp.spec) + (size_t)(c0 / 4) * bytes;
+  mbar_expect_tx(bar, NC / 4 * bytes);
 #pragma unroll 1
-  for (int b = 0; b < H / br; ++b) tma_load_2d(dst + (size_t)b * br * NC * es, fm, 2 * c0, b * br, bar);
+  for (int q = 0; q < NC / 4; ++q) bulk_load(dst + q * (bytes + fp_strip_pad(NC)), src + q * bytes, bytes, bar);
 }
 
 // Columns bx*NC .. bx*NC+NC-1 of candidate `is` in workspace slot `ws`, by
@@ -99,12 +109,12 @@ __device__ __forceinline__ void load_fp_strip(const FpDesc& fp, int c0, char* ds
 // MODE 0: every thread loads and stores its own elements.  MODE >= 1: the
 // strip comes into shared memory by TMA tile copies through `map` (the
 // workspace spectra as a [slots*H][W] float tensor) and leaves the same way.
-// MODE 2: the fingerprint strip too comes by TMA, into the strip buffer once
+// MODE 2: the fingerprint's strips come by bulk copies, into the strip buffer once
 // stage B has taken its inputs (the packed column-0 scratch then sits after
-// the buffer).  MODE 3 and 4: the fingerprint strip comes by TMA into its own
+// the buffer).  MODE 3 and 4: they come into their own
 // region after the strip buffer, copied from the start together with the
-// strip (MODE 4 sizes the region for FP16 bins: FP32 fingerprints are then
-// loaded per thread).  A TMA wait that runs out raises a.err and abandons the
+// strip (MODE 4 sizes the region for FP16 bins and takes FP16 fingerprints
+// only).  A TMA wait that runs out raises a.err and abandons the
 // candidate.
 // PART splits the pass for forward units (candidates that share a frame and
 // a grid node): PART 1 runs the forward column FFT only and stores its
@@ -132,10 +142,7 @@ __device__ __forceinline__ void col_body(const PassArgs& a, int is, int ws, int 
 
   constexpr int BR = tma_box_rows(H, NC);
   __shared__ uint64_t s_bar, s_fbar;
-  const int fes = fp.dtype == kF32 ? 8 : 4;
-  // the fingerprint strip comes by TMA (boxes of at least 16 bytes; MODE 3/4:
-  // a region sized for its bins), else by per-thread loads
-  const bool fp_tma = FPT && fp.tmaps != nullptr && NC * fes >= 16 && (!FPSEP || fes <= fp_region_bin(MODE));
+  const bool fp32 = MODE != 4 && fp.dtype == kF32;   // MODE 4 takes FP16 fingerprints only (launch_fixed_wave)
   if constexpr (TMA) {
     static_assert(BR > 0, "no TMA box for this strip");
     if (t == 0) {
@@ -148,7 +155,7 @@ __device__ __forceinline__ void col_body(const PassArgs& a, int is, int ws, int 
       mbar_expect_tx(&s_bar, H * NC * 8 + (a.stall ? 16 : 0));   // the test hook waits for bytes that never come
 #pragma unroll 1
       for (int b = 0; b < H / BR; ++b) tma_load_2d(sm + b * BR * NC, map, 2 * c0, src_ws * H + b * BR, &s_bar);
-      if (FPSEP && fp_tma) load_fp_strip<H, NC>(fp, c0, fpsm, &s_fbar);
+      if (FPSEP) load_fp_strips<H, NC>(fp, c0, fpsm, &s_fbar);
       if constexpr (PFD > 0) {   // the strip PFD strips on, into L2
         const int n = is * (Wh / NC) + bx + PFD, s2 = n / (Wh / NC), b2 = n - s2 * (Wh / NC);
         if (s2 < a.nitems) {
@@ -157,7 +164,7 @@ __device__ __forceinline__ void col_body(const PassArgs& a, int is, int ws, int 
         }
       }
     }
-    if (!block_wait(&s_bar, 0, a.err, FPSEP && fp_tma ? &s_fbar : nullptr)) return;
+    if (!block_wait(&s_bar, 0, a.err, FPSEP ? &s_fbar : nullptr)) return;
   }
 
   float2* Z = a.spec + (size_t)ws * H * Wh;
@@ -196,11 +203,9 @@ __device__ __forceinline__ void col_body(const PassArgs& a, int is, int ws, int 
     for (int r = 0; r < RB; ++r) v[0][r] = src[r * RA * NC];
   }
   if constexpr (FPT && !FPSEP) {   // the strip buffer is free: the fingerprint's strip goes there
-    if (fp_tma) {
-      fence_proxy_async_smem();
-      __syncthreads();
-      if (t == 0) load_fp_strip<H, NC>(fp, c0, fpsm, &s_fbar);
-    }
+    fence_proxy_async_smem();
+    __syncthreads();
+    if (t == 0) load_fp_strips<H, NC>(fp, c0, fpsm, &s_fbar);
   }
   if constexpr (PART != 2) {
     if (act_b) {
@@ -217,15 +222,13 @@ __device__ __forceinline__ void col_body(const PassArgs& a, int is, int ws, int 
       for (int r = 0; r < RB; ++r) dst[r * RA * NC] = v[0][r];
     }
   } else {
-    // fingerprint bin i of column cc of the strip
-    auto fp_bin = [&](int i, int cc) -> float2 {
-      if (fp_tma) {
-        if (fp.dtype == kF32) return reinterpret_cast<const float2*>(fpsm)[i * NC + cc];
-        return __half22float2(reinterpret_cast<const __half2*>(fpsm)[i * NC + cc]);
-      }
-      return load_spec(fp.spec, fp.dtype, (size_t)i * Wh + c0 + cc);
+    // fingerprint bin i of the strip's first column
+    auto fp_bin0 = [&](int i) -> float2 {
+      const char* p = FPT ? fpsm : static_cast<const char*>(fp.spec);
+      if (fp32) return reinterpret_cast<const float2*>(p)[i * 4];
+      return __half22float2(reinterpret_cast<const __half2*>(p)[i * 4]);
     };
-    if (FPT && fp_tma) {
+    if constexpr (FPT) {
       if (!block_wait(&s_fbar, 0, a.err)) return;
     } else {
       __syncthreads();   // every strip value read
@@ -244,7 +247,7 @@ __device__ __forceinline__ void col_body(const PassArgs& a, int is, int ws, int 
 #pragma unroll 1
         for (int i = j; i < H; i += RA) {
           const int im = i == 0 ? 0 : H - i;
-          X0[H + i] = packed_col0_product(X0[i], X0[im], fp_bin(i, 0), fp_bin(im, 0));
+          X0[H + i] = packed_col0_product(X0[i], X0[im], fp_bin0(i), fp_bin0(im));
         }
 #pragma unroll
         for (int r = 0; r < RB; ++r) v[0][r] = X0[H + j + r * RA];
@@ -252,21 +255,22 @@ __device__ __forceinline__ void col_body(const PassArgs& a, int is, int ws, int 
       __syncthreads();
     }
     if (act_b && col != 0) {
-      if (fp_tma && fp.dtype == kF32) {
-        const float2* f = reinterpret_cast<const float2*>(fpsm) + j * NC + c;
+      // this thread's bins, in shared memory or the spectrum's own strips
+      const int e0 = ((FPT ? c >> 2 : 0) * H + j) * 4 + (c & 3);
+      const char* f = FPT ? fpsm + (c >> 2) * fp_strip_pad(NC)
+                          : static_cast<const char*>(fp.spec) + (size_t)(col >> 2) * (H * 4 * (fp32 ? 8 : 4));
+      if (fp32) {
+        const float2* p = reinterpret_cast<const float2*>(f) + e0;
 #pragma unroll
-        for (int r = 0; r < RB; ++r) v[0][r] = c_conj_mul(v[0][r], f[r * RA * NC]);
-      } else if (fp_tma) {
-        const __half2* f = reinterpret_cast<const __half2*>(fpsm) + j * NC + c;
-#pragma unroll
-        for (int r = 0; r < RB; ++r) v[0][r] = c_conj_mul(v[0][r], __half22float2(f[r * RA * NC]));
+        for (int r = 0; r < RB; ++r) v[0][r] = c_conj_mul(v[0][r], FPT ? p[r * RA * 4] : __ldg(p + r * RA * 4));
       } else {
+        const __half2* p = reinterpret_cast<const __half2*>(f) + e0;
 #pragma unroll
         for (int r = 0; r < RB; ++r)
-          v[0][r] = c_conj_mul(v[0][r], load_spec(fp.spec, fp.dtype, (size_t)(j + r * RA) * Wh + col));
+          v[0][r] = c_conj_mul(v[0][r], __half22float2(FPT ? p[r * RA * 4] : __ldg(p + r * RA * 4)));
       }
     }
-    if (FPT && !FPSEP && fp_tma) __syncthreads();   // every fingerprint bin read before the buffer is rewritten
+    if (FPT && !FPSEP) __syncthreads();   // every fingerprint bin read before the buffer is rewritten
     if (act_b) {
       DftP<RB, true>::run(v[0]);
       float2* dst = sm + j * LB * NC + c;

@@ -33,10 +33,10 @@ struct WorkItem {
 
 // Fingerprint spectrum as the kernels see it.
 struct FpDesc {
-  const void* spec;    // packed [H][W/2] complex, float2 or __half2
+  const void* spec;          // packed half spectrum, float2 or __half2
   int dtype;                 // kF32 or kF16
   const float* inv_scale;    // device scalar: multiply the correlation by it to undo the storage scale
-  const void* tmaps;         // device CUtensorMap[4] of the spectrum (strips of 2, 4, 8, 16 columns), or nullptr
+  int strips;                // layout: 0 [H][W/2], 1 strips of 4 columns, [W/8][H][4] (planned sizes)
 };
 
 // Per-row statistics of one candidate's correlation surface.
@@ -189,6 +189,14 @@ __device__ __forceinline__ float2 load_spec(const void* p, int dtype, size_t i) 
   if (dtype == kF32) return __ldg(reinterpret_cast<const float2*>(p) + i);
   __half2 h = reinterpret_cast<const __half2*>(p)[i];
   return __half22float2(h);
+}
+
+// fingerprint bin i of column col (H rows, Wh columns): its place, and its value
+__device__ __forceinline__ size_t fp_index(const FpDesc& fp, int i, int col, int H, int Wh) {
+  return fp.strips ? ((size_t)(col >> 2) * H + i) * 4 + (col & 3) : (size_t)i * Wh + col;
+}
+__device__ __forceinline__ float2 load_fp(const FpDesc& fp, int i, int col, int H, int Wh) {
+  return load_spec(fp.spec, fp.dtype, fp_index(fp, i, col, H, Wh));
 }
 
 }  // namespace prnu

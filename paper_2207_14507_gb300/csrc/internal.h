@@ -91,12 +91,12 @@ struct ProfScope {
 void launch_row_forward(const PassArgs& a, bool warp, const float* mean_sub, float2* out, cudaStream_t s,
                         LaunchCounter& lc);
 // mode 0: forward FFT, multiply by the fingerprint, inverse FFT (in place)
-// mode 1: forward FFT only, written to out_f32 / out_f16 scaled by *scale
+// mode 1: forward FFT only, written to out_f32 / out_f16 scaled by *scale (out_strips: the layout, FpDesc)
 // mode 2: multiply only by the fingerprint (packed spectra, in place)  [naive path]
 // mode 3: forward only, in place (float2)                               [naive path]
 // mode 4: inverse only, in place (float2)                               [naive path]
 void launch_col(const PassArgs& a, int mode, float2* out_f32, void* out_f16, const float* scale,
-                cudaStream_t s, LaunchCounter& lc);
+                cudaStream_t s, LaunchCounter& lc, int out_strips = 0);
 // widths with a two-stage plan (a.prow.ra; row_generic.cuh)
 void launch_row_forward2(const PassArgs& a, bool warp, const float* mean_sub, float2* out, cudaStream_t s,
                          LaunchCounter& lc);
@@ -196,8 +196,8 @@ inline ResidLayout padded_layout(int H, int W) {
 struct Fingerprint {
   int H = 0, W = 0;
   int dtype = kF32;
-  void* d_spec = nullptr;    // spectrum, then (at tmap_off) the TMA descriptors of the column pass, if any
-  size_t tmap_off = 0;       // 0: no descriptors
+  void* d_spec = nullptr;    // spectrum
+  int strips = 0;            // its layout (FpDesc)
   float* d_scal = nullptr;   // [mean, scale, inv_scale]
   size_t bytes = 0;
   int refs = 0;
@@ -206,8 +206,7 @@ struct Fingerprint {
 
 // the kernels' view of a cached fingerprint
 inline FpDesc fp_desc(const Fingerprint& f) {
-  return FpDesc{f.d_spec, f.dtype, f.d_scal + 2,
-                f.tmap_off ? static_cast<const char*>(f.d_spec) + f.tmap_off : nullptr};
+  return FpDesc{f.d_spec, f.dtype, f.d_scal + 2, f.strips};
 }
 
 struct DeviceBuf {

@@ -96,7 +96,8 @@ __global__ void __launch_bounds__(512, 2) k_row_forward(PassArgs a, const float*
 // mode 0: fwd FFT, x conj(.) * K0^, inv FFT;  1: fwd FFT to out (fingerprint);
 // 2: product only;  3: fwd FFT only;  4: inv FFT only (modes 2-4 in place).
 __global__ void __launch_bounds__(512, 2) k_col(PassArgs a, int mode, float2* __restrict__ out_f32,
-                                              __half2* __restrict__ out_f16, const float* __restrict__ out_scale) {
+                                              __half2* __restrict__ out_f16, const float* __restrict__ out_scale,
+                                              int out_strips) {
   extern __shared__ float2 smem[];
   const int T = blockDim.x, tid = threadIdx.x;
   const int H = a.H, Wh = a.W >> 1;
@@ -122,8 +123,9 @@ __global__ void __launch_bounds__(512, 2) k_col(PassArgs a, int mode, float2* __
       const int i = e >> lg, col = c0 + (e & (NC - 1));
       if (col >= Wh) continue;
       const float2 v = make_float2(buf[e].x * s, buf[e].y * s);
-      if (out_f16) out_f16[(size_t)i * Wh + col] = __float22half2_rn(v);
-      else out_f32[(size_t)i * Wh + col] = v;
+      const size_t o = fp_index(FpDesc{nullptr, kF32, nullptr, out_strips}, i, col, H, Wh);
+      if (out_f16) out_f16[o] = __float22half2_rn(v);
+      else out_f32[o] = v;
     }
     return;
   }
@@ -133,7 +135,7 @@ __global__ void __launch_bounds__(512, 2) k_col(PassArgs a, int mode, float2* __
     for (int e = tid; e < n; e += T) {
       const int i = e >> lg, col = c0 + (e & (NC - 1));
       if (col == 0 || col >= Wh) continue;
-      const float2 s = load_spec(fp.spec, fp.dtype, (size_t)i * Wh + col);
+      const float2 s = load_fp(fp, i, col, H, Wh);
       buf[e] = c_conj_mul(buf[e], s);
     }
     if (c0 == 0) {
@@ -142,8 +144,7 @@ __global__ void __launch_bounds__(512, 2) k_col(PassArgs a, int mode, float2* __
       for (int i = tid; i <= (H >> 1); i += T) {
         const int im = (H - i) % H;
         const float2 F = buf[i << lg], Fm = buf[im << lg];
-        const float2 S = load_spec(fp.spec, fp.dtype, (size_t)i * Wh);
-        const float2 Sm = load_spec(fp.spec, fp.dtype, (size_t)im * Wh);
+        const float2 S = load_fp(fp, i, 0, H, Wh), Sm = load_fp(fp, im, 0, H, Wh);
         const float2 A = make_float2(0.5f * (F.x + Fm.x), 0.5f * (F.y - Fm.y));
         const float2 B = make_float2(0.5f * (F.y + Fm.y), 0.5f * (Fm.x - F.x));
         const float2 Ka = make_float2(0.5f * (S.x + Sm.x), 0.5f * (S.y - Sm.y));
@@ -463,7 +464,7 @@ void launch_row_forward(const PassArgs& a, bool warp, const float* mean_sub, flo
 }
 
 void launch_col(const PassArgs& a, int mode, float2* out_f32, void* out_f16, const float* scale, cudaStream_t s,
-                LaunchCounter& lc) {
+                LaunchCounter& lc, int out_strips) {
   if (mode == 0 && a.pcol.ra) {
     launch_col2(a, s, lc);
     return;
@@ -476,7 +477,7 @@ void launch_col(const PassArgs& a, int mode, float2* out_f32, void* out_f16, con
   const size_t sm = 2 * (size_t)a.H * nc * sizeof(float2);
   __half2* o16 = reinterpret_cast<__half2*>(out_f16);
   ProfScope ps(lc, kKindColumn, s);
-  k_col<<<g, b, sm, s>>>(a, mode, out_f32, o16, scale);
+  k_col<<<g, b, sm, s>>>(a, mode, out_f32, o16, scale, out_strips);
   PRNU_LAUNCH_CHECK();
   lc.n++;
 }

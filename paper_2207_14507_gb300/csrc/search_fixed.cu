@@ -1,10 +1,9 @@
 // search_fixed.cu -- registry and launchers of the compile-time-planned kernels
 // (search_fixed.cuh): the sizes they exist for, the TMA descriptors of their
-// spectra and fingerprints, and the launches of a wave.
+// spectra, and the launches of a wave.
 #include <cudaTypedefs.h>
 
 #include <algorithm>
-#include <cstring>
 #include <mutex>
 
 #include "internal.h"
@@ -70,34 +69,6 @@ bool encode_spec_map(CUtensorMap* m, const float2* base, int W, long long rows, 
 
 }  // namespace
 
-static_assert(4 * sizeof(CUtensorMap) == kFpTmapBytes, "four 128-byte descriptors per fingerprint");
-
-bool encode_fp_tmaps(const void* spec, int dtype, int H, int W, void* out) {
-  if (!find_fixed(H, W)) return false;
-  PFN_cuTensorMapEncodeTiled_v12000 enc = tensor_map_encoder();
-  if (!enc) return false;
-  const int es = dtype == kF32 ? 8 : 4;   // bytes per complex bin
-  const int ncs[4] = {2, 4, 8, 16};
-  CUtensorMap* m = reinterpret_cast<CUtensorMap*>(out);
-  for (int k = 0; k < 4; ++k) {
-    const int br = tma_box_rows(H, ncs[k], es);
-    if (ncs[k] * es < 16) {   // a box row narrower than 16 bytes: no descriptor (the kernel loads per thread)
-      memset(&m[k], 0, sizeof(CUtensorMap));
-      continue;
-    }
-    if (br <= 0) return false;
-    const cuuint64_t dims[2] = {(cuuint64_t)W, (cuuint64_t)H};
-    const cuuint64_t strides[1] = {(cuuint64_t)W * (es / 2)};
-    const cuuint32_t box[2] = {(cuuint32_t)(2 * ncs[k]), (cuuint32_t)br};
-    const cuuint32_t el[2] = {1, 1};
-    if (enc(&m[k], es == 8 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2,
-            const_cast<void*>(spec), dims, strides, box, el, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
-            CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-      return false;
-  }
-  return true;
-}
-
 void launch_fixed_wave(const PassArgs& a, const FixedShape& fs, int col_variant, cudaStream_t s, LaunchCounter& lc) {
   // forward units (several candidates of one frame and node): the row pass
   // and the forward column FFT per unit, into slots a.nitems + u; the product
@@ -106,21 +77,13 @@ void launch_fixed_wave(const PassArgs& a, const FixedShape& fs, int col_variant,
   const int nunits = units ? a.nunits : a.nitems;
   int v = std::max(0, std::min(col_variant, (int)fs.cols.size() - 1));
   // a variant whose fingerprint region holds FP16 bins only (mode 4) steps
-  // aside for FP32 fingerprints: the first variant that copies FP32 bins by TMA
-  // into a region of their own, else into the strip buffer
-  if (fs.cols[v].mode == 4 && a.fp_f32) {
-    auto first = [&](int mode) {
-      for (int k = 0; k < (int)fs.cols.size(); ++k)
-        if (fs.cols[k].mode == mode) return k;
-      return -1;
-    };
-    v = first(3) >= 0 ? first(3) : first(2) >= 0 ? first(2) : v;
-  }
-  const FixedCol& fv = fs.cols[v];
-  // forward units take the split pass (its inverse half in the variant's fingerprint mode)
-  const bool sep = fv.mode >= 3 && fs.col_inv_sep.fn && (fs.col_inv_sep.mode == 3 || !a.fp_f32);
-  const bool sep_h = fv.mode >= 3 && fs.col_inv_h.fn && !a.fp_f32;
-  const FixedCol& fc = units ? (sep_h ? fs.col_inv_h : sep ? fs.col_inv_sep : fs.col_inv) : fv;
+  // aside for FP32 fingerprints
+  if (fs.cols[v].mode == 4 && a.fp_f32) v = fs.f32_col;
+  // forward units take the split pass, its inverse half in the mode that is
+  // fastest for the wave's fingerprints (the bits are the same in all)
+  const bool sep = fs.col_inv_sep.fn && (fs.col_inv_sep.mode == 3 || !a.fp_f32);
+  const bool sep_h = fs.col_inv_h.fn && !a.fp_f32;
+  const FixedCol& fc = units ? (sep_h ? fs.col_inv_h : sep ? fs.col_inv_sep : fs.col_inv) : fs.cols[v];
   const FixedRow& fr = fs.row_for(a.pairs_per_block);
   const int Wh = a.W / 2;
   void* args[] = {const_cast<PassArgs*>(&a)};

@@ -422,25 +422,25 @@ __device__ __forceinline__ void row_forward_task(const PassArgs& a, int is, int 
 // adjacent columns per thread, loads and stores by every thread itself, L2
 // only.  The same steps as col_body (col_pass.cuh).
 
-// The fingerprint bins (i, col0) and (i, col0 + 1) for i = j + r*NS.
-template <int R, int NS, int Wh>
+// The fingerprint bins (i, col0) and (i, col0 + 1) for i = j + r*NS, from the
+// strip layout (col0 even: one vector).
+template <int R, int NS, int H>
 __device__ __forceinline__ void load_fp_pair(const FpDesc& fp, int j, int col0, float2 (&s)[2][R]) {
-  const size_t b = ((size_t)j * Wh + col0) / 2;
+  const size_t b = (((size_t)(col0 >> 2) * H + j) * 4 + (col0 & 3)) / 2;
   if (fp.dtype == kF32) {
     const float4* p = reinterpret_cast<const float4*>(fp.spec) + b;
 #pragma unroll
-    for (int r = 0; r < R; ++r) split2(__ldg(p + (size_t)r * NS * (Wh / 2)), s[0][r], s[1][r]);
+    for (int r = 0; r < R; ++r) split2(__ldg(p + r * NS * 2), s[0][r], s[1][r]);
   } else {
     const float2* p = reinterpret_cast<const float2*>(fp.spec) + b;   // two __half2
 #pragma unroll
     for (int r = 0; r < R; ++r) {
-      const float2 u = __ldg(p + (size_t)r * NS * (Wh / 2));
+      const float2 u = __ldg(p + r * NS * 2);
       s[0][r] = __half22float2(*reinterpret_cast<const __half2*>(&u.x));
       s[1][r] = __half22float2(*reinterpret_cast<const __half2*>(&u.y));
     }
   }
 }
-
 template <class SP, int W, int NC, int T>
 __device__ __forceinline__ void col_task(const PassArgs& a, int is, int ws, int bx, float2* sm) {
   constexpr int H = SP::N, Wh = W / 2;
@@ -521,8 +521,7 @@ __device__ __forceinline__ void col_task(const PassArgs& a, int is, int ws, int 
         for (int r = 0; r < FL::R; ++r) {
           const int i = j + r * FL::NS;
           const int im = i == 0 ? 0 : H - i;
-          v[it][0][r] = packed_col0_product(v[it][0][r], sm[im], load_spec(fp.spec, fp.dtype, (size_t)i * Wh),
-                                            load_spec(fp.spec, fp.dtype, (size_t)im * Wh));
+          v[it][0][r] = packed_col0_product(v[it][0][r], sm[im], load_fp(fp, i, 0, H, Wh), load_fp(fp, im, 0, H, Wh));
         }
       }
     }
@@ -533,7 +532,7 @@ __device__ __forceinline__ void col_task(const PassArgs& a, int is, int ws, int 
     const int j = j0 + it * TJ;
     if (FL::NB % TJ != 0 && j >= FL::NB) continue;
     float2 sf[2][FL::R];
-    load_fp_pair<FL::R, FL::NS, Wh>(fp, j, col0, sf);
+    load_fp_pair<FL::R, FL::NS, H>(fp, j, col0, sf);
 #pragma unroll
     for (int r = 0; r < FL::R; ++r) {
       if (col0 != 0) v[it][0][r] = c_conj_mul(v[it][0][r], sf[0][r]);

@@ -15,9 +15,6 @@ __host__ __device__ constexpr int tma_box_rows(int H, int NC, int esize = 8) {
   return 0;
 }
 
-// the descriptor of strips of NC columns among a fingerprint's four
-__host__ __device__ constexpr int fp_tmap_index(int NC) { return NC == 2 ? 0 : NC == 4 ? 1 : NC == 8 ? 2 : 3; }
-
 // one instantiated column-pass variant: columns per block, threads, shared
 // memory; with tma the kernel moves its strip by TMA tile copies of br rows
 // and takes a CUtensorMap of the workspace spectra as a second argument,
@@ -74,9 +71,10 @@ struct FixedShape {
   std::vector<FixedRow> rows;
   std::vector<FixedCol> cols;
   int default_col;           // the column variant of the default tuning
+  int f32_col;               // the one that takes a mode-4 variant's place for FP32 fingerprints
   FixedCol col_fwd, col_inv; // the column pass split for forward units (k_col_fwd_fx, k_col_inv_fx)
-  FixedCol col_inv_sep;      // k_col_inv_fx with the fingerprint strip in its own region (mode 3/4), taken
-                             // with a column variant of that mode; fn null where none is instantiated
+  FixedCol col_inv_sep;      // k_col_inv_fx with the fingerprint's strips in their own region (mode 3/4), taken
+                             // instead where its mode holds the wave's fingerprints; fn null where none is instantiated
   FixedCol col_inv_h;        // the same with a region for FP16 bins (mode 4) and more blocks per SM, taken
                              // instead when every fingerprint of the wave is FP16; fn null where none
   FixedPersist persist;
@@ -109,12 +107,5 @@ void launch_persistent(const PassArgs& a, const PersistArgs& p, const FixedShape
                        LaunchCounter& lc);
 
 constexpr int kPersistSlots = 8;
-
-// TMA descriptors (CUtensorMap, 128 bytes each) of a fingerprint spectrum
-// [H][W/2] (float2 for kF32, __half2 for kF16) for column strips of 2, 4, 8
-// and 16 columns, written to host memory `out` (4 descriptors).  False when
-// the frame size has no compile-time-planned kernels or the driver lacks TMA.
-bool encode_fp_tmaps(const void* spec, int dtype, int H, int W, void* out);
-constexpr size_t kFpTmapBytes = 4 * 128;
 
 }  // namespace prnu

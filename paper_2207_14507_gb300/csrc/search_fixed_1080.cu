@@ -11,16 +11,19 @@ FixedShape fixed_shape_1080() {
   // the row inverse takes 2.46 unbounded (50 registers, 10 blocks), 2.33 for 7,
   // the row forward 4.43 unbounded, 4.17 for 7, 4.30 for 9.
   using D = ShapeDef<Spec<1920, 16, 15, 8>, 128, ColPlan<1080, 36, 30>, Spec<1080, 9, 12, 10>>;
-  // us per candidate of the column variants (FP32 / FP16 fingerprints, waves of
-  // 512): 4-column strips, mode 4 with 4 blocks per SM - / 3.83, mode 3 with 3
-  // blocks 4.25 / 4.33, mode 2 4.70 / 4.83, mode 1 4.61 / 4.73, mode 0 5.50,
-  // 8-column strips 7.40 (mode 1), 6.7 (mode 3), 4.04 (mode 4, 2 blocks).  The
-  // three-stage plan: 5.38 / 5.30.
-  return D::make({D::row<2>(), D::row<1, 8, 8>()},
-                 {D::col<4, 4, 4>(), D::col<4, 3, 2>(), D::col<4, 3, 1>(), D::col<4, 3, 0>(), D::col<8, 1, 1>(),
-                  D::col<4, 3, 3>()},
-                 {D::col_fwd<4, 4>(), D::col_inv<4, 3>(), D::col_inv<4, 3, 3>(), D::col_inv<4, 4, 4>()},
-                 D::persist<192, 2, 4, Spec<1920, 16, 12, 10>>());
+  // us per candidate of the column variants (FP32 / FP16 fingerprints): 4-column
+  // strips, mode 4 with 4 blocks per SM - / 3.40; mode 1 with 4 blocks 3.72 /
+  // 3.58 (3 blocks 4.02 / 4.00); mode 2 with 4 blocks 3.75 / 3.74 (3 blocks 3.89 /
+  // 3.93); mode 3 with 3 blocks 3.82 / 3.89; mode 0 4.79; 8-column strips 7.2 (mode
+  // 1, 1 block), 3.72 (mode 4, 2 blocks, FP16).  Three stages with the fingerprint
+  // by 32-byte TMA rows: 5.38 / 5.30.
+  FixedShape s = D::make({D::row<2>(), D::row<1, 8, 8>()},
+                         {D::col<4, 4, 4>(), D::col<4, 4, 2>(), D::col<4, 4, 1>(), D::col<4, 3, 0>(), D::col<8, 1, 1>(),
+                          D::col<4, 3, 3>()},
+                         {D::col_fwd<4, 4>(), D::col_inv<4, 3>(), D::col_inv<4, 3, 3>(), D::col_inv<4, 4, 4>()},
+                         D::persist<192, 2, 4, Spec<1920, 16, 12, 10>>());
+  s.f32_col = 2;
+  return s;
 }
 
 }  // namespace prnu

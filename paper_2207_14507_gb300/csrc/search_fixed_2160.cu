@@ -10,12 +10,15 @@ FixedShape fixed_shape_2160() {
   // blocks 12.5; 16 x 16 x 15: 11.2), row forward FP16 17.4 (3 blocks 17.9, 6 blocks
   // 20.9; 16 x 16 x 15: 19.8).
   using D = ShapeDef<Spec<3840, 16, 15, 16>, 256, ColPlan<2160, 48, 45>, Spec<2160, 15, 12, 12>>;
-  // us per candidate (FP32 / FP16 fingerprints), 2 blocks per SM: mode 4 - / 18.8,
-  // with the L2 prefetch 18.0; mode 2 20.7 / 20.5; mode 1 25.2 / 25.0; mode 0 26
-  // (8-column strips, 1 block: 24 to 28).  The three-stage plan: 21.9 (FP16).
-  return D::make({D::row<2>(), D::row<1, 4, 4>()},
-                 {D::col<4, 2, 4, 152>(), D::col<4, 2, 2, 152>(), D::col<4, 2, 1>(), D::col<4, 2, 0>()},
-                 {D::col_fwd<4, 2>(), D::col_inv<4, 2>(), D::col_inv<4, 2, 4>()}, D::persist<256, 2, 4>());
+  // us per candidate (FP32 / FP16 fingerprints), 2 blocks per SM: mode 2 with the L2
+  // prefetch 17.0 / 16.7 (without 19.4 / 18.1), mode 4 with it - / 17.0 (without
+  // 18.4); mode 1 20.0 / 18.9; mode 0 22 / 21.  Three stages with the fingerprint by
+  // 32-byte TMA rows: 21.9 (FP16).
+  FixedShape s = D::make({D::row<2>(), D::row<1, 4, 4>()},
+                         {D::col<4, 2, 4, 152>(), D::col<4, 2, 2, 152>(), D::col<4, 2, 1>(), D::col<4, 2, 0>()},
+                         {D::col_fwd<4, 2>(), D::col_inv<4, 2>(), D::col_inv<4, 2, 4>()}, D::persist<256, 2, 4>());
+  s.f32_col = s.default_col = 1;
+  return s;
 }
 
 }  // namespace prnu

@@ -9,14 +9,17 @@ FixedShape fixed_shape_720() {
   // idle in the warp's gathers).  Registers for 5 blocks per SM: row inverse 1.10
   // us a candidate (unbounded 1.12, 4 blocks 1.15, 7 blocks 1.30; 160 threads 1.33).
   using D = ShapeDef<Spec<1280, 16, 10, 8>, 80, ColPlan<720, 30, 24>, Spec<720, 9, 10, 8>>;
-  // us per candidate (FP32 / FP16 fingerprints): 8-column strips, mode 4 with 3
-  // blocks per SM - / 1.56, mode 3 with 2 blocks 1.79 / 1.80, mode 2 2.27, mode 1
-  // 2.12 / 1.99; 4-column strips, mode 3 1.77 / 1.82, mode 4 1.66 to 1.69, mode 2 2.18.
-  return D::make({D::row<2, 5, 5>(), D::row<4>()},
-                 {D::col<8, 3, 4>(), D::col<8, 2, 1>(), D::col<8, 2, 2>(), D::col<8, 2, 0>(), D::col<4, 4, 2>(),
-                  D::col<4, 4, 3>()},
-                 {D::col_fwd<8, 3>(), D::col_inv<8, 2>(), D::col_inv<8, 2, 3>(), D::col_inv<8, 3, 4>()},
-                 D::persist<160, 2, 4>());
+  // us per candidate (FP32 / FP16 fingerprints): 4-column strips, mode 4 with 6
+  // blocks per SM - / 1.33 (5 blocks 1.36), mode 2 with 5 blocks 1.45 / 1.42 (4
+  // blocks 1.66 / 1.59), mode 3 with 4 blocks 1.49; 8-column strips, mode 4 with 3
+  // blocks - / 1.46, mode 2 1.53, mode 3 1.77, mode 1 1.89.
+  FixedShape s = D::make({D::row<2, 5, 5>(), D::row<4>()},
+                         {D::col<4, 6, 4>(), D::col<8, 2, 1>(), D::col<4, 5, 2>(), D::col<8, 2, 0>(), D::col<8, 3, 2>(),
+                          D::col<4, 4, 3>()},
+                         {D::col_fwd<4, 6>(), D::col_inv<4, 4>(), D::col_inv<4, 4, 3>(), D::col_inv<4, 6, 4>()},
+                         D::persist<160, 2, 4>());
+  s.f32_col = 2;
+  return s;
 }
 
 }  // namespace prnu
