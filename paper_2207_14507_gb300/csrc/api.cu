@@ -101,6 +101,12 @@ FftPlan make_plan_at(int n, int tw_base) {
   if (col2_radices(n, &p.ra, &p.rb)) {
     p.tw_fwd = off;
     p.tw_inv = off + stage_tw_len(p.rb, p.ra);
+    off = p.tw_inv + stage_tw_len(p.ra, p.rb);
+  }
+  if ((p.ra == 0 || p.ra > 32) && row3_radices(n, p.r3)) {
+    p.w3[0] = off;
+    p.w3[1] = off + stage_tw_len(p.r3[1], p.r3[0]);
+    p.inv3 = (unsigned)(((1ull << 32) + p.r3[0] - 1) / p.r3[0]);
   }
   return p;
 }
@@ -131,6 +137,10 @@ static void append_plan_twiddles(const FftPlan& p, std::vector<float4>& tab) {
   if (p.ra) {
     stage(p.rb, p.ra);
     stage(p.ra, p.rb);
+  }
+  if (p.r3[0]) {
+    stage(p.r3[1], p.r3[0]);
+    stage(p.r3[2], p.r3[0] * p.r3[1]);
   }
 }
 

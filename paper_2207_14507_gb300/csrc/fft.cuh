@@ -230,7 +230,10 @@ constexpr int kMaxFft = 4096;
 // for j < 2^16) and the place of its twiddles in the table (fft_plan.cuh), in
 // float4.  ra, rb: where n is the product of two radices that one thread can
 // hold, the two-stage plan of the column pass (col_generic.cuh), with the
-// twiddles of its second forward and second inverse stage; else 0.
+// twiddles of its second forward and second inverse stage; else 0.  r3: where
+// one thread cannot hold radices of such a plan in few registers, the row
+// passes' three radices (row_generic.cuh), w3 the twiddles of the second and
+// third stage, inv3 the reciprocal of r3[0]; else 0.
 struct FftPlan {
   int n;
   int nstages;
@@ -240,6 +243,8 @@ struct FftPlan {
   int tw[kMaxStages];
   int min_radix;
   int ra, rb, tw_fwd, tw_inv;
+  int r3[3], w3[2];
+  unsigned inv3;
 };
 
 // float4 entries of a stage's twiddles

@@ -42,6 +42,8 @@ FftPlan make_plan_at(int n, int tw_base);
 FftPlan make_plan(int n, const std::vector<int>& tw_offsets);
 // the two-stage plan of length n (col_generic.cuh, row_generic.cuh), false if it has none
 bool col2_radices(int n, int* ra, int* rb);
+// the three-stage row plan of length n (row_generic.cuh), false if it has none
+bool row3_radices(int n, int r[3]);
 void allow_col2();
 bool is_5smooth(int n);
 // threads per row FFT and registers-per-thread class (1, 2 or 4 butterflies)
@@ -97,11 +99,7 @@ void launch_row_forward(const PassArgs& a, bool warp, const float* mean_sub, flo
 // mode 4: inverse only, in place (float2)                               [naive path]
 void launch_col(const PassArgs& a, int mode, float2* out_f32, void* out_f16, const float* scale,
                 cudaStream_t s, LaunchCounter& lc, int out_strips = 0);
-// widths with a two-stage plan (a.prow.ra; row_generic.cuh)
-void launch_row_forward2(const PassArgs& a, bool warp, const float* mean_sub, float2* out, cudaStream_t s,
-                         LaunchCounter& lc);
-void launch_row_inverse2(const PassArgs& a, float* c_out, cudaStream_t s, LaunchCounter& lc);
-void allow_row2();
+void allow_rows();
 // mode 0 of a height with a two-stage plan (a.pcol.ra)
 void launch_col2(const PassArgs& a, cudaStream_t s, LaunchCounter& lc);
 void launch_row_inverse(const PassArgs& a, float* c_out, cudaStream_t s, LaunchCounter& lc);

@@ -41,7 +41,8 @@ constexpr size_t kOffSpecX = 0;
 constexpr size_t kOffSpecK = kOffSpecX + kSpecBytes;
 constexpr size_t kOffStats = kOffSpecK + kSpecBytes;
 constexpr size_t kOffTw = kOffStats + (size_t)kMaxSide * sizeof(RowStat);
-constexpr size_t kOffItem = kOffTw + 2 * (size_t)kMaxSide * sizeof(float4);   // a plan takes fewer entries than 4096
+constexpr int kTwLen = 2 * kMaxSide;   // float4 entries, more than any plan takes
+constexpr size_t kOffItem = kOffTw + 2 * (size_t)kTwLen * sizeof(float4);
 constexpr size_t kOffFp = kOffItem + 256;
 constexpr size_t kOffResult = kOffFp + 256;
 constexpr size_t kOffScal = kOffResult + 256;
@@ -70,6 +71,10 @@ __global__ void k_noalloc_twiddles(FftPlan p, float4* __restrict__ tw) {
   if (p.ra) {
     stage(p.rb, p.ra, p.tw_fwd);
     stage(p.ra, p.rb, p.tw_inv);
+  }
+  if (p.r3[0]) {
+    stage(p.r3[1], p.r3[0], p.w3[0]);
+    stage(p.r3[2], p.r3[0] * p.r3[1], p.w3[1]);
   }
 }
 
@@ -138,9 +143,9 @@ extern "C" int pce_score_noalloc(const float* d_X, const float* d_K, int H, int 
     float* scal = reinterpret_cast<float*>(base + kOffScal);   // mean, scale, inv_scale
     double* partials = reinterpret_cast<double*>(base + kOffPartials);
 
-    // twiddle tables: length W at tw[0], length H at tw[kMaxSide] (the
+    // twiddle tables: length W at tw[0], length H at tw[kTwLen] (the
     // offsets are set here, not looked up, so H == W needs no special case)
-    const FftPlan prow = make_plan_at(W, 0), pcol = make_plan_at(H, kMaxSide);
+    const FftPlan prow = make_plan_at(W, 0), pcol = make_plan_at(H, kTwLen);
     k_noalloc_twiddles<<<8, 256, 0, s>>>(prow, tw);
     PRNU_CUDA_TRY(cudaGetLastError());
     k_noalloc_twiddles<<<8, 256, 0, s>>>(pcol, tw);

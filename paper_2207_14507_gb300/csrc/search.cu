@@ -2,13 +2,13 @@
 //
 // Per candidate (frame f, fingerprint p, grid node (lambda, theta)) the fused
 // path runs four kernels over a wave of candidates:
-//   k_row_forward : inverse warp of the residual (Eq. 4, bilinear, zero
+//   k_row_forward{2,3} (row_generic.cuh): inverse warp of the residual (Eq. 4, bilinear, zero
 //                   outside) fused with the row FFT; two real rows share one
 //                   complex FFT; output is the packed half spectrum
 //                   [H][W/2] complex whose column 0 holds (DC, Nyquist) pairs;
 //   k_col         : column FFT, product conj(X^) K0^ with the cached
 //                   fingerprint spectrum, inverse column FFT, in place;
-//   k_row_inverse : inverse row FFT (two rows per complex FFT) and per-row
+//   k_row_inverse{2,3}: inverse row FFT (two rows per complex FFT) and per-row
 //                   max / first arg-max / sum of squares of C;
 //   k_finalize    : peak over rows, energy outside the cyclic 11x11 window
 //                   (the window's rows are recomputed from the spectrum) and
@@ -26,70 +26,6 @@
 namespace prnu {
 
 // ---------------------------------------------------------------- kernels
-
-// Warp (optional) + row FFT of two rows per thread group; writes the packed
-// half spectrum of both rows.  grid = (ceil((H/2)/ppb), wave), block = ppb*T.
-// Without WARP the input is the single image at a.resid (minus *mean_sub).
-// 64 registers (two blocks of 512): unbounded the kernel takes 68 and loses a
-// third at 1440 x 2560 (21.0 against 14.5 us a candidate)
-template <int DT, bool WARP>
-__global__ void __launch_bounds__(512, 2) k_row_forward(PassArgs a, const float* __restrict__ mean_sub,
-                                                      float2* __restrict__ out_override) {
-  extern __shared__ float2 smem[];
-  const int T = a.row_threads;
-  const int grp = threadIdx.x / T, t = threadIdx.x - grp * T;
-  const int H = a.H, W = a.W, Wh = W >> 1;
-  const int pair = blockIdx.x * a.pairs_per_block + grp;
-  const bool active = pair < (H >> 1);
-  const int slot = blockIdx.y;
-  float2* buf = smem + (size_t)grp * 2 * row_smem_len(W);
-  float2* buf2 = buf + row_smem_len(W);
-  const int y0 = 2 * pair, y1 = y0 + 1;
-  if (active) {
-    if constexpr (WARP) {
-      const WorkItem it = item_of(a, slot);
-      size_t base;
-      const void* Rf = frame_of(a, it.frame, &base);
-      const float cx = 0.5f * (float)(W - 1), cy = 0.5f * (float)(H - 1);
-      const float dy0 = (float)y0 - cy, dy1 = (float)y1 - cy;
-      const float bx0 = fmaf(it.a12, dy0, cx), by0 = fmaf(it.a22, dy0, cy);
-      const float bx1 = fmaf(it.a12, dy1, cx), by1 = fmaf(it.a22, dy1, cy);
-      for (int x = t; x < W; x += T) {
-        const float dx = (float)x - cx;
-        const float v0 = bilinear<DT>(Rf, base, H, W, a.rpitch, fmaf(it.a11, dx, bx0), fmaf(it.a21, dx, by0));
-        const float v1 = bilinear<DT>(Rf, base, H, W, a.rpitch, fmaf(it.a11, dx, bx1), fmaf(it.a21, dx, by1));
-        buf[rpad(x)] = make_float2(v0, v1);
-      }
-    } else {
-      const float m = mean_sub ? *mean_sub : 0.f;
-      for (int x = t; x < W; x += T) {
-        const float v0 = load_store_type<DT>(a.resid, (size_t)y0 * W + x) - m;
-        const float v1 = load_store_type<DT>(a.resid, (size_t)y1 * W + x) - m;
-        buf[rpad(x)] = make_float2(v0, v1);
-      }
-    }
-  }
-  __syncthreads();
-  buf = fft_row<false>(buf, buf2, a.prow, a.tw, active ? t : (1 << 28), T);
-  if (active) {
-    float2* o0 = (out_override ? out_override : a.spec + (size_t)slot * H * Wh) + (size_t)y0 * Wh;
-    float2* o1 = o0 + Wh;
-    for (int k = t; k < Wh; k += T) {
-      float2 A, B;
-      if (k == 0) {
-        const float2 z0 = buf[rpad(0)], zn = buf[rpad(Wh)];
-        A = make_float2(z0.x, zn.x);
-        B = make_float2(z0.y, zn.y);
-      } else {
-        const float2 zk = buf[rpad(k)], zm = buf[rpad(W - k)];
-        A = make_float2(0.5f * (zk.x + zm.x), 0.5f * (zk.y - zm.y));
-        B = make_float2(0.5f * (zk.y + zm.y), 0.5f * (zm.x - zk.x));
-      }
-      o0[k] = A;
-      o1[k] = B;
-    }
-  }
-}
 
 // Column pass over a strip of 1 << col_log2 columns of one candidate's packed
 // spectrum.  grid = (ceil((W/2) >> lg), wave), block = T.
@@ -162,55 +98,6 @@ __global__ void __launch_bounds__(512, 2) k_col(PassArgs a, int mode, float2* __
     const int i = e >> lg, col = c0 + (e & (NC - 1));
     if (col < Wh) Z[(size_t)i * Wh + col] = buf[e];
   }
-}
-
-// Inverse row FFT of two rows per group; per-row max / first arg-max / sum of
-// squares into a.stats, or (c_out != nullptr) the rows of C themselves.
-__global__ void __launch_bounds__(512, 2) k_row_inverse(PassArgs a, float* __restrict__ c_out) {
-  extern __shared__ float2 smem[];
-  const int T = a.row_threads;
-  const int grp = threadIdx.x / T, t = threadIdx.x - grp * T;
-  const int H = a.H, W = a.W, Wh = W >> 1;
-  const int ppb = a.pairs_per_block;
-  const int pair = blockIdx.x * ppb + grp;
-  const bool active = pair < (H >> 1);
-  const int slot = blockIdx.y;
-  float2* buf = smem + (size_t)grp * 2 * row_smem_len(W);
-  float2* buf2 = buf + row_smem_len(W);
-  WarpRed* red = reinterpret_cast<WarpRed*>(smem + (size_t)ppb * 2 * row_smem_len(W)) + grp * 32;
-  const float2* Z = a.spec + (size_t)slot * H * Wh;
-  if (active) build_full_row(buf, Z + (size_t)(2 * pair) * Wh, Z + (size_t)(2 * pair + 1) * Wh, W, t, T);
-  __syncthreads();
-  const int tl = active ? t : (1 << 28);
-  if (c_out) {
-    buf = fft_row<true>(buf, buf2, a.prow, a.tw, tl, T);
-    if (active) {
-      float* ra = c_out + (size_t)(2 * pair) * W;
-      for (int x = t; x < W; x += T) {
-        const float2 v = buf[rpad(x)];
-        ra[x] = v.x;
-        ra[W + x] = v.y;
-      }
-    }
-    return;
-  }
-  // the last stage's outputs go to the statistics from registers
-  float ma = -INFINITY, mb = -INFINITY;
-  int ia = INT_MAX, ib = INT_MAX;
-  float2 sq = make_float2(0.f, 0.f);
-  const int last = a.prow.nstages - 1;
-  buf = fft_row<true>(buf, buf2, a.prow, a.tw, tl, T, last);
-  plan_stage_any<true>(
-      a.prow, last, a.tw, tl, T, [=](int i) { return buf[rpad(i)]; },
-      [&](int x, float2 v) {
-        better_f(ma, ia, v.x, x);
-        better_f(mb, ib, v.y, x);
-        sq = __ffma2_rn(v, v, sq);
-      });
-  const float sa = sq.x, sb = sq.y;
-  row_stats_warp(ma, ia, mb, ib, sa, sb, t, reinterpret_cast<RowRed*>(red));
-  __syncthreads();
-  if (active && t == 0) row_stats_final(reinterpret_cast<const RowRed*>(red), T >> 5, a.stats + (size_t)slot * H + 2 * pair);
 }
 
 // Finalisation (search_common.cuh): window pairs b0 .. b1-1 and the row shares of
@@ -437,32 +324,6 @@ __global__ void k_naive_final(const float* __restrict__ C, int H, int W, const W
     if (e_ != cudaSuccess) throw Error{PRNU_ECUDA, std::string(__func__) + ": " + cudaGetErrorString(e_)}; \
   } while (0)
 
-void launch_row_forward(const PassArgs& a, bool warp, const float* mean_sub, float2* out, cudaStream_t s,
-                        LaunchCounter& lc) {
-  if (a.prow.ra) {
-    launch_row_forward2(a, warp, mean_sub, out, s, lc);
-    return;
-  }
-  int T, maxb;
-  row_launch_shape(a.prow, &T, &maxb);
-  PRNU_CHECK_ARG(T == a.row_threads, "row thread count mismatch");
-  const int ppb = a.pairs_per_block;
-  dim3 g((a.H / 2 + ppb - 1) / ppb, a.nitems), b(ppb * T);
-  const size_t sm = row_smem_bytes(a.W, ppb);
-  ProfScope ps(lc, kKindRowForward, s);
-  if (warp) {
-    if (a.rdtype == kF32) k_row_forward<kF32, true><<<g, b, sm, s>>>(a, mean_sub, out);
-    else if (a.rdtype == kF16) k_row_forward<kF16, true><<<g, b, sm, s>>>(a, mean_sub, out);
-    else k_row_forward<kBF16, true><<<g, b, sm, s>>>(a, mean_sub, out);
-  } else {
-    if (a.rdtype == kF32) k_row_forward<kF32, false><<<g, b, sm, s>>>(a, mean_sub, out);
-    else if (a.rdtype == kF16) k_row_forward<kF16, false><<<g, b, sm, s>>>(a, mean_sub, out);
-    else k_row_forward<kBF16, false><<<g, b, sm, s>>>(a, mean_sub, out);
-  }
-  PRNU_LAUNCH_CHECK();
-  lc.n++;
-}
-
 void launch_col(const PassArgs& a, int mode, float2* out_f32, void* out_f16, const float* scale, cudaStream_t s,
                 LaunchCounter& lc, int out_strips) {
   if (mode == 0 && a.pcol.ra) {
@@ -478,22 +339,6 @@ void launch_col(const PassArgs& a, int mode, float2* out_f32, void* out_f16, con
   __half2* o16 = reinterpret_cast<__half2*>(out_f16);
   ProfScope ps(lc, kKindColumn, s);
   k_col<<<g, b, sm, s>>>(a, mode, out_f32, o16, scale, out_strips);
-  PRNU_LAUNCH_CHECK();
-  lc.n++;
-}
-
-void launch_row_inverse(const PassArgs& a, float* c_out, cudaStream_t s, LaunchCounter& lc) {
-  if (a.prow.ra) {
-    launch_row_inverse2(a, c_out, s, lc);
-    return;
-  }
-  int T, maxb;
-  row_launch_shape(a.prow, &T, &maxb);
-  const int ppb = a.pairs_per_block;
-  dim3 g((a.H / 2 + ppb - 1) / ppb, a.nitems), b(ppb * T);
-  const size_t sm = row_smem_bytes(a.W, ppb);
-  ProfScope ps(lc, kKindRowInverse, s);
-  k_row_inverse<<<g, b, sm, s>>>(a, c_out);
   PRNU_LAUNCH_CHECK();
   lc.n++;
 }
@@ -601,18 +446,11 @@ static void allow_smem(K k) {
 }
 
 void set_kernel_attributes() {
-  allow_smem(k_row_forward<kF32, true>);
-  allow_smem(k_row_forward<kF16, true>);
-  allow_smem(k_row_forward<kBF16, true>);
-  allow_smem(k_row_forward<kF32, false>);
-  allow_smem(k_row_forward<kF16, false>);
-  allow_smem(k_row_forward<kBF16, false>);
   allow_smem(k_col);
-  allow_smem(k_row_inverse);
   allow_smem(k_finalize);
   allow_smem(k_finalize_part);
   allow_col2();
-  allow_row2();
+  allow_rows();
   cudaGetLastError();
 }
 
