@@ -47,6 +47,21 @@ constexpr int kPairs = kIn / 2;
 constexpr int kBand = kTS + 3;       // coefficients of the synthesis
 constexpr int kLevels = 4;
 
+// a byte as a float: in the low mantissa bits of 2^23, minus 2^23
+__device__ __forceinline__ float byte_float(uint32_t v) { return __uint_as_float(0x4B000000u | v) - 8388608.f; }
+
+// elements i, i + 1 of out, i even and out aligned to the pair
+template <int DT>
+__device__ __forceinline__ void store_pair(void* out, size_t i, float a, float b) {
+  if constexpr (DT == kF32) *reinterpret_cast<float2*>(reinterpret_cast<float*>(out) + i) = make_float2(a, b);
+  else if constexpr (DT == kF16) *reinterpret_cast<__half2*>(reinterpret_cast<__half*>(out) + i) = __floats2half2_rn(a, b);
+  else *reinterpret_cast<__nv_bfloat162*>(reinterpret_cast<__nv_bfloat16*>(out) + i) = __floats2bfloat162_rn(a, b);
+}
+__device__ __forceinline__ void copy4_async(float* dst, const float* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(__cvta_generic_to_global(src))
+               : "memory");
+}
+
 // index i >= 0 of an axis of n samples, periodic
 __device__ __forceinline__ int wrap_up(int i, int n) { return i < n ? i : i % n; }
 // index i >= -3, periodic
@@ -57,8 +72,11 @@ __device__ __forceinline__ int mirror(int i, int n) { return i < n ? i : 2 * n -
 // One level of the analysis: the h x w image (LEVEL0: the uint8 frame, mirrored
 // to that size; else X, dense, of frame stride fstride) to its three detail
 // bands in A (quadrant layout, pitch Wp) and, unless LL is null, its low-low
-// band (dense h/2 x w/2).  8 full-HD frames, all levels: 84 us, where a
-// kernel per axis with 8 global loads an output took 255.
+// band (dense h/2 x w/2).  A thread loads pairs of columns of pairs of rows, from
+// one moving address where the tile holds no edge.  8 full-HD frames, all levels:
+// 70 us (single samples, each with its edge tests: 84; a kernel per axis with 8
+// global loads an output: 255); the first level, 38 of them, issues in 60% of
+// cycles and uses 48% of the L1 pipe.
 template <bool LEVEL0>
 __global__ void __launch_bounds__(256) k_wav_analyse(const uint8_t* __restrict__ frames, size_t pitch, int H, int W,
                                                      const float* __restrict__ X, size_t fstride, int h, int w, int Wp,
@@ -68,18 +86,51 @@ __global__ void __launch_bounds__(256) k_wav_analyse(const uint8_t* __restrict__
   const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
   const int n0 = blockIdx.x * kTS, m0 = blockIdx.y * kTS, f = blockIdx.z;
   const int w2 = w / 2, h2 = h / 2;
-  auto sample = [&](int y, int x) -> float {
-    if (LEVEL0) return (float)__ldg(frames + ((size_t)f * H + mirror(y, H)) * pitch + mirror(x, W));
-    return __ldg(X + (size_t)f * fstride + (size_t)y * w + x);
+  // row pair p, column pair c; LEVEL0 frames by byte pairs where these are aligned
+  // and not mirrored
+  const bool even = LEVEL0 && ((reinterpret_cast<uintptr_t>(frames) | pitch) & 1) == 0;
+  auto pair = [&](int y, int x) -> float2 {
+    if (!LEVEL0) return __ldg(reinterpret_cast<const float2*>(X + (size_t)f * fstride + (size_t)y * w + x));
+    const uint8_t* row = frames + ((size_t)f * H + mirror(y, H)) * pitch;
+    if (even && x + 1 < W) {
+      const unsigned v = __ldg(reinterpret_cast<const uint16_t*>(row + x));
+      return make_float2(byte_float(v & 255u), byte_float(v >> 8));
+    }
+    return make_float2(byte_float(__ldg(row + mirror(x, W))), byte_float(__ldg(row + mirror(x + 1, W))));
   };
-  for (int p = wp; p < kPairs; p += 8) {
-    const int ya = wrap_up(2 * (m0 + p), h), yb = wrap_up(2 * (m0 + p) + 1, h);
+  // no edge of the image inside the tile: one address, moved by constant steps
+  const bool inner = 2 * m0 + kIn <= (LEVEL0 ? min(h, H) : h) && 2 * n0 + kIn <= (LEVEL0 ? min(w, W) : w) && (even || !LEVEL0);
+  int p = threadIdx.x / kPairs, c = threadIdx.x - p * kPairs;
+  const size_t pt = LEVEL0 ? pitch : (size_t)w;
+  size_t at = (size_t)(2 * (m0 + p)) * pt + 2 * (n0 + c) + (LEVEL0 ? (size_t)f * H * pitch : (size_t)f * fstride);
 #pragma unroll
-    for (int q = 0; q < 3; ++q) {
-      const int i = lane + 32 * q;
-      if (i >= kIn) break;
-      const int x = wrap_up(2 * n0 + i, w);
-      in[p * (kIn + 2) + i] = make_float2(sample(ya, x), sample(yb, x));
+  for (int e = 0; e < (kPairs * kPairs + 255) / 256; ++e) {
+    if (p < kPairs) {
+      float2 a, b;
+      if (inner) {
+        if (LEVEL0) {
+          const unsigned va = __ldg(reinterpret_cast<const uint16_t*>(frames + at));
+          const unsigned vb = __ldg(reinterpret_cast<const uint16_t*>(frames + at + pt));
+          a = make_float2(byte_float(va & 255u), byte_float(va >> 8));
+          b = make_float2(byte_float(vb & 255u), byte_float(vb >> 8));
+        } else {
+          a = __ldg(reinterpret_cast<const float2*>(X + at));
+          b = __ldg(reinterpret_cast<const float2*>(X + at + pt));
+        }
+      } else {
+        const int x = wrap_up(2 * (n0 + c), w);   // w is even: a pair does not wrap inside
+        a = pair(wrap_up(2 * (m0 + p), h), x);
+        b = pair(wrap_up(2 * (m0 + p) + 1, h), x);
+      }
+      *reinterpret_cast<float4*>(in + p * (kIn + 2) + 2 * c) = make_float4(a.x, b.x, a.y, b.y);
+    }
+    c += 256 % kPairs;
+    p += 256 / kPairs;
+    at += 2 * (256 / kPairs) * pt + 2 * (256 % kPairs);
+    if (c >= kPairs) {
+      c -= kPairs;
+      ++p;
+      at += 2 * pt - 2 * kPairs;
     }
   }
   __syncthreads();
@@ -130,17 +181,21 @@ __global__ void __launch_bounds__(256) k_wav_analyse(const uint8_t* __restrict__
 // the 3, 5, 7 and 9 wide windows go along rows first (four sums a pixel, each a
 // pair more than the last), then along columns.  The smallest of max(0, mean -
 // s0) is max(0, smallest mean - s0): subtraction and max are monotone in
-// floating point too.  8 full-HD frames: 121 us; 80 shared loads a
-// coefficient in a kernel per level took 211.
-constexpr int kSX = 32, kSY = 32, kSR = 4;
+// floating point too.  A tile of 56 rows and its borders are 64, two whole
+// turns of the row sums' lanes, and 7 rows of a column in a thread share the sums of
+// two and of four rows that lie in several windows.  8 full-HD frames: 63 us, issue
+// in 73% of cycles (tiles of 32 rows, 4 to a thread, each with its own sums: 121; 80
+// shared loads a coefficient in a kernel per level: 211).
+constexpr int kSX = 32, kSK = 7, kSY = 8 * kSK, kSR = 4;
 // FAST: the quotients c s0 / den have no subnormal or overflowing part
 template <bool FAST>
 __global__ void __launch_bounds__(256) k_wav_shrink(const float* __restrict__ A, int Hp, int Wp, size_t fstride, float s0sq,
                                                     float* __restrict__ T) {
-  // row pitches that put 8 lanes of consecutive rows in distinct 16-byte banks
+  // row pitches that put lanes of consecutive rows in distinct banks
   constexpr int SW = kSX + 2 * kSR + 4, SH = kSY + 2 * kSR, HW = kSX + 1;
+  static_assert(SH == 64, "two rows a lane of the row sums");
   __shared__ __align__(16) float sq[SH * SW];
-  __shared__ __align__(16) float4 hs[SH * HW];
+  __shared__ float2 ha[SH * HW], hb[SH * HW];   // (3, 5) and (7, 9) wide sums along rows
   const int f = blockIdx.z / 3, b = blockIdx.z - 3 * f;
   int h2 = Hp / 2, w2 = Wp / 2, tile = blockIdx.x, tx = (w2 + kSX - 1) / kSX, n = tx * ((h2 + kSY - 1) / kSY);
   while (tile >= n) {   // the level of this tile
@@ -154,21 +209,28 @@ __global__ void __launch_bounds__(256) k_wav_shrink(const float* __restrict__ A,
   const int oy = b == 0 ? 0 : h2, ox = b == 1 ? 0 : w2;
   const float* band = A + (size_t)f * fstride + (size_t)oy * Wp + ox;
   const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
-  for (int sy = wp; sy < SH; sy += 8) {
-    const int y = by0 + sy - kSR;
-    const float* row = band + (size_t)y * Wp;
+  {
+    constexpr int C = kSX + 2 * kSR;
+    static_assert(SH * C % 256 == 0, "whole steps of the block");
+    int sy = threadIdx.x / C, sx = threadIdx.x - sy * C;
 #pragma unroll
-    for (int q = 0; q < 2; ++q) {
-      const int sx = lane + 32 * q, x = bx0 + sx - kSR;
-      if (sx >= kSX + 2 * kSR) break;
+    for (int e = 0; e < SH * C / 256; ++e) {
+      const int y = by0 + sy - kSR, x = bx0 + sx - kSR;
       float c = 0.f;
-      if ((unsigned)y < (unsigned)h2 && (unsigned)x < (unsigned)w2) c = __ldg(row + x);
+      if ((unsigned)y < (unsigned)h2 && (unsigned)x < (unsigned)w2) c = __ldg(band + (size_t)y * Wp + x);
       sq[sy * SW + sx] = c * c;
+      sx += 256 % C;
+      sy += 256 / C;
+      if (sx >= C) {
+        sx -= C;
+        ++sy;
+      }
     }
   }
   __syncthreads();
-  for (int sy = lane; sy < SH; sy += 32) {   // four adjacent pixels of a row, a lane per row
-    const int x4 = wp * 4;
+#pragma unroll
+  for (int q = 0; q < 2; ++q) {   // four adjacent pixels of a row, a lane per row
+    const int sy = lane + 32 * q, x4 = wp * 4;
     const float4* p = reinterpret_cast<const float4*>(sq + sy * SW + x4);
     const float4 q0 = p[0], q1 = p[1], q2 = p[2];
     const float v[12] = {q0.x, q0.y, q0.z, q0.w, q1.x, q1.y, q1.z, q1.w, q2.x, q2.y, q2.z, q2.w};
@@ -176,39 +238,57 @@ __global__ void __launch_bounds__(256) k_wav_shrink(const float* __restrict__ A,
     for (int i = 0; i < 4; ++i) {
       const float s1 = v[i + 3] + v[i + 4] + v[i + 5], s2 = s1 + (v[i + 2] + v[i + 6]);
       const float s3 = s2 + (v[i + 1] + v[i + 7]);
-      hs[sy * HW + x4 + i] = make_float4(s1, s2, s3, s3 + (v[i] + v[i + 8]));
+      ha[sy * HW + x4 + i] = make_float2(s1, s2);
+      hb[sy * HW + x4 + i] = make_float2(s3, s3 + (v[i] + v[i + 8]));
     }
   }
   __syncthreads();
   const int x = bx0 + lane;
   if (x >= w2) return;
-  // four adjacent rows of a column
-  const int y0 = wp * 4;
-  float2 ra[12], rb[12];   // (3, 5) and (7, 9) wide sums
+  // kSK adjacent rows of a column; sums of two and four rows are shared by the
+  // rows whose windows hold them
+  const int y0 = wp * kSK;
+  float m[kSK];
+  {
+    const float2* src = ha + y0 * HW + lane;   // r[i] of row y0 + i - kSR
+    float2 r[kSK + 2 * kSR], p[kSK + 2 * kSR];
 #pragma unroll
-  for (int i = 0; i < 12; ++i) {
-    const float4 q = hs[(y0 + i) * HW + lane];
-    ra[i] = make_float2(q.x, q.y);
-    rb[i] = make_float2(q.z, q.w);
+    for (int i = 2; i < kSK + 6; ++i) r[i] = src[i * HW];
+#pragma unroll
+    for (int i = 2; i < kSK + 5; ++i) p[i] = __fadd2_rn(r[i], r[i + 1]);
+#pragma unroll
+    for (int k = 0; k < kSK; ++k) {
+      const int i = k + kSR;
+      m[k] = fminf((p[i - 1].x + r[i + 1].x) * (1.f / 9.f), (p[i - 2].y + p[i + 1].y + r[i].y) * (1.f / 25.f));
+    }
   }
-  float* const To = T + (size_t)f * fstride + (size_t)oy * Wp + ox;
+  {
+    const float2* src = hb + y0 * HW + lane;
+    float2 r[kSK + 2 * kSR], p[kSK + 2 * kSR], q[kSK + 2 * kSR];
 #pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    const int y = by0 + y0 + k, i = k + 4;
-    if (y >= h2) break;
-    const float c = __ldg(band + (size_t)y * Wp + x);
-    float2 ma = __fadd2_rn(ra[i], __fadd2_rn(ra[i - 1], ra[i + 1]));
-    float2 mb = __fadd2_rn(rb[i], __fadd2_rn(rb[i - 1], rb[i + 1]));
-    ma.y += ra[i - 2].y + ra[i + 2].y;
-    mb = __fadd2_rn(mb, __fadd2_rn(rb[i - 2], rb[i + 2]));
-    mb = __fadd2_rn(mb, __fadd2_rn(rb[i - 3], rb[i + 3]));
-    mb.y += rb[i - 4].y + rb[i + 4].y;
-    const float m = fminf(fminf(ma.x * (1.f / 9.f), ma.y * (1.f / 25.f)), fminf(mb.x * (1.f / 49.f), mb.y * (1.f / 81.f)));
-    const float den = fmaxf(m - s0sq, 0.f) + s0sq, num = c * s0sq;
+    for (int i = 0; i < kSK + 8; ++i) r[i] = src[i * HW];
+#pragma unroll
+    for (int i = 0; i < kSK + 7; ++i) p[i] = __fadd2_rn(r[i], r[i + 1]);
+#pragma unroll
+    for (int i = 0; i < kSK + 5; ++i) q[i] = __fadd2_rn(p[i], p[i + 2]);
+#pragma unroll
+    for (int k = 0; k < kSK; ++k) {
+      const int i = k + kSR;
+      const float s7 = q[i - 3].x + (p[i + 1].x + r[i + 3].x), s9 = (q[i - 4].y + q[i].y) + r[i + 4].y;
+      m[k] = fminf(m[k], fminf(s7 * (1.f / 49.f), s9 * (1.f / 81.f)));
+    }
+  }
+  float* To = T + (size_t)f * fstride + (size_t)(oy + by0 + y0) * Wp + ox + x;
+  const float* co = band + (size_t)(by0 + y0) * Wp + x;
+#pragma unroll
+  for (int k = 0; k < kSK; ++k) {
+    if (by0 + y0 + k >= h2) break;
+    const float c = __ldg(co + (size_t)k * Wp);
+    const float den = fmaxf(m[k] - s0sq, 0.f) + s0sq, num = c * s0sq;
     float r;
     if (FAST) r = refined_quotient(num, den);
     else r = den > 0.f ? num / den : 0.f;
-    To[(size_t)y * Wp + x] = r;
+    To[(size_t)k * Wp] = r;
   }
 }
 
@@ -216,8 +296,9 @@ __global__ void __launch_bounds__(256) k_wav_shrink(const float* __restrict__ A,
 // and the low-low image LL (dense h/2 x w/2; null: zero) to the h x w image.
 // OUT 0: dense into Y.  The last level: OUT 1 stores R = I W (or W) in `out`
 // (dense [F][H][W]), OUT 2 the per-block sum of R^2 in partials, OUT 3
-// R * scale[f].  8 full-HD frames, all levels: 104 us, where a kernel per
-// axis and one for the residual took 400.
+// R * scale[f].  8 full-HD frames, all levels: 79 us (loads through registers, a
+// sample at a time: 104; a kernel per axis and one for the residual: 400), 51 of
+// them in the last level, whose 66 MB of output HBM takes in 10.
 template <int DT, int OUT>
 __global__ void __launch_bounds__(256) k_wav_synth(const float* __restrict__ D, const float* __restrict__ LL, size_t fstride,
                                                    int h, int w, int Wp, float* __restrict__ Y,
@@ -231,18 +312,40 @@ __global__ void __launch_bounds__(256) k_wav_synth(const float* __restrict__ D, 
   const int n0 = blockIdx.x * kTS, m0 = blockIdx.y * kTS, fl = blockIdx.z, f = f0 + fl;
   const int w2 = w / 2, h2 = h / 2;
   const size_t fo = (size_t)fl * fstride;
-  for (int r = wp; r < kBand; r += 8) {
-    const int m = wrap_both(m0 + r - 3, h2);
+  {   // asynchronous copies: all of a thread's are in flight together
+    constexpr int C = kTS + 4;
+    const bool inner = m0 >= 3 && n0 >= 3 && m0 + kTS <= h2 && n0 + kTS < w2;   // no edge inside the tile
+    int r = threadIdx.x / C, c = threadIdx.x - r * C;
+    const float* d = D + fo + (size_t)max(m0 + r - 3, 0) * Wp + max(n0 + c - 3, 0);
+    const float* ll = LL + fo + (size_t)max(m0 + r - 3, 0) * w2 + max(n0 + c - 3, 0);
+    const size_t dh = (size_t)h2 * Wp;
 #pragma unroll
-    for (int q = 0; q < 2; ++q) {
-      const int c = lane + 32 * q;
-      if (c >= kTS + 4) break;
-      const int n = wrap_both(n0 + c - 3, w2);
-      B[0][r][c] = LL ? __ldg(LL + fo + (size_t)m * w2 + n) : 0.f;
-      B[1][r][c] = __ldg(D + fo + (size_t)(h2 + m) * Wp + n);
-      B[2][r][c] = __ldg(D + fo + (size_t)m * Wp + w2 + n);
-      B[3][r][c] = __ldg(D + fo + (size_t)(h2 + m) * Wp + w2 + n);
+    for (int e = 0; e < (kBand * C + 255) / 256; ++e) {
+      if (r < kBand) {
+        if (!inner) {
+          const int m = wrap_both(m0 + r - 3, h2), n = wrap_both(n0 + c - 3, w2);
+          d = D + fo + (size_t)m * Wp + n;
+          ll = LL + fo + (size_t)m * w2 + n;
+        }
+        float* b = &B[0][0][0] + threadIdx.x + 256 * e;
+        if (LL) copy4_async(b, ll);
+        else *b = 0.f;
+        copy4_async(b + kBand * C, d + dh);
+        copy4_async(b + 2 * kBand * C, d + w2);
+        copy4_async(b + 3 * kBand * C, d + dh + w2);
+      }
+      c += 256 % C;
+      r += 256 / C;
+      d += 256 / C * Wp + 256 % C;
+      ll += 256 / C * w2 + 256 % C;
+      if (c >= C) {
+        c -= C;
+        ++r;
+        d += Wp - C;
+        ll += w2 - C;
+      }
     }
+    asm volatile("cp.async.wait_all;" ::: "memory");
   }
   __syncthreads();
   // columns: outputs 2i and 2i + 1 take coefficients i - 3 .. i; a thread takes
@@ -276,6 +379,8 @@ __global__ void __launch_bounds__(256) k_wav_synth(const float* __restrict__ D, 
   // rows: a warp takes a pair of rows, a lane outputs 2n and 2n + 1 of both
   const int x = 2 * (n0 + lane);
   const float s = OUT == 3 ? scale[f] : 1.f;
+  const bool even_in = ((reinterpret_cast<uintptr_t>(frames) | pitch) & 1) == 0;
+  const bool even_out = W % 2 == 0 && reinterpret_cast<uintptr_t>(out) % (DT == kF32 ? 8 : 4) == 0;
   float sq[kTS / 8];
 #pragma unroll
   for (int k = 0; k < kTS / 8; ++k) {
@@ -302,15 +407,25 @@ __global__ void __launch_bounds__(256) k_wav_synth(const float* __restrict__ D, 
         const bool two = x + 1 < W;
         if (weight) {
           const uint8_t* I = frames + ((size_t)f * H + y + e) * pitch + x;
-          r.x *= (float)__ldg(I);
-          r.y *= two ? (float)__ldg(I + 1) : 0.f;
+          if (two && even_in) {
+            const unsigned v = __ldg(reinterpret_cast<const uint16_t*>(I));
+            r.x *= byte_float(v & 255u);
+            r.y *= byte_float(v >> 8);
+          } else {
+            r.x *= byte_float(__ldg(I));
+            r.y *= two ? byte_float(__ldg(I + 1)) : 0.f;
+          }
         }
         if (OUT == 2) {
           sq[k] += fmaf(r.x, r.x, two ? r.y * r.y : 0.f);
         } else {
           const size_t o = ((size_t)f * H + y + e) * W + x;
-          store_store_type<DT>(out, o, r.x * s);
-          if (two) store_store_type<DT>(out, o + 1, r.y * s);
+          if (even_out) {
+            store_pair<DT>(out, o, r.x * s, r.y * s);
+          } else {
+            store_store_type<DT>(out, o, r.x * s);
+            if (two) store_store_type<DT>(out, o + 1, r.y * s);
+          }
         }
       }
     }
