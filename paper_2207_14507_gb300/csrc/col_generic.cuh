@@ -4,9 +4,9 @@
 // RA or RB rows at an odd pitch between stages) with the strides and the radix
 // as run-time values, the strip loaded and stored by every thread itself.
 // Three ping-pong stages each way with runtime radices (k_col) take the other
-// heights.  Microseconds a candidate: 480 x 640 2.13 -> 0.82, 900 x
-// 1600 10.9 -> 3.5, 1440 x 2560 26.4 -> 12.8; latency bounds it (12 to 16 warps per
-// SM, strips in 64-byte rows straight from L2).
+// heights.  Microseconds a candidate: 480 x 640 2.13 -> 0.62, 900 x
+// 1600 10.9 -> 3.5, 1440 x 2560 26.4 -> 12.1, 1500 x 2000 21.5 -> 9.9; latency bounds it
+// (12 to 24 warps per SM, strips in 64- or 32-byte rows straight from L2).
 #pragma once
 #include "common.cuh"
 #include "fft_plan.cuh"
@@ -34,44 +34,56 @@ __host__ __device__ constexpr int col2_rows(int ra, int rb) {
 }
 __host__ __device__ constexpr int col2_threads(int ra, int rb, int nc) { return nc * (ra > rb ? ra : rb); }
 
-// f(R as a compile-time constant); BIG: radices 25 to 48, else 3 to 32
+// The radices of a kernel's switch: each set costs its largest radix' registers.
+enum ColSet { kColTo27, kColTo32, kColTo40, kColTo54 };
+__host__ __device__ constexpr bool col_set_has(ColSet set, int r) {
+  constexpr int lo[] = {3, 4, 5, 6, 8, 9, 10, 12, 15, 16, 18, 20, 24}, hi[] = {25, 27, 30, 32, 36, 40, 45, 48, 50, 54};
+  const int top = set == kColTo27 ? 27 : set == kColTo32 ? 32 : set == kColTo40 ? 40 : 54;
+  if (r > top) return false;
+  if (set == kColTo27 || set == kColTo32)
+    for (int q : lo)
+      if (q == r) return true;
+  for (int q : hi)
+    if (q == r) return true;
+  return false;
+}
 template <int R>
 struct RadixC {
   static constexpr int value = R;
 };
-template <bool BIG, class F>
+// f(R as a compile-time constant); R is in the set (checked before the launch)
+template <ColSet SET, class F>
 __device__ __forceinline__ void with_radix(int R, F&& f) {
-  if constexpr (BIG) {
-    switch (R) {
-      case 25: f(RadixC<25>{}); break;
-      case 27: f(RadixC<27>{}); break;
-      case 30: f(RadixC<30>{}); break;
-      case 32: f(RadixC<32>{}); break;
-      case 36: f(RadixC<36>{}); break;
-      case 40: f(RadixC<40>{}); break;
-      case 45: f(RadixC<45>{}); break;
-      default: f(RadixC<48>{}); break;
-    }
-  } else {
-    switch (R) {
-      case 3: f(RadixC<3>{}); break;
-      case 4: f(RadixC<4>{}); break;
-      case 5: f(RadixC<5>{}); break;
-      case 6: f(RadixC<6>{}); break;
-      case 8: f(RadixC<8>{}); break;
-      case 9: f(RadixC<9>{}); break;
-      case 10: f(RadixC<10>{}); break;
-      case 12: f(RadixC<12>{}); break;
-      case 15: f(RadixC<15>{}); break;
-      case 16: f(RadixC<16>{}); break;
-      case 18: f(RadixC<18>{}); break;
-      case 20: f(RadixC<20>{}); break;
-      case 24: f(RadixC<24>{}); break;
-      case 25: f(RadixC<25>{}); break;
-      case 27: f(RadixC<27>{}); break;
-      case 30: f(RadixC<30>{}); break;
-      default: f(RadixC<32>{}); break;
-    }
+  switch (R) {
+#define PRNU_RADIX(r)                                    \
+  case r:                                                \
+    if constexpr (col_set_has(SET, r)) f(RadixC<r>{});   \
+    break;
+    PRNU_RADIX(3)
+    PRNU_RADIX(4)
+    PRNU_RADIX(5)
+    PRNU_RADIX(6)
+    PRNU_RADIX(8)
+    PRNU_RADIX(9)
+    PRNU_RADIX(10)
+    PRNU_RADIX(12)
+    PRNU_RADIX(15)
+    PRNU_RADIX(16)
+    PRNU_RADIX(18)
+    PRNU_RADIX(20)
+    PRNU_RADIX(24)
+    PRNU_RADIX(25)
+    PRNU_RADIX(27)
+    PRNU_RADIX(30)
+    PRNU_RADIX(32)
+    PRNU_RADIX(36)
+    PRNU_RADIX(40)
+    PRNU_RADIX(45)
+    PRNU_RADIX(48)
+    PRNU_RADIX(50)
+    PRNU_RADIX(54)
+#undef PRNU_RADIX
+    default: break;
   }
 }
 
@@ -174,8 +186,7 @@ struct Col2 {
 };
 
 // grid = (ceil((W/2) / NC), candidates); block = col2_threads(ra, rb, NC).
-// BIG: radices 25 to 48, at least one above 32; else 3 to 32.
-template <int NC, bool BIG, int MAXT, int MINB>
+template <int NC, ColSet SET, int MAXT, int MINB>
 __global__ void __launch_bounds__(MAXT, MINB) k_col2(PassArgs a) {
   extern __shared__ float2 smem[];
   const int c = threadIdx.x % NC, slot = blockIdx.y;
@@ -183,11 +194,11 @@ __global__ void __launch_bounds__(MAXT, MINB) k_col2(PassArgs a) {
   const FpDesc fp = a.fps[it.fp];
   const Col2<NC> w{a, smem, a.spec + (size_t)slot * a.H * (a.W >> 1), fp, c, (int)threadIdx.x / NC,
                    (int)blockIdx.x * NC + c};
-  with_radix<BIG>(a.pcol.ra, [&](auto r) { w.template forward<decltype(r)::value>(); });
+  with_radix<SET>(a.pcol.ra, [&](auto r) { w.template forward<decltype(r)::value>(); });
   __syncthreads();
-  with_radix<BIG>(a.pcol.rb, [&](auto r) { w.template middle<decltype(r)::value>(); });
+  with_radix<SET>(a.pcol.rb, [&](auto r) { w.template middle<decltype(r)::value>(); });
   __syncthreads();
-  with_radix<BIG>(a.pcol.ra, [&](auto r) { w.template inverse<decltype(r)::value>(); });
+  with_radix<SET>(a.pcol.ra, [&](auto r) { w.template inverse<decltype(r)::value>(); });
 }
 
 }  // namespace prnu

@@ -138,7 +138,7 @@ __global__ void __launch_bounds__(128, MINB) k_row_forward2(PassArgs a, const fl
   float2* sm = smem + (size_t)grp * rb * odd_pitch(ra);
   load_row_pair<DT>(a, slot, 2 * pair, mean_sub, warp, t, kRow2Threads, sm);
   __syncwarp();
-  with_radix<false>(ra, [&](auto rc) {
+  with_radix<kColTo32>(ra, [&](auto rc) {
     constexpr int R = decltype(rc)::value;
     float2 u[R];
     if (t < rb) {
@@ -154,7 +154,7 @@ __global__ void __launch_bounds__(128, MINB) k_row_forward2(PassArgs a, const fl
     }
   });
   __syncwarp();
-  with_radix<false>(rb, [&](auto rc) {
+  with_radix<kColTo32>(rb, [&](auto rc) {
     constexpr int R = decltype(rc)::value;
     float2 v[R];
     if (t < ra) {
@@ -186,7 +186,7 @@ __global__ void __launch_bounds__(128, MINB) k_row_inverse2(PassArgs a, float* _
   if (pair >= (H >> 1)) return;
   float2* sm = smem + (size_t)grp * rb * odd_pitch(ra);
   const float2* pa = a.spec + ((size_t)slot * H + 2 * pair) * Wh;
-  with_radix<false>(ra, [&](auto rc) {
+  with_radix<kColTo32>(ra, [&](auto rc) {
     constexpr int R = decltype(rc)::value;
     if (t >= rb) return;
     float2 u[R];
@@ -198,7 +198,7 @@ __global__ void __launch_bounds__(128, MINB) k_row_inverse2(PassArgs a, float* _
   });
   __syncwarp();
   PairStat ps;
-  with_radix<false>(rb, [&](auto rc) {
+  with_radix<kColTo32>(rb, [&](auto rc) {
     constexpr int R = decltype(rc)::value;
     if (t >= ra) return;
     float2 v[R];

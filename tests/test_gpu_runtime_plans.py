@@ -1,5 +1,5 @@
 """Frame sizes without compile-time plans: two-stage passes with runtime radices
-(3 to 32, and 25 to 48 for heights), three stages for the wider rows, and the
+(3 to 32, and 25 to 54 for heights), three stages for the wider rows, and the
 ping-pong stages that take the other heights.
 
 Each length stands for other radices as a height and as a width; the candidates
@@ -20,7 +20,8 @@ SIZES = [(16, 18), (18, 972), (20, 250), (24, 1350), (30, 1200), (54, 640), (50,
          (640, 30), (768, 60), (972, 32), (1000, 24), (1200, 20), (1250, 50), (1350, 36), (2304, 16), (64, 1250),
          (48, 1500), (2000, 40), (96, 96), (120, 1600), (1440, 128),
          (20, 1458), (18, 2000), (16, 2048), (18, 2430), (16, 2916), (18, 3456), (16, 3750), (20, 4000), (18, 4050),
-         (16, 4096)]
+         (16, 4096), (1458, 18), (1500, 16), (1536, 20), (1600, 18), (1944, 16), (2250, 16), (2400, 18), (2592, 16),
+         (2916, 18), (3000, 16)]
 
 
 @pytest.fixture(scope="module")
