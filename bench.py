@@ -142,7 +142,8 @@ def hbm_peak():
 
 # the sources that define the planned-plan kernels' device code (and the
 # launch shapes chosen for them); host-only files do not change the counters
-KERNEL_SOURCES = ("common.cuh", "fft.cuh", "fft_fixed.cuh", "search_common.cuh",
+KERNEL_SOURCES = ("col_generic.cuh", "col_pass.cuh", "common.cuh", "fft.cuh", "fft_fixed.cuh",
+                  "fft_packed.cuh", "fft_plan.cuh", "search_common.cuh",
                   "search_fixed.cu", "search_fixed.cuh", "search_fixed.h", "search_fixed_256.cu",
                   "search_fixed_720.cu", "search_fixed_1080.cu", "search_fixed_2160.cu", "tma.cuh")
 

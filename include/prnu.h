@@ -417,10 +417,10 @@ int prnu_server_stats_get(prnu_ctx* ctx, prnu_server_stats* out);
 /* ---------------------------------------------------------------- tuning */
 
 /* Launch configuration of the fused path for one frame size: columns per
- * column-pass block and row pairs per row block of the generic kernels (sides
- * that are the product of two radices up to 48 have two-stage passes with
- * their own blocks and take neither), the
- * candidates per wave (per-candidate spectra kept in the workspace), and which
+ * column-pass block of the generic kernels (heights that are the product of two
+ * radices up to 54 have passes with their own blocks, which it does not change),
+ * row pairs per row block of the planned kernels, the candidates per wave
+ * (per-candidate spectra kept in the workspace), and which
  * compile-time-planned column kernel to use where the size has them
  * (1920x1080, 1280x720, 3840x2160, 256x256). */
 typedef struct {

@@ -10,10 +10,12 @@
 // (67% of its peak, a quarter of it bank conflicts and spilled registers) and
 // by the barriers between its stages.  At 1080p FP32 (ncu, 64 candidates):
 // 3.5 M -> 2.3 M warp instructions a candidate, L1 data pipe 67% -> 49%, L1 hit
-// rate of the twiddles 49% -> 99%, 5.38 -> 4.25 us a candidate.  What bounds it
-// now is latency: 13.5 warps per SM (registers and the strips' shared memory),
-// no unit above 50%.  Each size's variants and their times stand at its
-// registry entry (search_fixed_<rows>.cu).
+// rate of the twiddles 49% -> 99%, 5.38 -> 4.25 us a candidate; with the
+// fingerprint in contiguous strips (load_fp_strips) 3.72.  What bounds it
+// now is the movement of the strip, two TMA copies in rows of 32 bytes (with the
+// fingerprint's a third, movement alone took 3.35 of 4.18 us), and latency: 13.5 to 18
+// warps per SM (registers and the strips' shared memory), no other unit above 50%.  Each size's variants and
+// their times stand at its registry entry (search_fixed_<rows>.cu).
 //
 //   stage A : butterfly j < RB reads x[j + r RB], r < RA; writes j RA + r
 //   stage B : butterfly j < RA reads x[j + r RA], r < RB, twiddle w_H^(rj);

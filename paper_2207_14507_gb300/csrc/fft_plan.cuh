@@ -5,7 +5,7 @@
 // thread loads one butterfly's R inputs, transforms them in registers and
 // stores the R outputs before it takes the next butterfly, so no register
 // state crosses a barrier.  Two layouts:
-//  * row layout: one FFT per thread group, element i at i + (i >> 4) (one
+//  * row layout: one FFT per block (the finalisation), element i at i + (i >> 4) (one
 //    float2 of padding every 16 keeps the strided stores off one bank);
 //  * column layout: NC = 1 << lg interleaved FFTs (columns), element i of
 //    column c at i*NC + c; butterflies are spread over all threads of the block.
@@ -78,15 +78,13 @@ __device__ __forceinline__ void plan_stage_any(const FftPlan& p, int s, const fl
   }
 }
 
-// The first `stages` stages of the FFT of the data in `a` (row layout), using
-// `b` as the second buffer.  Every thread of the block must call it (it holds
-// barriers); a thread of a group without a row passes t >= n so that it owns
-// no butterfly.  The caller synchronises before the call; the result is in the
-// returned buffer and is visible to the whole block on return.
+// The FFT of the data in `a` (row layout), using `b` as the second buffer.  Every
+// thread of the block must call it (it holds barriers).  The caller synchronises
+// before the call; the result is in the returned buffer and is visible to the
+// whole block on return.
 template <bool INV>
-__device__ float2* fft_row(float2* a, float2* b, const FftPlan& p, const float4* __restrict__ tab, int t, int T,
-                           int stages) {
-  for (int s = 0; s < stages; ++s) {
+__device__ float2* fft_row(float2* a, float2* b, const FftPlan& p, const float4* __restrict__ tab, int t, int T) {
+  for (int s = 0; s < p.nstages; ++s) {
     plan_stage_any<INV>(
         p, s, tab, t, T, [=](int i) { return a[rpad(i)]; }, [=](int i, float2 v) { b[rpad(i)] = v; });
     __syncthreads();
@@ -95,10 +93,6 @@ __device__ float2* fft_row(float2* a, float2* b, const FftPlan& p, const float4*
     b = x;
   }
   return a;
-}
-template <bool INV>
-__device__ float2* fft_row(float2* a, float2* b, const FftPlan& p, const float4* __restrict__ tab, int t, int T) {
-  return fft_row<INV>(a, b, p, tab, t, T, p.nstages);
 }
 
 // The FFTs of the 1 << lg columns in `a` (column layout).

@@ -778,7 +778,7 @@ struct ShapeDef {
   static constexpr int FT = (RTI + 31) / 32 * 32;   // of a row pair in the finalisation: whole warps
   static_assert(CS::N == H, "column plans of one length");
   // NC columns per block, at least MINB resident blocks per SM
-  // MODE: 0 plain loads and stores, 1 strip by TMA, 2 strip and fingerprint by TMA
+  // MODE: 0 plain loads and stores, 1 strip by TMA, 2 strip by TMA and fingerprint by bulk copies
   static FixedCol col_entry(void* fn, int nc, int mode) {
     allow_max_dynamic_smem(fn);
     return FixedCol{nc, nc * CP::lanes, col_pass_smem<CP>(nc, mode), fn, mode != 0, tma_box_rows(H, nc), mode};

@@ -26,7 +26,7 @@ struct FixedCol {
   void* fn;
   bool tma;
   int br;
-  int mode;   // 0 plain loads, 1 strip by TMA, 2 fingerprint by TMA into the strip buffer, 3/4 into its own region
+  int mode;   // 0 plain loads, 1 strip by TMA, 2 fingerprint by bulk copies into the strip buffer, 3/4 into its own region
 };
 
 // one instantiated pair of row kernels: row pairs per block, threads per pair
