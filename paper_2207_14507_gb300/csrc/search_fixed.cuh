@@ -601,6 +601,7 @@ __device__ __forceinline__ double window_pair_energy(const PassArgs& a, const fl
 template <class SP, int T, int PPB>
 __device__ __forceinline__ void finalize_task(const PassArgs& a, int is, int ws, float2* smem, int tx) {
   constexpr int W = SP::N, Wh = W / 2, L = row_len2(W), TB = T * PPB;
+  static_assert(T % 32 == 0, "groups of whole warps: their shares end in warp reductions");
   __shared__ double red[kFinParts][T / 32];
   const int t = tx, grp = t / T, tg = t - grp * T;
   const RowStat* st = a.stats + (size_t)ws * a.H;
