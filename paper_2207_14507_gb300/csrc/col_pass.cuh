@@ -140,6 +140,14 @@ __device__ __forceinline__ void col_body(const PassArgs& a, int is, int ws, int 
   const int c0 = bx * NC, col = c0 + c;
   const WorkItem wi = item_of(a, is);
   const FpDesc fp = a.fps[wi.fp];
+  if constexpr (MODE == 4 && PART != 1) {
+    // an FP32 strip is twice the region: whoever launched this variant for it
+    // (launch_fixed_wave takes another) gets an error, not the memory behind
+    if (fp.dtype == kF32) {
+      if (threadIdx.x == 0 && a.err) atomicExch(a.err, 1);
+      return;
+    }
+  }
   char* const fpsm = reinterpret_cast<char*>(sm) + (FPSEP ? col_buf_bytes<CP>(NC) : 0);
 
   constexpr int BR = tma_box_rows(H, NC);

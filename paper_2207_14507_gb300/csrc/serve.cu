@@ -36,6 +36,7 @@
 #include <algorithm>
 #include <chrono>
 #include <cstring>
+#include <tuple>
 
 #include "search_fixed.h"
 #include "server.h"
@@ -127,10 +128,13 @@ struct Server::Impl {
     cudaEvent_t ev = nullptr;
   };
 
+  // fp_f32 (device loops): some fingerprint is FP32.  A loop's graph holds one
+  // column variant, and those whose fingerprint region is sized for FP16 bins
+  // must never meet an FP32 spectrum, so such queries have a loop of their own.
   struct SizeKey {
-    int H, W, dtype;
+    int H, W, dtype, fp_f32 = 0;
     bool operator<(const SizeKey& o) const {
-      return H != o.H ? H < o.H : W != o.W ? W < o.W : dtype < o.dtype;
+      return std::tie(H, W, dtype, fp_f32) < std::tie(o.H, o.W, o.dtype, o.fp_f32);
     }
   };
 
@@ -546,10 +550,14 @@ struct Server::Impl {
 
   // ---------------------------------------------------------------- device loop (holds mu)
 
+  static bool any_f32(const Query& q) {
+    return std::any_of(q.fps.begin(), q.fps.end(), [](const auto& f) { return f->dtype == kF32; });
+  }
+
   // The device loop of q's size class; nullptr where the size has no planned
   // kernels for q's tuning (its queries take host waves).
   DevLoop* loop_for(const Query& q) {
-    const SizeKey key{q.H, q.W, q.dtype};
+    const SizeKey key{q.H, q.W, q.dtype, any_f32(q)};
     auto it = loops.find(key);
     if (it != loops.end() && it->second && it->second->dead) {
       retired.push_back(std::move(it->second));   // kept until its queries are reported
@@ -620,7 +628,7 @@ struct Server::Impl {
     c.rdtype = L.key.dtype;
     c.wave = L.wave;
     c.budget = kLoopWaves;
-    c.fp_f32 = L.key.dtype == kF32 ? 1 : 0;   // half residuals: FP16 fingerprints expected (FP32 ones still correct)
+    c.fp_f32 = L.key.fp_f32;
     c.spec = ws_spec;
     c.stats = ws_stats;
     const size_t slot = (size_t)L.key.H * (L.key.W / 2) * sizeof(float2);
@@ -742,7 +750,7 @@ struct Server::Impl {
         hu[nunits++] = count + u * S;
       }
       grouped = grouped || S > 1;
-      for (auto& f : q.fps) fp_f32 = fp_f32 || f->dtype == kF32;
+      fp_f32 = fp_f32 || any_f32(q);
       count += take;
       q.next += take;
       if (q.next == n) finished.push_back(&q);

@@ -101,6 +101,30 @@ def test_device_loop_many_small_queries(prnu):
                                         for q in qs)
 
 
+@pytest.mark.parametrize("H,W", [(256, 256), (720, 1280), (1080, 1920), (2160, 3840)])
+def test_device_loop_takes_fp32_fingerprints_with_half_residuals(prnu, H, W):
+    """Half residuals against FP32, mixed and FP16 fingerprints in one context,
+    one and several per frame: the column variants that stage FP16 bins only
+    take none of the FP32 ones, and every query equals the host loop's."""
+    qs = [_query(H, W, 1, P, True, 20 + P) for P in (1, 2, 1, 2, 2)]
+    stores = [(prnu.PRNU_F32,), (prnu.PRNU_F32, prnu.PRNU_F32), (prnu.PRNU_F16,), (prnu.PRNU_F16, prnu.PRNU_F16),
+              (prnu.PRNU_F16, prnu.PRNU_F32)]
+    flags = prnu.PRNU_WEIGHT_BY_INTENSITY | prnu.PRNU_NORMALISE
+    out = {}
+    for mode in (prnu.PRNU_LOOP_HOST, prnu.PRNU_LOOP_DEVICE):
+        with prnu.Context(0) as ctx:
+            ctx.prnu_server_set_loop(mode)
+            ids = []
+            for q, st in zip(qs, stores):
+                hs = [ctx.prnu_fingerprint_term(torch.from_numpy(K).to(DEV), d) for K, d in zip(q["fps"], st)]
+                ids.append(ctx.query_submit(q["frames"], hs, q["g"], windows=q["windows"], dtype=prnu.PRNU_F16,
+                                            flags=flags))
+            out[mode] = [ctx.query_poll(i, q["F"], q["P"], timeout_us=300_000_000) for i, q in zip(ids, qs)]
+    for h, d in zip(out[prnu.PRNU_LOOP_HOST], out[prnu.PRNU_LOOP_DEVICE]):
+        assert h.tobytes() == d.tobytes()
+        assert d[0, 0]["pce"] > 60   # the matching fingerprint, whatever its storage
+
+
 def test_loop_mode_rules(prnu):
     with prnu.Context(0) as ctx:
         with pytest.raises(prnu.PrnuError) as e:
