@@ -149,7 +149,9 @@ int prnu_fingerprint_release(prnu_ctx* ctx, uint64_t handle);
  *   C(d) = sum_x X(x) K0_p((x + d) mod (H, W))  over all H*W cyclic shifts;
  *   PCE  = sgn(C*) C*^2 / E, C* = max C (first in row-major order on ties),
  *          E = mean of C^2 outside the cyclic 11x11 window around the peak
- *          (E == 0: PCE = 0 for a zero peak, +-inf otherwise);
+ *          (E == 0: PCE = 0 for a zero peak, +-inf otherwise; where C holds no
+ *          ordered value, as a NaN or an infinity in the residual or the
+ *          fingerprint makes it: PCE and peak -inf, shift (0, 0));
  * then keeps, per (f, p), the candidate of largest PCE (ties: lowest index).
  *  d_resid:  [F][H][W] residuals of type `dtype` (from prnu_residual).
  *  d_scale:  [F] or NULL; when given, the reported peak is divided by d_scale[f].
@@ -320,8 +322,9 @@ int eis_invert_video(prnu_ctx* ctx, const void* d_resid, int dtype, const float*
                      double* gamma, double* mean_gamma, int* decision, prnu_result* best, int* from_reg,
                      prnu_stream stream);
 
-/* PCE of one aligned pair (Eq. 3, no warp): d_X device float [H][W] against the
- * cached fingerprint `fp_handle`.  Host outputs; any of them may be NULL.
+/* PCE of one aligned pair (Eq. 3, no warp, scored as eis_grid_search scores a
+ * candidate): d_X device float [H][W] against the cached fingerprint
+ * `fp_handle`.  Host outputs; any of them may be NULL.
  * Synchronous (waits for `stream`). */
 int pce_score(prnu_ctx* ctx, const float* d_X, uint64_t fp_handle, int H, int W,
               double* pce, int* dy, int* dx, float* peak, prnu_stream stream);

@@ -42,7 +42,7 @@ struct FpDesc {
 // Per-row statistics of one candidate's correlation surface.
 struct RowStat {
   float max;
-  int arg;             // column of the first maximum
+  int arg;             // column of the first maximum; INT_MAX where no value is ordered (NaN)
   double sumsq;        // sum of C^2 over the row
 };
 

@@ -22,7 +22,7 @@ struct WarpRed {
   double sb;
 };
 
-__device__ __forceinline__ void better_f(float& v, int& i, float v2, int i2) {
+__host__ __device__ __forceinline__ void better_f(float& v, int& i, float v2, int i2) {
   if (v2 > v || (v2 == v && i2 < i)) {
     v = v2;
     i = i2;
@@ -164,7 +164,7 @@ __device__ __forceinline__ void row_stats_final(const RowRed* red, int nw, RowSt
   st[1] = RowStat{r.mb, r.ib, (double)r.sb + (double)r.cb};
 }
 // cyclic distance between indices a and b modulo n
-__device__ __forceinline__ int cdist(int a, int b, int n) {
+__host__ __device__ __forceinline__ int cdist(int a, int b, int n) {
   int d = a - b;
   if (d < 0) d = -d;
   return d < n - d ? d : n - d;
@@ -326,7 +326,7 @@ __host__ __device__ inline size_t row_smem_bytes(int W, int ppb) {
 constexpr int kFinPairParts = 6, kFinRowParts = 3, kFinParts = kFinRowParts + kFinPairParts;
 
 // the b-th row pair of the window around row py (11 rows cover 6 pairs)
-__device__ __forceinline__ int window_pair(int py, int b, int H) {
+__host__ __device__ __forceinline__ int window_pair(int py, int b, int H) {
   return (((py - kHalfWindow + H) % H >> 1) + b) % (H >> 1);
 }
 
@@ -334,15 +334,22 @@ struct FinPeak {
   float peak;
   int py, px;
 };
+// Row y's maximum into the running maximum (v, i) over rows.  A row without an
+// ordered value (NaN throughout) has its arg outside [0, W) and no part in it.
+__host__ __device__ __forceinline__ void take_row(float& v, int& i, const RowStat& r, int y, int W) {
+  if ((unsigned)r.arg < (unsigned)W) better_f(v, i, r.max, y * W + r.arg);
+}
+// the peak from it; of a surface without an ordered value: -infinity at (0, 0)
+__host__ __device__ __forceinline__ FinPeak peak_at(float v, int i, int W) {
+  if (i == INT_MAX) i = 0;
+  return FinPeak{v, i / W, i - (i / W) * W};
+}
 // the first maximum over all rows, by the TB threads of the block; holds barriers
 __device__ __forceinline__ FinPeak block_peak(const RowStat* st, int H, int W, int t, int TB, WarpRed* red) {
   __shared__ FinPeak s_peak;
   float bv = -INFINITY;
   int bi = INT_MAX;
-  for (int y = t; y < H; y += TB) {
-    const RowStat r = ld_l2(st + y);
-    better_f(bv, bi, r.max, y * W + r.arg);
-  }
+  for (int y = t; y < H; y += TB) take_row(bv, bi, ld_l2(st + y), y, W);
   warp_maxarg(bv, bi);
   if ((t & 31) == 0) {
     red[t >> 5].ma = bv;
@@ -351,8 +358,7 @@ __device__ __forceinline__ FinPeak block_peak(const RowStat* st, int H, int W, i
   __syncthreads();
   if (t == 0) {
     for (int k = 1; k < TB >> 5; ++k) better_f(bv, bi, red[k].ma, red[k].ia);
-    if (bi == INT_MAX) bi = 0;
-    s_peak = FinPeak{bv, bi / W, bi - (bi / W) * W};
+    s_peak = peak_at(bv, bi, W);
   }
   __syncthreads();
   return s_peak;
@@ -391,10 +397,11 @@ __device__ __forceinline__ double part_total(const double* red_part, int nw) {
 }
 
 // Where a candidate's parts wait when several blocks compute them: in its own
-// spectrum, dead but for the window's rows, eight rows from the peak.
+// spectrum, dead but for the window's rows: in the row pair (two rows hold the
+// parts even at W = 16) half the rows, at least eight, from the peak.
+__host__ __device__ __forceinline__ int fin_scratch_row(int py, int H) { return (py + H / 2) % H & ~1; }
 __device__ __forceinline__ double* fin_scratch(const PassArgs& a, int ws, int py) {
-  const int H = a.H, row = (py + H / 2) % H & ~1;
-  return reinterpret_cast<double*>(a.spec + ((size_t)ws * H + row) * (a.W >> 1));
+  return reinterpret_cast<double*>(a.spec + ((size_t)ws * a.H + fin_scratch_row(py, a.H)) * (a.W >> 1));
 }
 
 // one thread: PCE and result of candidate `is`
@@ -406,7 +413,8 @@ __device__ __forceinline__ void finish_candidate(const PassArgs& a, int is, cons
   const double E = etot / ((double)H * (double)W - (double)kWindowCount);
   const double pk = (double)p.peak;
   double pce;
-  if (E > 0.0) pce = (pk < 0 ? -1.0 : 1.0) * pk * pk / E;
+  if (p.peak == -INFINITY) pce = -INFINITY;   // no ordered value
+  else if (E > 0.0) pce = (pk < 0 ? -1.0 : 1.0) * pk * pk / E;
   else pce = pk == 0.0 ? 0.0 : (pk < 0 ? -INFINITY : INFINITY);
   const FpDesc fp = a.fps[it.fp];
   double pv = pk / ((double)H * (double)W) * (double)(*fp.inv_scale);
