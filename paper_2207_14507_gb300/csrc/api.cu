@@ -1211,7 +1211,7 @@ int prnu_fingerprint_estimate(prnu_ctx* ctx, const uint8_t* d_frames, int L, int
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     PRNU_CUDA_TRY(cudaStreamWaitEvent(s, ctx->last_done, 0));
     const size_t accb = (sizeof(unsigned long long) * L + 255) & ~(size_t)255;
-    ensure_buf(ctx, ctx->ws_resid, accb + sizeof(unsigned long long) * residual_partials_needed(L, H, W));
+    ensure_buf(ctx, ctx->ws_resid, accb + sizeof(unsigned long long) * fp_estimate_slots(L, H, W));
     auto* acc = reinterpret_cast<unsigned long long*>(ctx->ws_resid.p);
     auto* slots = reinterpret_cast<unsigned long long*>(reinterpret_cast<char*>(ctx->ws_resid.p) + accb);
     launch_fp_estimate(d_frames, pitch, L, H, W, slots, acc, d_K, s, ctx->launches);

@@ -175,8 +175,9 @@ size_t wavelet_partials_needed(int F, int H, int W);
 // fingerprint resampling with T taps per axis; w, idx: (H + W) * T scratch weights and input indices
 void launch_fp_resize(const float* K, int Hin, int Win, size_t pitch, double scale, int y0, int x0, int T, float* w,
                       int* idx, int H, int W, float* out, cudaStream_t s, LaunchCounter& lc);
-// Eq. 2's estimate over L frames into K [H][W]; slots: residual_partials_needed(L,
-// H, W) of 8 bytes, acc: L (scratch)
+// Eq. 2's estimate over L frames into K [H][W]; slots: fp_estimate_slots(L, H, W)
+// of 8 bytes, acc: L (scratch)
+size_t fp_estimate_slots(int L, int H, int W);
 void launch_fp_estimate(const uint8_t* frames, size_t pitch, int L, int H, int W, unsigned long long* slots,
                         unsigned long long* acc, float* K, cudaStream_t s, LaunchCounter& lc);
 // dense [F][H][W] residuals -> the zero-bordered layout the compile-time-planned

@@ -9,6 +9,7 @@
 //   W = (x - mu) nu2 / var = 9 D nu2 / V   where var >= nu2 (and V > 0),
 //   W = x - mu = D / 9                      elsewhere,
 // and R = x W (PRNU_WEIGHT_BY_INTENSITY) or W.
+#include <algorithm>
 #include <type_traits>
 
 #include "internal.h"
@@ -26,6 +27,7 @@ namespace {
 // 243 us instead of 737; what bounds it is instruction issue (63%),
 // 34 instructions a pixel and pass.
 constexpr int kBX = 32, kPX = 4;   // lanes of a block's row, pixels of a thread
+constexpr int kMomentFrames = 1024;   // frames of the estimate whose noise powers one launch sums
 
 // rows per thread: 8, but 2 where 8 would leave the GPU's 152 SMs with less
 // than two blocks each
@@ -727,7 +729,12 @@ __global__ void k_fp_resize(const float* __restrict__ K, size_t pitch, const flo
 void launch_fp_estimate(const uint8_t* frames, size_t pitch, int L, int H, int W, unsigned long long* slots,
                         unsigned long long* acc, float* K, cudaStream_t s, LaunchCounter& lc) {
   ProfScope ps(lc, kKindResidual, s);
-  launch_moments(frames, L, H, W, pitch, resid_rows(L, H, W), slots, acc, s, lc);
+  // frames are a grid dimension of at most 65535: the noise powers come in
+  // runs of kMomentFrames, which reuse the slots of the first
+  const int rpt = resid_rows(std::min(L, kMomentFrames), H, W);
+  for (int l0 = 0; l0 < L; l0 += kMomentFrames)
+    launch_moments(frames + (size_t)l0 * H * pitch, std::min(kMomentFrames, L - l0), H, W, pitch, rpt, slots, acc + l0, s,
+                   lc);
   const dim3 g = resid_grid(1, H, W, 2), b(kBX, 8);
   const bool vec = rows_aligned4(frames, pitch), lng = L > 256;
   const bool vec_out = W % 4 == 0 && reinterpret_cast<uintptr_t>(K) % 16 == 0;
@@ -773,6 +780,8 @@ void launch_literal_residuals(const uint8_t* frames, size_t pitch, int H, int W,
 size_t literal_partials_needed(int nr, int H, int W) {
   return (size_t)nr * ((W + kLX - 1) / kLX) * ((H + kLY - 1) / kLY);
 }
+
+size_t fp_estimate_slots(int L, int H, int W) { return residual_partials_needed(std::min(L, kMomentFrames), H, W); }
 
 size_t residual_partials_needed(int F, int H, int W) {
   const dim3 g = resid_grid(F, H, W, resid_rows(F, H, W));

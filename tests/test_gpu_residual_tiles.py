@@ -68,3 +68,12 @@ def test_estimate_tile_edges(ctx, L, H, W, pad, offset):
     ref = oracle.fingerprint_estimate(host)
     assert got[0, 0] == 0
     assert np.max(np.abs(got - ref)) <= 1e-6 * np.abs(ref).max() + 1e-30
+
+
+@pytest.mark.parametrize("L,H,W", [(1025, 70, 130), (65537, 3, 5), (70000, 2, 4)])
+def test_estimate_of_many_frames(ctx, L, H, W):
+    """More frames than one launch's grid holds, and than one run of noise powers."""
+    host, dev = _frames(L, H, W, W, 0, L)
+    got = ctx.prnu_fingerprint_estimate(dev).double().cpu().numpy()
+    ref = oracle.fingerprint_estimate(host)
+    assert np.max(np.abs(got - ref)) <= 1e-6 * np.abs(ref).max()
