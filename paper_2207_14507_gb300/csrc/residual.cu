@@ -680,9 +680,9 @@ __global__ void __launch_bounds__(256) k_lit_apply(const float* __restrict__ X, 
 
 // Taps of one axis (Sec. 3's resampling): output sample o at input position
 // u = (first + o + 0.5) / scale - 0.5, tent weights max(0, 1 - |j - u| a) with a
-// = min(scale, 1), indices clamped to the axis, normalised; T taps per sample
-// (zero weight beyond its support).  In double, one thread per sample of both
-// axes (y first).
+// = min(scale, 1), indices clamped to the axis, normalised; a sample's taps of
+// nonzero weight first, then zero weights up to T.  In double, one thread per
+// sample of both axes (y first).
 struct TapAxis {
   int n_in, first, n;
   float* w;
@@ -699,14 +699,19 @@ __global__ void k_fp_taps(TapAxis ay, TapAxis ax, double scale, int T) {
   const int lo = (int)floor(u - 1.0 / a);
   double tot = 0.0;
   for (int k = 0; k < T; ++k) tot += fmax(1.0 - fabs((double)(lo + k) - u) * a, 0.0);
+  int m = 0;
   for (int k = 0; k < T; ++k) {
-    t.w[(size_t)o * T + k] = (float)(fmax(1.0 - fabs((double)(lo + k) - u) * a, 0.0) / tot);
-    t.idx[(size_t)o * T + k] = min(max(lo + k, 0), t.n_in - 1);
+    const double v = fmax(1.0 - fabs((double)(lo + k) - u) * a, 0.0);
+    if (v == 0.0) continue;
+    t.w[(size_t)o * T + m] = (float)(v / tot);
+    t.idx[(size_t)o * T + m++] = min(max(lo + k, 0), t.n_in - 1);
   }
+  for (; m < T; ++m) t.w[(size_t)o * T + m] = 0.f;
 }
 
 // Fingerprint resampling: out(y, x) = sum_a sum_b wy[y][a] wx[x][b] K(iy[y][a], ix[x][b]),
-// T taps per axis (unused taps have weight 0).
+// T taps per axis, the first zero weight ends them (a sample without weight has
+// no part in the sum: it may hold an infinity or a NaN).
 __global__ void k_fp_resize(const float* __restrict__ K, size_t pitch, const float* __restrict__ wy,
                             const int* __restrict__ iy, const float* __restrict__ wx, const int* __restrict__ ix,
                             int T, int H, int W, float* __restrict__ out) {
@@ -715,10 +720,14 @@ __global__ void k_fp_resize(const float* __restrict__ K, size_t pitch, const flo
   float acc = 0.f;
   for (int a = 0; a < T; ++a) {
     const float w = wy[(size_t)y * T + a];
-    if (w == 0.f) continue;
+    if (w == 0.f) break;
     const float* row = K + (size_t)iy[(size_t)y * T + a] * pitch;
     float r = 0.f;
-    for (int b = 0; b < T; ++b) r = fmaf(wx[(size_t)x * T + b], __ldg(row + ix[(size_t)x * T + b]), r);
+    for (int b = 0; b < T; ++b) {
+      const float v = wx[(size_t)x * T + b];
+      if (v == 0.f) break;
+      r = fmaf(v, __ldg(row + ix[(size_t)x * T + b]), r);
+    }
     acc = fmaf(w, r, acc);
   }
   out[(size_t)y * W + x] = acc;

@@ -52,3 +52,22 @@ def test_resize_rejects_bad_crops(prnu):
             with pytest.raises(prnu.PrnuError) as e:
                 ctx.prnu_fingerprint_resize(K, *args)
             assert e.value.code == prnu.PRNU_EINVAL
+
+
+@pytest.mark.parametrize("scale,y0,x0,H,W", [(1.0, 2, 3, 60, 100), (0.5, 0, 0, 36, 64), (0.48, 1, 2, 30, 50),
+                                             (1.5, 5, 6, 90, 150)])
+def test_resize_keeps_a_non_finite_sample_to_its_own_outputs(prnu, scale, y0, x0, H, W):
+    """An infinity and a NaN in the fingerprint reach the outputs that weigh
+    them and no others (a tap of weight zero has no part in a sum)."""
+    K = np.random.default_rng(3).standard_normal((72, 128)).astype(np.float32)
+    bad = K.copy()
+    bad[20, 0], bad[31, 77], bad[71, 127] = np.inf, np.nan, -np.inf
+    wy = oracle.resize_weights(72, scale, y0, H) != 0
+    wx = oracle.resize_weights(128, scale, x0, W) != 0
+    hit = (wy.astype(int) @ ~np.isfinite(bad) @ wx.T.astype(int)) > 0
+    with prnu.Context(0) as ctx:
+        want, got = (ctx.prnu_fingerprint_resize(torch.from_numpy(k).to(DEV), scale, y0, x0, H, W).cpu().numpy()
+                     for k in (K, bad))
+    assert hit.any() and not hit.all()
+    np.testing.assert_array_equal(~np.isfinite(got), hit)
+    np.testing.assert_array_equal(got[~hit], want[~hit])
