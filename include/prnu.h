@@ -428,7 +428,10 @@ int prnu_server_stats_get(prnu_ctx* ctx, prnu_server_stats* out);
  * (1920x1080, 1280x720, 3840x2160, 256x256). */
 typedef struct {
     int col_width;        /* 4, 8 or 16 */
-    int pairs_per_block;  /* 1, 2 or 4 */
+    int pairs_per_block;  /* with compile-time-planned kernels: one the size has a plan for
+                             (256x256 8, 4; 1280x720 2, 4; 1920x1080 1, 2; 3840x2160 1, 2), or 1 or
+                             2 for its default where it has none of these; other sizes take 1, 2
+                             and 4 and run the same whichever */
     int wave;             /* candidates in flight, >= 1 (default: up to 1024, with at most
                              16 GB of spectra and a quarter of the context's HBM budget) */
     int variant;          /* compile-time-planned column kernel variant for this size

@@ -215,11 +215,11 @@ Tuning tuning_for(prnu_ctx* c, int H, int W) {
       break;
     }
   }
-  // the planned kernels run one row pair per block best; waves of up to 1024
-  // candidates (up to 16 GB of spectra) amortise the per-wave finalisation and
-  // tail: 1024 against 512 gains 0.7% at 1080p, 512 against 129 1% at 4K
+  // waves of up to 1024 candidates (up to 16 GB of spectra) amortise the
+  // per-wave finalisation and tail: 1024 against 512 gains 0.7% at 1080p, 512
+  // against 129 1% at 4K
   const FixedShape* fs = find_fixed(H, W);
-  t.ppb = fs ? 1 : 2;
+  t.ppb = fs ? fs->row_for(1).ppb : 2;   // (other sizes have no use for it)
   // sizes without compile-time-planned kernels run the generic ones (-1), so
   // that what prnu_get_tuning reports is accepted by prnu_set_tuning
   t.variant = fs ? fs->default_col : -1;
@@ -1631,22 +1631,19 @@ int prnu_set_tuning(prnu_ctx* ctx, int H, int W, const prnu_tuning* cfg) {
     for (int k = 0; k <= 4; ++k)
       if (cfg->col_width == (1 << k)) lg = k;
     PRNU_CHECK_ARG(lg >= 0, "col_width must be 1, 2, 4, 8 or 16");
-    PRNU_CHECK_ARG(cfg->pairs_per_block == 1 || cfg->pairs_per_block == 2 || cfg->pairs_per_block == 4,
-                   "pairs_per_block must be 1, 2 or 4");
-    PRNU_CHECK_ARG(cfg->wave >= 1, "wave must be >= 1");
-    FftPlan pc = make_plan(H, ctx->tw_off), pr = make_plan(W, ctx->tw_off);
-    int T, mb;
-    col_launch_shape(pc, lg, &T, &mb);
-    PRNU_CHECK_ARG(2 * (size_t)H * (1u << lg) * sizeof(float2) <= 227 * 1024, "column strip exceeds shared memory");
-    row_launch_shape(pr, &T, &mb);
-    PRNU_CHECK_ARG(T * cfg->pairs_per_block <= 512, "row block exceeds 512 threads");
     const FixedShape* fs = find_fixed(H, W);
+    const int ppb = cfg->pairs_per_block;
+    PRNU_CHECK_ARG(ppb == 1 || ppb == 2 || (fs ? fs->row_for(ppb).ppb == ppb : ppb == 4),
+                   fs ? "pairs_per_block must be 1, 2 or one this frame size has a plan for"
+                      : "pairs_per_block must be 1, 2 or 4");
+    PRNU_CHECK_ARG(cfg->wave >= 1, "wave must be >= 1");
+    PRNU_CHECK_ARG(2 * (size_t)H * (1u << lg) * sizeof(float2) <= 227 * 1024, "column strip exceeds shared memory");
     PRNU_CHECK_ARG(cfg->variant >= -1 && cfg->variant < (fs ? (int)fs->cols.size() : 0),
                    "variant out of range for this frame size (-1 = generic kernels)");
     PRNU_CHECK_ARG(cfg->persistent >= 0 && cfg->persistent <= 2, "persistent must be 0, 1 or 2");
     PRNU_CHECK_ARG(cfg->streams >= 0 && cfg->streams <= 2, "streams must be 0, 1 or 2");
     PRNU_CHECK_ARG(cfg->share_forward == 0 || cfg->share_forward == 1, "share_forward must be 0 or 1");
-    ctx->tuning[{H, W}] = Tuning{lg, cfg->pairs_per_block, cfg->wave, cfg->variant, cfg->persistent,
+    ctx->tuning[{H, W}] = Tuning{lg, ppb, cfg->wave, cfg->variant, cfg->persistent,
                                  cfg->streams == 2 ? 2 : 1, cfg->share_forward};
   });
 }

@@ -217,7 +217,7 @@ class Server;
 
 struct Tuning {
   int col_log2 = 3;   // generic kernels: columns per column-pass block = 1 << col_log2
-  int ppb = 2;        // generic kernels: row pairs per row block
+  int ppb = 2;        // compile-time-planned shapes: row pairs per row block
   int wave = 64;      // candidates in flight
   int variant = 0;    // compile-time-planned column variant; -1 = generic kernels only
   int persistent = 0; // compile-time-planned shapes: one persistent launch per call instead of waves

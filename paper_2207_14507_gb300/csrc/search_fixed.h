@@ -78,7 +78,8 @@ struct FixedShape {
   FixedCol col_inv_h;        // the same with a region for FP16 bins (mode 4) and more blocks per SM, taken
                              // instead when every fingerprint of the wave is FP16; fn null where none
   FixedPersist persist;
-  // the row kernels with `ppb` pairs per block, else the first variant
+  // the row kernels with `ppb` pairs per block, else the first variant (what
+  // the default tuning asks row_for(1) for)
   const FixedRow& row_for(int ppb) const {
     for (auto& r : rows)
       if (r.ppb == ppb) return r;
