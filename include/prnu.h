@@ -435,7 +435,9 @@ typedef struct {
     int wave;             /* candidates in flight, >= 1 (default: up to 1024, with at most
                              16 GB of spectra and a quarter of the context's HBM budget) */
     int variant;          /* compile-time-planned column kernel variant for this size
-                             (0.. n-1), or -1 for the generic runtime-plan kernels */
+                             (0.. n-1, 0 the default; the bits are the same in all, and
+                             which kernel another number names may change), or -1 for
+                             the generic runtime-plan kernels */
     int persistent;       /* 0: waves, one launch sequence each (default).
                              1: sizes with compile-time-planned kernels run a whole call
                              as one persistent launch that schedules every phase of every

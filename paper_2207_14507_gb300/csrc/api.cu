@@ -222,7 +222,7 @@ Tuning tuning_for(prnu_ctx* c, int H, int W) {
   t.ppb = fs ? fs->row_for(1).ppb : 2;   // (other sizes have no use for it)
   // sizes without compile-time-planned kernels run the generic ones (-1), so
   // that what prnu_get_tuning reports is accepted by prnu_set_tuning
-  t.variant = fs ? fs->default_col : -1;
+  t.variant = fs ? 0 : -1;
   // within a quarter of the context's HBM budget (spectra and row statistics)
   const size_t per_item = (size_t)H * (W / 2) * sizeof(float2) + (size_t)H * sizeof(RowStat);
   t.wave = (int)std::max<size_t>(1, std::min<size_t>((size_t)default_wave(H, W), c->budget / 4 / per_item));

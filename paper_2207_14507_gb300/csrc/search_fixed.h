@@ -69,8 +69,7 @@ struct PersistArgs {
 struct FixedShape {
   int W, H;
   std::vector<FixedRow> rows;
-  std::vector<FixedCol> cols;
-  int default_col;           // the column variant of the default tuning
+  std::vector<FixedCol> cols;  // the first is the default tuning's
   int f32_col;               // the one that takes a mode-4 variant's place for FP32 fingerprints
   FixedCol col_fwd, col_inv; // the column pass split for forward units (k_col_fwd_fx, k_col_inv_fx)
   FixedCol col_inv_sep;      // k_col_inv_fx with the fingerprint's strips in their own region (mode 3/4), taken

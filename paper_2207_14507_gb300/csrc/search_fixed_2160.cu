@@ -14,11 +14,9 @@ FixedShape fixed_shape_2160() {
   // prefetch 17.0 / 16.7 (without 19.4 / 18.1), mode 4 with it - / 17.0 (without
   // 18.4); mode 1 20.0 / 18.9; mode 0 22 / 21.  Three stages with the fingerprint by
   // 32-byte TMA rows: 21.9 (FP16).
-  FixedShape s = D::make({D::row<2>(), D::row<1, 4, 4>()},
-                         {D::col<4, 2, 4, 152>(), D::col<4, 2, 2, 152>(), D::col<4, 2, 1>(), D::col<4, 2, 0>()},
-                         {D::col_fwd<4, 2>(), D::col_inv<4, 2>(), D::col_inv<4, 2, 4>()}, D::persist<256, 2, 4>());
-  s.f32_col = s.default_col = 1;
-  return s;
+  return D::make({D::row<2>(), D::row<1, 4, 4>()},
+                 {D::col<4, 2, 2, 152>(), D::col<4, 2, 4, 152>(), D::col<4, 2, 1>(), D::col<4, 2, 0>()},
+                 {D::col_fwd<4, 2>(), D::col_inv<4, 2>(), D::col_inv<4, 2, 4>()}, D::persist<256, 2, 4>());
 }
 
 }  // namespace prnu

@@ -13,12 +13,10 @@ FixedShape fixed_shape_256() {
   // us per candidate: 4-column strips, mode 3 with 12 blocks per SM 0.104 (the
   // default); 8-column strips, mode 1 with 8 blocks 0.109, mode 2 0.109, mode 3 0.110;
   // 16-column strips, mode 2 0.115, mode 3 0.124.
-  FixedShape s = D::make({D::row<8, 6, 6>(), D::row<4>()},
-                         {D::col<16, 4, 2>(), D::col<8, 8, 1>(), D::col<4, 12, 3>()},
-                         {D::col_fwd<16, 4>(), D::col_inv<16, 4>(), D::col_inv<16, 3, 3>()},
-                         D::persist<32, 8, 16>());
-  s.default_col = 2;
-  return s;
+  return D::make({D::row<8, 6, 6>(), D::row<4>()},
+                 {D::col<4, 12, 3>(), D::col<8, 8, 1>(), D::col<16, 4, 2>()},
+                 {D::col_fwd<16, 4>(), D::col_inv<16, 4>(), D::col_inv<16, 3, 3>()},
+                 D::persist<32, 8, 16>());
 }
 
 }  // namespace prnu

@@ -3,11 +3,11 @@
 The column pass multiplies each frame column spectrum by the fingerprint's
 (Eq. 3, the cross-correlation by FFT).  Where the fingerprint strip comes
 from is a launch choice only:
-* mode 2 copies it by TMA into the strip buffer once the last forward stage
+* mode 2 copies it in bulk into the strip buffer once the last forward stage
   has taken its inputs;
 * mode 3 copies it, from the start, into a region of its own;
 * mode 4 does the same with a region sized for FP16 bins.  A wave with an FP32
-  fingerprint then takes the first mode-2/3 variant.
+  fingerprint then takes the size's variant for these (mode 1 or 2).
 
 With the shared forward pass and FP16 fingerprints only, the split inverse
 half runs a mode-4 kernel with more blocks per SM at 720p and 1080p.
@@ -26,7 +26,7 @@ pytestmark = pytest.mark.gpu
 DEV = "cuda:0"
 # (H, W): column variant indices of mode 2 and of mode 3/4 (the registry order
 # of the compile-time-planned kernels)
-MODES = {(256, 256): (0, 2), (720, 1280): (2, 0), (1080, 1920): (1, 0), (2160, 3840): (1, 0)}
+MODES = {(256, 256): (2, 0), (720, 1280): (2, 0), (1080, 1920): (1, 0), (2160, 3840): (0, 1)}
 
 
 @pytest.fixture(scope="module")

@@ -36,6 +36,7 @@ def test_every_row_plan_can_be_set(prnu, H, W):
         h = ctx.prnu_fingerprint_term(torch.from_numpy(wl.fingerprints[0]).to(DEV))
         t = ctx.prnu_get_tuning(H, W)
         assert t["pairs_per_block"] == PLANS[(H, W)][0]
+        assert t["variant"] == 0   # the binding's default argument
         _set(ctx, H, W, t)
         out = []
         for ppb in sorted({*PLANS[(H, W)], 1, 2}):   # 1 and 2 were always taken
