@@ -92,12 +92,15 @@ __device__ __forceinline__ void load_full_bins(float2 (&u)[R], const float2* __r
 }
 
 // Maxima, first arg-maxima and sums of squares of a thread's values of two rows,
-// its positions met in increasing order.
+// its positions met in increasing order.  The squares go to kSums plain FP32
+// sums (at most 8 terms each of the 32 a thread can have), which are joined,
+// and added up over the warp, in compensated FP32.
 struct PairStat {
+  static constexpr int kSums = 4;
   float ma = -INFINITY, mb = -INFINITY;
   int ia = INT_MAX, ib = INT_MAX;
-  float2 sq = make_float2(0.f, 0.f);
-  __device__ __forceinline__ void add(int x, float2 v) {
+  float2 sq[kSums] = {};
+  __device__ __forceinline__ void add(int x, int k, float2 v) {   // the thread's k-th value
     if (v.x > ma) {
       ma = v.x;
       ia = x;
@@ -106,7 +109,7 @@ struct PairStat {
       mb = v.y;
       ib = x;
     }
-    sq = __ffma2_rn(v, v, sq);
+    sq[k % kSums] = __ffma2_rn(v, v, sq[k % kSums]);
   }
   // over the warp
   __device__ __forceinline__ RowRed reduce() {
@@ -115,12 +118,15 @@ struct PairStat {
     const int kb = __reduce_max_sync(0xffffffffu, float_key(mb));
     ia = __reduce_min_sync(0xffffffffu, float_key(ma) == ka ? ia : INT_MAX);
     ib = __reduce_min_sync(0xffffffffu, float_key(mb) == kb ? ib : INT_MAX);
+    float2 s = sq[0], c = make_float2(0.f, 0.f);
+#pragma unroll
+    for (int k = 1; k < kSums; ++k) csum_add2(s, c, sq[k]);
 #pragma unroll
     for (int o = 16; o; o >>= 1) {
-      sq.x += __shfl_xor_sync(0xffffffffu, sq.x, o);
-      sq.y += __shfl_xor_sync(0xffffffffu, sq.y, o);
+      c = __fadd2_rn(c, make_float2(__shfl_xor_sync(0xffffffffu, c.x, o), __shfl_xor_sync(0xffffffffu, c.y, o)));
+      csum_add2(s, c, make_float2(__shfl_xor_sync(0xffffffffu, s.x, o), __shfl_xor_sync(0xffffffffu, s.y, o)));
     }
-    return RowRed{key_float(ka), ia, key_float(kb), ib, sq.x, 0.f, sq.y, 0.f};
+    return RowRed{key_float(ka), ia, key_float(kb), ib, s.x, c.x, s.y, c.y};
   }
 };
 
@@ -217,7 +223,7 @@ __global__ void __launch_bounds__(128, MINB) k_row_inverse2(PassArgs a, float* _
       return;
     }
 #pragma unroll
-    for (int r = 0; r < R; ++r) ps.add(t + r * ra, v[r]);
+    for (int r = 0; r < R; ++r) ps.add(t + r * ra, r, v[r]);
   });
   if (c_out) return;
   const RowRed red = ps.reduce();
@@ -375,7 +381,7 @@ __global__ void __launch_bounds__(kRow3Bound, MINB) k_row_inverse3(PassArgs a, f
       return;
     }
 #pragma unroll
-    for (int r = 0; r < R; ++r) ps.add(x + r * step, u[r]);
+    for (int r = 0; r < R; ++r) ps.add(x + r * step, r, u[r]);
   });
   if (c_out) return;
   const RowRed red = ps.reduce();

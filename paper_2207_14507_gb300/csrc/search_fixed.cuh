@@ -285,7 +285,7 @@ __device__ __forceinline__ void row_inverse_body(const PassArgs& a, int ws, int 
   // maximum is kept without comparing indices
   float ma = -INFINITY, mb = -INFINITY;
   int ia = INT_MAX, ib = INT_MAX;
-  float2 sq = make_float2(0.f, 0.f);
+  float2 sqs[GL::IT] = {};   // a sum per butterfly: at most 16 terms
 #pragma unroll
   for (int r = 0; r < GL::R; ++r) {
 #pragma unroll
@@ -301,9 +301,12 @@ __device__ __forceinline__ void row_inverse_body(const PassArgs& a, int ws, int 
         mb = u.y;
         ib = x;
       }
-      sq = __ffma2_rn(u, u, sq);
+      sqs[it] = __ffma2_rn(u, u, sqs[it]);
     }
   }
+  float2 sq = sqs[0];
+#pragma unroll
+  for (int it = 1; it < GL::IT; ++it) sq = __fadd2_rn(sq, sqs[it]);
   // across the warp: the max by an integer reduction of the order-preserving
   // key, then the least index among the lanes that hold it (across the half
   // warp by shuffles where groups share warps); energies by an FP32 butterfly (warps are combined
