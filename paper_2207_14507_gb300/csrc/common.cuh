@@ -161,6 +161,44 @@ __device__ __forceinline__ void csum_square2(float2& s, float2& c, float2 v) {
   csum_add2(s, c, p);
 }
 
+// Sums over the warp of N values a lane has (N a power of two up to 32), each
+// by the usual butterfly; lane l returns that of value l * N / 32.  A lane
+// hands on the half it does not keep, so N sums take hardly more shuffles than
+// one (N = 8: 9, one: 5).
+template <int N, int O = 16>
+__device__ __forceinline__ float warp_sums(float (&v)[N], int lane) {
+  if constexpr (N == 1) {
+    v[0] += __shfl_xor_sync(0xffffffffu, v[0], O);
+    if constexpr (O > 1) return warp_sums<1, O / 2>(v, lane);
+    return v[0];
+  } else {
+    const bool up = lane & O;
+    float h[N / 2];
+#pragma unroll
+    for (int i = 0; i < N / 2; ++i)
+      h[i] = (up ? v[i + N / 2] : v[i]) + __shfl_xor_sync(0xffffffffu, up ? v[i] : v[i + N / 2], O);
+    if constexpr (O > 1) return warp_sums<N / 2, O / 2>(h, lane);
+    else return h[0];
+  }
+}
+
+// A block's total of N values a thread: FP32 sums of the 32 lanes' values
+// (warp_sums), everything past them in double.  Returned to thread 0 of a
+// block of 8 warps; part: 8 N doubles of shared memory.  Holds a barrier.
+template <int N>
+__device__ __forceinline__ double block_sum(float (&v)[N], int lane, int warp, double* part) {
+  const float s = warp_sums(v, lane);
+  if (lane % (32 / N) == 0) part[warp * N + lane * N / 32] = (double)s;
+  __syncthreads();
+  double t = 0.0;
+  if (warp == 0) {
+    for (int k = lane; k < 8 * N; k += 32) t += part[k];
+#pragma unroll
+    for (int o = 16; o; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+  }
+  return t;
+}
+
 // ---------------------------------------------------------------- storage loads / stores
 
 template <int DT>

@@ -221,7 +221,8 @@ __global__ void __launch_bounds__(kBX * 8) k_resid_apply(const uint8_t* __restri
                                                          int weight, void* __restrict__ out,
                                                          double* __restrict__ partials, float* __restrict__ scale,
                                                          ResidLayout lay, bool vec_out) {
-  __shared__ double part[8];
+  constexpr int NS = RPT < 4 ? RPT : 4;
+  __shared__ double part[MODE == 1 ? 8 * NS : 1];
   __shared__ float2 s_nu2;
   const int f = blockIdx.z, tx = threadIdx.x;
   if (tx == 0 && threadIdx.y == 0) s_nu2 = noise_power(acc[f], H, W);   // once per block: the FP64 pipe is narrow
@@ -229,9 +230,9 @@ __global__ void __launch_bounds__(kBX * 8) k_resid_apply(const uint8_t* __restri
   const float2 nu2 = s_nu2;
   const float s = MODE == 2 ? scale[f] : 1.f;
   const int x = (blockIdx.x * kBX + tx) * kPX, y0 = (blockIdx.y * 8 + threadIdx.y) * RPT;
-  float sq[RPT];
+  float sq[NS];   // of rows k, k + NS
 #pragma unroll
-  for (int k = 0; k < RPT; ++k) sq[k] = 0.f;
+  for (int k = 0; k < NS; ++k) sq[k] = 0.f;
   if (x < W && y0 < H) {
     for_rows<RPT>(FrameRows<VEC>{frames + (size_t)f * H * pitch, pitch, H, W, x, y0},
                        [&](int k, const Row6& p, float2 va, float2 vb, float2 da, float2 db) {
@@ -243,7 +244,7 @@ __global__ void __launch_bounds__(kBX * 8) k_resid_apply(const uint8_t* __restri
                            if (x + 1 >= W) r.y = 0.f;
                            if (x + 2 >= W) r.z = 0.f;
                            if (x + 3 >= W) r.w = 0.f;
-                           sq[k] = fmaf(r.x, r.x, r.y * r.y) + fmaf(r.z, r.z, r.w * r.w);
+                           sq[k % NS] += fmaf(r.x, r.x, r.y * r.y) + fmaf(r.z, r.z, r.w * r.w);
                          } else {
                            if (MODE == 2) r = make_float4(r.x * s, r.y * s, r.z * s, r.w * s);
                            store4<DT>(out, (size_t)f * lay.fpitch + lay.roff + (size_t)(y0 + k) * lay.rpitch + x, r, W - x,
@@ -252,21 +253,10 @@ __global__ void __launch_bounds__(kBX * 8) k_resid_apply(const uint8_t* __restri
                        });
   }
   if (MODE == 0 && scale && blockIdx.x == 0 && blockIdx.y == 0 && tx == 0 && threadIdx.y == 0) scale[f] = 1.f;
-  if (MODE == 1) {   // pairwise over a thread's rows, float within a warp, double across warps and blocks
-#pragma unroll
-    for (int o = RPT / 2; o; o >>= 1)
-#pragma unroll
-      for (int k = 0; k < o; ++k) sq[k] += sq[k + o];
-    float v = sq[0];
-#pragma unroll
-    for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    if (tx == 0) part[threadIdx.y] = (double)v;
-    __syncthreads();
-    if (threadIdx.y == 0 && tx == 0) {
-      double t = 0;
-      for (int k = 0; k < 8; ++k) t += part[k];
+  if constexpr (MODE == 1) {   // float over a warp's 128 pixels of one or two rows, double beyond
+    const double t = block_sum(sq, tx, threadIdx.y, part);
+    if (threadIdx.y == 0 && tx == 0)
       partials[(size_t)f * gridDim.x * gridDim.y + blockIdx.y * gridDim.x + blockIdx.x] = t;
-    }
   }
 }
 
@@ -547,7 +537,7 @@ __global__ void __launch_bounds__(256) k_lit_moments(const uint8_t* __restrict__
                                                      const WorkItem* __restrict__ renders,
                                                      double* __restrict__ partials, float* __restrict__ X) {
   __shared__ __align__(16) float tile[kLTY * kLP];
-  __shared__ double part[8];
+  __shared__ double part[8 * 4];
   const WorkItem it = renders[blockIdx.z];
   const uint8_t* fr = frames + (size_t)it.frame * H * pitch;
   const float cx = 0.5f * (float)(W - 1), cy = 0.5f * (float)(H - 1);
@@ -608,18 +598,12 @@ __global__ void __launch_bounds__(256) k_lit_moments(const uint8_t* __restrict__
       mid = dn;
     }
   }
-  // float within a warp, double across warps and blocks: the FP64 pipe is a
-  // small fraction of the FP32 one, so it takes one add per warp
-  float v = (acc[0].x + acc[1].x) + (acc[0].y + acc[1].y);
-#pragma unroll
-  for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  if (lane == 0) part[wp] = (double)v;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double s = 0.0;
-    for (int k = 0; k < 8; ++k) s += part[k];
+  // float over 128 pixels (4 rows of every other column of the warp's band),
+  // double beyond: the FP64 pipe is a small fraction of the FP32 one
+  float v[4] = {acc[0].x, acc[0].y, acc[1].x, acc[1].y};
+  const double s = block_sum(v, lane, wp, part);
+  if (threadIdx.x == 0)
     partials[(size_t)blockIdx.z * gridDim.x * gridDim.y + blockIdx.y * gridDim.x + blockIdx.x] = s;
-  }
 }
 
 // one block per render: nu2 = (fixed-order sum of the block partials) / (H W)

@@ -307,7 +307,7 @@ __global__ void __launch_bounds__(256) k_wav_synth(const float* __restrict__ D, 
                                                    const float* __restrict__ scale) {
   __shared__ __align__(16) float B[4][kBand][kTS + 4];         // the four bands, coefficient n at n - n0 + 3
   __shared__ __align__(16) float2 T[kTS][2][kTS + 4];          // (row 2i, row 2i + 1) after the column filters
-  __shared__ double part[8];
+  __shared__ double part[OUT == 2 ? kTS : 1];
   const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
   const int n0 = blockIdx.x * kTS, m0 = blockIdx.y * kTS, fl = blockIdx.z, f = f0 + fl;
   const int w2 = w / 2, h2 = h / 2;
@@ -381,11 +381,10 @@ __global__ void __launch_bounds__(256) k_wav_synth(const float* __restrict__ D, 
   const float s = OUT == 3 ? scale[f] : 1.f;
   const bool even_in = ((reinterpret_cast<uintptr_t>(frames) | pitch) & 1) == 0;
   const bool even_out = W % 2 == 0 && reinterpret_cast<uintptr_t>(out) % (DT == kF32 ? 8 : 4) == 0;
-  float sq[kTS / 8];
+  float sq[kTS / 8] = {};   // R^2 over 2 x 2 pixels (OUT 2)
 #pragma unroll
   for (int k = 0; k < kTS / 8; ++k) {
     const int i = wp + 8 * k, y = 2 * (m0 + i);
-    sq[k] = 0.f;
     if (OUT == 0 ? (y >= h || x >= w) : (y >= H || x >= W)) continue;
     float2 a = dup(0.f), b = dup(0.f);
 #pragma unroll
@@ -430,17 +429,9 @@ __global__ void __launch_bounds__(256) k_wav_synth(const float* __restrict__ D, 
       }
     }
   }
-  if (OUT == 2) {   // pairwise in a thread, float within a warp, double across warps and blocks
-    float v = (sq[0] + sq[1]) + (sq[2] + sq[3]);
-#pragma unroll
-    for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    if (lane == 0) part[wp] = (double)v;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      double t = 0.0;
-      for (int k = 0; k < 8; ++k) t += part[k];
-      partials[(size_t)f * gridDim.x * gridDim.y + blockIdx.y * gridDim.x + blockIdx.x] = t;
-    }
+  if constexpr (OUT == 2) {   // float over a warp's two rows of 64 pixels, double beyond
+    const double t = block_sum(sq, lane, wp, part);
+    if (threadIdx.x == 0) partials[(size_t)f * gridDim.x * gridDim.y + blockIdx.y * gridDim.x + blockIdx.x] = t;
   }
 }
 
