@@ -59,6 +59,38 @@ def test_residual_tile_edges(ctx, F, H, W, pad, offset):
             assert np.max(np.abs(got[f] - ref * want)) <= (2.0 ** -11 * 1.01 if norm else 2e-6) * top
 
 
+def _ieee_residual(x, weight):
+    """The residual in IEEE single precision, from the exact integer moments."""
+    H, W = x.shape
+    p = np.pad(x.astype(np.int64), 1, mode="edge")
+    win = [p[dy:dy + H, dx:dx + W] for dy in range(3) for dx in range(3)]
+    s1, s2 = sum(win), sum(w * w for w in win)
+    V, D = 9 * s2 - s1 * s1, 9 * p[1:-1, 1:-1] - s1
+    nu2 = float(V.sum()) / (81.0 * float(H) * float(W))
+    f = np.float32
+    wiener = (V > 0) & (V.astype(f) >= f(81.0 * nu2))
+    num = np.where(wiener, f(9) * D.astype(f) * f(nu2), D.astype(f))
+    w = num / np.where(wiener, V, 9).astype(f)
+    return x.astype(f) * w if weight else w
+
+
+@pytest.mark.parametrize("sigma", [0.4, 1.5, 6.0, 25.0, 100.0])
+def test_residual_has_the_bits_of_ieee_division(ctx, sigma):
+    """W = 9 D nu2 / V or D / 9 by a reciprocal and one correction: the rounded
+    quotient itself, as V is an integer below 1.31e6 (the argument stands at
+    residual_w)."""
+    rng = np.random.default_rng(int(10 * sigma))
+    base = rng.uniform(20, 235, size=(8, 1, 1)) + 40 * np.sin(np.arange(600) / 50)
+    host = np.clip(np.rint(base + sigma * rng.standard_normal((8, 500, 600))), 0, 255).astype(np.uint8)
+    host[0] = rng.choice([0, 255], size=host[0].shape)    # the largest V
+    for weight in (0, 1):
+        out = torch.empty(host.shape, dtype=torch.float32, device=DEV)
+        ctx.prnu_residual(torch.from_numpy(host).to(DEV), out, flags=weight)
+        got = out.cpu().numpy()
+        for f in range(len(host)):
+            np.testing.assert_array_equal(got[f], _ieee_residual(host[f], weight))
+
+
 @pytest.mark.parametrize("L,H,W,pad,offset", [(1, 5, 3, 0, 1), (3, 16, 128, 0, 0), (20, 33, 130, 2, 0), (300, 18, 37, 0, 0)])
 def test_estimate_tile_edges(ctx, L, H, W, pad, offset):
     host, dev = _frames(L, H, W, W + pad, offset, 7 * L + W)
