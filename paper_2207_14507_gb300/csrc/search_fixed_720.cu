@@ -13,11 +13,14 @@ FixedShape fixed_shape_720() {
   // blocks per SM - / 1.33 (5 blocks 1.36), mode 2 with 5 blocks 1.45 / 1.42 (4
   // blocks 1.66 / 1.59), mode 3 with 4 blocks 1.49; 8-column strips, mode 4 with 3
   // blocks - / 1.46, mode 2 1.53, mode 3 1.77, mode 1 1.89.
+  // The persistent launch: three row pairs of 128 threads to a block, 14.8 us a
+  // candidate (FP32 and FP16); 160 threads, two pairs, spills more at 96
+  // registers and takes 18.3 (17.6 with scalar butterflies); 8-column strips 18.5.
   FixedShape s = D::make({D::row<2, 5, 5>(), D::row<4>()},
                          {D::col<4, 6, 4>(), D::col<8, 2, 1>(), D::col<4, 5, 2>(), D::col<8, 2, 0>(), D::col<8, 3, 2>(),
                           D::col<4, 4, 3>()},
                          {D::col_fwd<4, 6>(), D::col_inv<4, 4>(), D::col_inv<4, 4, 3>(), D::col_inv<4, 6, 4>()},
-                         D::persist<160, 2, 4>());
+                         D::persist<128, 3, 4>());
   s.f32_col = 2;
   return s;
 }
