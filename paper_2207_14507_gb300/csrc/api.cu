@@ -359,8 +359,6 @@ void enqueue_search(prnu_ctx* c, const SearchCall& call, prnu_result* d_out, dou
   const int ngroups = ((int)call.group_start.size() - 1) * share;
   const FftPlan prow = make_plan(W, c->tw_off), pcol = make_plan(H, c->tw_off);
   Tuning tn = tuning_for(c, H, W);
-  int rowT, rowMB;
-  row_launch_shape(prow, &rowT, &rowMB);
   // waves hold whole forward units (share items each)
   const int wave = naive ? 1 : std::max(share, std::min(tn.wave, n) / share * share);
   const FixedShape* fs = (!naive && tn.variant >= 0) ? find_fixed(H, W) : nullptr;
@@ -432,9 +430,8 @@ void enqueue_search(prnu_ctx* c, const SearchCall& call, prnu_result* d_out, dou
   a.pcol = pcol;
   a.err = c->d_err;
   a.stall = c->debug_stall;
-  a.pairs_per_block = naive ? 2 : tn.ppb;
+  a.pairs_per_block = tn.ppb;
   a.col_log2 = tn.col_log2;
-  a.row_threads = rowT;
   a.share = share;
   a.units = nullptr;
   a.unit_of = nullptr;
@@ -1156,7 +1153,7 @@ int prnu_residual(prnu_ctx* ctx, const uint8_t* d_frames, int F, int H, int W, s
     float* scale = d_scale;
     if (!scale && (flags & PRNU_NORMALISE))
       scale = reinterpret_cast<float*>(reinterpret_cast<char*>(partials) + ((sizeof(double) * np + 255) & ~(size_t)255));
-    launch_residual(d_frames, F, H, W, pitch, flags, out_dtype, d_out, scale, acc, partials, (int)np, s,
+    launch_residual(d_frames, F, H, W, pitch, flags, out_dtype, d_out, scale, acc, partials, s,
                     ctx->launches);
     PRNU_CUDA_TRY(cudaEventRecord(ctx->last_done, s));
   });
@@ -1250,8 +1247,6 @@ int prnu_fingerprint_term(prnu_ctx* ctx, const float* d_K, int H, int W, int sto
     ensure_buf(ctx, ctx->ws_misc, 2 * nblk * sizeof(double));
     ensure_buf(ctx, ctx->ws_spec, (size_t)H * Wh * sizeof(float2));
     const FftPlan prow = make_plan(W, ctx->tw_off), pcol = make_plan(H, ctx->tw_off);
-    int rowT, rowMB;
-    row_launch_shape(prow, &rowT, &rowMB);
     Tuning tn = tuning_for(ctx, H, W);
     launch_fp_stats(d_K, H, W, reinterpret_cast<double*>(ctx->ws_misc.p), nblk, f->d_scal, f->d_scal + 1,
                     f->d_scal + 2, half, s, ctx->launches);
@@ -1268,7 +1263,6 @@ int prnu_fingerprint_term(prnu_ctx* ctx, const float* d_K, int H, int W, int sto
     a.pcol = pcol;
     a.pairs_per_block = tn.ppb;
     a.col_log2 = tn.col_log2;
-    a.row_threads = rowT;
     launch_row_forward(a, false, f->d_scal, nullptr, s, ctx->launches);
     launch_col(a, 1, half ? nullptr : reinterpret_cast<float2*>(f->d_spec), half ? f->d_spec : nullptr,
                f->d_scal + 1, s, ctx->launches, f->strips);
@@ -1496,8 +1490,6 @@ int pce_score(prnu_ctx* ctx, const float* d_X, uint64_t fp_handle, int H, int W,
                                reinterpret_cast<FpDesc*>(ctx->ws_fpdesc.p));
     PRNU_CUDA_TRY(cudaGetLastError());
     const FftPlan prow = make_plan(W, ctx->tw_off), pcol = make_plan(H, ctx->tw_off);
-    int rowT, rowMB;
-    row_launch_shape(prow, &rowT, &rowMB);
     Tuning tn = tuning_for(ctx, H, W);
     PassArgs a{};
     a.resid = d_X;
@@ -1518,7 +1510,6 @@ int pce_score(prnu_ctx* ctx, const float* d_X, uint64_t fp_handle, int H, int W,
     a.pcol = pcol;
     a.pairs_per_block = tn.ppb;
     a.col_log2 = tn.col_log2;
-    a.row_threads = rowT;
     a.err = ctx->d_err;
     a.stall = ctx->debug_stall;
     a.fp_f32 = fd.dtype == kF32;

@@ -76,7 +76,6 @@ struct PassArgs {
   FftPlan prow, pcol;
   int pairs_per_block;
   int col_log2;               // columns per column-pass block = 1 << col_log2
-  int row_threads;            // threads per row FFT
   // Optional per-slot indirection, used when one wave mixes candidates of
   // several queries (serving): item and result of slot s live at
   // item_ptrs[s] / result_ptrs[s], and frame f's residual at frame_ptrs[f].

@@ -148,7 +148,7 @@ struct ResidLayout {
 };
 // lay == nullptr: dense [F][H][W]
 void launch_residual(const uint8_t* frames, int F, int H, int W, size_t pitch, int flags, int dtype, void* out,
-                     float* scale, unsigned long long* acc, double* partials, int max_partials, cudaStream_t s,
+                     float* scale, unsigned long long* acc, double* partials, cudaStream_t s,
                      LaunchCounter& lc, const ResidLayout* lay = nullptr);
 size_t residual_partials_needed(int F, int H, int W);
 // frame-literal residuals (Sec. 3.2): for render r of renders[nr] (frame

@@ -158,8 +158,6 @@ extern "C" int pce_score_noalloc(const float* d_X, const float* d_K, int H, int 
     k_noalloc_descriptors<<<1, 1, 0, s>>>(it, fd, ditem, dfp);
     PRNU_CUDA_TRY(cudaGetLastError());
 
-    int rowT, rowMB;
-    row_launch_shape(prow, &rowT, &rowMB);
     int lg = 0;
     for (int k = 4; k >= 0; --k)
       if (2 * (size_t)H * (1u << k) * sizeof(float2) <= 112 * 1024) {
@@ -179,9 +177,7 @@ extern "C" int pce_score_noalloc(const float* d_X, const float* d_K, int H, int 
     a.tw = tw;
     a.prow = prow;
     a.pcol = pcol;
-    a.pairs_per_block = 2;
     a.col_log2 = lg;
-    a.row_threads = rowT;
 
     // fingerprint term: spectrum of K - mean(K), FP32.  Its row spectrum goes
     // to specX (free until X's row pass) so that the column pass reads one

@@ -785,7 +785,7 @@ size_t residual_partials_needed(int F, int H, int W) {
 }
 
 void launch_residual(const uint8_t* frames, int F, int H, int W, size_t pitch, int flags, int dtype, void* out,
-                     float* scale, unsigned long long* acc, double* partials, int /*max_partials*/, cudaStream_t s,
+                     float* scale, unsigned long long* acc, double* partials, cudaStream_t s,
                      LaunchCounter& lc, const ResidLayout* lay) {
   const ResidLayout l = lay ? *lay : ResidLayout{W, (size_t)H * W, 0};
   const int rpt = resid_rows(F, H, W);

@@ -106,15 +106,6 @@ __device__ __forceinline__ void csum_add(float& s, float& c, float b) {
   s = t;
   c += e;
 }
-__device__ __forceinline__ void warp_csum(float& s, float& c) {
-#pragma unroll
-  for (int o = 16; o; o >>= 1) {
-    const float s2 = __shfl_xor_sync(0xffffffffu, s, o);
-    const float c2 = __shfl_xor_sync(0xffffffffu, c, o);
-    c += c2;
-    csum_add(s, c, s2);
-  }
-}
 
 // Per-warp partial statistics of a row pair (rows a and b).
 struct RowRed {
@@ -126,18 +117,6 @@ struct RowRed {
 };
 static_assert(sizeof(RowRed) == sizeof(WarpRed), "row reductions share the WarpRed scratch");
 
-// Reduce the per-thread row statistics of a row pair to one RowRed per warp
-// (lane 0 writes red[warp]).  Per thread: FP32 partial over its few elements;
-// across the warp: compensated FP32.
-__device__ __forceinline__ void row_stats_warp(float ma, int ia, float mb, int ib, float sa, float sb, int t,
-                                               RowRed* red) {
-  float ca = 0.f, cb = 0.f;
-  warp_maxarg(ma, ia);
-  warp_maxarg(mb, ib);
-  warp_csum(sa, ca);
-  warp_csum(sb, cb);
-  if ((t & 31) == 0) red[t >> 5] = RowRed{ma, ia, mb, ib, sa, ca, sb, cb};
-}
 // Order-preserving map of a float to a signed int (for max reductions on
 // integer units): x < y  <=>  key(x) < key(y) for non-NaN x, y; -0 and +0 both
 // map to 0, as they compare equal.

@@ -81,9 +81,7 @@ void launch_fixed_wave(const PassArgs& a, const FixedShape& fs, int col_variant,
   if (fs.cols[v].mode == 4 && a.fp_f32) v = fs.f32_col;
   // forward units take the split pass, its inverse half in the mode that is
   // fastest for the wave's fingerprints (the bits are the same in all)
-  const bool sep = fs.col_inv_sep.fn && (fs.col_inv_sep.mode == 3 || !a.fp_f32);
-  const bool sep_h = fs.col_inv_h.fn && !a.fp_f32;
-  const FixedCol& fc = units ? (sep_h ? fs.col_inv_h : sep ? fs.col_inv_sep : fs.col_inv) : fs.cols[v];
+  const FixedCol& fc = units ? (fs.col_inv_h.fn && !a.fp_f32 ? fs.col_inv_h : fs.col_inv) : fs.cols[v];
   const FixedRow& fr = fs.row_for(a.pairs_per_block);
   const int Wh = a.W / 2;
   void* args[] = {const_cast<PassArgs*>(&a)};

@@ -765,11 +765,6 @@ __global__ void __launch_bounds__(RT * PPB, RT * PPB <= 384 ? 2 : 1)
 
 // ---------------------------------------------------------------- registry
 
-template <class K>
-void allow(K k) {
-  allow_max_dynamic_smem(k);
-}
-
 // row pairs of the 11-row window recomputed at once by the finalisation
 constexpr int kFinPairs = 3;
 
@@ -797,7 +792,7 @@ struct ShapeDef {
   static FixedCol col_fwd() {
     return col_entry((void*)k_col_fwd_fx<CP, W, NC, MINB>, NC, 1);
   }
-  template <int NC, int MINB, int MODE = 2>
+  template <int NC, int MINB, int MODE>
   static FixedCol col_inv() {
     return col_entry((void*)k_col_inv_fx<CP, W, NC, MINB, MODE>, NC, MODE);
   }
@@ -861,9 +856,8 @@ struct ShapeDef {
     }
     return f;
   }
-  // split: the forward half, the inverse half (mode 2) and, optionally, the
-  // inverse half with the fingerprint strip in its own region (mode 3/4) and
-  // the one for FP16 fingerprints only (mode 4, more blocks per SM)
+  // split: the forward half, the inverse half and, optionally, the one for FP16
+  // fingerprints only (mode 4)
   static FixedShape make(std::vector<FixedRow> rows, std::vector<FixedCol> cols, std::vector<FixedCol> split,
                          FixedPersist ps) {
     FixedShape s{};
@@ -873,8 +867,7 @@ struct ShapeDef {
     s.cols = std::move(cols);
     s.col_fwd = split.at(0);
     s.col_inv = split.at(1);
-    if (split.size() > 2) s.col_inv_sep = split[2];
-    if (split.size() > 3) s.col_inv_h = split[3];
+    if (split.size() > 2) s.col_inv_h = split[2];
     s.persist = ps;
     return s;
   }

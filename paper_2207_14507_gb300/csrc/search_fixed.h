@@ -72,10 +72,8 @@ struct FixedShape {
   std::vector<FixedCol> cols;  // the first is the default tuning's
   int f32_col;               // the one that takes a mode-4 variant's place for FP32 fingerprints
   FixedCol col_fwd, col_inv; // the column pass split for forward units (k_col_fwd_fx, k_col_inv_fx)
-  FixedCol col_inv_sep;      // k_col_inv_fx with the fingerprint's strips in their own region (mode 3/4), taken
-                             // instead where its mode holds the wave's fingerprints; fn null where none is instantiated
-  FixedCol col_inv_h;        // the same with a region for FP16 bins (mode 4) and more blocks per SM, taken
-                             // instead when every fingerprint of the wave is FP16; fn null where none
+  FixedCol col_inv_h;        // k_col_inv_fx with a fingerprint region for FP16 bins (mode 4), taken instead when
+                             // every fingerprint of the wave is FP16; fn null where none is instantiated
   FixedPersist persist;
   // the row kernels with `ppb` pairs per block, else the first variant (what
   // the default tuning asks row_for(1) for)

@@ -22,7 +22,7 @@ FixedShape fixed_shape_1080() {
   FixedShape s = D::make({D::row<2>(), D::row<1, 8, 8>()},
                          {D::col<4, 4, 4>(), D::col<4, 4, 2>(), D::col<4, 4, 1>(), D::col<4, 3, 0>(), D::col<8, 1, 1>(),
                           D::col<4, 3, 3>()},
-                         {D::col_fwd<4, 4>(), D::col_inv<4, 3>(), D::col_inv<4, 3, 3>(), D::col_inv<4, 4, 4>()},
+                         {D::col_fwd<4, 4>(), D::col_inv<4, 3, 3>(), D::col_inv<4, 4, 4>()},
                          D::persist<128, 3, 4>());
   s.f32_col = 2;
   return s;

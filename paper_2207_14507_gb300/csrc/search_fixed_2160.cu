@@ -16,7 +16,7 @@ FixedShape fixed_shape_2160() {
   // 32-byte TMA rows: 21.9 (FP16).
   return D::make({D::row<2>(), D::row<1, 4, 4>()},
                  {D::col<4, 2, 2, 152>(), D::col<4, 2, 4, 152>(), D::col<4, 2, 1>(), D::col<4, 2, 0>()},
-                 {D::col_fwd<4, 2>(), D::col_inv<4, 2>(), D::col_inv<4, 2, 4>()}, D::persist<256, 2, 4>());
+                 {D::col_fwd<4, 2>(), D::col_inv<4, 2, 2>(), D::col_inv<4, 2, 4>()}, D::persist<256, 2, 4>());
 }
 
 }  // namespace prnu

@@ -19,7 +19,7 @@ FixedShape fixed_shape_720() {
   FixedShape s = D::make({D::row<2, 5, 5>(), D::row<4>()},
                          {D::col<4, 6, 4>(), D::col<8, 2, 1>(), D::col<4, 5, 2>(), D::col<8, 2, 0>(), D::col<8, 3, 2>(),
                           D::col<4, 4, 3>()},
-                         {D::col_fwd<4, 6>(), D::col_inv<4, 4>(), D::col_inv<4, 4, 3>(), D::col_inv<4, 6, 4>()},
+                         {D::col_fwd<4, 6>(), D::col_inv<4, 4, 3>(), D::col_inv<4, 6, 4>()},
                          D::persist<128, 3, 4>());
   s.f32_col = 2;
   return s;

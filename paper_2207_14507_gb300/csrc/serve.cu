@@ -526,7 +526,7 @@ struct Server::Impl {
     const ResidLayout lay = padded_layout(q.H, q.W);
     PRNU_CUDA_TRY(cudaMemsetAsync(q.d_resid, 0, resid_bytes, s_copy));
     launch_residual(frames, q.F, q.H, q.W, pitch, q.flags, q.dtype, q.d_resid, d_scale + q.frame_slot0, q.d_acc,
-                    q.d_partials, (int)residual_partials_needed(q.F, q.H, q.W), s_copy, ctx->launches, &lay);
+                    q.d_partials, s_copy, ctx->launches, &lay);
     k_set_frame_ptrs<<<(q.F + 127) / 128, 128, 0, s_copy>>>(d_frame_ptrs + q.frame_slot0,
                                                             reinterpret_cast<const char*>(q.d_resid), q.F,
                                                             lay.fpitch * elem_size(q.dtype));
@@ -717,8 +717,6 @@ struct Server::Impl {
     const Tuning tn = best->second.front()->tn;
     // the twiddle offsets are fixed when the context is created
     const FftPlan prow = make_plan(W, ctx->tw_off), pcol = make_plan(H, ctx->tw_off);
-    int rowT, rowMB;
-    row_launch_shape(prow, &rowT, &rowMB);
     const int wave = std::max(1, std::min(tn.wave, kMaxWave));
     void** hi = slot.h_tab;
     void** hr = slot.h_tab + kMaxWave;
@@ -778,7 +776,6 @@ struct Server::Impl {
     a.pcol = pcol;
     a.pairs_per_block = tn.ppb;
     a.col_log2 = tn.col_log2;
-    a.row_threads = rowT;
     a.item_ptrs = reinterpret_cast<const WorkItem* const*>(slot.d_tab);
     a.result_ptrs = reinterpret_cast<CandResult* const*>(slot.d_tab + kMaxWave);
     a.frame_ptrs = d_frame_ptrs;

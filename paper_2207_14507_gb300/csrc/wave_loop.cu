@@ -236,8 +236,6 @@ void WaveLoop::rewind(cudaStream_t s) {
 void WaveLoop::capture(cudaGraph_t into, bool units, int items, int nunits) {
   const WaveLoopConfig& c = cfg_;
   const FftPlan prow = make_plan(c.W, ctx_->tw_off), pcol = make_plan(c.H, ctx_->tw_off);
-  int rowT, rowMB;
-  row_launch_shape(prow, &rowT, &rowMB);
   PassArgs a{};
   a.err = c.err;
   a.stall = c.stall;
@@ -259,7 +257,6 @@ void WaveLoop::capture(cudaGraph_t into, bool units, int items, int nunits) {
   a.pcol = pcol;
   a.pairs_per_block = c.ppb;
   a.col_log2 = c.col_log2;
-  a.row_threads = rowT;
   a.item_ptrs = items_;
   a.result_ptrs = results_;
   a.frame_ptrs = c.frame_ptrs;
