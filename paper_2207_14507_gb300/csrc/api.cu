@@ -80,7 +80,7 @@ bool is_5smooth(int n) {
   return n == 1;
 }
 
-FftPlan make_plan_at(int n, int tw_base) {
+FftPlan make_plan(int n) {
   FftPlan p{};
   PRNU_CHECK_ARG(n >= 2 && n <= kMaxFft && is_5smooth(n), "FFT length must be 5-smooth in [2, 4096]");
   std::vector<int> cur, best;
@@ -88,7 +88,7 @@ FftPlan make_plan_at(int n, int tw_base) {
   PRNU_CHECK_ARG(!best.empty() && (int)best.size() <= kMaxStages, "no FFT plan");
   p.n = n;
   p.nstages = (int)best.size();
-  int ns = 1, off = tw_base;
+  int ns = 1, off = 0;
   for (int i = 0; i < p.nstages; ++i) {
     p.radix[i] = best[i];
     p.ns[i] = ns;
@@ -111,13 +111,9 @@ FftPlan make_plan_at(int n, int tw_base) {
   return p;
 }
 
-FftPlan make_plan(int n, const std::vector<int>& tw_offsets) {
-  PRNU_CHECK_ARG(n >= 2 && n <= kMaxFft && tw_offsets[n] >= 0, "no twiddles for this FFT length");
-  return make_plan_at(n, tw_offsets[n]);
-}
-
-// The twiddles of plan p, appended to the table.
-static void append_plan_twiddles(const FftPlan& p, std::vector<float4>& tab) {
+// The twiddles of plan p.
+static std::vector<float4> plan_table(const FftPlan& p) {
+  std::vector<float4> tab;
   std::vector<float2> w(p.n);   // exp(-2 pi i k / n)
   for (int k = 0; k < p.n; ++k) {
     const double a = 2.0 * 3.14159265358979323846 * (double)k / (double)p.n;
@@ -141,7 +137,29 @@ static void append_plan_twiddles(const FftPlan& p, std::vector<float4>& tab) {
   if (p.r3[0]) {
     stage(p.r3[1], p.r3[0]);
     stage(p.r3[2], p.r3[0] * p.r3[1]);
+  }  return tab;
+}
+
+FftPlan plan_for(prnu_ctx* c, int n) {
+  std::lock_guard<std::mutex> lk(c->plan_mu);
+  auto it = c->plans.find(n);
+  if (it != c->plans.end()) return it->second.first;
+  FftPlan p = make_plan(n);
+  const std::vector<float4> tab = plan_table(p);
+  const size_t bytes = tab.size() * sizeof(float4);
+  void* d = ctx_alloc(c, bytes);
+  cudaStream_t s = nullptr;   // of its own: the table is there for every stream on return, and none is waited for
+  cudaError_t e = cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(d, tab.data(), bytes, cudaMemcpyHostToDevice, s);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+  if (s) cudaStreamDestroy(s);
+  if (e != cudaSuccess) {
+    ctx_free(c, d, bytes);
+    throw Error{PRNU_ECUDA, std::string("twiddle table: ") + cudaGetErrorString(e)};
   }
+  p.tab = reinterpret_cast<const float4*>(d);
+  c->plans[n] = {p, bytes};
+  return p;
 }
 
 void row_launch_shape(const FftPlan& p, int* threads, int* maxb) {
@@ -206,7 +224,6 @@ Tuning tuning_for(prnu_ctx* c, int H, int W) {
   auto it = c->tuning.find({H, W});
   if (it != c->tuning.end()) return it->second;
   Tuning t;
-  FftPlan pc = make_plan(H, c->tw_off);
   t.col_log2 = 0;
   for (int lg = 4; lg >= 0; --lg) {
     const size_t sm = 2 * (size_t)H * (1u << lg) * sizeof(float2);
@@ -357,7 +374,7 @@ void enqueue_search(prnu_ctx* c, const SearchCall& call, prnu_result* d_out, dou
   const int n = (int)call.items.size();
   const int share = std::max(call.share, 1);
   const int ngroups = ((int)call.group_start.size() - 1) * share;
-  const FftPlan prow = make_plan(W, c->tw_off), pcol = make_plan(H, c->tw_off);
+  const FftPlan prow = plan_for(c, W), pcol = plan_for(c, H);
   Tuning tn = tuning_for(c, H, W);
   // waves hold whole forward units (share items each)
   const int wave = naive ? 1 : std::max(share, std::min(tn.wave, n) / share * share);
@@ -425,7 +442,6 @@ void enqueue_search(prnu_ctx* c, const SearchCall& call, prnu_result* d_out, dou
   a.results = reinterpret_cast<CandResult*>(c->ws_results.p);
   a.fps = reinterpret_cast<const FpDesc*>(c->ws_fpdesc.p);
   a.scale = call.scale;
-  a.tw = c->d_tw;
   a.prow = prow;
   a.pcol = pcol;
   a.err = c->d_err;
@@ -1067,18 +1083,6 @@ int prnu_create(prnu_ctx** out, int device, size_t hbm_budget_bytes) {
     size_t fr = 0, tot = 0;
     PRNU_CUDA_TRY(cudaMemGetInfo(&fr, &tot));
     c->budget = hbm_budget_bytes ? hbm_budget_bytes : (size_t)(0.9 * (double)fr);
-    // stage twiddles of the plans of every length a side can have
-    c->tw_off.assign(kMaxFft + 1, -1);
-    std::vector<float4> tw;
-    for (int n = 16; n <= kMaxFft; n += 2) {
-      if (!is_5smooth(n)) continue;
-      c->tw_off[n] = (int)tw.size();
-      append_plan_twiddles(make_plan(n, c->tw_off), tw);
-    }
-    const size_t twb = tw.size() * sizeof(float4);
-    c->d_tw = reinterpret_cast<float4*>(ctx_alloc(c.get(), twb));
-    c->tw_bytes = twb;
-    PRNU_CUDA_TRY(cudaMemcpy(c->d_tw, tw.data(), twb, cudaMemcpyHostToDevice));
     PRNU_CUDA_TRY(cudaEventCreateWithFlags(&c->last_done, cudaEventDisableTiming));
     PRNU_CUDA_TRY(cudaEventCreateWithFlags(&c->stage_free, cudaEventDisableTiming));
     PRNU_CUDA_TRY(cudaEventRecord(c->last_done, 0));
@@ -1114,7 +1118,7 @@ int prnu_destroy(prnu_ctx* ctx) {
                          &ctx->ws_lit, &ctx->ws_litx, &ctx->ws_litpart, &ctx->ws_renders, &ctx->ws_resize,
                          &ctx->ws_wav, &ctx->ws_corr})
       ctx_free(ctx, b->p, b->bytes);
-    ctx_free(ctx, ctx->d_tw, ctx->tw_bytes);
+    for (auto& kv : ctx->plans) ctx_free(ctx, const_cast<float4*>(kv.second.first.tab), kv.second.second);
     ctx_free(ctx, ctx->d_err, sizeof(int));
     if (ctx->h_pinned) cudaFreeHost(ctx->h_pinned);
     if (ctx->h_err) cudaFreeHost(ctx->h_err);
@@ -1246,7 +1250,7 @@ int prnu_fingerprint_term(prnu_ctx* ctx, const float* d_K, int H, int W, int sto
     const int nblk = 256;
     ensure_buf(ctx, ctx->ws_misc, 2 * nblk * sizeof(double));
     ensure_buf(ctx, ctx->ws_spec, (size_t)H * Wh * sizeof(float2));
-    const FftPlan prow = make_plan(W, ctx->tw_off), pcol = make_plan(H, ctx->tw_off);
+    const FftPlan prow = plan_for(ctx, W), pcol = plan_for(ctx, H);
     Tuning tn = tuning_for(ctx, H, W);
     launch_fp_stats(d_K, H, W, reinterpret_cast<double*>(ctx->ws_misc.p), nblk, f->d_scal, f->d_scal + 1,
                     f->d_scal + 2, half, s, ctx->launches);
@@ -1258,7 +1262,6 @@ int prnu_fingerprint_term(prnu_ctx* ctx, const float* d_K, int H, int W, int sto
     a.item0 = 0;
     a.nitems = 1;
     a.spec = reinterpret_cast<float2*>(ctx->ws_spec.p);
-    a.tw = ctx->d_tw;
     a.prow = prow;
     a.pcol = pcol;
     a.pairs_per_block = tn.ppb;
@@ -1489,7 +1492,7 @@ int pce_score(prnu_ctx* ctx, const float* d_X, uint64_t fp_handle, int H, int W,
     k_set_pair<<<1, 1, 0, s>>>(it, fd, reinterpret_cast<WorkItem*>(ctx->ws_items.p),
                                reinterpret_cast<FpDesc*>(ctx->ws_fpdesc.p));
     PRNU_CUDA_TRY(cudaGetLastError());
-    const FftPlan prow = make_plan(W, ctx->tw_off), pcol = make_plan(H, ctx->tw_off);
+    const FftPlan prow = plan_for(ctx, W), pcol = plan_for(ctx, H);
     Tuning tn = tuning_for(ctx, H, W);
     PassArgs a{};
     a.resid = d_X;
@@ -1505,7 +1508,6 @@ int pce_score(prnu_ctx* ctx, const float* d_X, uint64_t fp_handle, int H, int W,
     a.stats = reinterpret_cast<RowStat*>(ctx->ws_stats.p);
     a.results = reinterpret_cast<CandResult*>(ctx->ws_results.p);
     a.fps = reinterpret_cast<const FpDesc*>(ctx->ws_fpdesc.p);
-    a.tw = ctx->d_tw;
     a.prow = prow;
     a.pcol = pcol;
     a.pairs_per_block = tn.ppb;

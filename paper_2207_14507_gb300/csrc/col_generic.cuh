@@ -123,7 +123,7 @@ struct Col2 {
       const int step = odd_pitch(ra) * NC;
 #pragma unroll
       for (int r = 0; r < R; ++r) v[r] = src[r * step];
-      plan_twiddles<R, false>(v, j, ra, a.tw + a.pcol.tw_fwd);
+      plan_twiddles<R, false>(v, j, ra, a.pcol.tab + a.pcol.tw_fwd);
       DftP<R, false>::run(v);
     }
     __syncthreads();   // every strip value read
@@ -175,7 +175,7 @@ struct Col2 {
     const int step = odd_pitch(rb) * NC;
 #pragma unroll
     for (int r = 0; r < R; ++r) u[r] = src[r * step];
-    plan_twiddles<R, true>(u, j, rb, a.tw + a.pcol.tw_inv);
+    plan_twiddles<R, true>(u, j, rb, a.pcol.tab + a.pcol.tw_inv);
     DftP<R, true>::run(u);
     if (col >= Wh) return;
     float2* dst = Z + (size_t)j * Wh + col;

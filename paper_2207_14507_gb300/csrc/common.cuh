@@ -72,7 +72,6 @@ struct PassArgs {
   CandResult* results;        // [all items]
   const FpDesc* fps;          // [P]
   const float* scale;         // [F] or nullptr
-  const float4* tw;           // stage twiddles of the runtime plans
   FftPlan prow, pcol;
   int pairs_per_block;
   int col_log2;               // columns per column-pass block = 1 << col_log2

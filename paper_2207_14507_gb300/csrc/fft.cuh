@@ -227,14 +227,15 @@ constexpr int kMaxFft = 4096;
 
 // A length-n plan: radices in execution order; per stage the product of the
 // earlier radices, ceil(2^32 / ns) (j mod ns by one high multiplication, exact
-// for j < 2^16) and the place of its twiddles in the table (fft_plan.cuh), in
-// float4.  ra, rb: where n is the product of two radices that one thread can
+// for j < 2^16) and the place of its twiddles in the plan's table tab
+// (fft_plan.cuh), in float4.  ra, rb: where n is the product of two radices that one thread can
 // hold, the two-stage plan of the column pass (col_generic.cuh), with the
 // twiddles of its second forward and second inverse stage; else 0.  r3: where
 // one thread cannot hold radices of such a plan in few registers, the row
 // passes' three radices (row_generic.cuh), w3 the twiddles of the second and
 // third stage, inv3 the reciprocal of r3[0]; else 0.
 struct FftPlan {
+  const float4* tab;
   int n;
   int nstages;
   int radix[kMaxStages];

@@ -41,10 +41,10 @@ __device__ __forceinline__ void plan_twiddles(float2 (&v)[R], int k, int ns, con
 
 // One stage: butterflies j = t, t + T, ..: inputs ld(i), outputs st(i, v).
 template <int R, bool INV, class Ld, class St>
-__device__ __forceinline__ void plan_stage(const FftPlan& p, int s, const float4* __restrict__ tab, int t, int T, Ld&& ld,
+__device__ __forceinline__ void plan_stage(const FftPlan& p, int s, int t, int T, Ld&& ld,
                                            St&& st) {
   const int nb = p.n / R, ns = p.ns[s];
-  const float4* tw = tab + p.tw[s];
+  const float4* tw = p.tab + p.tw[s];
   for (int j = t; j < nb; j += T) {
     float2 v[R];
 #pragma unroll
@@ -61,20 +61,20 @@ __device__ __forceinline__ void plan_stage(const FftPlan& p, int s, const float4
   }
 }
 template <bool INV, class Ld, class St>
-__device__ __forceinline__ void plan_stage_any(const FftPlan& p, int s, const float4* __restrict__ tab, int t, int T,
+__device__ __forceinline__ void plan_stage_any(const FftPlan& p, int s, int t, int T,
                                                Ld&& ld, St&& st) {
   switch (p.radix[s]) {
-    case 2: plan_stage<2, INV>(p, s, tab, t, T, ld, st); break;
-    case 3: plan_stage<3, INV>(p, s, tab, t, T, ld, st); break;
-    case 4: plan_stage<4, INV>(p, s, tab, t, T, ld, st); break;
-    case 5: plan_stage<5, INV>(p, s, tab, t, T, ld, st); break;
-    case 6: plan_stage<6, INV>(p, s, tab, t, T, ld, st); break;
-    case 8: plan_stage<8, INV>(p, s, tab, t, T, ld, st); break;
-    case 9: plan_stage<9, INV>(p, s, tab, t, T, ld, st); break;
-    case 10: plan_stage<10, INV>(p, s, tab, t, T, ld, st); break;
-    case 12: plan_stage<12, INV>(p, s, tab, t, T, ld, st); break;
-    case 15: plan_stage<15, INV>(p, s, tab, t, T, ld, st); break;
-    default: plan_stage<16, INV>(p, s, tab, t, T, ld, st); break;
+    case 2: plan_stage<2, INV>(p, s, t, T, ld, st); break;
+    case 3: plan_stage<3, INV>(p, s, t, T, ld, st); break;
+    case 4: plan_stage<4, INV>(p, s, t, T, ld, st); break;
+    case 5: plan_stage<5, INV>(p, s, t, T, ld, st); break;
+    case 6: plan_stage<6, INV>(p, s, t, T, ld, st); break;
+    case 8: plan_stage<8, INV>(p, s, t, T, ld, st); break;
+    case 9: plan_stage<9, INV>(p, s, t, T, ld, st); break;
+    case 10: plan_stage<10, INV>(p, s, t, T, ld, st); break;
+    case 12: plan_stage<12, INV>(p, s, t, T, ld, st); break;
+    case 15: plan_stage<15, INV>(p, s, t, T, ld, st); break;
+    default: plan_stage<16, INV>(p, s, t, T, ld, st); break;
   }
 }
 
@@ -83,10 +83,10 @@ __device__ __forceinline__ void plan_stage_any(const FftPlan& p, int s, const fl
 // before the call; the result is in the returned buffer and is visible to the
 // whole block on return.
 template <bool INV>
-__device__ float2* fft_row(float2* a, float2* b, const FftPlan& p, const float4* __restrict__ tab, int t, int T) {
+__device__ float2* fft_row(float2* a, float2* b, const FftPlan& p, int t, int T) {
   for (int s = 0; s < p.nstages; ++s) {
     plan_stage_any<INV>(
-        p, s, tab, t, T, [=](int i) { return a[rpad(i)]; }, [=](int i, float2 v) { b[rpad(i)] = v; });
+        p, s, t, T, [=](int i) { return a[rpad(i)]; }, [=](int i, float2 v) { b[rpad(i)] = v; });
     __syncthreads();
     float2* x = a;
     a = b;
@@ -97,11 +97,11 @@ __device__ float2* fft_row(float2* a, float2* b, const FftPlan& p, const float4*
 
 // The FFTs of the 1 << lg columns in `a` (column layout).
 template <bool INV>
-__device__ float2* fft_col(float2* a, float2* b, const FftPlan& p, const float4* __restrict__ tab, int t, int T, int lg) {
+__device__ float2* fft_col(float2* a, float2* b, const FftPlan& p, int t, int T, int lg) {
   const int c = t & ((1 << lg) - 1);   // T is a multiple of the columns: a thread keeps its column
   for (int s = 0; s < p.nstages; ++s) {
     plan_stage_any<INV>(
-        p, s, tab, t >> lg, T >> lg, [=](int i) { return a[(i << lg) + c]; },
+        p, s, t >> lg, T >> lg, [=](int i) { return a[(i << lg) + c]; },
         [=](int i, float2 v) { b[(i << lg) + c] = v; });
     __syncthreads();
     float2* x = a;

@@ -37,9 +37,10 @@ void set_error(const std::string& msg);
 
 // ---------------------------------------------------------------- plans
 
-// the plan of length n, its twiddles from entry tw_base (tw_offsets[n]) of the table
-FftPlan make_plan_at(int n, int tw_base);
-FftPlan make_plan(int n, const std::vector<int>& tw_offsets);
+// the plan of length n, its table to be set
+FftPlan make_plan(int n);
+// the same with the context's table, made when a length is first asked for
+FftPlan plan_for(prnu_ctx* c, int n);
 // the two-stage plan of length n (col_generic.cuh, row_generic.cuh), false if it has none
 bool col2_radices(int n, int* ra, int* rb);
 // the three-stage row plan of length n (row_generic.cuh), false if it has none
@@ -239,14 +240,13 @@ struct prnu_ctx {
   std::recursive_mutex mu;
   std::map<uint64_t, std::shared_ptr<prnu::Fingerprint>> fps;
   uint64_t next_handle = 1;
-  float4* d_tw = nullptr;
-  std::vector<int> tw_off;   // offset per length, -1 where no side has it
+  std::mutex plan_mu;        // of plans alone (the server's thread asks too)
+  std::map<int, std::pair<prnu::FftPlan, size_t>> plans;   // by length, with the bytes of its table
   prnu::LaunchCounter launches;
   cudaEvent_t last_done = nullptr;
   // call workspace
   prnu::DeviceBuf ws_spec, ws_stats, ws_items, ws_results, ws_groups, ws_out, ws_fpdesc, ws_misc, ws_resid,
       ws_persist, ws_pad, ws_lit, ws_litx, ws_litpart, ws_renders, ws_resize, ws_wav, ws_corr;
-  size_t tw_bytes = 0;
   prnu::CandResult* h_res = nullptr;   // pinned: pce_score's result
   int* h_err = nullptr;           // pinned: error flag of the last persistent launch or TMA wait
   int* d_err = nullptr;           // device flag the wave kernels raise when a bounded wait gives up

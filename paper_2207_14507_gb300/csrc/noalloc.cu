@@ -143,12 +143,13 @@ extern "C" int pce_score_noalloc(const float* d_X, const float* d_K, int H, int 
     float* scal = reinterpret_cast<float*>(base + kOffScal);   // mean, scale, inv_scale
     double* partials = reinterpret_cast<double*>(base + kOffPartials);
 
-    // twiddle tables: length W at tw[0], length H at tw[kTwLen] (the
-    // offsets are set here, not looked up, so H == W needs no special case)
-    const FftPlan prow = make_plan_at(W, 0), pcol = make_plan_at(H, kTwLen);
+    // twiddle tables: length W at tw[0], length H at tw[kTwLen]
+    FftPlan prow = make_plan(W), pcol = make_plan(H);
+    prow.tab = tw;
+    pcol.tab = tw + kTwLen;
     k_noalloc_twiddles<<<8, 256, 0, s>>>(prow, tw);
     PRNU_CUDA_TRY(cudaGetLastError());
-    k_noalloc_twiddles<<<8, 256, 0, s>>>(pcol, tw);
+    k_noalloc_twiddles<<<8, 256, 0, s>>>(pcol, tw + kTwLen);
     PRNU_CUDA_TRY(cudaGetLastError());
 
     WorkItem it{};
@@ -174,7 +175,6 @@ extern "C" int pce_score_noalloc(const float* d_X, const float* d_K, int H, int 
     a.stats = stats;
     a.results = dres;
     a.fps = dfp;
-    a.tw = tw;
     a.prow = prow;
     a.pcol = pcol;
     a.col_log2 = lg;

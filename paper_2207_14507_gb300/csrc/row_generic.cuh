@@ -167,7 +167,7 @@ __global__ void __launch_bounds__(128, MINB) k_row_forward2(PassArgs a, const fl
       const int step = odd_pitch(ra);
 #pragma unroll
       for (int r = 0; r < R; ++r) v[r] = sm[t + r * step];
-      plan_twiddles<R, false>(v, t, ra, a.tw + a.prow.tw_fwd);
+      plan_twiddles<R, false>(v, t, ra, a.prow.tab + a.prow.tw_fwd);
       DftP<R, false>::run(v);
     }
     __syncwarp();
@@ -211,7 +211,7 @@ __global__ void __launch_bounds__(128, MINB) k_row_inverse2(PassArgs a, float* _
     const int step = odd_pitch(ra);
 #pragma unroll
     for (int r = 0; r < R; ++r) v[r] = sm[t + r * step];
-    plan_twiddles<R, true>(v, t, ra, a.tw + a.prow.tw_fwd);
+    plan_twiddles<R, true>(v, t, ra, a.prow.tab + a.prow.tw_fwd);
     DftP<R, true>::run(v);
     if (c_out) {
       float* oa = c_out + (size_t)(2 * pair) * W;
@@ -307,7 +307,7 @@ struct Row3 {
       }
       __syncthreads();
       if (t < r1 * r3) {
-        plan_twiddles<R, INV>(u, k, r1, a.tw + a.prow.w3[0]);
+        plan_twiddles<R, INV>(u, k, r1, a.prow.tab + a.prow.w3[0]);
         DftP<R, INV>::run(u);
         float2* dst = sm + q * row3_pitch(r1, R) + k;
 #pragma unroll
@@ -326,7 +326,7 @@ struct Row3 {
       if (t < nb) {
 #pragma unroll
         for (int r = 0; r < R; ++r) u[r] = sm[t + r * L];
-        plan_twiddles<R, INV>(u, t, nb, a.tw + a.prow.w3[1]);
+        plan_twiddles<R, INV>(u, t, nb, a.prow.tab + a.prow.w3[1]);
         DftP<R, INV>::run(u);
       }
       if (SYNC) __syncthreads();

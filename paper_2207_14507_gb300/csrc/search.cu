@@ -50,7 +50,7 @@ __global__ void __launch_bounds__(512, 2) k_col(PassArgs a, int mode, float2* __
   }
   __syncthreads();
   if (mode == 0 || mode == 1 || mode == 3) {
-    float2* r = fft_col<false>(buf, buf2, a.pcol, a.tw, tid, T, lg);
+    float2* r = fft_col<false>(buf, buf2, a.pcol, tid, T, lg);
     if (r != buf) { buf2 = buf; buf = r; }
   }
   if (mode == 1) {
@@ -93,7 +93,7 @@ __global__ void __launch_bounds__(512, 2) k_col(PassArgs a, int mode, float2* __
     }
     __syncthreads();
   }
-  if (mode == 0 || mode == 4) buf = fft_col<true>(buf, buf2, a.pcol, a.tw, tid, T, lg);
+  if (mode == 0 || mode == 4) buf = fft_col<true>(buf, buf2, a.pcol, tid, T, lg);
   for (int e = tid; e < n; e += T) {
     const int i = e >> lg, col = c0 + (e & (NC - 1));
     if (col < Wh) Z[(size_t)i * Wh + col] = buf[e];
@@ -117,7 +117,7 @@ __device__ void finalize_parts(const PassArgs& a, int s, const FinPeak& pk, int 
     const int p = window_pair(pk.py, b, H);
     build_full_row(bufA, Z + (size_t)(2 * p) * Wh, Z + (size_t)(2 * p + 1) * Wh, W, t, T);
     __syncthreads();
-    const float2* buf = fft_row<true>(bufA, bufB, a.prow, a.tw, t, T);
+    const float2* buf = fft_row<true>(bufA, bufB, a.prow, t, T);
     PairEnergy e;
     for (int x = t; x < W; x += T)
       if (cdist(x, pk.px, W) > kHalfWindow) e.add(buf[rpad(x)]);

@@ -715,8 +715,7 @@ struct Server::Impl {
     const SizeKey key = best->first;
     const int H = key.H, W = key.W;
     const Tuning tn = best->second.front()->tn;
-    // the twiddle offsets are fixed when the context is created
-    const FftPlan prow = make_plan(W, ctx->tw_off), pcol = make_plan(H, ctx->tw_off);
+    const FftPlan prow = plan_for(ctx, W), pcol = plan_for(ctx, H);
     const int wave = std::max(1, std::min(tn.wave, kMaxWave));
     void** hi = slot.h_tab;
     void** hr = slot.h_tab + kMaxWave;
@@ -771,7 +770,6 @@ struct Server::Impl {
     a.stats = ws_stats;
     a.fps = d_fpdesc;
     a.scale = d_scale;
-    a.tw = ctx->d_tw;
     a.prow = prow;
     a.pcol = pcol;
     a.pairs_per_block = tn.ppb;

@@ -235,7 +235,7 @@ void WaveLoop::rewind(cudaStream_t s) {
 // the live counts read on the device.
 void WaveLoop::capture(cudaGraph_t into, bool units, int items, int nunits) {
   const WaveLoopConfig& c = cfg_;
-  const FftPlan prow = make_plan(c.W, ctx_->tw_off), pcol = make_plan(c.H, ctx_->tw_off);
+  const FftPlan prow = plan_for(ctx_, c.W), pcol = plan_for(ctx_, c.H);
   PassArgs a{};
   a.err = c.err;
   a.stall = c.stall;
@@ -252,7 +252,6 @@ void WaveLoop::capture(cudaGraph_t into, bool units, int items, int nunits) {
   a.stats = c.stats;
   a.fps = c.fps;
   a.scale = c.scale;
-  a.tw = ctx_->d_tw;
   a.prow = prow;
   a.pcol = pcol;
   a.pairs_per_block = c.ppb;

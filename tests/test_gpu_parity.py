@@ -387,6 +387,16 @@ def test_constant_frames_score_zero(ctx, prnu):
     assert np.all(res["pce"] == 0.0) and np.all(res["cand_idx"] == 0)
 
 
+def test_twiddles_take_what_the_sizes_in_use_need(prnu):
+    """A budget of 1.25 MB holds a context, its tables and a small frame's
+    search (tables of every length would take twice that)."""
+    g = torch.Generator(device=DEV).manual_seed(3)
+    X, K = torch.randn((2, 64, 96), generator=g, device=DEV)
+    with prnu.Context(0, hbm_budget_bytes=1_250_000) as small, prnu.Context(0) as large:
+        r = [c.pce_score(X, c.prnu_fingerprint_term(K)) for c in (small, large)]
+    assert r[0] == r[1]
+
+
 def test_launch_counter_advances(ctx, prnu):
     n0 = ctx.prnu_launch_count()
     frames = torch.zeros((1, 32, 32), dtype=torch.uint8, device=DEV)
