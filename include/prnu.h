@@ -339,7 +339,7 @@ int pce_score(prnu_ctx* ctx, const float* d_X, uint64_t fp_handle, int H, int W,
  * point needs no context and no fingerprint handle and allocates nothing: it
  * computes the PCE of d_X (device float [H][W]) against the fingerprint d_K
  * (device float [H][W], mean removed inside) in a fixed static device scratch
- * array of about 8.5 MB that every GPU loading the library holds until exit.
+ * array of about 8.7 MB that every GPU loading the library holds until exit.
  *  - H*W must not exceed 2^20 pixels (e.g. 1280x720, 1024x1024), with the
  *    size rule of pce_score; larger frames return PRNU_EINVAL.
  *  - All calls share the scratch array, which keeps the last call's contents;
@@ -392,8 +392,8 @@ int query_latency(prnu_ctx* ctx, uint64_t qid, double* queued_ms, double* total_
 /* Request loop of the server.  PRNU_LOOP_HOST: a host thread forms every
  * wave (its candidate, result and frame tables) and launches its kernels.
  * PRNU_LOOP_DEVICE: for frame sizes with compile-time-planned kernels, the
- * loop runs on the GPU.  One CUDA graph per frame size and storage type
- * repeats, in a WHILE node:
+ * loop runs on the GPU.  One CUDA graph per frame size, residual storage type
+ * and kind of fingerprints (all FP16, or some FP32) repeats, in a WHILE node:
  *  - a scheduler kernel takes the next candidates of the admitted queries
  *    (whole forward units, in admission order) from a host-mapped ring and
  *    builds the wave's tables on the device;
@@ -499,8 +499,8 @@ int prnu_profile_end(prnu_ctx* ctx, prnu_kernel_stat* out, int max, int* n_out);
  * persistent kernel's dependency counts) waits for one arrival more than will
  * ever come: each such wait runs out (about a second), the kernel raises the
  * context's device error flag and abandons its candidate, the results of that
- * call are undefined, and the next search call on the context fails with
- * PRNU_EDEVICE_ABORT.  The context stays usable.  Value 0 turns it off.
+ * call are undefined, and it, or if it was asynchronous the next search or
+ * pce_score on the context, fails with PRNU_EDEVICE_ABORT.  The context stays usable.  Value 0 turns it off.
  * Errors: PRNU_EINVAL (NULL context, unknown key). */
 enum { PRNU_DEBUG_STALL_DEVICE_WAITS = 1 };
 int prnu_debug_set(prnu_ctx* ctx, int key, int value);

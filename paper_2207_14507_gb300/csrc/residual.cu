@@ -24,7 +24,7 @@ namespace {
 // sums as sums over rows (kept for the next row), then over columns.  Against
 // one pixel per thread from a shared-memory tile with 9 integer loads a pixel,
 // 30 full-HD frames to normalised FP16 (three passes, the frames in L2) take
-// 243 us instead of 737; what bounds it is instruction issue (63%),
+// 246 us instead of 737; what bounds it is instruction issue (63%),
 // 34 instructions a pixel and pass.
 constexpr int kBX = 32, kPX = 4;   // lanes of a block's row, pixels of a thread
 constexpr int kMomentFrames = 1024;   // frames of the estimate whose noise powers one launch sums

@@ -11,15 +11,15 @@
 // base plus a multiple of one stride, and no block barrier is needed.  The
 // ping-pong stages that every width took before spent 153 warp instructions a
 // complex point on their indices (58 in the compile-time plans).  Microseconds a
-// candidate (row forward, row inverse): 480 x 640 1.37, 1.20 -> 0.84, 0.53; 540 x
-// 960 2.84, 2.40 -> 1.35, 0.76.
+// candidate (row forward, row inverse): 480 x 640 1.37, 1.20 -> 0.84, 0.54; 540 x
+// 960 2.84, 2.40 -> 1.35, 0.78.
 //
 // Three stages for every other even width: a block per row pair, a thread per
 // butterfly of the stage that has most, in the same manner (Row3, below).  Two stages
 // of radices up to 48 at 168 registers and the ping-pong stages, which took these
 // widths, left too few warps for the gathers of the warp (us a candidate, row
-// forward, row inverse): 900 x 1600 6.13, 3.77 -> 4.47, 2.57; 1440 x 2560 14.0, 11.5 ->
-// 12.0, 7.1; 500 x 4000 11.2, 9.9 -> 8.3, 5.2.  Per pixel the two stages stay ahead
+// forward, row inverse): 900 x 1600 6.13, 3.77 -> 4.47, 2.65; 1440 x 2560 14.0, 11.5 ->
+// 11.9, 7.2; 500 x 4000 11.2, 9.9 -> 8.1, 5.3.  Per pixel the two stages stay ahead
 // where they apply (540 x 960: 2.6, 1.5 us a megapixel against 3.1, 1.8 at 900 x 1600).
 #pragma once
 #include "col_generic.cuh"

@@ -22,7 +22,8 @@
 //  host   : the server thread forms each wave's tables and launches its
 //           kernels;
 //  device : for frame sizes with compile-time-planned kernels, one CUDA graph
-//           per size class holds the whole loop.  A WHILE node repeats a body:
+//           per size class (frame size, storage type, whether a fingerprint
+//           is FP32) holds the whole loop.  A WHILE node repeats a body:
 //           a scheduler kernel takes the next candidates of the ready queries
 //           from a host-mapped ring, builds the wave tables on the device and
 //           picks the branch of a SWITCH node that holds the wave kernels
