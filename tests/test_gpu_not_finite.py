@@ -77,3 +77,37 @@ def test_search_frames_beside_it_keep_their_bits(ctx, H, W, n, persistent, dtype
         ctx.prnu_set_tuning(H, W, t["col_width"], t["pairs_per_block"], t["wave"], t["variant"], t["persistent"])
         for h in hs:
             ctx.prnu_fingerprint_release(h)
+
+
+@pytest.mark.parametrize("loop", ["PRNU_LOOP_HOST", "PRNU_LOOP_DEVICE"])
+@pytest.mark.parametrize("H,W", [(720, 1280), (480, 640)])
+def test_served_beside_a_fingerprint_with_a_nan(prnu, H, W, loop):
+    """Queries of a good and of a NaN fingerprint in shared waves."""
+    g = synth.Grid(0.99, 0.005, 5, -0.5, 0.25, 5)
+    frames = (128 + 20 * _images(H, W, 2)).clamp_(0, 255).to(torch.uint8)
+    K = _images(H, W, 1, 6)[0]
+    bad = K.clone()
+    bad[1, 1] = np.nan
+    with prnu.Context(0) as c:
+        c.prnu_server_set_loop(getattr(prnu, loop))
+        hs = [c.prnu_fingerprint_term(k) for k in (K, bad)]
+        alone = c.query_poll(c.query_submit(frames, hs[:1], g), 2, 1, 60_000_000)
+        ids = [(c.query_submit(frames, f, g), f) for f in (hs[1:], hs[:1], hs[::-1], hs[1:], hs[:1])]
+        out = [c.query_poll(i, 2, len(f), 60_000_000) for i, f in ids]
+    for res, (_, f) in zip(out, ids):
+        for p, h in enumerate(f):
+            for frame in range(2):
+                r = res[frame, p]
+                assert _no_peak(r) if h == hs[1] else r.tobytes() == alone[frame, 0].tobytes()
+
+
+def test_correction_beside_a_frame_with_a_nan(ctx):
+    R = _images(256, 256, 3)
+    h = ctx.prnu_fingerprint_term(_images(256, 256, 1, 6)[0])
+    want, n = ctx.eis_correction(R, [h], max_iter=2, th_half1=5)
+    R[1, 100, 100] = np.inf
+    got, m = ctx.eis_correction(R, [h], max_iter=2, th_half1=5)
+    for f in (0, 2):
+        assert got[f].tobytes() == want[f].tobytes() and m[f] == n[f]
+    assert _no_peak(got[1, 0])
+    ctx.prnu_fingerprint_release(h)
